@@ -35,11 +35,15 @@ struct sv_ctx {
   double2* lam = nullptr;
   double* epart = nullptr;    // kRedBlocks energy partials
   double* scal = nullptr;     // [0] energy
-  // circuit-sized buffers, grown on demand
-  DOp* ops = nullptr;
+  // circuit-sized buffers, grown on demand.  blob holds the staged circuit's records, uploaded
+  // in one copy: ops, fused-pass items and permutation tables.
+  unsigned char* blob = nullptr;
+  size_t blob_cap = 0;
+  DOp* ops = nullptr;         // (in blob)
+  FItem* items = nullptr;     // (in blob) fused-pass items of the staged circuit
   Rot* coef = nullptr;
-  double* contrib = nullptr;
-  size_t ops_cap = 0, coef_cap = 0, contrib_cap = 0;
+  RotT* rt = nullptr;
+  size_t coef_cap = 0, rt_cap = 0;
   double* gpart = nullptr;    // n_ops x kRedBlocks gradient partials
   size_t gpart_cap = 0;
   double* theta = nullptr;
@@ -47,8 +51,6 @@ struct sv_ctx {
   size_t theta_cap = 0, grad_cap = 0;
   double* etraj = nullptr;
   size_t etraj_cap = 0;
-  FItem* items = nullptr;     // fused-pass items of the staged circuit
-  size_t items_cap = 0;
   HostPlan plan;              // fused passes of the staged circuit (empty: per-op kernels)
   // psi checkpoints of commuting layers (sv_set_checkpoint_bytes): the staged circuit's fused
   // passes are planned in chunks, each either a checkpointed layer or a run of other ops
@@ -57,9 +59,8 @@ struct sv_ctx {
   // whole-state diagonal + permutation segments (k_dp.cu) need a third state buffer
   double2* scratch = nullptr;
   bool scratch_failed = false;
-  uint32_t* dp_tab = nullptr;   // permutation tables of the staged segments
-  size_t dp_tab_cap = 0;
-  double2* dp_phase = nullptr;  // their phase tables (written from theta every evaluation)
+  double2* dp_phase = nullptr;  // phase tables of the staged segments (written from theta every
+                                // evaluation)
   size_t dp_phase_cap = 0;
   enum { CH_PASSES = 0, CH_LAYER = 1, CH_DP = 2 };
   struct Chunk {
@@ -234,17 +235,15 @@ sv_status sv_destroy(sv_ctx* c) {
   cudaFree(c->lam);
   cudaFree(c->epart);
   cudaFree(c->scal);
-  cudaFree(c->ops);
+  cudaFree(c->blob);
   cudaFree(c->coef);
-  cudaFree(c->contrib);
+  cudaFree(c->rt);
   cudaFree(c->gpart);
   cudaFree(c->theta);
   cudaFree(c->grad);
   cudaFree(c->etraj);
-  cudaFree(c->items);
   for (double2* p : c->ck) cudaFree(p);
   cudaFree(c->scratch);
-  cudaFree(c->dp_tab);
   cudaFree(c->dp_phase);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   cudaGetLastError();
@@ -435,28 +434,44 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc);
 
 sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune) {
   const size_t n_ops = hc.ops.size();
-  SV_CUDA(grow(c->ops, c->ops_cap, n_ops), c);
   SV_CUDA(grow(c->coef, c->coef_cap, n_ops), c);
-  SV_CUDA(grow(c->contrib, c->contrib_cap, n_ops), c);
+  SV_CUDA(grow(c->rt, c->rt_cap, n_ops), c);
   SV_CUDA(grow(c->gpart, c->gpart_cap, std::max<size_t>(1, n_ops) * kRedBlocks), c);
   SV_CUDA(grow(c->theta, c->theta_cap, (size_t)hc.n_params), c);
   SV_CUDA(grow(c->grad, c->grad_cap, (size_t)hc.n_params), c);
-  if (n_ops)
-    SV_CUDA(cudaMemcpyAsync(c->ops, hc.ops.data(), n_ops * sizeof(DOp), cudaMemcpyHostToDevice,
-                            c->stream), c);
   int m = fused_tile_bits();
   if (may_tune && c->tune && c->n >= kFusedMinQubits && n_ops > 0) m = tune_tile_bits(c, hc);
   if (m <= 0) return SV_ECUDA;
   return plan_circuit(c, hc, m);
 }
 
-// Fused-pass plan of a staged circuit with tiles of tile_bits bits (see stage_circuit).
+static int single_op(const sv_ctx* c, int p);
+
+// Tile size and lowest contiguous bits of the fused passes of a run of ops.  Tiles of tile_bits
+// bits leave a small state in fewer tiles than the 152 SMs, one block each (17 qubits: 64 tiles
+// of 2^11, 24 us per 9-gate pass).  Below 18 qubits a tile of n - 7 bits gives 128 blocks, and
+// fewer contiguous low bits (the state sits in L2, where a 16- or 32-byte access costs no burst)
+// leave its other bits for gate wires: two passes still cover every qubit of a layer.  Runs of
+// gates on many wires (excitations) that the smaller tile would cut into over half as many
+// passes again keep the larger one, a pass costing a few microseconds whatever its tiles.
+static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan& plan) {
+  plan_passes(ops, n, tile_bits, plan);
+  const int m = std::max({n - 7, (n + 1) / 2, 4 + kMinLowBitsL2});  // (a gate has up to 4 wires)
+  if (n > 17 || m >= tile_bits) return;
+  HostPlan small;
+  plan_passes(ops, n, m, small, std::max(0, std::min(kMinLowBitsL2, 2 * m - n)));
+  if (2 * small.passes.size() <= 3 * plan.passes.size()) std::swap(plan, small);
+}
+
+// Fused-pass plan of a staged circuit with tiles of tile_bits bits (see stage_circuit), and its
+// upload.
 static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
   const size_t n_ops = hc.ops.size();
   c->tile_bits = tile_bits;
   c->plan.passes.clear();
   c->plan.items.clear();
   c->chunks.clear();
+  std::vector<uint32_t> tabs;  // permutation tables of the whole-state segments
   if (c->n >= kFusedMinQubits && n_ops > 0) {
     // commuting layers that get a psi checkpoint: as many as the budget (and the device) allow
     std::vector<std::pair<int, int>> layers = commuting_layers(hc.ops, 2);
@@ -483,7 +498,6 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
       }
     }
     const bool use_dp = c->scratch != nullptr && c->n >= kDpMinQubits;
-    std::vector<uint32_t> tabs;
     auto is_diag = [&](int t) { return t == SV_GATE_RZ || t == SV_GATE_CZ; };
     auto is_perm = [&](int t) { return t == SV_GATE_CNOT || t == SV_GATE_X; };
     // a run of RZ/CZ (at most kDpMaxRz / kDpMaxCz) then at least two CNOT/X gates, from l
@@ -506,7 +520,7 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
     auto plan_chunk = [&](int kind, int first, int count, int ckid) {
       const std::vector<DOp> sub(hc.ops.begin() + first, hc.ops.begin() + first + count);
       HostPlan sp;
-      plan_passes(sub, c->n, tile_bits, sp);
+      plan_run(sub, c->n, tile_bits, sp);
       sv_ctx::Chunk ch{};
       ch.kind = kind;
       ch.first = first;
@@ -596,26 +610,50 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
       }
     }
     flush((int)n_ops);
-    SV_CUDA(grow(c->items, c->items_cap, std::max<size_t>(1, c->plan.items.size())), c);
-    if (!c->plan.items.empty())
-      SV_CUDA(cudaMemcpyAsync(c->items, c->plan.items.data(),
-                              c->plan.items.size() * sizeof(FItem), cudaMemcpyHostToDevice,
-                              c->stream), c);
-    const size_t n_dp = tabs.size() / kDpTableWords;
-    if (n_dp) {
-      SV_CUDA(grow(c->dp_tab, c->dp_tab_cap, tabs.size()), c);
-      SV_CUDA(grow(c->dp_phase, c->dp_phase_cap, n_dp * kDpPhaseEntries), c);
-      SV_CUDA(cudaMemcpyAsync(c->dp_tab, tabs.data(), tabs.size() * sizeof(uint32_t),
-                              cudaMemcpyHostToDevice, c->stream), c);
-      for (sv_ctx::Chunk& ch : c->chunks) {
-        if (ch.kind != sv_ctx::CH_DP) continue;
-        DpArgs& d = ch.dp;
-        double2* ph = c->dp_phase + (size_t)ch.ck * kDpPhaseEntries;
-        d.perm = c->dp_tab + (size_t)ch.ck * kDpTableWords;
-        d.phase_lo = d.phase_lo_w = ph;
-        d.phase_b1 = d.phase_b1_w = ph + 2048;
-        d.phase_b2 = d.phase_b2_w = ph + 3072;
-      }
+  }
+  // one upload: ops (with the number of blocks that write each op's gradient shares), items and
+  // permutation tables
+  std::vector<DOp> ops(hc.ops);
+  for (size_t l = 0; l < n_ops; ++l) ops[l].flags = adjoint_blocks(c->n, ops[l]);
+  for (const sv_ctx::Chunk& ch : c->chunks) {
+    if (ch.kind == sv_ctx::CH_DP) {
+      for (int l = ch.first; l < ch.first + ch.count; ++l) ops[l].flags = kRedBlocks;
+      continue;
+    }
+    for (int p = ch.p0; p < ch.p1; ++p) {
+      const FPass& P = c->plan.passes[p];
+      if (ch.kind == sv_ctx::CH_PASSES && single_op(c, p) >= 0) continue;
+      for (int i = P.first_item; i < P.first_item + P.n_items; ++i)
+        for (int g = 0; g < c->plan.items[i].count; ++g)
+          ops[c->plan.items[i].op + g].flags = pass_blocks(P);
+    }
+  }
+  auto align = [](size_t v) { return (v + 255) / 256 * 256; };
+  const size_t o_items = align(n_ops * sizeof(DOp));
+  const size_t o_tabs = align(o_items + c->plan.items.size() * sizeof(FItem));
+  std::vector<unsigned char> blob(o_tabs + tabs.size() * sizeof(uint32_t));
+  if (n_ops) std::memcpy(blob.data(), ops.data(), n_ops * sizeof(DOp));
+  if (!c->plan.items.empty())
+    std::memcpy(blob.data() + o_items, c->plan.items.data(), c->plan.items.size() * sizeof(FItem));
+  if (!tabs.empty())
+    std::memcpy(blob.data() + o_tabs, tabs.data(), tabs.size() * sizeof(uint32_t));
+  SV_CUDA(grow(c->blob, c->blob_cap, blob.size()), c);
+  if (!blob.empty())
+    SV_CUDA(cudaMemcpyAsync(c->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice,
+                            c->stream), c);
+  c->ops = (DOp*)c->blob;
+  c->items = (FItem*)(c->blob + o_items);
+  const size_t n_dp = tabs.size() / kDpTableWords;
+  if (n_dp) {
+    SV_CUDA(grow(c->dp_phase, c->dp_phase_cap, n_dp * kDpPhaseEntries), c);
+    for (sv_ctx::Chunk& ch : c->chunks) {
+      if (ch.kind != sv_ctx::CH_DP) continue;
+      DpArgs& d = ch.dp;
+      double2* ph = c->dp_phase + (size_t)ch.ck * kDpPhaseEntries;
+      d.perm = (const uint32_t*)(c->blob + o_tabs) + (size_t)ch.ck * kDpTableWords;
+      d.phase_lo = d.phase_lo_w = ph;
+      d.phase_b1 = d.phase_b1_w = ph + 2048;
+      d.phase_b2 = d.phase_b2_w = ph + 3072;
     }
   }
   return SV_OK;
@@ -646,7 +684,7 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
                          double2** psi_out) {
   const int n_ops = (int)hc.ops.size();
   *psi_out = c->psi;
-  SV_CUDA(launch_prep_coefs(c->ops, n_ops, theta_dev, c->coef, c->stream), c);
+  SV_CUDA(launch_prep_coefs(c->ops, n_ops, theta_dev, c->coef, c->rt, c->stream), c);
   if (!c->chunks.empty()) {
     double2* psi = c->psi;
     for (const sv_ctx::Chunk& ch : c->chunks) {
@@ -665,7 +703,7 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
         if (op >= 0)
           SV_CUDA(launch_apply_op(psi, c->n, hc.ops[op], c->coef + op, false, c->stream), c);
         else
-          SV_CUDA(launch_fpass(psi, c->plan.passes[p], c->items, c->ops, c->coef, theta_dev,
+          SV_CUDA(launch_fpass(psi, c->plan.passes[p], c->items, c->ops, c->coef, c->rt,
                                c->stream), c);
       }
     }
@@ -783,9 +821,10 @@ sv_status sv_tile_bits(const sv_ctx* c, int32_t* tile_bits) {
 }
 
 // psi = |ref>, forward, lambda = H psi, adjoint sweep; energy -> energy_dev[0], gradient ->
-// grad_dev.  Everything stream-ordered on c->stream.
+// grad_dev; with theta_upd set also the descent step (see launch_finish).  Everything stream-ordered on c->stream.
 sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
-                       const double* theta_dev, double* energy_dev, double* grad_dev) {
+                       const double* theta_dev, double* energy_dev, double* grad_dev,
+                       double* theta_upd, double lr, double* traj) {
   SV_CUDA(launch_init_basis(c->psi, c->n, c->ref, c->stream), c);
   double2* psi = nullptr;
   sv_status st = forward(c, hc, theta_dev, true, &psi);
@@ -793,12 +832,8 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
   double2* lam = psi == c->lam ? c->psi : c->lam;
   SV_CUDA(launch_hpsi(psi, lam, c->n, H->groups, H->n_groups, H->tables, c->epart,
                       c->stream), c);
-  SV_CUDA(launch_sum(c->epart, kRedBlocks, energy_dev, c->stream), c);
   const int n_ops = (int)hc.ops.size();
   if (!c->chunks.empty()) {
-    // passes over fewer tiles than kRedBlocks launch fewer blocks: their other partials are 0
-    SV_CUDA(cudaMemsetAsync(c->gpart, 0, (size_t)std::max(1, n_ops) * kRedBlocks * sizeof(double),
-                            c->stream), c);
     for (int ci = (int)c->chunks.size() - 1; ci >= 0; --ci) {
       const sv_ctx::Chunk& ch = c->chunks[ci];
       if (ch.kind == sv_ctx::CH_PASSES) {
@@ -810,7 +845,7 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
                                       c->stream), c);
           } else {
             SV_CUDA(launch_bpass(psi, lam, c->plan.passes[p], c->items, c->ops, c->coef,
-                                 theta_dev, c->gpart, c->stream), c);
+                                 c->rt, c->gpart, c->stream), c);
           }
         }
       } else if (ch.kind == sv_ctx::CH_LAYER) {
@@ -818,11 +853,10 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
         // end, then the layer un-applied to lambda alone; psi before the layer is the
         // checkpoint itself (the buffer is not needed again in this sweep)
         for (int p = ch.p0; p < ch.p1; ++p)
-          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->items, c->ops, c->gpart,
-                               c->stream), c);
+          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->items, c->gpart, c->stream), c);
         for (int p = ch.p1 - 1; p >= ch.p0; --p)
-          SV_CUDA(launch_fpass_inv(lam, c->plan.passes[p], c->items, c->ops, c->coef,
-                                   theta_dev, c->stream), c);
+          SV_CUDA(launch_fpass_inv(lam, c->plan.passes[p], c->items, c->ops, c->coef, c->rt,
+                                   c->stream), c);
         psi = c->ck[ch.ck];
       } else {
         // diagonal + permutation: psi gathered and un-phased into a free buffer, then lambda
@@ -846,8 +880,8 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
       SV_CUDA(launch_adjoint_op(c->psi, c->lam, c->n, op, c->coef + l, part, c->stream), c);
     }
   }
-  SV_CUDA(launch_reduce_grads(c->ops, n_ops, c->gpart, hc.n_params, c->contrib, grad_dev,
-                              c->stream), c);
+  SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, energy_dev,
+                        theta_upd, lr, traj, c->stream), c);
   return SV_OK;
 }
 
@@ -948,9 +982,9 @@ sv_status svqe::vqe_enqueue(sv_ctx* c, const HostCircuit& hc, const sv_ham* H, c
     SV_CUDA(cudaMemcpyAsync(c->theta, theta_in, hc.n_params * sizeof(double),
                             cudaMemcpyHostToDevice, c->stream), c);
   for (int t = 0; t < n_steps; ++t) {
-    if ((st = adjoint_core(c, hc, H, c->theta, c->scal, c->grad)) != SV_OK) return st;
-    SV_CUDA(launch_gd_update(c->theta, c->grad, hc.n_params, lr, c->scal, c->etraj + t,
-                             c->stream), c);
+    if ((st = adjoint_core(c, hc, H, c->theta, c->scal, c->grad, c->theta, lr, c->etraj + t)) !=
+        SV_OK)
+      return st;
   }
   if (hc.n_params)
     SV_CUDA(cudaMemcpyAsync(theta_out, c->theta, hc.n_params * sizeof(double),

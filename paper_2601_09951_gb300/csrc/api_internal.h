@@ -19,7 +19,8 @@ namespace svqe {
 sv_status stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune = false);
 // psi = |ref>, forward, lambda = H psi, adjoint sweep; stream-ordered.
 sv_status adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
-                       const double* theta_dev, double* energy_dev, double* grad_dev);
+                       const double* theta_dev, double* energy_dev, double* grad_dev,
+                       double* theta_upd = nullptr, double lr = 0.0, double* traj = nullptr);
 // n_steps of gradient descent, enqueued on the context's stream without synchronising:
 // theta_in is read before the call returns; theta_out (n_params) and energy_out (n_steps)
 // are written when the stream reaches them (pinned host memory for real asynchrony).

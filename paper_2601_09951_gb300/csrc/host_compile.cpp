@@ -251,8 +251,8 @@ struct Unit {      // a schedulable unit: one op, or a run of RZ ops (diagonal i
 };
 }  // namespace
 
-void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan) {
-  const int min_low = n <= kL2Qubits ? kMinLowBitsL2 : kMinLowBits;
+void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan, int min_low) {
+  if (min_low < 0) min_low = n <= kL2Qubits ? kMinLowBitsL2 : kMinLowBits;
   plan.passes.clear();
   plan.items.clear();
   std::vector<Unit> units;
@@ -313,6 +313,7 @@ void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan) {
     P.c = c;
     P.first_item = (int)plan.items.size();
     P.n_items = (int)take.size();
+    P.diag = -1;
     int slot = 0;
     for (int u : take) {
       const Unit& U = units[u];
@@ -341,6 +342,7 @@ void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan) {
         L.flip = loc(L.flip);
         it.local = L;
       }
+      if (U.kind == 1) P.diag = (int)plan.items.size() - P.first_item;
       plan.items.push_back(it);
       done[u] = 1;
       --left;

@@ -55,13 +55,14 @@ std::vector<std::pair<int, int>> commuting_layers(const std::vector<DOp>& ops, i
 // move ahead of ops skipped for this pass only if it shares no qubit with them (so it
 // commutes with them).  Runs of >= 3 consecutive RZ gates become one diagonal item (at most
 // one per pass, at most kMaxSlots RZ gates).  A pass holds at most kMaxSlots gradient slots.
-// Every tile includes the kMinLowBits lowest bits (kMinLowBitsL2 for n <= kL2Qubits).
+// Every tile includes the min_low lowest bits; min_low < 0 selects kMinLowBits (kMinLowBitsL2
+// for n <= kL2Qubits).
 constexpr int kMaxSlots = kMaxSlotsDev;
 struct HostPlan {
   std::vector<FPass> passes;
   std::vector<FItem> items;
 };
-void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan);
+void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan, int min_low = -1);
 
 // A Pauli sum grouped by X mask.  Every group's f(k) = sum_t c_t (-i)^{popc(x&z_t)}
 // (-1)^{popc(z_t&k)} is tabulated over the kz bits of the union zu of its z masks, so that

@@ -7,10 +7,18 @@
 //           parameterised item's 2 Im<lambda|G|psi> in a per-thread shared-memory slot (one
 //           DADD per item per tile instead of a warp reduction), un-applies the items to both,
 //           and reduces every slot once at the end into partial[op * kRedBlocks + block] (one
-//           block per tile up to kRedBlocks; the caller zeroes the partials beforehand, so the
-//           entries of blocks a small pass does not launch read as zero).
+//           block per tile up to kRedBlocks).
 // A run of RZ gates is one diagonal phase per amplitude: half tables over the tile's local
 // bits times a per-tile factor for the RZ gates on outer bits.
+//
+// What bounds these kernels is the FP64 pipe (2 FMA/clk/SM), so the RY and RX gates of a pass
+// run without their normalisation: R(phi) = cos phi [[1, -t], [t, 1]] with t = tan phi is two
+// FMAs per real pair where three shears are three, and the product of the cosines multiplies
+// the tile once, when it is stored (RotT; cot and sin where |sin| > |cos|, so every factor
+// dropped lies in [0.707, 1]).  Two such gates on different bits share one trip through shared
+// memory.  The pass's items and coefficients are staged in shared memory by one warp while the
+// tile's loads are in flight: read one at a time from global memory they cost a round trip per
+// gate and tile, which is most of a pass when a state of 2^13 to 2^20 amplitudes sits in L2.
 #include <algorithm>
 
 #include "launch.h"
@@ -25,6 +33,7 @@ constexpr int kFT = 256;  // threads per CTA of the fused kernels
 struct DiagS {
   double2 cs[kMaxSlotsDev];  // (cos phi, sin phi) per RZ gate of the item
   int loc[kMaxSlotsDev];     // local bit, or -1 - global bit for a gate on an outer bit
+  int par[kMaxSlotsDev];     // whether the gate has a gradient
   double2 tl[64];            // phase over local bits [0, hl)
   double2 th[64];            // phase over local bits [hl, m), times the tile's outer factor
   double2 th0[64];           // phase over local bits [hl, m) alone
@@ -55,19 +64,18 @@ __device__ __forceinline__ uint64_t pdep64(uint64_t v, uint64_t m) {
 
 // Per-CTA setup of a diagonal item: cos/sin, local bits and the inner half tables.
 __device__ void diag_setup(DiagS& D, const FPass& P, const FItem& it, const DOp* gops,
-                           const double* theta) {
+                           const RotT* rt) {
   if (threadIdx.x == 0) {
     D.m_rz = it.count;
     D.hl = P.m / 2;
   }
   if ((int)threadIdx.x < it.count) {
-    const DOp op = gops[it.op + threadIdx.x];
-    const double t = op.param >= 0 ? theta[op.param] : op.fixed;
-    double s, c;
-    sincos(0.5 * t, &s, &c);
-    D.cs[threadIdx.x] = make_double2(c, s);
-    const uint64_t b = 1ull << op.bit0;
-    D.loc[threadIdx.x] = (P.tile_mask & b) ? __popcll(P.tile_mask & (b - 1ull)) : -1 - op.bit0;
+    const RotT r = rt[it.op + threadIdx.x];  // (cos, sin) of an RZ gate
+    D.cs[threadIdx.x] = make_double2(r.t, r.c);
+    const int bit0 = gops[it.op + threadIdx.x].bit0;
+    const uint64_t b = 1ull << bit0;
+    D.loc[threadIdx.x] = (P.tile_mask & b) ? __popcll(P.tile_mask & (b - 1ull)) : -1 - bit0;
+    D.par[threadIdx.x] = gops[it.op + threadIdx.x].param >= 0;
   }
   __syncthreads();
   const int hl = D.hl;
@@ -110,48 +118,190 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Tile-local index j -> global amplitude index.
-__device__ __forceinline__ uint64_t gidx(const uint64_t* hoff, uint32_t j, int c,
-                                         uint64_t outer) {
-  return hoff[j >> c] | (uint64_t)(j & ((1u << c) - 1u)) | outer;
+// A thread's amplitudes of a tile are j = tid + i nt, i < 2^m / nt (nt threads, a power of
+// two): the global index of j is g ^ the bits of i, g the spread of tid over the tile's bits and
+// h[q] the global bit of local bit log2(nt) + q.
+struct TileMap {
+  uint32_t g, h[3];
+  int cnt;  // amplitudes per thread (at most 8); 0 for a thread beyond the tile
+};
+
+__device__ __forceinline__ TileMap tile_map(const FPass& P) {
+  TileMap T;
+  const int lt = 31 - __clz((int)blockDim.x);
+  uint32_t m = (uint32_t)P.tile_mask, v = threadIdx.x;
+  T.g = 0;
+  for (int b = 0; b < lt && m; ++b) {
+    const uint32_t low = m & (0u - m);
+    if (v & 1u) T.g |= low;
+    v >>= 1;
+    m &= m - 1u;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    T.h[q] = m & (0u - m);
+    m &= m - 1u;
+  }
+  T.cnt = P.m > lt ? 1 << (P.m - lt) : (threadIdx.x < (1u << P.m) ? 1 : 0);
+  return T;
+}
+__device__ __forceinline__ uint32_t tile_idx(const TileMap& T, int i) {
+  return T.g ^ ((i & 1) ? T.h[0] : 0u) ^ ((i & 2) ? T.h[1] : 0u) ^ ((i & 4) ? T.h[2] : 0u);
 }
 
-__device__ void setup_hoff(uint64_t* hoff, const FPass& P) {
-  const uint64_t hm = P.tile_mask & ~((1ull << P.c) - 1ull);
-  for (int j = threadIdx.x; j < (1 << (P.m - P.c)); j += blockDim.x) hoff[j] = pdep64(j, hm);
-}
-
-enum FKind { F_SWAP = 0, F_H = 1, F_ROTY = 2, F_ROTX = 3, F_ROTZ = 4, F_NEG = 5 };
+enum FKind { F_SWAP = 0, F_H = 1, F_EXC = 2, F_ROTZ = 3, F_NEG = 4, F_RY = 5, F_RX = 6, F_DIAG = 7 };
 
 __device__ __forceinline__ int fkind_of(int type) {
   switch (type) {
     case SV_GATE_H: return F_H;
-    case SV_GATE_RY: case SV_GATE_SINGLE_EXC: case SV_GATE_DOUBLE_EXC: return F_ROTY;
-    case SV_GATE_RX: return F_ROTX;
+    case SV_GATE_RY: return F_RY;
+    case SV_GATE_RX: return F_RX;
+    case SV_GATE_SINGLE_EXC: case SV_GATE_DOUBLE_EXC: return F_EXC;
     case SV_GATE_RZ: return F_ROTZ;
     case SV_GATE_CZ: return F_NEG;
     default: return F_SWAP;
   }
 }
 
-// One pair of one kind with oriented coefficients (the caller takes the inverse).
+// An item as the tile loops read it, in shared memory, its coefficients oriented (inverted for
+// un-applying).
+struct SItem {
+  double p, q;     // RY, RX: p = t (see RotT); the other rotations: lifting coefficients a, b
+  double f;        // factor of the item's gradient sum (see stage_items)
+  uint32_t lo, fl;
+  uint8_t sb[4];
+  int16_t kind, k;
+  int16_t mode, slot;  // RY, RX: RotT::mode; the others: Rot::k
+  int op, count;
+};
+constexpr int kChunk = 32;  // items staged at a time, one lane of the first warp each
+
+// a * b for a value held as an unevaluated sum hi + lo (error about 2^-104).
+__device__ __forceinline__ void dd_mul(double& ah, double& al, double bh, double bl) {
+  const double p = ah * bh;
+  double e = fma(ah, bh, dneg(p));
+  e = fma(ah, bl, e);
+  e = fma(al, bh, e);
+  ah = p + e;
+  al = e - (ah - p);
+}
+
+// Stage items [base, base + cnt) of the pass (cnt <= kChunk), by the first warp.  scale and
+// scale_lo (that warp's lanes) are multiplied by the factors the chunk's RY and RX gates
+// leave out.  With grad set (the backward pass, chunks and items in reverse order) fac is the
+// square of the factors left out by the chunks already un-applied, and item j's sums of
+// lambda psi, taken when the items after it have been un-applied to both, carry their inverse:
+// f is the correction.
+__device__ __forceinline__ void stage_items(SItem* S, const FItem* items, int base, int cnt,
+                                            const Rot* coef, const RotT* rt, bool inv, bool grad,
+                                            double& scale, double& scale_lo, double& fac) {
+  const int lane = threadIdx.x;
+  double c = 1.0, clo = 0.0;
+  SItem o;
+  if (lane < cnt) {
+    const FItem it = items[base + lane];
+    o.lo = (uint32_t)it.local.lo_or;
+    o.fl = (uint32_t)it.local.flip;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) o.sb[b] = it.local.sb[b];
+    o.k = (int16_t)it.local.k;
+    o.slot = (int16_t)it.slot;
+    o.op = it.op;
+    o.count = it.count;
+    o.kind = (int16_t)(it.kind == 1 ? F_DIAG : fkind_of(it.local.type));
+    o.p = o.q = 0.0;
+    o.mode = 0;
+    if (o.kind == F_RY || o.kind == F_RX) {
+      const RotT r = rt[it.op];
+      o.p = inv ? dneg(r.t) : r.t;
+      // the inverse of (t x - y, x + t y) is (t x + y, t y - x), the same factor left out
+      o.mode = (int16_t)(r.mode ? (inv ? 2 : 1) : 0);
+      if (r.mode && inv) o.p = r.t;
+      c = r.c;
+      clo = r.clo;
+    } else if (o.kind == F_EXC || o.kind == F_ROTZ) {
+      Rot r = coef[it.op];
+      if (inv) r = rot_inverse(r);
+      o.p = r.a;
+      o.q = r.b;
+      o.mode = (int16_t)r.k;
+    }
+  }
+  // nothing left out (a chunk of excitations, say): every factor is one
+  const bool none = __ballot_sync(0xffffffffu, c != 1.0) == 0u;
+  if (grad) o.f = fac;
+  if (grad && !none) {
+    // product of c^2 over the items after this one (lanes above), times the earlier chunks'
+    double w = c * c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double v = __shfl_down_sync(0xffffffffu, w, d);
+      if (lane + d < 32) w *= v;
+    }
+    const double nx = __shfl_down_sync(0xffffffffu, w, 1);
+    o.f = fac * (lane == 31 ? 1.0 : nx);
+    fac *= __shfl_sync(0xffffffffu, w, 0);
+  }
+  if (!none) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const double h = __shfl_xor_sync(0xffffffffu, c, d);
+      const double l = __shfl_xor_sync(0xffffffffu, clo, d);
+      dd_mul(c, clo, h, l);
+    }
+    dd_mul(scale, scale_lo, __shfl_sync(0xffffffffu, c, 0), __shfl_sync(0xffffffffu, clo, 0));
+  }
+  if (lane < cnt) S[lane] = o;
+}
+
+// (x, y) <- the rotation without its factor.
+__device__ __forceinline__ void rot_t(int mode, double t, double& x, double& y) {
+  const double u = x, v = y;
+  if (mode == 0) {
+    x = fma(dneg(t), v, u);
+    y = fma(t, u, v);
+  } else if (mode == 1) {
+    x = fma(t, u, dneg(v));
+    y = fma(t, v, u);
+  } else {
+    x = fma(t, u, v);
+    y = fma(t, v, dneg(u));
+  }
+}
+
+template <bool ROTX>
+__device__ __forceinline__ void pair_t(int mode, double t, double2& x, double2& y) {
+  if (ROTX) {
+    // x' = c x - i s y, y' = c y - i s x: R(phi) on (im x, re y), R(-phi) on (re x, im y), the
+    // latter as R(phi) on (im y, re x)
+    rot_t(mode, t, y.y, x.x);
+    rot_t(mode, t, x.y, y.x);
+  } else {
+    rot_t(mode, t, x.x, y.x);
+    rot_t(mode, t, x.y, y.y);
+  }
+}
+
+// One pair of one of the normalised kinds.
 template <int KIND>
-__device__ __forceinline__ void fapply(const Rot& r, double2& x, double2& y) {
+__device__ __forceinline__ void fapply(const SItem& s, double2& x, double2& y) {
   if (KIND == F_SWAP) {
     const double2 t = x; x = y; y = t;
   } else if (KIND == F_H) {
-    pair_apply(SV_GATE_H, r, false, x, y);
-  } else if (KIND == F_ROTY) {
+    pair_apply(SV_GATE_H, Rot{}, false, x, y);
+  } else if (KIND == F_EXC) {
+    const Rot r{s.p, s.q, s.mode, 0};
     rot_apply(r, x.x, y.x);
     rot_apply(r, x.y, y.y);
-  } else if (KIND == F_ROTX) {
-    const Rot m = rot_inverse(r);
-    rot_apply(m, x.x, y.y);
-    rot_apply(r, x.y, y.x);
   } else if (KIND == F_ROTZ) {
+    const Rot r{s.p, s.q, s.mode, 0};
     const Rot m = rot_inverse(r);
     rot_apply(m, x.x, x.y);
     rot_apply(r, y.x, y.y);
+  } else if (KIND == F_RY) {
+    pair_t<false>(s.mode, s.p, x, y);
+  } else if (KIND == F_RX) {
+    pair_t<true>(s.mode, s.p, x, y);
   }
 }
 
@@ -159,7 +309,7 @@ __device__ __forceinline__ void fapply(const Rot& r, double2& x, double2& y) {
 template <int KIND>
 __device__ __forceinline__ void fgrad(const double2& lx, const double2& ly, const double2& px,
                                       const double2& py, double& acc) {
-  if (KIND == F_ROTX) {
+  if (KIND == F_RX) {
     acc = fma(lx.x, py.y, acc);
     acc = fma(dneg(lx.y), py.x, acc);
     acc = fma(ly.x, px.y, acc);
@@ -169,7 +319,7 @@ __device__ __forceinline__ void fgrad(const double2& lx, const double2& ly, cons
     acc = fma(dneg(lx.y), px.x, acc);
     acc = fma(dneg(ly.x), py.y, acc);
     acc = fma(ly.y, py.x, acc);
-  } else if (KIND == F_ROTY) {
+  } else if (KIND == F_RY || KIND == F_EXC) {
     acc = fma(ly.x, px.x, acc);
     acc = fma(ly.y, px.y, acc);
     acc = fma(dneg(lx.x), py.x, acc);
@@ -177,214 +327,350 @@ __device__ __forceinline__ void fgrad(const double2& lx, const double2& ly, cons
   }
 }
 
+__device__ __forceinline__ uint32_t item_index(const SItem& s, uint32_t p) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (t < s.k) {
+      const uint32_t low = p & ((1u << s.sb[t]) - 1u);
+      p = ((p >> s.sb[t]) << (s.sb[t] + 1)) | low;
+    }
+  }
+  return p | s.lo;
+}
+
 template <int KIND>
-__device__ __forceinline__ void tile_op_k(double2* v, uint32_t M, const DOp& op, const Rot& r) {
-  const uint32_t np = M >> op.k;
-  const uint32_t lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
-  for (uint32_t p = threadIdx.x; p < np; p += kFT) {
-    const uint32_t i = (uint32_t)insert_zeros(p, op.sb, op.k) | lo;
+__device__ __forceinline__ void tile_op_k(double2* v, uint32_t M, const SItem& s) {
+  const uint32_t np = M >> s.k, nt = blockDim.x;
+  for (uint32_t p = threadIdx.x; p < np; p += nt) {
+    const uint32_t i = item_index(s, p);
     if (KIND == F_NEG) {
       v[i] = make_double2(dneg(v[i].x), dneg(v[i].y));
     } else {
-      double2 x = v[i], y = v[i ^ fl];
-      fapply<KIND>(r, x, y);
+      double2 x = v[i], y = v[i ^ s.fl];
+      fapply<KIND>(s, x, y);
       v[i] = x;
-      v[i ^ fl] = y;
+      v[i ^ s.fl] = y;
     }
   }
 }
 
-__device__ __forceinline__ void tile_op(double2* v, uint32_t M, const DOp& op, const Rot& rf,
-                                        bool inv) {
-  const Rot r = inv ? rot_inverse(rf) : rf;
-  switch (fkind_of(op.type)) {
-    case F_SWAP: tile_op_k<F_SWAP>(v, M, op, r); break;
-    case F_H: tile_op_k<F_H>(v, M, op, r); break;
-    case F_ROTY: tile_op_k<F_ROTY>(v, M, op, r); break;
-    case F_ROTX: tile_op_k<F_ROTX>(v, M, op, r); break;
-    case F_ROTZ: tile_op_k<F_ROTZ>(v, M, op, r); break;
-    default: tile_op_k<F_NEG>(v, M, op, r); break;
+__device__ __forceinline__ void tile_op(double2* v, uint32_t M, const SItem& s) {
+  switch (s.kind) {
+    case F_SWAP: tile_op_k<F_SWAP>(v, M, s); break;
+    case F_H: tile_op_k<F_H>(v, M, s); break;
+    case F_EXC: tile_op_k<F_EXC>(v, M, s); break;
+    case F_ROTZ: tile_op_k<F_ROTZ>(v, M, s); break;
+    case F_RY: tile_op_k<F_RY>(v, M, s); break;
+    case F_RX: tile_op_k<F_RX>(v, M, s); break;
+    default: tile_op_k<F_NEG>(v, M, s); break;
   }
 }
 
-// Adjoint step of one op on the psi and lambda tiles: gradient share into acc (if grad), then
-// un-apply to both.
+// The four amplitudes of a block on two single-bit items: i, i | f0, i | f1, i | f0 | f1.
+__device__ __forceinline__ uint32_t quad_index(uint32_t f0, uint32_t f1, uint32_t p) {
+  const uint32_t l0 = min(f0, f1) - 1u, l1 = max(f0, f1) - 1u;
+  p = ((p & ~l0) << 1) | (p & l0);
+  return ((p & ~l1) << 1) | (p & l1);
+}
+
+// Two RY (or RX) gates on different bits in one trip, s0 first.
+template <bool ROTX>
+__device__ __forceinline__ void tile_op2(double2* v, uint32_t M, const SItem& s0,
+                                         const SItem& s1) {
+  const uint32_t f0 = s0.fl, f1 = s1.fl, nt = blockDim.x;
+  const int m0 = s0.mode, m1 = s1.mode;
+  const double t0 = s0.p, t1 = s1.p;
+  for (uint32_t p = threadIdx.x; p < (M >> 2); p += nt) {
+    const uint32_t i = quad_index(f0, f1, p);
+    double2 a = v[i], b = v[i | f0], c = v[i | f1], d = v[i | f0 | f1];
+    pair_t<ROTX>(m0, t0, a, b);
+    pair_t<ROTX>(m0, t0, c, d);
+    pair_t<ROTX>(m1, t1, a, c);
+    pair_t<ROTX>(m1, t1, b, d);
+    v[i] = a;
+    v[i | f0] = b;
+    v[i | f1] = c;
+    v[i | f0 | f1] = d;
+  }
+}
+
+// Adjoint step of one item on the psi and lambda tiles: gradient share into acc, then un-apply
+// to both.
 template <int KIND>
-__device__ __forceinline__ void tile_adj_k(double2* tp, double2* tl, uint32_t M, const DOp& op,
-                                           const Rot& ri, bool grad, double& acc) {
-  const uint32_t np = M >> op.k;
-  const uint32_t lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
-  for (uint32_t p = threadIdx.x; p < np; p += kFT) {
-    const uint32_t a = (uint32_t)insert_zeros(p, op.sb, op.k) | lo;
+__device__ __forceinline__ void tile_adj_k(double2* tp, double2* tl, uint32_t M, const SItem& s,
+                                           double& acc) {
+  const uint32_t np = M >> s.k, nt = blockDim.x;
+  const bool grad = s.slot >= 0;
+  for (uint32_t p = threadIdx.x; p < np; p += nt) {
+    const uint32_t a = item_index(s, p);
     if (KIND == F_NEG) {
       tp[a] = make_double2(dneg(tp[a].x), dneg(tp[a].y));
       tl[a] = make_double2(dneg(tl[a].x), dneg(tl[a].y));
     } else {
-      double2 px = tp[a], py = tp[a ^ fl], lx = tl[a], ly = tl[a ^ fl];
+      const uint32_t b = a ^ s.fl;
+      double2 px = tp[a], py = tp[b], lx = tl[a], ly = tl[b];
       if (grad) fgrad<KIND>(lx, ly, px, py, acc);
-      fapply<KIND>(ri, px, py);
-      fapply<KIND>(ri, lx, ly);
+      fapply<KIND>(s, px, py);
+      fapply<KIND>(s, lx, ly);
       tp[a] = px;
-      tp[a ^ fl] = py;
+      tp[b] = py;
       tl[a] = lx;
-      tl[a ^ fl] = ly;
+      tl[b] = ly;
     }
   }
+}
+
+// The same for two RY (or RX) gates on different bits, s0 un-applied first.
+template <bool ROTX>
+__device__ __forceinline__ void tile_adj2(double2* tp, double2* tl, uint32_t M, const SItem& s0,
+                                          const SItem& s1, double& acc0, double& acc1) {
+  constexpr int KIND = ROTX ? F_RX : F_RY;
+  const uint32_t f0 = s0.fl, f1 = s1.fl, nt = blockDim.x;
+  const int m0 = s0.mode, m1 = s1.mode;
+  const double t0 = s0.p, t1 = s1.p;
+  const bool g0 = s0.slot >= 0, g1 = s1.slot >= 0;
+  for (uint32_t p = threadIdx.x; p < (M >> 2); p += nt) {
+    const uint32_t i = quad_index(f0, f1, p), j = i | f0, k = i | f1, l = j | f1;
+    double2 pa = tp[i], pb = tp[j], pc = tp[k], pd = tp[l];
+    double2 la = tl[i], lb = tl[j], lc = tl[k], ld = tl[l];
+    if (g0) {
+      fgrad<KIND>(la, lb, pa, pb, acc0);
+      fgrad<KIND>(lc, ld, pc, pd, acc0);
+    }
+    pair_t<ROTX>(m0, t0, pa, pb);
+    pair_t<ROTX>(m0, t0, pc, pd);
+    pair_t<ROTX>(m0, t0, la, lb);
+    pair_t<ROTX>(m0, t0, lc, ld);
+    if (g1) {
+      fgrad<KIND>(la, lc, pa, pc, acc1);
+      fgrad<KIND>(lb, ld, pb, pd, acc1);
+    }
+    pair_t<ROTX>(m1, t1, pa, pc);
+    pair_t<ROTX>(m1, t1, pb, pd);
+    pair_t<ROTX>(m1, t1, la, lc);
+    pair_t<ROTX>(m1, t1, lb, ld);
+    tp[i] = pa;
+    tp[j] = pb;
+    tp[k] = pc;
+    tp[l] = pd;
+    tl[i] = la;
+    tl[j] = lb;
+    tl[k] = lc;
+    tl[l] = ld;
+  }
+}
+
+// Whether items a and b (in processing order) share a trip.
+__device__ __forceinline__ bool can_pair(const SItem& a, const SItem& b) {
+  return a.kind == b.kind && (a.kind == F_RY || a.kind == F_RX) && a.fl != b.fl;
 }
 
 // INV: apply the pass's items inverted, in reverse order (un-applying the pass).
 template <bool INV>
-__global__ void __launch_bounds__(kFT) k_fpass(double2* __restrict__ psi, FPass P,
+__global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPass P,
                                                const FItem* __restrict__ items,
                                                const DOp* __restrict__ gops,
                                                const Rot* __restrict__ coef,
-                                               const double* __restrict__ theta) {
+                                               const RotT* __restrict__ rt) {
   extern __shared__ double2 tile[];
-  __shared__ uint64_t hoff[1 << (11 - kMinLowBitsL2)];
   __shared__ DiagS D;
-  const uint32_t M = 1u << P.m;
+  __shared__ SItem its[kChunk];
+  __shared__ double s_scale;
+  const uint32_t M = 1u << P.m, nt = blockDim.x;
   const uint64_t ntiles = 1ull << __popcll(P.outer_mask);
-  int diag = -1;
-  for (int i = 0; i < P.n_items; ++i)
-    if (items[P.first_item + i].kind == 1) diag = i;
-  setup_hoff(hoff, P);
-  if (diag >= 0) diag_setup(D, P, items[P.first_item + diag], gops, theta);
-  __syncthreads();
+  const int nch = (P.n_items + kChunk - 1) / kChunk;
+  const TileMap T = tile_map(P);
+  items += P.first_item;
+  bool staged = false;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint64_t outer = pdep64(t, P.outer_mask);
-    for (uint32_t j = threadIdx.x; j < M; j += kFT)
-      cp_async16(&tile[j], &psi[gidx(hoff, j, P.c, outer)]);
-    cp_async_wait_all();
-    if (diag >= 0) diag_tile(D, P, outer);
-    __syncthreads();
-    for (int ii = 0; ii < P.n_items; ++ii) {
-      const int i = INV ? P.n_items - 1 - ii : ii;
-      const FItem it = items[P.first_item + i];
-      if (it.kind == 0) {
-        tile_op(tile, M, it.local, coef[it.op], INV);
-      } else if (INV) {
-        for (uint32_t j = threadIdx.x; j < M; j += kFT)
-          tile[j] = cmul_conj(tile[j], diag_phase(D, j));
-      } else {
-        for (uint32_t j = threadIdx.x; j < M; j += kFT) tile[j] = cmul(tile[j], diag_phase(D, j));
-      }
-      __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < T.cnt) cp_async16(&tile[threadIdx.x + i * nt], &psi[outer | tile_idx(T, i)]);
+    if (P.diag >= 0) {
+      if (!staged) diag_setup(D, P, items[P.diag], gops, rt);
+      diag_tile(D, P, outer);
     }
-    for (uint32_t j = threadIdx.x; j < M; j += kFT) psi[gidx(hoff, j, P.c, outer)] = tile[j];
+    double sc = 1.0, sc_lo = 0.0, fac = 1.0;
+    for (int ch = 0; ch < nch; ++ch) {
+      const int base = (INV ? nch - 1 - ch : ch) * kChunk;
+      const int cnt = min(kChunk, P.n_items - base);
+      if (!staged || nch > 1) {
+        if (threadIdx.x < 32) {
+          stage_items(its, items, base, cnt, coef, rt, INV, false, sc, sc_lo, fac);
+          if (ch == nch - 1 && threadIdx.x == 0) s_scale = sc;
+        }
+      }
+      if (ch == 0) cp_async_wait_all();
+      __syncthreads();
+      for (int ii = 0; ii < cnt;) {
+        const int i = INV ? cnt - 1 - ii : ii;
+        const SItem& s = its[i];
+        if (s.kind == F_DIAG) {
+          if (INV) {
+            for (uint32_t j = threadIdx.x; j < M; j += nt)
+              tile[j] = cmul_conj(tile[j], diag_phase(D, j));
+          } else {
+            for (uint32_t j = threadIdx.x; j < M; j += nt)
+              tile[j] = cmul(tile[j], diag_phase(D, j));
+          }
+          ++ii;
+        } else if (ii + 1 < cnt && can_pair(s, its[INV ? i - 1 : i + 1])) {
+          const SItem& s1 = its[INV ? i - 1 : i + 1];
+          if (s.kind == F_RX) tile_op2<true>(tile, M, s, s1);
+          else tile_op2<false>(tile, M, s, s1);
+          ii += 2;
+        } else {
+          tile_op(tile, M, s);
+          ++ii;
+        }
+        __syncthreads();
+      }
+    }
+    staged = true;
+    const double f = s_scale;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < T.cnt) {
+        const double2 v = tile[threadIdx.x + i * nt];
+        psi[outer | tile_idx(T, i)] = f == 1.0 ? v : make_double2(f * v.x, f * v.y);
+      }
     __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(kFT) k_bpass(double2* __restrict__ psi,
+__global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
                                                double2* __restrict__ lam, FPass P,
                                                const FItem* __restrict__ items,
                                                const DOp* __restrict__ gops,
                                                const Rot* __restrict__ coef,
-                                               const double* __restrict__ theta,
+                                               const RotT* __restrict__ rt,
                                                double* __restrict__ partial) {
   extern __shared__ double2 smem[];
-  __shared__ uint64_t hoff[1 << (11 - kMinLowBitsL2)];
   __shared__ DiagS D;
-  __shared__ double red[kFT / 32];
-  const uint32_t M = 1u << P.m;
+  __shared__ SItem its[kChunk];
+  __shared__ double s_scale;
+  __shared__ int s_op[kMaxSlotsDev];      // op and gradient factor of each slot
+  __shared__ double s_fac[kMaxSlotsDev];
+  const uint32_t M = 1u << P.m, nt = blockDim.x;
   double2* tp = smem;
   double2* tlam = smem + M;
-  double* accp = (double*)(smem + 2 * M);  // [n_slots][kFT]
+  double* accp = (double*)(smem + 2 * M);  // [n_slots][nt]
   const uint64_t ntiles = 1ull << __popcll(P.outer_mask);
-  const int tid = threadIdx.x;
-  int diag = -1;
-  for (int i = 0; i < P.n_items; ++i)
-    if (items[P.first_item + i].kind == 1) diag = i;
-  for (int s = 0; s < P.n_slots; ++s) accp[s * kFT + tid] = 0.0;
-  setup_hoff(hoff, P);
-  if (diag >= 0) diag_setup(D, P, items[P.first_item + diag], gops, theta);
-  __syncthreads();
+  const int tid = threadIdx.x, lt = 31 - __clz((int)nt);
+  const int nch = (P.n_items + kChunk - 1) / kChunk;
+  const TileMap T = tile_map(P);
+  items += P.first_item;
+  for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
+  bool staged = false;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint64_t outer = pdep64(t, P.outer_mask);
-    for (uint32_t j = tid; j < M; j += kFT) {
-      const uint64_t k = gidx(hoff, j, P.c, outer);
-      cp_async16(&tp[j], &psi[k]);
-      cp_async16(&tlam[j], &lam[k]);
-    }
-    cp_async_wait_all();
-    if (diag >= 0) diag_tile(D, P, outer);
-    __syncthreads();
-    for (int i = P.n_items - 1; i >= 0; --i) {
-      const FItem it = items[P.first_item + i];
-      if (it.kind == 0) {
-        const DOp& op = it.local;
-        const Rot ri = rot_inverse(coef[it.op]);
-        const bool gr = it.slot >= 0;
-        double acc = 0.0;
-        switch (fkind_of(op.type)) {
-          case F_SWAP: tile_adj_k<F_SWAP>(tp, tlam, M, op, ri, false, acc); break;
-          case F_H: tile_adj_k<F_H>(tp, tlam, M, op, ri, false, acc); break;
-          case F_ROTY: tile_adj_k<F_ROTY>(tp, tlam, M, op, ri, gr, acc); break;
-          case F_ROTX: tile_adj_k<F_ROTX>(tp, tlam, M, op, ri, gr, acc); break;
-          case F_ROTZ: tile_adj_k<F_ROTZ>(tp, tlam, M, op, ri, gr, acc); break;
-          default: tile_adj_k<F_NEG>(tp, tlam, M, op, ri, false, acc); break;
-        }
-        if (gr) accp[it.slot * kFT + tid] += acc;
-      } else {
-        // gradients of the RZ gates: 2 Im<lambda|Z_q/2|psi> = sum_k s_q(k) Im(conj(l_k) p_k)
-        double W = 0.0;
-        double hi[3] = {0.0, 0.0, 0.0};  // RZ gates on local bits 8..10 (vary within a thread)
-        for (uint32_t j = tid; j < M; j += kFT) {
-          const double2 pk = tp[j], lk = tlam[j];
-          const double w = fma(lk.x, pk.y, dneg(lk.y) * pk.x);
-          W += w;
 #pragma unroll
-          for (int q = 0; q < 3; ++q) hi[q] += ((j >> (8 + q)) & 1u) ? dneg(w) : w;
-          const double2 ph = diag_phase(D, j);
-          tp[j] = cmul_conj(pk, ph);
-          tlam[j] = cmul_conj(lk, ph);
-        }
-        int s = it.slot;
-        for (int g = 0; g < it.count; ++g) {
-          const DOp op = gops[it.op + g];
-          if (op.param < 0) continue;
-          const int lb = D.loc[g];
-          double v;
-          if (lb < 0) {
-            v = ((outer >> (-1 - lb)) & 1ull) ? dneg(W) : W;
-          } else if (lb < 8) {
-            v = ((tid >> lb) & 1) ? dneg(W) : W;
-          } else {
-            v = lb == 8 ? hi[0] : lb == 9 ? hi[1] : hi[2];
+    for (int i = 0; i < 8; ++i)
+      if (i < T.cnt) {
+        const uint64_t k = outer | tile_idx(T, i);
+        cp_async16(&tp[tid + i * nt], &psi[k]);
+        cp_async16(&tlam[tid + i * nt], &lam[k]);
+      }
+    if (P.diag >= 0) {
+      if (!staged) diag_setup(D, P, items[P.diag], gops, rt);
+      diag_tile(D, P, outer);
+    }
+    double sc = 1.0, sc_lo = 0.0, fac = 1.0;
+    for (int ch = nch - 1; ch >= 0; --ch) {
+      const int base = ch * kChunk;
+      const int cnt = min(kChunk, P.n_items - base);
+      if (!staged || nch > 1) {
+        if (tid < 32) {
+          stage_items(its, items, base, cnt, coef, rt, true, true, sc, sc_lo, fac);
+          if (!staged && tid < cnt && its[tid].slot >= 0 && its[tid].kind != F_DIAG) {
+            s_op[its[tid].slot] = its[tid].op;
+            s_fac[its[tid].slot] = its[tid].f;
           }
-          accp[s * kFT + tid] += v;
-          ++s;
+          if (ch == 0 && tid == 0) s_scale = sc;
         }
       }
+      if (ch == nch - 1) cp_async_wait_all();
       __syncthreads();
+      for (int i = cnt - 1; i >= 0;) {
+        const SItem& s = its[i];
+        if (s.kind == F_DIAG) {
+          // gradients of the RZ gates: 2 Im<lambda|Z_q/2|psi> = sum_k s_q(k) Im(conj(l_k) p_k)
+          double W = 0.0;
+          double hi[3] = {0.0, 0.0, 0.0};  // RZ gates on local bits that vary within a thread
+          for (uint32_t j = tid; j < M; j += nt) {
+            const double2 pk = tp[j], lk = tlam[j];
+            const double w = fma(lk.x, pk.y, dneg(lk.y) * pk.x);
+            W += w;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) hi[q] += ((j >> (lt + q)) & 1u) ? dneg(w) : w;
+            const double2 ph = diag_phase(D, j);
+            tp[j] = cmul_conj(pk, ph);
+            tlam[j] = cmul_conj(lk, ph);
+          }
+          int sl = s.slot;
+          for (int g = 0; g < s.count; ++g) {
+            if (!D.par[g]) continue;
+            const int lb = D.loc[g];
+            double v;
+            if (lb < 0) {
+              v = ((outer >> (-1 - lb)) & 1ull) ? dneg(W) : W;
+            } else if (lb < lt) {
+              v = ((tid >> lb) & 1) ? dneg(W) : W;
+            } else {
+              v = lb == lt ? hi[0] : lb == lt + 1 ? hi[1] : hi[2];
+            }
+            accp[sl * nt + tid] += v;
+            if (!staged && tid == 0) {
+              s_op[sl] = s.op + g;
+              s_fac[sl] = s.f;
+            }
+            ++sl;
+          }
+          --i;
+        } else if (i > 0 && can_pair(s, its[i - 1])) {
+          const SItem& s1 = its[i - 1];
+          double a0 = 0.0, a1 = 0.0;
+          if (s.kind == F_RX) tile_adj2<true>(tp, tlam, M, s, s1, a0, a1);
+          else tile_adj2<false>(tp, tlam, M, s, s1, a0, a1);
+          if (s.slot >= 0) accp[s.slot * nt + tid] += a0;
+          if (s1.slot >= 0) accp[s1.slot * nt + tid] += a1;
+          i -= 2;
+        } else {
+          double acc = 0.0;
+          switch (s.kind) {
+            case F_SWAP: tile_adj_k<F_SWAP>(tp, tlam, M, s, acc); break;
+            case F_H: tile_adj_k<F_H>(tp, tlam, M, s, acc); break;
+            case F_EXC: tile_adj_k<F_EXC>(tp, tlam, M, s, acc); break;
+            case F_ROTZ: tile_adj_k<F_ROTZ>(tp, tlam, M, s, acc); break;
+            case F_RY: tile_adj_k<F_RY>(tp, tlam, M, s, acc); break;
+            case F_RX: tile_adj_k<F_RX>(tp, tlam, M, s, acc); break;
+            default: tile_adj_k<F_NEG>(tp, tlam, M, s, acc); break;
+          }
+          if (s.slot >= 0) accp[s.slot * nt + tid] += acc;
+          --i;
+        }
+        __syncthreads();
+      }
     }
-    for (uint32_t j = tid; j < M; j += kFT) {
-      const uint64_t k = gidx(hoff, j, P.c, outer);
-      psi[k] = tp[j];
-      lam[k] = tlam[j];
-    }
+    staged = true;
+    const double f = s_scale;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < T.cnt) {
+        const uint64_t k = outer | tile_idx(T, i);
+        const double2 p = tp[tid + i * nt], l = tlam[tid + i * nt];
+        psi[k] = f == 1.0 ? p : make_double2(f * p.x, f * p.y);
+        lam[k] = f == 1.0 ? l : make_double2(f * l.x, f * l.y);
+      }
     __syncthreads();
   }
-  // one block reduction per slot, written to the slot's op
-  int s = 0;
-  for (int i = 0; i < P.n_items; ++i) {
-    const FItem it = items[P.first_item + i];
-    if (it.slot < 0) continue;
-    const int cnt = it.kind == 0 ? 1 : it.count;
-    for (int g = 0; g < cnt; ++g) {
-      const int op = it.op + g;
-      if (gops[op].param < 0) continue;
-      double v = warp_sum(accp[s * kFT + tid]);
-      if ((tid & 31) == 0) red[tid >> 5] = v;
-      __syncthreads();
-      if (tid < 32) {
-        double u = tid < kFT / 32 ? red[tid] : 0.0;
-        u = warp_sum(u);
-        if (tid == 0) partial[(size_t)op * kRedBlocks + blockIdx.x] = u;
-      }
-      __syncthreads();
-      ++s;
-    }
+  // one warp reduces a slot: every thread's sum in a fixed order, to the slot's op
+  for (int s = tid >> 5; s < P.n_slots; s += (int)(nt >> 5)) {
+    double v = 0.0;
+    for (uint32_t j = tid & 31; j < nt; j += 32) v += accp[s * nt + j];
+    v = warp_sum(v);
+    if ((tid & 31) == 0) partial[(size_t)s_op[s] * kRedBlocks + blockIdx.x] = s_fac[s] * v;
   }
 }
 
@@ -397,57 +683,60 @@ __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
                                                const FItem* __restrict__ items,
                                                double* __restrict__ partial) {
   extern __shared__ double2 smem[];
-  __shared__ uint64_t hoff[1 << (11 - kMinLowBitsL2)];
-  __shared__ double red[kFT / 32];
-  const uint32_t M = 1u << P.m;
+  __shared__ SItem its[kChunk];
+  const uint32_t M = 1u << P.m, nt = blockDim.x;
   double2* tp = smem;
   double2* tlam = smem + M;
-  double* accp = (double*)(smem + 2 * M);  // [n_slots][kFT]
+  double* accp = (double*)(smem + 2 * M);  // [n_slots][nt]
   const uint64_t ntiles = 1ull << __popcll(P.outer_mask);
   const int tid = threadIdx.x;
-  for (int s = 0; s < P.n_slots; ++s) accp[s * kFT + tid] = 0.0;
-  setup_hoff(hoff, P);
-  __syncthreads();
+  const TileMap T = tile_map(P);
+  items += P.first_item;
+  for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint64_t outer = pdep64(t, P.outer_mask);
-    for (uint32_t j = tid; j < M; j += kFT) {
-      const uint64_t k = gidx(hoff, j, P.c, outer);
-      cp_async16(&tp[j], &psi[k]);
-      cp_async16(&tlam[j], &lam[k]);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    for (int i = 0; i < P.n_items; ++i) {
-      const FItem it = items[P.first_item + i];
-      if (it.kind != 0 || it.slot < 0) continue;
-      const DOp& op = it.local;
-      const uint32_t np = M >> op.k;
-      const uint32_t lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
-      const int kind = fkind_of(op.type);
-      double acc = 0.0;
-      for (uint32_t p = tid; p < np; p += kFT) {
-        const uint32_t a = (uint32_t)insert_zeros(p, op.sb, op.k) | lo;
-        const double2 px = tp[a], py = tp[a ^ fl], lx = tlam[a], ly = tlam[a ^ fl];
-        if (kind == F_ROTX) fgrad<F_ROTX>(lx, ly, px, py, acc);
-        else if (kind == F_ROTZ) fgrad<F_ROTZ>(lx, ly, px, py, acc);
-        else fgrad<F_ROTY>(lx, ly, px, py, acc);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < T.cnt) {
+        const uint64_t k = outer | tile_idx(T, i);
+        cp_async16(&tp[tid + i * nt], &psi[k]);
+        cp_async16(&tlam[tid + i * nt], &lam[k]);
       }
-      accp[it.slot * kFT + tid] += acc;
+    cp_async_wait_all();
+    for (int base = 0; base < P.n_items; base += kChunk) {
+      const int cnt = min(kChunk, P.n_items - base);
+      if (tid < cnt) {
+        const FItem it = items[base + tid];
+        SItem o;
+        o.kind = (int16_t)fkind_of(it.local.type);
+        o.slot = (int16_t)it.slot;
+        o.fl = (uint32_t)it.local.flip;
+        its[tid] = o;
+      }
+      __syncthreads();
+      for (int i = 0; i < cnt; ++i) {
+        const SItem& s = its[i];
+        if (s.slot < 0) continue;
+        const uint32_t fl = s.fl, low = fl - 1u;  // RY or RX: one bit
+        double acc = 0.0;
+        for (uint32_t p = tid; p < (M >> 1); p += nt) {
+          const uint32_t a = ((p & ~low) << 1) | (p & low);
+          const double2 px = tp[a], py = tp[a | fl], lx = tlam[a], ly = tlam[a | fl];
+          if (s.kind == F_RX) fgrad<F_RX>(lx, ly, px, py, acc);
+          else fgrad<F_RY>(lx, ly, px, py, acc);
+        }
+        accp[s.slot * nt + tid] += acc;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
-  for (int i = 0; i < P.n_items; ++i) {
-    const FItem it = items[P.first_item + i];
-    if (it.kind != 0 || it.slot < 0) continue;
-    double v = warp_sum(accp[it.slot * kFT + tid]);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    __syncthreads();
-    if (tid < 32) {
-      double u = tid < kFT / 32 ? red[tid] : 0.0;
-      u = warp_sum(u);
-      if (tid == 0) partial[(size_t)it.op * kRedBlocks + blockIdx.x] = u;
-    }
-    __syncthreads();
+  for (int i = tid >> 5; i < P.n_items; i += (int)(nt >> 5)) {
+    const int slot = items[i].slot;
+    if (slot < 0) continue;
+    double v = 0.0;
+    for (uint32_t j = tid & 31; j < nt; j += 32) v += accp[slot * nt + j];
+    v = warp_sum(v);
+    if ((tid & 31) == 0) partial[(size_t)items[i].op * kRedBlocks + blockIdx.x] = v;
   }
 }
 
@@ -455,17 +744,27 @@ __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
 
 int fused_tile_bits() { return 11; }
 
+namespace {
+// Threads of a pass: two to eight amplitudes each, so that a small tile's gates still fill
+// whole warps and no thread holds more than TileMap allows.
+int pass_threads(int m) { return std::min(kFT, std::max(32, 1 << (m > 0 ? m - 1 : 0))); }
 size_t fpass_smem(int m) { return ((size_t)1 << m) * sizeof(double2); }
 size_t bpass_smem(int m, int slots) {
-  return 2 * ((size_t)1 << m) * sizeof(double2) + (size_t)slots * kFT * sizeof(double);
+  return 2 * ((size_t)1 << m) * sizeof(double2) + (size_t)slots * pass_threads(m) * sizeof(double);
+}
+}  // namespace
+
+int pass_blocks(const FPass& P) {
+  const uint64_t ntiles = 1ull << __builtin_popcountll(P.outer_mask);
+  return (int)std::min<uint64_t>(ntiles, kRedBlocks);
 }
 
 cudaError_t fused_prepare() {
   cudaError_t e = cudaFuncSetAttribute(k_fpass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fpass_smem(12));
+                                       (int)fpass_smem(11));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_fpass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)fpass_smem(12));
+                           (int)fpass_smem(11));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_gpass, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)bpass_smem(11, kMaxSlotsDev));
@@ -475,37 +774,31 @@ cudaError_t fused_prepare() {
 }
 
 cudaError_t launch_fpass(double2* psi, const FPass& P, const FItem* items, const DOp* gops,
-                         const Rot* coef, const double* theta, cudaStream_t s) {
-  const uint64_t ntiles = 1ull << __builtin_popcountll(P.outer_mask);
-  const int grid = (int)std::min<uint64_t>(ntiles, kRedBlocks);
-  k_fpass<false><<<grid, kFT, fpass_smem(P.m), s>>>(psi, P, items, gops, coef, theta);
+                         const Rot* coef, const RotT* rt, cudaStream_t s) {
+  k_fpass<false><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(psi, P, items, gops,
+                                                                           coef, rt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fpass_inv(double2* v, const FPass& P, const FItem* items, const DOp* gops,
-                             const Rot* coef, const double* theta, cudaStream_t s) {
-  const uint64_t ntiles = 1ull << __builtin_popcountll(P.outer_mask);
-  const int grid = (int)std::min<uint64_t>(ntiles, kRedBlocks);
-  k_fpass<true><<<grid, kFT, fpass_smem(P.m), s>>>(v, P, items, gops, coef, theta);
+                             const Rot* coef, const RotT* rt, cudaStream_t s) {
+  k_fpass<true><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(v, P, items, gops,
+                                                                          coef, rt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const FItem* items, const DOp* gops, double* partial, cudaStream_t s) {
-  (void)gops;
-  const uint64_t ntiles = 1ull << __builtin_popcountll(P.outer_mask);
-  const int grid = (int)std::min<uint64_t>(ntiles, kRedBlocks);
-  k_gpass<<<grid, kFT, bpass_smem(P.m, P.n_slots), s>>>(psi, lam, P, items, partial);
+                         const FItem* items, double* partial, cudaStream_t s) {
+  k_gpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(psi, lam, P, items,
+                                                                              partial);
   return cudaGetLastError();
 }
 
 cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const FItem* items,
-                         const DOp* gops, const Rot* coef, const double* theta, double* partial,
+                         const DOp* gops, const Rot* coef, const RotT* rt, double* partial,
                          cudaStream_t s) {
-  const uint64_t ntiles = 1ull << __builtin_popcountll(P.outer_mask);
-  const int grid = (int)std::min<uint64_t>(ntiles, kRedBlocks);
-  k_bpass<<<grid, kFT, bpass_smem(P.m, P.n_slots), s>>>(psi, lam, P, items, gops, coef,
-                                                               theta, partial);
+  k_bpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(
+      psi, lam, P, items, gops, coef, rt, partial);
   return cudaGetLastError();
 }
 

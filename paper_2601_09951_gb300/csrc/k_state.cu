@@ -63,9 +63,26 @@ __global__ void k_init_basis(double2* __restrict__ psi, uint64_t N, uint64_t b) 
 }
 
 __global__ void k_prep_coefs(const DOp* __restrict__ ops, int n_ops,
-                             const double* __restrict__ theta, Rot* __restrict__ coefs) {
+                             const double* __restrict__ theta, Rot* __restrict__ coefs,
+                             RotT* __restrict__ rt) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < n_ops) coefs[g] = make_coef(ops[g], theta).r;
+  if (g >= n_ops) return;
+  const int type = ops[g].type, param = ops[g].param;
+  Rot r{0.0, 0.0, 0, 0};
+  RotT u{0.0, 1.0, 0.0, 0, 0};
+  if (is_param_type(type)) {
+    double s, c;
+    sincos(0.5 * (param >= 0 ? theta[param] : ops[g].fixed), &s, &c);
+    r = make_rot_cs(c, s);
+    if (type == SV_GATE_RZ) {
+      u.t = c;
+      u.c = s;
+    } else if (type == SV_GATE_RY || type == SV_GATE_RX) {
+      u = make_rott(c, s);
+    }
+  }
+  coefs[g] = r;
+  if (rt) rt[g] = u;
 }
 
 template <int KIND>
@@ -340,35 +357,46 @@ __global__ void k_sum(const double* __restrict__ partial, int count, double* __r
   if (threadIdx.x == 0) out[0] = t;
 }
 
-// One warp per op: contrib[l] = sum_b partial[l * kRedBlocks + b] (lane-strided, fixed order).
-__global__ void k_op_contrib(const DOp* __restrict__ ops, int n_ops,
-                             const double* __restrict__ partial, double* __restrict__ contrib) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, l = threadIdx.x & 31;
-  if (w >= n_ops) return;
-  double v = 0.0;
-  if (ops[w].param >= 0)
-    for (int b = l; b < kRedBlocks; b += 32) v += partial[(size_t)w * kRedBlocks + b];
-  v = warp_sum(v);
-  if (l == 0) contrib[w] = v;
-}
-
-__global__ void k_param_sum(const DOp* __restrict__ ops, int n_ops,
-                            const double* __restrict__ contrib, int n_params,
-                            double* __restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per parameter: it finds the parameter's ops 32 at a time and adds each op's block
+// shares (lane-strided, fixed order) in op order; the block after the last parameter sums the
+// energy.  Scanning the op list by a whole warp replaces one thread per parameter walking it
+// alone, which took 34 us for 400 parameters; only the blocks that wrote are read, so nothing
+// has to be zeroed first.
+__global__ void k_finish(const DOp* __restrict__ ops, int n_ops,
+                         const double* __restrict__ partial, int n_params,
+                         double* __restrict__ grad, const double* __restrict__ epart,
+                         double* __restrict__ energy, double* __restrict__ theta_upd, double lr,
+                         double* __restrict__ traj) {
+  __shared__ double red[32];
+  if (blockIdx.x == gridDim.x - 1) {
+    if (!epart) return;
+    double v = 0.0;
+    for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) v += epart[i];
+    const double t = block_sum(v, red);
+    if (threadIdx.x == 0) {
+      energy[0] = t;
+      if (traj) traj[0] = t;
+    }
+    return;
+  }
+  const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, l = threadIdx.x & 31;
   if (p >= n_params) return;
   double g = 0.0;
-  for (int l = 0; l < n_ops; ++l)
-    if (ops[l].param == p) g += contrib[l];
-  grad[p] = g;
-}
-
-__global__ void k_gd_update(double* __restrict__ theta, const double* __restrict__ grad, int n,
-                            double lr, const double* __restrict__ energy,
-                            double* __restrict__ traj) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < n) theta[p] = fma(-lr, grad[p], theta[p]);
-  if (p == 0 && traj) traj[0] = energy[0];
+  for (int o0 = 0; o0 < n_ops; o0 += 32) {
+    unsigned hit = __ballot_sync(0xffffffffu, o0 + l < n_ops && ops[o0 + l].param == p);
+    while (hit) {
+      const int o = o0 + __ffs(hit) - 1;
+      hit &= hit - 1u;
+      const int nb = ops[o].flags;
+      double v = 0.0;
+      for (int b = l; b < nb; b += 32) v += partial[(size_t)o * kRedBlocks + b];
+      g += warp_sum(v);
+    }
+  }
+  if (l == 0) {
+    grad[p] = g;
+    if (theta_upd) theta_upd[p] = fma(-lr, g, theta_upd[p]);
+  }
 }
 
 inline int grid_for(uint64_t work) {
@@ -388,9 +416,9 @@ cudaError_t launch_init_basis(double2* psi, int n, uint64_t b, cudaStream_t s) {
 }
 
 cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Rot* coefs,
-                              cudaStream_t s) {
+                              RotT* rt, cudaStream_t s) {
   if (n_ops <= 0) return cudaSuccess;
-  k_prep_coefs<<<(n_ops + 127) / 128, 128, 0, s>>>(ops, n_ops, theta, coefs);
+  k_prep_coefs<<<(n_ops + 31) / 32, 32, 0, s>>>(ops, n_ops, theta, coefs, rt);
   return cudaGetLastError();
 }
 
@@ -409,10 +437,12 @@ cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef,
   return cudaGetLastError();
 }
 
+int adjoint_blocks(int n, const DOp& op) { return grid_for(1ull << (n - op.k)); }
+
 cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, const Rot* coef,
                               double* partial, cudaStream_t s) {
   const uint64_t npairs = 1ull << (n - op.k);
-  const int g = partial ? kRedBlocks : grid_for(npairs);
+  const int g = grid_for(npairs);
   switch (kind_of(op.type)) {
     case K_SWAP: k_adjoint<K_SWAP><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, nullptr); break;
     case K_H: k_adjoint<K_H><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, nullptr); break;
@@ -439,22 +469,12 @@ cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_grads(const DOp* ops, int n_ops, const double* partial, int n_params,
-                                double* contrib, double* grad, cudaStream_t s) {
-  if (n_ops > 0) {
-    const int warps_per_block = 8;
-    k_op_contrib<<<(n_ops + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0,
-                   s>>>(ops, n_ops, partial, contrib);
-  }
-  if (n_params > 0)
-    k_param_sum<<<(n_params + 127) / 128, 128, 0, s>>>(ops, n_ops, contrib, n_params, grad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gd_update(double* theta, const double* grad, int n, double lr,
-                             const double* energy, double* traj, cudaStream_t s) {
-  k_gd_update<<<(n + 127) / 128 > 0 ? (n + 127) / 128 : 1, 128, 0, s>>>(theta, grad, n, lr,
-                                                                         energy, traj);
+cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
+                          double* grad, const double* epart, double* energy, double* theta_upd,
+                          double lr, double* traj, cudaStream_t s) {
+  const int per = kThreads / 32;
+  k_finish<<<(n_params + per - 1) / per + 1, kThreads, 0, s>>>(
+      ops, n_ops, partial, n_params, grad, epart, energy, theta_upd, lr, traj);
   return cudaGetLastError();
 }
 

@@ -13,13 +13,16 @@ constexpr int kRedBlocks = 1216;  // 152 SMs x 8
 constexpr int kThreads = 256;
 
 cudaError_t launch_init_basis(double2* psi, int n, uint64_t b, cudaStream_t s);
+// Coefficients of every op at theta: the lifting form, and (rt != nullptr) the unnormalised form
+// that the fused passes use.
 cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Rot* coefs,
-                              cudaStream_t s);
+                              RotT* rt, cudaStream_t s);
 // Apply (inv = false) or un-apply one op on psi; coef points at the op's Rot.
 cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef, bool inv,
                             cudaStream_t s);
-// Adjoint step for one op: if the op is parameterised, partial[b] (b < kRedBlocks) receives
-// block b's share of 2 Im<lambda|G|psi>; then psi and lambda are un-applied.
+// Adjoint step for one op: if the op is parameterised, partial[b] (b < adjoint_blocks(n, op))
+// receives block b's share of 2 Im<lambda|G|psi>; then psi and lambda are un-applied.
+int adjoint_blocks(int n, const DOp& op);
 cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, const Rot* coef,
                               double* partial, cudaStream_t s);
 // lambda = H psi (if lam != nullptr) and partial[b] = block b's share of Re<psi|H psi>.
@@ -27,12 +30,13 @@ cudaError_t launch_hpsi(const double2* psi, double2* lam, int n, const DGroup* g
                         int n_groups, const double2* tables, double* partial, cudaStream_t s);
 // out[0] = sum of partial[0..count) in a fixed order.
 cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream_t s);
-// grad[p] = sum over ops l with param p (in op order) of sum_b partial[l * kRedBlocks + b].
-cudaError_t launch_reduce_grads(const DOp* ops, int n_ops, const double* partial, int n_params,
-                                double* contrib, double* grad, cudaStream_t s);
-// theta -= lr * grad (n entries); optionally records energy[0] into traj[step].
-cudaError_t launch_gd_update(double* theta, const double* grad, int n, double lr,
-                             const double* energy, double* traj, cudaStream_t s);
+// The end of an evaluation, in one launch: grad[p] = sum over ops l with param p (in op order)
+// of sum_b partial[l * kRedBlocks + b] over the op's ops[l].flags blocks, and (epart != nullptr)
+// energy[0] = the sum of epart[0..kRedBlocks).  With theta_upd set also the descent step
+// theta_upd[p] -= lr * grad[p] and (traj != nullptr) traj[0] = the energy.
+cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
+                          double* grad, const double* epart, double* energy, double* theta_upd,
+                          double lr, double* traj, cudaStream_t s);
 
 }  // namespace svqe
 
@@ -47,10 +51,12 @@ constexpr int kDpMinQubits = 14;
 int fused_tile_bits();
 cudaError_t fused_prepare();
 cudaError_t launch_fpass(double2* psi, const FPass& P, const FItem* items, const DOp* gops,
-                         const Rot* coef, const double* theta, cudaStream_t s);
+                         const Rot* coef, const RotT* rt, cudaStream_t s);
 // The pass's items inverted and in reverse order, on v (un-applying the pass).
 cudaError_t launch_fpass_inv(double2* v, const FPass& P, const FItem* items, const DOp* gops,
-                             const Rot* coef, const double* theta, cudaStream_t s);
+                             const Rot* coef, const RotT* rt, cudaStream_t s);
+// Blocks a pass launches: one per tile, at most kRedBlocks.
+int pass_blocks(const FPass& P);
 // Whole-state diagonal + permutation segment of the single-state path (k_dp.cu): a run of
 // RZ/CZ gates followed by a run of CNOT/X gates, applied in one out-of-place streaming pass
 // for n >= 14.  perm: the permutation P of the CNOT/X run (gates in order) as three
@@ -100,12 +106,11 @@ cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2*
 // Gradient shares only (psi and lambda unchanged) of a pass whose items are single ops:
 // partial[op * kRedBlocks + b] as for launch_bpass.
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const FItem* items, const DOp* gops, double* partial, cudaStream_t s);
+                         const FItem* items, double* partial, cudaStream_t s);
 // Backward pass: partial[op * kRedBlocks + b] receives block b's gradient share of every
-// parameterised op of the pass, for the min(tiles, kRedBlocks) blocks launched; the caller
-// zeroes the partials beforehand.
+// parameterised op of the pass, for the pass_blocks(P) blocks launched.
 cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const FItem* items,
-                         const DOp* gops, const Rot* coef, const double* theta, double* partial,
+                         const DOp* gops, const Rot* coef, const RotT* rt, double* partial,
                          cudaStream_t s);
 
 // One instance of a compiled batch (device record).  steps, lr and etraj_off are used when

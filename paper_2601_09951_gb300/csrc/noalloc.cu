@@ -43,8 +43,7 @@ constexpr size_t kOffPsi = 0;
 constexpr size_t kOffLam = kOffPsi + align256(kStateBytes);
 constexpr size_t kOffOps = kOffLam + align256(kStateBytes);
 constexpr size_t kOffCoef = kOffOps + align256(sizeof(DOp) * SV_NOALLOC_MAX_GATES);
-constexpr size_t kOffContrib = kOffCoef + align256(sizeof(Rot) * SV_NOALLOC_MAX_GATES);
-constexpr size_t kOffGpart = kOffContrib + align256(sizeof(double) * SV_NOALLOC_MAX_GATES);
+constexpr size_t kOffGpart = kOffCoef + align256(sizeof(Rot) * SV_NOALLOC_MAX_GATES);
 constexpr size_t kOffEpart =
     kOffGpart + align256(sizeof(double) * (size_t)kRedBlocks * SV_NOALLOC_MAX_GATES);
 // A register of n qubits has at most 2^n distinct X masks, hence at most 2^n groups.
@@ -219,13 +218,13 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
   double2* lam = (double2*)(base + kOffLam);
   DOp* ops = (DOp*)(base + kOffOps);
   Rot* coef = (Rot*)(base + kOffCoef);
-  double* contrib = (double*)(base + kOffContrib);
   double* gpart = (double*)(base + kOffGpart);
   double* epart = (double*)(base + kOffEpart);
   DGroup* groups = (DGroup*)(base + kOffGroups);
   unsigned* flag = (unsigned*)(base + kOffFlag);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n_ops = (int)hc.ops.size();
+  for (DOp& op : hc.ops) op.flags = adjoint_blocks(n, op);
   for (int i0 = 0; i0 < n_ops; i0 += kOpChunk) {
     OpChunk c;
     const int cnt = n_ops - i0 < kOpChunk ? n_ops - i0 : kOpChunk;
@@ -237,16 +236,15 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
                                        flag);
   NA_CUDA(cudaGetLastError());
   NA_CUDA(launch_init_basis(psi, n, ref, s));
-  NA_CUDA(launch_prep_coefs(ops, n_ops, theta_dev, coef, s));
+  NA_CUDA(launch_prep_coefs(ops, n_ops, theta_dev, coef, nullptr, s));
   for (int l = 0; l < n_ops; ++l) NA_CUDA(launch_apply_op(psi, n, hc.ops[l], coef + l, false, s));
   NA_CUDA(launch_hpsi(psi, lam, n, groups, n_groups, (const double2*)tables_dev, epart, s));
-  NA_CUDA(launch_sum(epart, kRedBlocks, energy_dev, s));
   for (int l = n_ops - 1; l >= 0; --l) {
     double* part = hc.ops[l].param >= 0 ? gpart + (size_t)l * kRedBlocks : nullptr;
     NA_CUDA(launch_adjoint_op(psi, lam, n, hc.ops[l], coef + l, part, s));
   }
-  if (n_ops || hc.n_params)
-    NA_CUDA(launch_reduce_grads(ops, n_ops, gpart, hc.n_params, contrib, grad_dev, s));
+  NA_CUDA(launch_finish(ops, n_ops, gpart, hc.n_params, grad_dev, epart, energy_dev, nullptr, 0.0,
+                        nullptr, s));
   k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
   NA_CUDA(cudaGetLastError());
   return SV_OK;

@@ -50,9 +50,7 @@ __device__ __forceinline__ uint32_t pext64(uint64_t i, uint64_t m) {
 }
 
 // Rotation coefficients for R(phi), computed once per gate (not per amplitude).
-__device__ __forceinline__ Rot make_rot(double phi) {
-  double s, c;
-  sincos(phi, &s, &c);
+__device__ __forceinline__ Rot make_rot_cs(double c, double s) {
   Rot r;
   double cr, sr;
   if (fabs(c) >= fabs(s)) {
@@ -64,6 +62,40 @@ __device__ __forceinline__ Rot make_rot(double phi) {
   r.b = sr;
   r.pad = 0;
   return r;
+}
+
+__device__ __forceinline__ Rot make_rot(double phi) {
+  double s, c;
+  sincos(phi, &s, &c);
+  return make_rot_cs(c, s);
+}
+
+// The unnormalised form (see RotT) from c = cos phi, s = sin phi.  The factor is that of the
+// rounded t: r = 1 / sqrt(1 + t^2) with 1 + t^2 held in two doubles, and one Newton step for
+// the low part.
+__device__ __forceinline__ RotT make_rott(double c, double s) {
+  RotT o;
+  o.mode = fabs(s) > fabs(c) ? 1 : 0;
+  const double num = o.mode ? c : s, den = o.mode ? s : c;
+  const double t = num / den;
+  const double p = t * t, e = fma(t, t, dneg(p));
+  const double a = 1.0 + p, al = (p - (a - 1.0)) + e;
+  const double r = 1.0 / sqrt(a);
+  const double r2 = r * r, r2e = fma(r, r, dneg(r2));
+  double res = fma(dneg(r2), a, 1.0);
+  res = fma(dneg(r2e), a, res);
+  res = fma(dneg(r2), al, res);
+  const double lo = 0.5 * r * res;
+  double h = r + lo, l = lo - (h - r);
+  if (den < 0.0) {
+    h = dneg(h);
+    l = dneg(l);
+  }
+  o.t = t;
+  o.c = h;
+  o.clo = l;
+  o.pad = 0;
+  return o;
 }
 
 // Coefficients of R(-phi) from those of R(phi).

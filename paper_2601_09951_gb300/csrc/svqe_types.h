@@ -18,7 +18,8 @@ struct DOp {
   int32_t k;       // number of inserted zero bits
   int32_t bit0;    // basis-index bit of the first wire (1-qubit gates)
   uint8_t sb[4];   // sorted bit positions of the wires
-  int32_t flags;   // kOpCS: the batched kernel wants (cos, sin) for this op (see below)
+  int32_t flags;   // batched kernel: kOpCS if it wants (cos, sin) for this op (see below);
+                   // single-state path: blocks that write gradient shares of this op
   uint64_t lo_or;  // bits set in the first amplitude of each pair
   uint64_t flip;   // XOR mask from the first to the second amplitude
   double fixed;    // angle when param < 0
@@ -39,6 +40,19 @@ struct Rot {
   int32_t pad;
 };
 static_assert(sizeof(Rot) == 24, "Rot layout");
+
+// The same rotation without its normalisation, for the fused passes of the single-state path:
+// with mode 0 (|cos| >= |sin|) t = tan phi and R(phi) = c [[1, -t], [t, 1]], c = cos phi; with
+// mode 1 t = cot phi and R(phi) = c [[t, -1], [1, t]], c = sin phi.  c + clo is the factor of
+// the rounded t to about 2^-100, +-1 / sqrt(1 + t^2), so that a pass which multiplies its
+// amplitudes by the product of its factors keeps their norm to one rounding.  For an RZ gate
+// t = cos phi and c = sin phi.
+struct RotT {
+  double t, c, clo;
+  int32_t mode;
+  int32_t pad;
+};
+static_assert(sizeof(RotT) == 32, "RotT layout");
 
 // An X-mask group of Pauli terms, (H psi)[k] += f(k) psi[k ^ x]:
 //   cls 0/1/2: f(k) = table[toff + pext(k, zu)], a real / imaginary / complex table over the
@@ -109,7 +123,8 @@ struct FPass {
   int32_t m, c;
   int32_t first_item, n_items;
   int32_t n_slots;  // gradient slots used by the pass's parameterised items
-  int32_t pad[3];
+  int32_t diag;     // index of the pass's diagonal item (kind 1), or -1
+  int32_t pad[2];
 };
 static_assert(sizeof(FPass) == 48, "FPass layout");
 

@@ -1,0 +1,75 @@
+"""GPU parity of the fused passes at the edges of their rules: registers on both sides of the tile
+rule (tiles of n - 7 bits below 18 qubits), angles on both sides of the quarter turns where the
+unnormalised rotations change form, RY and RX gates that share a trip or repeat a qubit, and
+passes of more items than are staged at a time.  Tolerances as in tests/parity.py."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2601_09951_gb300 import svqe
+from paper_2601_09951_gb300 import workloads as W
+from tests.parity import PSI_TOL, assert_energy, assert_grad
+
+pytestmark = pytest.mark.gpu
+
+# phi = theta / 2 on and beside the multiples of pi / 4 (form changes) and pi / 2 (zero cosine)
+ANGLES = [s * (k * np.pi / 2 + d) for k in range(5) for d in (-1e-9, 0.0, 1e-9) for s in (1, -1)]
+
+
+def _circuit(n, rng, n_rot, n_swap):
+    """n_rot RY/RX gates on few-to-all qubits (repeats included), fixed and free, with runs of
+    n_swap CNOT/X gates on the lowest qubits between them, and one of every other gate."""
+    cb = W.CircuitBuilder(n)
+    for q in range(n):
+        cb.add(W.H, (q,))
+    kinds = [W.RY, W.RY, W.RX]
+    for i in range(n_rot):
+        g = kinds[i // 4 % 3]
+        if i % 7 == 3:
+            cb.add(g, (int(rng.integers(n)),), angle=float(rng.choice(ANGLES)))
+        else:
+            cb.add(g, (int(rng.integers(n)),), param="new")
+        if i == n_rot // 2:
+            for j in range(n_swap):
+                a, b = (n - 1, n - 2) if n > 1 else (0, 0)
+                if j % 3 == 0 or n == 1:
+                    cb.add(W.X, (a,))
+                else:
+                    cb.add(W.CNOT, (a, b) if j % 3 == 1 else (b, a))
+    if n > 1:
+        cb.add(W.CZ, (0, n - 1))
+        cb.add(W.SINGLE_EXC, (n - 1, 0), param="new")
+    if n > 3:
+        cb.add(W.DOUBLE_EXC, (0, 1, n - 2, n - 1), param="new")
+    return cb.build()
+
+
+@pytest.mark.parametrize("n,n_rot,n_swap", [(1, 6, 3), (2, 9, 70), (5, 12, 33), (6, 20, 40),
+                                            (7, 20, 0), (12, 24, 35), (13, 24, 70), (14, 20, 3),
+                                            (17, 10, 40), (18, 8, 0)])
+def test_pass_edges(n, n_rot, n_swap):
+    rng = np.random.default_rng(900 + n)
+    circ = _circuit(n, rng, n_rot, n_swap)
+    theta = rng.uniform(-7, 7, circ["n_params"])
+    special = rng.permutation(circ["n_params"])[: circ["n_params"] // 2]
+    theta[special] = rng.choice(ANGLES, size=len(special))
+    ref = int(rng.integers(1 << n))
+    ctx = svqe.Context(n)
+    ctx.init_reference(ref)
+    ctx.apply_circuit(circ, theta)
+    want = oracle.state(circ, theta, ref)
+    assert np.max(np.abs(ctx.get_state() - want)) <= PSI_TOL
+    if n > 14:
+        # every parameter costs the oracle two to four whole energies: keep the first few
+        circ = dict(circ, params=np.where(np.asarray(circ["params"]) < 5, circ["params"], -1),
+                    fixed=np.where(np.asarray(circ["params"]) < 5, circ["fixed"], 0.37),
+                    n_params=5)
+        theta = theta[:5]
+    inst = {"circuit": circ, "ham": W.random_pauli_sum(rng, n, 12, 0.5, min(4, n), 1.0),
+            "ref": ref, "theta": theta}
+    ctx.init_reference(ref)
+    H = svqe.Ham(ctx, inst["ham"])
+    e, g = ctx.adjoint_grad(circ, theta, H)
+    e0, g0 = oracle.energy_grad(inst)
+    assert_energy(e, e0, inst["ham"], f"n={n}")
+    assert_grad(g, g0, inst["ham"], f"n={n}")
