@@ -36,14 +36,20 @@ struct sv_ctx {
   double* epart = nullptr;    // kRedBlocks energy partials
   double* scal = nullptr;     // [0] energy
   // circuit-sized buffers, grown on demand.  blob holds the staged circuit's records, uploaded
-  // in one copy: ops, fused-pass items and permutation tables.
+  // in one copy: ops, fused-pass items and preparation units.
   unsigned char* blob = nullptr;
   size_t blob_cap = 0;
   DOp* ops = nullptr;         // (in blob)
   FItem* items = nullptr;     // (in blob) fused-pass items of the staged circuit
+  PrepUnit* units = nullptr;  // (in blob)
+  int n_units = 0;
+  // what the preparation kernel derives from theta
   Rot* coef = nullptr;
-  RotT* rt = nullptr;
-  size_t coef_cap = 0, rt_cap = 0;
+  double2* cs = nullptr;
+  SItem* sitems = nullptr;
+  double* scales = nullptr;
+  double2* dptab = nullptr;
+  size_t coef_cap = 0, cs_cap = 0, sitems_cap = 0, scales_cap = 0, dptab_cap = 0;
   double* gpart = nullptr;    // n_ops x kRedBlocks gradient partials
   size_t gpart_cap = 0;
   double* theta = nullptr;
@@ -59,9 +65,6 @@ struct sv_ctx {
   // whole-state diagonal + permutation segments (k_dp.cu) need a third state buffer
   double2* scratch = nullptr;
   bool scratch_failed = false;
-  double2* dp_phase = nullptr;  // phase tables of the staged segments (written from theta every
-                                // evaluation)
-  size_t dp_phase_cap = 0;
   enum { CH_PASSES = 0, CH_LAYER = 1, CH_DP = 2 };
   struct Chunk {
     int kind;
@@ -217,7 +220,7 @@ sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
     return SV_ENOMEM;
   }
   c->ref = 0;
-  if (fused_prepare() != cudaSuccess || dp_prepare() != cudaSuccess ||
+  if (fused_prepare() != cudaSuccess ||
       launch_init_basis(c->psi, n, 0, c->stream) != cudaSuccess) {
     set_error("init kernel launch failed");
     sv_destroy(c);
@@ -237,14 +240,16 @@ sv_status sv_destroy(sv_ctx* c) {
   cudaFree(c->scal);
   cudaFree(c->blob);
   cudaFree(c->coef);
-  cudaFree(c->rt);
+  cudaFree(c->cs);
+  cudaFree(c->sitems);
+  cudaFree(c->scales);
+  cudaFree(c->dptab);
   cudaFree(c->gpart);
   cudaFree(c->theta);
   cudaFree(c->grad);
   cudaFree(c->etraj);
   for (double2* p : c->ck) cudaFree(p);
   cudaFree(c->scratch);
-  cudaFree(c->dp_phase);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   cudaGetLastError();
   delete c;
@@ -435,7 +440,7 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc);
 sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune) {
   const size_t n_ops = hc.ops.size();
   SV_CUDA(grow(c->coef, c->coef_cap, n_ops), c);
-  SV_CUDA(grow(c->rt, c->rt_cap, n_ops), c);
+  SV_CUDA(grow(c->cs, c->cs_cap, n_ops), c);
   SV_CUDA(grow(c->gpart, c->gpart_cap, std::max<size_t>(1, n_ops) * kRedBlocks), c);
   SV_CUDA(grow(c->theta, c->theta_cap, (size_t)hc.n_params), c);
   SV_CUDA(grow(c->grad, c->grad_cap, (size_t)hc.n_params), c);
@@ -471,7 +476,6 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
   c->plan.passes.clear();
   c->plan.items.clear();
   c->chunks.clear();
-  std::vector<uint32_t> tabs;  // permutation tables of the whole-state segments
   if (c->n >= kFusedMinQubits && n_ops > 0) {
     // commuting layers that get a psi checkpoint: as many as the budget (and the device) allow
     std::vector<std::pair<int, int>> layers = commuting_layers(hc.ops, 2);
@@ -544,14 +548,12 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
       ch.kind = sv_ctx::CH_DP;
       ch.first = first;
       ch.count = len;
-      ch.ck = (int)(tabs.size() / kDpTableWords);  // index of the segment's tables
+      ch.ck = -1;
       DpArgs& d = ch.dp;
       d.n = c->n;
-      d.N = c->N;
       for (int l = first; l < first + split; ++l) {
         const DOp& op = hc.ops[l];
         if (op.type == SV_GATE_RZ) {
-          d.rz_all[d.n_rz_all++] = l;
           if (op.param >= 0) {
             d.rz_op[d.n_rz] = l;
             d.rz_bit[d.n_rz] = op.bit0;
@@ -561,8 +563,7 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
           d.cz_mask[d.n_cz++] = (uint32_t)op.lo_or;
         }
       }
-      // P(k): the CNOT/X gates' conditional flips in order; tables over bits [0, 11),
-      // [11, 22), [22, 31), the first holding P(0)
+      // P(k): the CNOT/X gates' conditional flips in order, affine over GF(2)
       auto P = [&](uint32_t k) {
         for (int l = first + split; l < first + len; ++l) {
           const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
@@ -570,21 +571,15 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
         }
         return k;
       };
-      const uint32_t c0 = P(0);
+      d.c0 = P(0);
+      for (int b = 0; b < c->n; ++b) d.col[b] = P(1u << b) ^ d.c0;
       // delta = M^-1 e_0: the linear parts of the gates (a CNOT flips its target where its
       // control is set; an X is a constant) applied to e_0 in reverse order
-      uint32_t delta = 1u;
+      d.delta = 1u;
       for (int l = first + len - 1; l >= first + split; --l) {
         const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
-        if (lo && (delta & lo) == lo) delta ^= fl;
+        if (lo && (d.delta & lo) == lo) d.delta ^= fl;
       }
-      d.pair = delta >> 11;
-      d.pair_hi = d.pair ? 31 - __builtin_clz(d.pair) : 0;
-      for (int t = 0; t < 3; ++t)
-        for (uint32_t j = 0; j < 2048; ++j) {
-          const uint64_t k = (uint64_t)j << (11 * t);
-          tabs.push_back(k < c->N ? (t == 0 ? P((uint32_t)k) : P((uint32_t)k) ^ c0) : 0u);
-        }
       c->chunks.push_back(ch);
     };
     int i = 0, pass_start = 0;
@@ -611,13 +606,12 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
     }
     flush((int)n_ops);
   }
-  // one upload: ops (with the number of blocks that write each op's gradient shares), items and
-  // permutation tables
+  // one upload: ops (with the number of blocks that write each op's gradient shares), items
   std::vector<DOp> ops(hc.ops);
   for (size_t l = 0; l < n_ops; ++l) ops[l].flags = adjoint_blocks(c->n, ops[l]);
   for (const sv_ctx::Chunk& ch : c->chunks) {
     if (ch.kind == sv_ctx::CH_DP) {
-      for (int l = ch.first; l < ch.first + ch.count; ++l) ops[l].flags = kRedBlocks;
+      for (int l = ch.first; l < ch.first + ch.count; ++l) ops[l].flags = dp_blocks(c->n);
       continue;
     }
     for (int p = ch.p0; p < ch.p1; ++p) {
@@ -628,34 +622,42 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
           ops[c->plan.items[i].op + g].flags = pass_blocks(P);
     }
   }
+  std::vector<PrepUnit> units;
+  int n_dp = 0;
+  for (const sv_ctx::Chunk& ch : c->chunks) {
+    if (ch.kind == sv_ctx::CH_DP) {
+      int split = 0;
+      while (split < ch.count && (hc.ops[ch.first + split].type == SV_GATE_RZ ||
+                                  hc.ops[ch.first + split].type == SV_GATE_CZ))
+        ++split;
+      units.push_back(PrepUnit{1, ch.first, split, n_dp++});
+    }
+    for (int p = ch.p0; p < ch.p1; ++p)
+      units.push_back(PrepUnit{0, c->plan.passes[p].first_item, c->plan.passes[p].n_items, p});
+  }
   auto align = [](size_t v) { return (v + 255) / 256 * 256; };
   const size_t o_items = align(n_ops * sizeof(DOp));
-  const size_t o_tabs = align(o_items + c->plan.items.size() * sizeof(FItem));
-  std::vector<unsigned char> blob(o_tabs + tabs.size() * sizeof(uint32_t));
+  const size_t o_units = align(o_items + c->plan.items.size() * sizeof(FItem));
+  std::vector<unsigned char> blob(o_units + units.size() * sizeof(PrepUnit));
   if (n_ops) std::memcpy(blob.data(), ops.data(), n_ops * sizeof(DOp));
   if (!c->plan.items.empty())
     std::memcpy(blob.data() + o_items, c->plan.items.data(), c->plan.items.size() * sizeof(FItem));
-  if (!tabs.empty())
-    std::memcpy(blob.data() + o_tabs, tabs.data(), tabs.size() * sizeof(uint32_t));
+  if (!units.empty())
+    std::memcpy(blob.data() + o_units, units.data(), units.size() * sizeof(PrepUnit));
   SV_CUDA(grow(c->blob, c->blob_cap, blob.size()), c);
+  SV_CUDA(grow(c->sitems, c->sitems_cap, c->plan.items.size()), c);
+  SV_CUDA(grow(c->scales, c->scales_cap, c->plan.passes.size()), c);
+  if (n_dp) SV_CUDA(grow(c->dptab, c->dptab_cap, (size_t)n_dp * kDpTab), c);
   if (!blob.empty())
     SV_CUDA(cudaMemcpyAsync(c->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice,
                             c->stream), c);
   c->ops = (DOp*)c->blob;
   c->items = (FItem*)(c->blob + o_items);
-  const size_t n_dp = tabs.size() / kDpTableWords;
-  if (n_dp) {
-    SV_CUDA(grow(c->dp_phase, c->dp_phase_cap, n_dp * kDpPhaseEntries), c);
-    for (sv_ctx::Chunk& ch : c->chunks) {
-      if (ch.kind != sv_ctx::CH_DP) continue;
-      DpArgs& d = ch.dp;
-      double2* ph = c->dp_phase + (size_t)ch.ck * kDpPhaseEntries;
-      d.perm = (const uint32_t*)(c->blob + o_tabs) + (size_t)ch.ck * kDpTableWords;
-      d.phase_lo = d.phase_lo_w = ph;
-      d.phase_b1 = d.phase_b1_w = ph + 2048;
-      d.phase_b2 = d.phase_b2_w = ph + 3072;
-    }
-  }
+  c->units = (PrepUnit*)(c->blob + o_units);
+  c->n_units = (int)units.size();
+  n_dp = 0;
+  for (sv_ctx::Chunk& ch : c->chunks)
+    if (ch.kind == sv_ctx::CH_DP) ch.dp.tab = c->dptab + (size_t)kDpTab * n_dp++;
   return SV_OK;
 }
 
@@ -684,13 +686,13 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
                          double2** psi_out) {
   const int n_ops = (int)hc.ops.size();
   *psi_out = c->psi;
-  SV_CUDA(launch_prep_coefs(c->ops, n_ops, theta_dev, c->coef, c->rt, c->stream), c);
+  SV_CUDA(launch_prep(c->units, c->n_units, c->ops, c->items, theta_dev, c->n, c->coef, c->sitems,
+                      c->scales, c->cs, c->dptab, c->stream), c);
   if (!c->chunks.empty()) {
     double2* psi = c->psi;
     for (const sv_ctx::Chunk& ch : c->chunks) {
       if (ch.kind == sv_ctx::CH_DP) {
         double2* dst = free_buffer(c, psi, nullptr);
-        SV_CUDA(launch_dp_setup(ch.dp, c->ops, theta_dev, c->stream), c);
         SV_CUDA(launch_dp_fwd(psi, dst, ch.dp, c->stream), c);
         psi = dst;
         continue;
@@ -703,7 +705,7 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
         if (op >= 0)
           SV_CUDA(launch_apply_op(psi, c->n, hc.ops[op], c->coef + op, false, c->stream), c);
         else
-          SV_CUDA(launch_fpass(psi, c->plan.passes[p], c->items, c->ops, c->coef, c->rt,
+          SV_CUDA(launch_fpass(psi, c->plan.passes[p], c->sitems, c->ops, c->cs, c->scales + p,
                                c->stream), c);
       }
     }
@@ -844,8 +846,8 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
             SV_CUDA(launch_adjoint_op(psi, lam, c->n, hc.ops[op], c->coef + op, part,
                                       c->stream), c);
           } else {
-            SV_CUDA(launch_bpass(psi, lam, c->plan.passes[p], c->items, c->ops, c->coef,
-                                 c->rt, c->gpart, c->stream), c);
+            SV_CUDA(launch_bpass(psi, lam, c->plan.passes[p], c->sitems, c->ops, c->cs,
+                                 c->scales + p, c->gpart, c->stream), c);
           }
         }
       } else if (ch.kind == sv_ctx::CH_LAYER) {
@@ -853,10 +855,10 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
         // end, then the layer un-applied to lambda alone; psi before the layer is the
         // checkpoint itself (the buffer is not needed again in this sweep)
         for (int p = ch.p0; p < ch.p1; ++p)
-          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->items, c->gpart, c->stream), c);
+          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->sitems, c->gpart, c->stream), c);
         for (int p = ch.p1 - 1; p >= ch.p0; --p)
-          SV_CUDA(launch_fpass_inv(lam, c->plan.passes[p], c->items, c->ops, c->coef, c->rt,
-                                   c->stream), c);
+          SV_CUDA(launch_fpass_inv(lam, c->plan.passes[p], c->sitems, c->ops, c->cs,
+                                   c->scales + p, c->stream), c);
         psi = c->ck[ch.ck];
       } else {
         // diagonal + permutation: psi gathered and un-phased into a free buffer, then lambda

@@ -4,18 +4,25 @@
 // CNOT (and X) gates.  Fused shared-memory passes need four or more passes for such a run when
 // the CNOTs chain through all qubits (a ring or a ladder), each pass moving psi and lambda
 // through HBM for very little arithmetic.  Here the run is one streaming pass over the state:
-//   * the CNOT/X run is an affine map of the index bits over GF(2), P(k) = T0[k & 2047] ^
-//     T1[(k >> 11) & 2047] ^ T2[k >> 22], from three tables staged in shared memory;
+//   * the CNOT/X run is an affine map of the index bits over GF(2), P(k) = c0 ^ the columns of
+//     k's set bits;
 //   * the diagonal part is one phase per amplitude, e^{-i sum_q phi_q s_q(k)} (times -1 for
-//     the CZ gates that fire), from a table over the 11 low bits (staged) and a factor per
-//     block of 2048 amplitudes from two tables over the block index;
+//     the CZ gates that fire);
 //   * the RZ gradients 2 Im<lambda|Z_q/2|psi> = sum_k s_q(k) w_k, w_k = Im(conj(lambda_k)
 //     psi_k), are the same at either end of the diagonal part (the phase cancels in w_k), so
-//     they are taken from the un-phased lambda and psi: a per-thread sum for the bits fixed in
-//     a thread (0-7), three sums for the bits that vary within a block (8-10), and one sum per
-//     block-index bit (11 and up).
-// Blocks of 2048 consecutive amplitudes are handled by 256 threads, 8 amplitudes each (k =
-// base + tid + 256 i).  Out of place: the gather/scatter needs a second buffer.
+//     they are taken from the un-phased lambda and psi.
+// Blocks of 128 NA consecutive amplitudes are handled by 128 threads, NA (1 to 8) amplitudes
+// each (k = base + tid + 128 i), so P and the phase of an amplitude split into a part per
+// thread, one per i and one per block: a thread keeps its own part in registers, and the block
+// and i parts of 32 rounds are tabulated together.  The phases come from tables of 128 entries over
+// seven bits each (k_prep.cu).  Tables of 2048 entries staged per block (80 KB read through
+// 56 KB of shared memory) cost small states ten times their work and held large ones to four
+// blocks per SM: the lambda sweep took 94 us at 17 qubits and 610 us at 24, now 20 and 470.
+// Out of place: the gather/scatter needs a second buffer.
+//
+// Bound by the FP64 pipe on an HBM-resident state (8 operations per amplitude forward, 12.75 in
+// the lambda sweep, against 32 and 48 bytes).  The grid is at most 1024 blocks of 128 threads:
+// seven to an SM, so all are resident and no last wave runs short.
 #include <algorithm>
 
 #include "launch.h"
@@ -25,9 +32,10 @@ namespace svqe {
 
 namespace {
 
-constexpr int kDT = 256;     // threads per CTA
-constexpr int kDB = 11;      // bits per block
-constexpr int kDBlock = 1 << kDB;
+constexpr int kDT = 128;       // threads per CTA
+constexpr int kDTLog = kDpThreadLog;
+constexpr int kChunk = 32;     // rounds tabulated at a time
+constexpr int kMaxRound = 11;  // round bits (31 qubits: 2^21 blocks on 2^10 CTAs)
 
 __device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
   return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
@@ -36,247 +44,303 @@ __device__ __forceinline__ double2 cmul_conj(const double2& a, const double2& b)
   return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, dneg(a.x) * b.y));
 }
 
-// Dynamic shared memory of every k_dp kernel (56 KiB + reduction scratch).
-struct DpShared {
-  double2 p0[kDBlock];       // phase over the 11 low bits
-  uint32_t t[3][kDBlock];    // permutation tables
-  double red[kDT / 32];
-};
-
-__device__ __forceinline__ void dp_stage(DpShared& S, const DpArgs& a) {
-  for (int j = threadIdx.x; j < 3 * kDBlock; j += kDT) (&S.t[0][0])[j] = a.perm[j];
-  for (int j = threadIdx.x; j < kDBlock; j += kDT) S.p0[j] = a.phase_lo[j];
-  __syncthreads();
-}
-
-__device__ __forceinline__ uint32_t dp_map(const DpShared& S, uint64_t k) {
-  return S.t[0][k & (kDBlock - 1)] ^ S.t[1][(k >> kDB) & (kDBlock - 1)] ^ S.t[2][k >> (2 * kDB)];
-}
-
-__device__ __forceinline__ double2 dp_outer(const DpArgs& a, uint64_t blk) {
-  return cmul(a.phase_b1[blk & 1023], a.phase_b2[blk >> 10]);
-}
-
-// The block of visit index t (see DpArgs::pair): bit 0 of t selects pair, bit pair_hi of t
-// selects block bit 0, every other bit of t is the same block bit.  A bijection on the block
-// indices, because pair has bit pair_hi set.
-__device__ __forceinline__ uint64_t dp_block(const DpArgs& a, uint64_t t) {
-  if (a.pair <= 1u) return t;
-  const uint64_t ep = 1ull << a.pair_hi;
-  uint64_t b = t & ~(ep | 1ull);
-  if (t & 1ull) b ^= a.pair;
-  if (t & ep) b ^= 1ull;
+// The block of visit index t: bit 0 of t selects pair, bit pair_hi of t selects block bit 0,
+// every other bit of t is the same block bit.  A bijection on the block indices, because pair
+// has bit pair_hi set.  The amplitude P(k) ^ 1, which shares P(k)'s 32-byte sector, is
+// P(k ^ delta), delta = M^-1 e_0 (M the linear part of P); pair is delta's block part, so
+// adjacent CTAs read (or write) the two halves of the same sectors in the same round.
+__device__ __forceinline__ uint32_t dp_block(uint32_t pair, uint32_t t) {
+  if (pair <= 1u) return t;
+  const uint32_t ep = 1u << (31 - __clz((int)pair));
+  uint32_t b = t & ~(ep | 1u);
+  if (t & 1u) b ^= pair;
+  if (t & ep) b ^= 1u;
   return b;
 }
 
-__device__ __forceinline__ bool dp_cz(const DpArgs& a, uint64_t k) {
+__device__ __forceinline__ bool dp_cz(const DpArgs& a, uint32_t k) {
   uint32_t par = 0;
   for (int c = 0; c < a.n_cz; ++c) par ^= ((k & a.cz_mask[c]) == a.cz_mask[c]);
   return par & 1u;
 }
 
-// Forward: out[P(k)] = phase(k) in[k].
-__global__ void __launch_bounds__(kDT) k_dp_fwd(const double2* __restrict__ in,
-                                                double2* __restrict__ out, DpArgs a) {
-  extern __shared__ double2 dsm[];
-  DpShared& S = *reinterpret_cast<DpShared*>(dsm);
-  dp_stage(S, a);
-  const uint64_t nblk = a.N >> kDB;
-  for (uint64_t t = blockIdx.x; t < nblk; t += gridDim.x) {
-    const uint64_t blk = dp_block(a, t);
-    const double2 o = dp_outer(a, blk);
+template <int NA>
+struct DpShared {
+  double2 q[kChunk * NA];    // phases of the rounds' blocks times those of the i bits
+  uint32_t blk[kChunk];      // the rounds' blocks and their part of P (with c0)
+  uint32_t pc[kChunk];
+};
+
+// What a thread keeps for the whole launch: its part of P and of the phase.
+struct DpThread {
+  uint32_t pt;
+  double2 ph;
+};
+
+__device__ __forceinline__ DpThread dp_start(const DpArgs& a) {
+  DpThread t;
+  t.ph = a.tab[threadIdx.x];
+  t.pt = 0;
 #pragma unroll
-    for (int i = 0; i < kDBlock / kDT; ++i) {
-      const uint32_t j = threadIdx.x + i * kDT;
-      const uint64_t k = (blk << kDB) | j;
-      double2 v = cmul(in[k], cmul(S.p0[j], o));
-      if (a.n_cz && dp_cz(a, k)) v = make_double2(dneg(v.x), dneg(v.y));
-      out[dp_map(S, k)] = v;
+  for (int b = 0; b < kDTLog; ++b)
+    if ((threadIdx.x >> b) & 1u) t.pt ^= a.col[b];
+  return t;
+}
+
+// Tabulate rounds [r0, r0 + kChunk) of this CTA (visit indices t = blockIdx.x + r gridDim.x).
+template <int NA>
+__device__ __forceinline__ void dp_rounds(DpShared<NA>& S, const DpArgs& a, uint32_t r0,
+                                          uint32_t nblk) {
+  constexpr int BL = kDTLog + (NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0);
+  const int tid = threadIdx.x;
+  const uint32_t pair = a.delta >> BL;
+  const double2* pi = a.tab + 128;
+  const double2* po = a.tab + 136;
+  __syncthreads();
+  for (int j = tid; j < kChunk * NA; j += kDT) {
+    const int r = j / NA;
+    const uint32_t t = blockIdx.x + (r0 + r) * gridDim.x;
+    if (t >= nblk) break;
+    const uint32_t b = dp_block(pair, t);
+    if (j % NA == 0) {
+      uint32_t c = a.c0;
+      for (int i = BL; i < a.n; ++i)
+        if ((b >> (i - BL)) & 1u) c ^= a.col[i];
+      S.blk[r] = b;
+      S.pc[r] = c;
+    }
+    double2 p = po[b & 127u];
+    if (a.n > BL + 7) p = cmul(p, po[128 + ((b >> 7) & 127u)]);
+    if (a.n > BL + 14) p = cmul(p, po[256 + (b >> 14)]);
+    S.q[j] = NA > 1 ? cmul(p, pi[j % NA]) : p;
+  }
+  __syncthreads();
+}
+
+// Forward (BWD false): out[P(k)] = phase(k) in[k].  Backward: out[k] = conj(phase(k)) in[P(k)].
+template <int NA, bool BWD>
+__global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
+                                               double2* __restrict__ out, DpArgs a) {
+  __shared__ DpShared<NA> S;
+  constexpr int BL = kDTLog + (NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0);
+  const DpThread T = dp_start(a);
+  const uint32_t nblk = 1u << (a.n - BL);
+  for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
+    dp_rounds(S, a, r0, nblk);
+    for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
+      const uint32_t base = (S.blk[r] << BL) | threadIdx.x, pc = S.pc[r] ^ T.pt;
+      double2 v[NA];
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        uint32_t p = pc;
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if ((i >> b) & 1) p ^= a.col[kDTLog + b];
+        v[i] = in[BWD ? p : base | (i * kDT)];
+      }
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        uint32_t p = pc;
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if ((i >> b) & 1) p ^= a.col[kDTLog + b];
+        const uint32_t k = base | (i * kDT);
+        const double2 ph = cmul(T.ph, S.q[r * NA + i]);
+        double2 w = BWD ? cmul_conj(v[i], ph) : cmul(v[i], ph);
+        if (a.n_cz && dp_cz(a, k)) w = make_double2(dneg(w.x), dneg(w.y));
+        out[BWD ? k : p] = w;
+      }
     }
   }
 }
 
-// Backward, psi: out[k] = conj(phase(k)) in[P(k)].
-__global__ void __launch_bounds__(kDT) k_dp_bwd_psi(const double2* __restrict__ in,
-                                                    double2* __restrict__ out, DpArgs a) {
-  extern __shared__ double2 dsm[];
-  DpShared& S = *reinterpret_cast<DpShared*>(dsm);
-  dp_stage(S, a);
-  const uint64_t nblk = a.N >> kDB;
-  for (uint64_t t = blockIdx.x; t < nblk; t += gridDim.x) {
-    const uint64_t blk = dp_block(a, t);
-    const double2 o = dp_outer(a, blk);
+// Sum over the warp of 16 values per lane by recursive halving (16 DADD per lane instead of
+// 80); afterwards lanes 2j and 2j+1 hold the warp total of value j.
+__device__ __forceinline__ double warp_sum16(double (&v)[16]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < kDBlock / kDT; ++i) {
-      const uint32_t j = threadIdx.x + i * kDT;
-      const uint64_t k = (blk << kDB) | j;
-      double2 v = cmul_conj(in[dp_map(S, k)], cmul(S.p0[j], o));
-      if (a.n_cz && dp_cz(a, k)) v = make_double2(dneg(v.x), dneg(v.y));
-      out[k] = v;
+  for (int s = 0; s < 4; ++s) {
+    const int o = 16 >> s, h = 8 >> s;
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = up ? v[i] : v[i + h];
+      const double keep = up ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
     }
   }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Backward, lambda: out[k] = conj(phase(k)) lam[P(k)], and the RZ gradient shares from
-// w_k = Im(conj(out[k]) psi_b[k]) with psi_b the un-phased psi (k_dp_bwd_psi's output):
-// partial[op * kRedBlocks + block] for every parameterised RZ op of the segment.  The first
-// G = min(blocks, 1024) CTAs do the work, CTA c taking visit indices t = c, c + G, c + 2G, ...
-// (block dp_block(t)): bits of t below log2 G are fixed per CTA (their signs apply to the
-// CTA's total), and the bits above it are bits of the round r (one sum each, at most 10).
-// The other CTAs write zeros.
-__global__ void __launch_bounds__(kDT, 2) k_dp_bwd_lam(const double2* __restrict__ lam,
-                                                    const double2* __restrict__ psi_b,
-                                                    double2* __restrict__ out, DpArgs a,
-                                                    double* __restrict__ partial) {
-  extern __shared__ double2 dsm[];
-  DpShared& S = *reinterpret_cast<DpShared*>(dsm);
-  dp_stage(S, a);
-  const uint64_t nblk = a.N >> kDB;
-  const uint64_t G = nblk < 1024 ? nblk : 1024;
-  const int lg = __popcll(G - 1);  // log2 G
-  const int nrb = a.n - kDB - lg;  // round bits
-  constexpr int kMaxRound = 10;
+// w_k = Im(conj(out[k]) psi_b[k]) with psi_b the un-phased psi (k_dp<BWD>'s output):
+// partial[op * kRedBlocks + block] for every parameterised RZ op of the segment.  The number of
+// CTAs is a power of two, G: CTA c takes visit indices t = c, c + G, c + 2G, ..., so the bits of
+// t below log2 G are fixed per CTA (their signs apply to the CTA's total) and the bits above
+// are bits of the round r (one sum each, at most kMaxRound).
+template <int NA>
+__global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ lam,
+                                                   const double2* __restrict__ psi_b,
+                                                   double2* __restrict__ out, DpArgs a,
+                                                   double* __restrict__ partial) {
+  __shared__ DpShared<NA> S;
+  __shared__ double red[kDT / 32][32];
+  constexpr int NL = NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0;
+  constexpr int BL = kDTLog + NL;
+  const DpThread T = dp_start(a);
+  const uint32_t nblk = 1u << (a.n - BL);
+  const int lg = 31 - __clz((int)gridDim.x);
+  const int nrb = a.n - BL - lg;  // round bits
   double W = 0.0, mid[3] = {0.0, 0.0, 0.0}, hr[kMaxRound];
 #pragma unroll
   for (int b = 0; b < kMaxRound; ++b) hr[b] = 0.0;
-  if (blockIdx.x < G) {
-    uint64_t r = 0;
-    for (uint64_t t = blockIdx.x; t < nblk; t += G, ++r) {
-      const uint64_t blk = dp_block(a, t);
-      const double2 o = dp_outer(a, blk);
+  for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
+    dp_rounds(S, a, r0, nblk);
+    for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
+      const uint32_t base = (S.blk[r] << BL) | threadIdx.x, pc = S.pc[r] ^ T.pt;
       double wb = 0.0;
+      // four slots at a time: loads first, and their sums by a partial butterfly (2.75 DADD per
+      // amplitude instead of 4)
 #pragma unroll
-      for (int i = 0; i < kDBlock / kDT; ++i) {
-        const uint32_t j = threadIdx.x + i * kDT;
-        const uint64_t k = (blk << kDB) | j;
-        double2 v = cmul_conj(lam[dp_map(S, k)], cmul(S.p0[j], o));
-        if (a.n_cz && dp_cz(a, k)) v = make_double2(dneg(v.x), dneg(v.y));
-        out[k] = v;
-        const double2 p = psi_b[k];
-        const double w = fma(v.x, p.y, dneg(v.y) * p.x);
-        wb += w;
+      for (int i0 = 0; i0 < NA; i0 += 4) {
+        constexpr int U = NA < 4 ? NA : 4;
+        double2 v[U], p[U];
+        double w[U];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) mid[q] += ((i >> q) & 1) ? dneg(w) : w;
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u;
+          uint32_t src = pc;
+#pragma unroll
+          for (int b = 0; b < 3; ++b)
+            if ((i >> b) & 1) src ^= a.col[kDTLog + b];
+          v[u] = lam[src];
+          p[u] = psi_b[base | (i * kDT)];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u;
+          const uint32_t k = base | (i * kDT);
+          const double2 ph = cmul(T.ph, S.q[r * NA + i]);
+          double2 x = cmul_conj(v[u], ph);
+          if (a.n_cz && dp_cz(a, k)) x = make_double2(dneg(x.x), dneg(x.y));
+          out[k] = x;
+          w[u] = fma(x.x, p[u].y, dneg(x.y) * p[u].x);
+        }
+        double Sq;
+        if constexpr (U == 4) {
+          const double s01 = w[0] + w[1], d01 = w[0] - w[1];
+          const double s23 = w[2] + w[3], d23 = w[2] - w[3];
+          Sq = s01 + s23;
+          mid[0] += d01 + d23;
+          mid[1] += s01 - s23;
+          if (NA == 8) mid[2] += i0 ? dneg(Sq) : Sq;
+        } else if constexpr (U == 2) {
+          Sq = w[0] + w[1];
+          mid[0] += w[0] - w[1];
+        } else {
+          Sq = w[0];
+        }
+        wb += Sq;
       }
       W += wb;
 #pragma unroll
       for (int b = 0; b < kMaxRound; ++b)
-        if (b < nrb) hr[b] += ((r >> b) & 1ull) ? dneg(wb) : wb;
+        if (b < nrb) hr[b] += (((r0 + r) >> b) & 1u) ? dneg(wb) : wb;
     }
   }
-  // one CTA reduction per parameterised RZ op
-  const int tid = threadIdx.x;
-  for (int g = 0; g < a.n_rz; ++g) {
-    const int bit = a.rz_bit[g];
-    double v;
-    if (bit < 8) {
-      v = ((tid >> bit) & 1) ? dneg(W) : W;
-    } else if (bit < kDB) {
-      v = bit == 8 ? mid[0] : bit == 9 ? mid[1] : mid[2];
+  // CTA totals: 0 the whole sum, 1..7 signed by a thread bit, 8..10 by an i bit, 11.. by a round
+  // bit
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  {
+    double v[16];
+    v[0] = W;
+#pragma unroll
+    for (int b = 0; b < kDTLog; ++b) v[1 + b] = ((tid >> b) & 1) ? dneg(W) : W;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) v[8 + b] = mid[b];
+#pragma unroll
+    for (int b = 0; b < 5; ++b) v[11 + b] = hr[b];
+    const double t = warp_sum16(v);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = t;
+  }
+  if (nrb > 5) {
+    double v[16];
+#pragma unroll
+    for (int b = 0; b < 16; ++b) v[b] = b + 5 < kMaxRound ? hr[b + 5 < kMaxRound ? b + 5 : 0] : 0.0;
+    const double t = warp_sum16(v);
+    if ((lane & 1) == 0) red[warp][16 + (lane >> 1)] = t;
+  }
+  __syncthreads();
+  if (tid < a.n_rz) {
+    const int bit = a.rz_bit[tid];
+    const uint32_t pair = a.delta >> BL;
+    int j;
+    bool neg = false;
+    if (bit < kDTLog) {
+      j = 1 + bit;
+    } else if (bit < BL) {
+      j = 8 + bit - kDTLog;
     } else {
       // block bit jb of the block visited at t = blockIdx.x + r G is bit src of t, flipped by
       // t's bit 0 where pair has bit jb (dp_block); bits of t below lg are the CTA's, the
       // others the round's
-      const int jb = bit - kDB;
-      const bool paired = a.pair > 1u;
-      const bool t0 = blockIdx.x & 1u;
+      const int jb = bit - BL;
       int src = jb;
-      bool flip = false;
-      if (paired) {
-        if (jb == a.pair_hi) src = 0;
-        else if (jb == 0) src = a.pair_hi;
-        flip = jb != a.pair_hi && t0 && ((a.pair >> jb) & 1u);
+      if (pair > 1u) {
+        const int ph = 31 - __clz((int)pair);
+        if (jb == ph) src = 0;
+        else if (jb == 0) src = ph;
+        neg = jb != ph && (blockIdx.x & 1u) && ((pair >> jb) & 1u);
       }
       if (src < lg) {
-        v = ((blockIdx.x >> src) & 1u) ? dneg(W) : W;
+        j = 0;
+        neg ^= (blockIdx.x >> src) & 1u;
       } else {
-        v = 0.0;
-#pragma unroll
-        for (int b = 0; b < kMaxRound; ++b)
-          if (b == src - lg) v = hr[b];
+        j = 11 + src - lg;
       }
-      if (flip) v = dneg(v);
     }
-    v = warp_sum(v);
-    if ((tid & 31) == 0) S.red[tid >> 5] = v;
-    __syncthreads();
-    if (tid < 32) {
-      double u = tid < kDT / 32 ? S.red[tid] : 0.0;
-      u = warp_sum(u);
-      if (tid == 0) partial[(size_t)a.rz_op[g] * kRedBlocks + blockIdx.x] = u;
-    }
-    __syncthreads();
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < kDT / 32; ++w) v += red[w][j];
+    partial[(size_t)a.rz_op[tid] * kRedBlocks + blockIdx.x] = neg ? dneg(v) : v;
   }
 }
 
-// Phase tables from the step's coefficients: coef of an RZ op holds Rot(theta/2) in lifting
-// form, so (cos, sin) are recomputed here from theta (one thread per table entry).
-__global__ void k_dp_setup(DpArgs a, const DOp* __restrict__ ops, const double* __restrict__ theta) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  // entries: [0, 2048) low table, then 1024 + 1024 block tables
-  if (t >= kDBlock + 2048) return;
-  int lo_bit, nbits;
-  uint32_t idx;
-  double2* dst;
-  if (t < kDBlock) {
-    lo_bit = 0; nbits = kDB; idx = (uint32_t)t; dst = a.phase_lo_w + t;
-  } else if (t < kDBlock + 1024) {
-    lo_bit = kDB; nbits = 10; idx = (uint32_t)(t - kDBlock); dst = a.phase_b1_w + idx;
-  } else {
-    lo_bit = kDB + 10; nbits = 10; idx = (uint32_t)(t - kDBlock - 1024); dst = a.phase_b2_w + idx;
-  }
-  double2 p = make_double2(1.0, 0.0);
-  for (int g = 0; g < a.n_rz_all; ++g) {
-    const DOp op = ops[a.rz_all[g]];
-    const int b = op.bit0;
-    if (b < lo_bit || b >= lo_bit + nbits) continue;
-    const double th = op.param >= 0 ? theta[op.param] : op.fixed;
-    double s, c;
-    sincos(0.5 * th, &s, &c);
-    const bool one = (idx >> (b - lo_bit)) & 1u;
-    p = cmul(p, make_double2(c, one ? s : dneg(s)));  // e^{-i phi} on |0>, e^{+i phi} on |1>
-  }
-  *dst = p;
-}
+// Amplitudes per thread: as many as leave 128 blocks, up to eight (a block's set-up costs what
+// four hundred amplitudes do; one amplitude per thread in 1024 blocks took 11 us at 17 qubits).
+int dp_na(int n) { return n >= 17 ? 8 : n == 16 ? 4 : n == 15 ? 2 : 1; }
 
 }  // namespace
 
-cudaError_t dp_prepare() {
-  const int sm = (int)sizeof(DpShared);
-  cudaError_t e = cudaFuncSetAttribute(k_dp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_dp_bwd_psi, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_dp_bwd_lam, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-}
+int dp_block_log(int n) { return kDTLog + (n >= 17 ? 3 : n == 16 ? 2 : n == 15 ? 1 : 0); }
+int dp_blocks(int n) { return (int)std::min<uint64_t>(1ull << (n - dp_block_log(n)), 1024); }
 
-cudaError_t launch_dp_setup(const DpArgs& a, const DOp* ops, const double* theta,
-                            cudaStream_t s) {
-  k_dp_setup<<<(kDBlock + 2048 + 255) / 256, 256, 0, s>>>(a, ops, theta);
+#define DP_LAUNCH(K, ...)                                          \
+  switch (dp_na(a.n)) {                                            \
+    case 8: K(8)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
+    case 4: K(4)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
+    case 2: K(2)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
+    default: K(1)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;           \
+  }                                                                \
   return cudaGetLastError();
-}
-
-static int dp_grid(const DpArgs& a) {
-  const uint64_t nblk = a.N >> kDB;
-  return (int)std::min<uint64_t>(nblk, kRedBlocks);
-}
+#define DP_FWD(NA) k_dp<NA, false>
+#define DP_BWD(NA) k_dp<NA, true>
+#define DP_LAM(NA) k_dp_lam<NA>
 
 cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s) {
-  k_dp_fwd<<<dp_grid(a), kDT, sizeof(DpShared), s>>>(in, out, a);
-  return cudaGetLastError();
+  const int g = dp_blocks(a.n);
+  DP_LAUNCH(DP_FWD, in, out, a)
 }
 
-cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a,
-                              cudaStream_t s) {
-  k_dp_bwd_psi<<<dp_grid(a), kDT, sizeof(DpShared), s>>>(in, out, a);
-  return cudaGetLastError();
+cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s) {
+  const int g = dp_blocks(a.n);
+  DP_LAUNCH(DP_BWD, in, out, a)
 }
 
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
                               const DpArgs& a, double* partial, cudaStream_t s) {
-  // every block writes its share of every RZ op: the grid must be kRedBlocks
-  k_dp_bwd_lam<<<kRedBlocks, kDT, sizeof(DpShared), s>>>(lam, psi_b, out, a, partial);
-  return cudaGetLastError();
+  const int g = dp_blocks(a.n);
+  DP_LAUNCH(DP_LAM, lam, psi_b, out, a, partial)
 }
 
 }  // namespace svqe

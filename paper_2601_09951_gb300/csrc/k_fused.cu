@@ -14,11 +14,14 @@
 // What bounds these kernels is the FP64 pipe (2 FMA/clk/SM), so the RY and RX gates of a pass
 // run without their normalisation: R(phi) = cos phi [[1, -t], [t, 1]] with t = tan phi is two
 // FMAs per real pair where three shears are three, and the product of the cosines multiplies
-// the tile once, when it is stored (RotT; cot and sin where |sin| > |cos|, so every factor
+// the tile once, when it is stored (SItem; cot and sin where |sin| > |cos|, so every factor
 // dropped lies in [0.707, 1]).  Two such gates on different bits share one trip through shared
-// memory.  The pass's items and coefficients are staged in shared memory by one warp while the
-// tile's loads are in flight: read one at a time from global memory they cost a round trip per
-// gate and tile, which is most of a pass when a state of 2^13 to 2^20 amplitudes sits in L2.
+// memory.  The pass's items, coefficients included, are staged in shared memory by one warp while
+// the tile's loads are in flight: read one at a time from global memory they cost a round trip
+// per gate and tile, which is most of a pass when a state of 2^13 to 2^20 amplitudes sits in L2.
+// Nothing is computed per item here: one warp's FP64 instruction takes 64 clocks of its
+// scheduler's pipe, so a chain of 40 of them costs a block 1.2 us, once per block of every pass
+// (k_prep.cu does it once per evaluation).
 #include <algorithm>
 
 #include "launch.h"
@@ -51,31 +54,30 @@ __device__ __forceinline__ double2 rz_factor(const double2& cs, int bit) {
   return make_double2(cs.x, bit ? cs.y : dneg(cs.y));  // e^{-i phi} on |0>, e^{+i phi} on |1>
 }
 
-__device__ __forceinline__ uint64_t pdep64(uint64_t v, uint64_t m) {
-  uint64_t r = 0;
+__device__ __forceinline__ uint32_t pdep32(uint32_t v, uint32_t m) {
+  uint32_t r = 0;
   while (m) {
-    const uint64_t low = m & (0ull - m);
-    if (v & 1ull) r |= low;
+    const uint32_t low = m & (0u - m);
+    if (v & 1u) r |= low;
     v >>= 1;
-    m &= m - 1;
+    m &= m - 1u;
   }
   return r;
 }
 
 // Per-CTA setup of a diagonal item: cos/sin, local bits and the inner half tables.
-__device__ void diag_setup(DiagS& D, const FPass& P, const FItem& it, const DOp* gops,
-                           const RotT* rt) {
+__device__ void diag_setup(DiagS& D, const FPass& P, int op0, int count, const DOp* gops,
+                           const double2* cs) {
   if (threadIdx.x == 0) {
-    D.m_rz = it.count;
+    D.m_rz = count;
     D.hl = P.m / 2;
   }
-  if ((int)threadIdx.x < it.count) {
-    const RotT r = rt[it.op + threadIdx.x];  // (cos, sin) of an RZ gate
-    D.cs[threadIdx.x] = make_double2(r.t, r.c);
-    const int bit0 = gops[it.op + threadIdx.x].bit0;
+  if ((int)threadIdx.x < count) {
+    D.cs[threadIdx.x] = cs[op0 + threadIdx.x];
+    const int bit0 = gops[op0 + threadIdx.x].bit0;
     const uint64_t b = 1ull << bit0;
     D.loc[threadIdx.x] = (P.tile_mask & b) ? __popcll(P.tile_mask & (b - 1ull)) : -1 - bit0;
-    D.par[threadIdx.x] = gops[it.op + threadIdx.x].param >= 0;
+    D.par[threadIdx.x] = gops[op0 + threadIdx.x].param >= 0;
   }
   __syncthreads();
   const int hl = D.hl;
@@ -94,12 +96,21 @@ __device__ void diag_setup(DiagS& D, const FPass& P, const FItem& it, const DOp*
   __syncthreads();
 }
 
-// Per-tile: th = th0 * (product of the outer-bit RZ factors for this tile).
-__device__ void diag_tile(DiagS& D, const FPass& P, uint64_t outer) {
+// Per-tile: th = th0 * (product of the outer-bit RZ factors for this tile), the product by a
+// tree over the lanes of each warp that needs it.
+__device__ void diag_tile(DiagS& D, const FPass& P, uint32_t outer) {
+  const int nh = 1 << (P.m - D.hl), lane = threadIdx.x & 31;
+  if ((int)(threadIdx.x & ~31u) >= nh) return;
   double2 f = make_double2(1.0, 0.0);
-  for (int g = 0; g < D.m_rz; ++g)
-    if (D.loc[g] < 0) f = cmul(f, rz_factor(D.cs[g], (int)((outer >> (-1 - D.loc[g])) & 1ull)));
-  const int nh = 1 << (P.m - D.hl);
+  if (lane < D.m_rz && D.loc[lane] < 0)
+    f = rz_factor(D.cs[lane], (int)((outer >> (-1 - D.loc[lane])) & 1u));
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, f.x, o), y = __shfl_xor_sync(0xffffffffu, f.y, o);
+    f = cmul(f, make_double2(x, y));
+  }
+  f.x = __shfl_sync(0xffffffffu, f.x, 0);
+  f.y = __shfl_sync(0xffffffffu, f.y, 0);
   for (int j = threadIdx.x; j < nh; j += blockDim.x) D.th[j] = cmul(D.th0[j], f);
 }
 
@@ -149,109 +160,26 @@ __device__ __forceinline__ uint32_t tile_idx(const TileMap& T, int i) {
   return T.g ^ ((i & 1) ? T.h[0] : 0u) ^ ((i & 2) ? T.h[1] : 0u) ^ ((i & 4) ? T.h[2] : 0u);
 }
 
-enum FKind { F_SWAP = 0, F_H = 1, F_EXC = 2, F_ROTZ = 3, F_NEG = 4, F_RY = 5, F_RX = 6, F_DIAG = 7 };
-
-__device__ __forceinline__ int fkind_of(int type) {
-  switch (type) {
-    case SV_GATE_H: return F_H;
-    case SV_GATE_RY: return F_RY;
-    case SV_GATE_RX: return F_RX;
-    case SV_GATE_SINGLE_EXC: case SV_GATE_DOUBLE_EXC: return F_EXC;
-    case SV_GATE_RZ: return F_ROTZ;
-    case SV_GATE_CZ: return F_NEG;
-    default: return F_SWAP;
-  }
-}
-
-// An item as the tile loops read it, in shared memory, its coefficients oriented (inverted for
-// un-applying).
-struct SItem {
-  double p, q;     // RY, RX: p = t (see RotT); the other rotations: lifting coefficients a, b
-  double f;        // factor of the item's gradient sum (see stage_items)
-  uint32_t lo, fl;
-  uint8_t sb[4];
-  int16_t kind, k;
-  int16_t mode, slot;  // RY, RX: RotT::mode; the others: Rot::k
-  int op, count;
-};
 constexpr int kChunk = 32;  // items staged at a time, one lane of the first warp each
 
-// a * b for a value held as an unevaluated sum hi + lo (error about 2^-104).
-__device__ __forceinline__ void dd_mul(double& ah, double& al, double bh, double bl) {
-  const double p = ah * bh;
-  double e = fma(ah, bh, dneg(p));
-  e = fma(ah, bl, e);
-  e = fma(al, bh, e);
-  ah = p + e;
-  al = e - (ah - p);
-}
-
-// Stage items [base, base + cnt) of the pass (cnt <= kChunk), by the first warp.  scale and
-// scale_lo (that warp's lanes) are multiplied by the factors the chunk's RY and RX gates
-// leave out.  With grad set (the backward pass, chunks and items in reverse order) fac is the
-// square of the factors left out by the chunks already un-applied, and item j's sums of
-// lambda psi, taken when the items after it have been un-applied to both, carry their inverse:
-// f is the correction.
-__device__ __forceinline__ void stage_items(SItem* S, const FItem* items, int base, int cnt,
-                                            const Rot* coef, const RotT* rt, bool inv, bool grad,
-                                            double& scale, double& scale_lo, double& fac) {
+// Stage items [0, cnt) of the chunk at src (cnt <= kChunk) by the first warp, inverted for
+// un-applying: the inverse of (p x - y, x + p y) is (p x + y, p y - x) with the same factor left
+// out.
+__device__ __forceinline__ void stage_items(SItem* S, const SItem* src, int cnt, bool inv) {
   const int lane = threadIdx.x;
-  double c = 1.0, clo = 0.0;
-  SItem o;
-  if (lane < cnt) {
-    const FItem it = items[base + lane];
-    o.lo = (uint32_t)it.local.lo_or;
-    o.fl = (uint32_t)it.local.flip;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) o.sb[b] = it.local.sb[b];
-    o.k = (int16_t)it.local.k;
-    o.slot = (int16_t)it.slot;
-    o.op = it.op;
-    o.count = it.count;
-    o.kind = (int16_t)(it.kind == 1 ? F_DIAG : fkind_of(it.local.type));
-    o.p = o.q = 0.0;
-    o.mode = 0;
+  if (lane >= cnt) return;
+  SItem o = src[lane];
+  if (inv) {
     if (o.kind == F_RY || o.kind == F_RX) {
-      const RotT r = rt[it.op];
-      o.p = inv ? dneg(r.t) : r.t;
-      // the inverse of (t x - y, x + t y) is (t x + y, t y - x), the same factor left out
-      o.mode = (int16_t)(r.mode ? (inv ? 2 : 1) : 0);
-      if (r.mode && inv) o.p = r.t;
-      c = r.c;
-      clo = r.clo;
+      if (o.mode) o.mode = 2;
+      else o.p = dneg(o.p);
     } else if (o.kind == F_EXC || o.kind == F_ROTZ) {
-      Rot r = coef[it.op];
-      if (inv) r = rot_inverse(r);
-      o.p = r.a;
-      o.q = r.b;
-      o.mode = (int16_t)r.k;
+      o.p = dneg(o.p);
+      o.q = dneg(o.q);
+      o.mode = (int16_t)((4 - o.mode) & 3);
     }
   }
-  // nothing left out (a chunk of excitations, say): every factor is one
-  const bool none = __ballot_sync(0xffffffffu, c != 1.0) == 0u;
-  if (grad) o.f = fac;
-  if (grad && !none) {
-    // product of c^2 over the items after this one (lanes above), times the earlier chunks'
-    double w = c * c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const double v = __shfl_down_sync(0xffffffffu, w, d);
-      if (lane + d < 32) w *= v;
-    }
-    const double nx = __shfl_down_sync(0xffffffffu, w, 1);
-    o.f = fac * (lane == 31 ? 1.0 : nx);
-    fac *= __shfl_sync(0xffffffffu, w, 0);
-  }
-  if (!none) {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      const double h = __shfl_xor_sync(0xffffffffu, c, d);
-      const double l = __shfl_xor_sync(0xffffffffu, clo, d);
-      dd_mul(c, clo, h, l);
-    }
-    dd_mul(scale, scale_lo, __shfl_sync(0xffffffffu, c, 0), __shfl_sync(0xffffffffu, clo, 0));
-  }
-  if (lane < cnt) S[lane] = o;
+  S[lane] = o;
 }
 
 // (x, y) <- the rotation without its factor.
@@ -468,38 +396,34 @@ __device__ __forceinline__ bool can_pair(const SItem& a, const SItem& b) {
 // INV: apply the pass's items inverted, in reverse order (un-applying the pass).
 template <bool INV>
 __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPass P,
-                                               const FItem* __restrict__ items,
+                                               const SItem* __restrict__ items,
                                                const DOp* __restrict__ gops,
-                                               const Rot* __restrict__ coef,
-                                               const RotT* __restrict__ rt) {
+                                               const double2* __restrict__ cs,
+                                               const double* __restrict__ scale) {
   extern __shared__ double2 tile[];
   __shared__ DiagS D;
   __shared__ SItem its[kChunk];
-  __shared__ double s_scale;
   const uint32_t M = 1u << P.m, nt = blockDim.x;
   const uint64_t ntiles = 1ull << __popcll(P.outer_mask);
   const int nch = (P.n_items + kChunk - 1) / kChunk;
   const TileMap T = tile_map(P);
+  const double f = *scale;
   items += P.first_item;
   bool staged = false;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const uint64_t outer = pdep64(t, P.outer_mask);
+    const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
       if (i < T.cnt) cp_async16(&tile[threadIdx.x + i * nt], &psi[outer | tile_idx(T, i)]);
     if (P.diag >= 0) {
-      if (!staged) diag_setup(D, P, items[P.diag], gops, rt);
+      if (!staged) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
       diag_tile(D, P, outer);
     }
-    double sc = 1.0, sc_lo = 0.0, fac = 1.0;
     for (int ch = 0; ch < nch; ++ch) {
       const int base = (INV ? nch - 1 - ch : ch) * kChunk;
       const int cnt = min(kChunk, P.n_items - base);
       if (!staged || nch > 1) {
-        if (threadIdx.x < 32) {
-          stage_items(its, items, base, cnt, coef, rt, INV, false, sc, sc_lo, fac);
-          if (ch == nch - 1 && threadIdx.x == 0) s_scale = sc;
-        }
+        if (threadIdx.x < 32) stage_items(its, items + base, cnt, INV);
       }
       if (ch == 0) cp_async_wait_all();
       __syncthreads();
@@ -528,28 +452,33 @@ __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPa
       }
     }
     staged = true;
-    const double f = s_scale;
+    // (two loops: a select would issue the multiplications of an unscaled pass too)
+    if (f == 1.0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (i < T.cnt) {
-        const double2 v = tile[threadIdx.x + i * nt];
-        psi[outer | tile_idx(T, i)] = f == 1.0 ? v : make_double2(f * v.x, f * v.y);
-      }
+      for (int i = 0; i < 8; ++i)
+        if (i < T.cnt) psi[outer | tile_idx(T, i)] = tile[threadIdx.x + i * nt];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < T.cnt) {
+          const double2 v = tile[threadIdx.x + i * nt];
+          psi[outer | tile_idx(T, i)] = make_double2(f * v.x, f * v.y);
+        }
+    }
     __syncthreads();
   }
 }
 
 __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
                                                double2* __restrict__ lam, FPass P,
-                                               const FItem* __restrict__ items,
+                                               const SItem* __restrict__ items,
                                                const DOp* __restrict__ gops,
-                                               const Rot* __restrict__ coef,
-                                               const RotT* __restrict__ rt,
+                                               const double2* __restrict__ cs,
+                                               const double* __restrict__ scale,
                                                double* __restrict__ partial) {
   extern __shared__ double2 smem[];
   __shared__ DiagS D;
   __shared__ SItem its[kChunk];
-  __shared__ double s_scale;
   __shared__ int s_op[kMaxSlotsDev];      // op and gradient factor of each slot
   __shared__ double s_fac[kMaxSlotsDev];
   const uint32_t M = 1u << P.m, nt = blockDim.x;
@@ -560,34 +489,33 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
   const int tid = threadIdx.x, lt = 31 - __clz((int)nt);
   const int nch = (P.n_items + kChunk - 1) / kChunk;
   const TileMap T = tile_map(P);
+  const double f = *scale;
   items += P.first_item;
   for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
   bool staged = false;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const uint64_t outer = pdep64(t, P.outer_mask);
+    const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
       if (i < T.cnt) {
-        const uint64_t k = outer | tile_idx(T, i);
+        const uint32_t k = outer | tile_idx(T, i);
         cp_async16(&tp[tid + i * nt], &psi[k]);
         cp_async16(&tlam[tid + i * nt], &lam[k]);
       }
     if (P.diag >= 0) {
-      if (!staged) diag_setup(D, P, items[P.diag], gops, rt);
+      if (!staged) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
       diag_tile(D, P, outer);
     }
-    double sc = 1.0, sc_lo = 0.0, fac = 1.0;
     for (int ch = nch - 1; ch >= 0; --ch) {
       const int base = ch * kChunk;
       const int cnt = min(kChunk, P.n_items - base);
       if (!staged || nch > 1) {
         if (tid < 32) {
-          stage_items(its, items, base, cnt, coef, rt, true, true, sc, sc_lo, fac);
+          stage_items(its, items + base, cnt, true);
           if (!staged && tid < cnt && its[tid].slot >= 0 && its[tid].kind != F_DIAG) {
             s_op[its[tid].slot] = its[tid].op;
             s_fac[its[tid].slot] = its[tid].f;
           }
-          if (ch == 0 && tid == 0) s_scale = sc;
         }
       }
       if (ch == nch - 1) cp_async_wait_all();
@@ -614,7 +542,7 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
             const int lb = D.loc[g];
             double v;
             if (lb < 0) {
-              v = ((outer >> (-1 - lb)) & 1ull) ? dneg(W) : W;
+              v = ((outer >> (-1 - lb)) & 1u) ? dneg(W) : W;
             } else if (lb < lt) {
               v = ((tid >> lb) & 1) ? dneg(W) : W;
             } else {
@@ -654,15 +582,24 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
       }
     }
     staged = true;
-    const double f = s_scale;
+    if (f == 1.0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (i < T.cnt) {
-        const uint64_t k = outer | tile_idx(T, i);
-        const double2 p = tp[tid + i * nt], l = tlam[tid + i * nt];
-        psi[k] = f == 1.0 ? p : make_double2(f * p.x, f * p.y);
-        lam[k] = f == 1.0 ? l : make_double2(f * l.x, f * l.y);
-      }
+      for (int i = 0; i < 8; ++i)
+        if (i < T.cnt) {
+          const uint32_t k = outer | tile_idx(T, i);
+          psi[k] = tp[tid + i * nt];
+          lam[k] = tlam[tid + i * nt];
+        }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i < T.cnt) {
+          const uint32_t k = outer | tile_idx(T, i);
+          const double2 p = tp[tid + i * nt], l = tlam[tid + i * nt];
+          psi[k] = make_double2(f * p.x, f * p.y);
+          lam[k] = make_double2(f * l.x, f * l.y);
+        }
+    }
     __syncthreads();
   }
   // one warp reduces a slot: every thread's sum in a fixed order, to the slot's op
@@ -680,7 +617,7 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
 // no barrier between them.
 __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
                                                const double2* __restrict__ lam, FPass P,
-                                               const FItem* __restrict__ items,
+                                               const SItem* __restrict__ items,
                                                double* __restrict__ partial) {
   extern __shared__ double2 smem[];
   __shared__ SItem its[kChunk];
@@ -694,11 +631,11 @@ __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
   items += P.first_item;
   for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const uint64_t outer = pdep64(t, P.outer_mask);
+    const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
       if (i < T.cnt) {
-        const uint64_t k = outer | tile_idx(T, i);
+        const uint32_t k = outer | tile_idx(T, i);
         cp_async16(&tp[tid + i * nt], &psi[k]);
         cp_async16(&tlam[tid + i * nt], &lam[k]);
       }
@@ -706,12 +643,7 @@ __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
     for (int base = 0; base < P.n_items; base += kChunk) {
       const int cnt = min(kChunk, P.n_items - base);
       if (tid < cnt) {
-        const FItem it = items[base + tid];
-        SItem o;
-        o.kind = (int16_t)fkind_of(it.local.type);
-        o.slot = (int16_t)it.slot;
-        o.fl = (uint32_t)it.local.flip;
-        its[tid] = o;
+        its[tid] = items[base + tid];
       }
       __syncthreads();
       for (int i = 0; i < cnt; ++i) {
@@ -773,32 +705,32 @@ cudaError_t fused_prepare() {
                               (int)bpass_smem(11, kMaxSlotsDev));
 }
 
-cudaError_t launch_fpass(double2* psi, const FPass& P, const FItem* items, const DOp* gops,
-                         const Rot* coef, const RotT* rt, cudaStream_t s) {
+cudaError_t launch_fpass(double2* psi, const FPass& P, const SItem* items, const DOp* gops,
+                         const double2* cs, const double* scale, cudaStream_t s) {
   k_fpass<false><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(psi, P, items, gops,
-                                                                           coef, rt);
+                                                                           cs, scale);
   return cudaGetLastError();
 }
 
-cudaError_t launch_fpass_inv(double2* v, const FPass& P, const FItem* items, const DOp* gops,
-                             const Rot* coef, const RotT* rt, cudaStream_t s) {
+cudaError_t launch_fpass_inv(double2* v, const FPass& P, const SItem* items, const DOp* gops,
+                             const double2* cs, const double* scale, cudaStream_t s) {
   k_fpass<true><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(v, P, items, gops,
-                                                                          coef, rt);
+                                                                          cs, scale);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const FItem* items, double* partial, cudaStream_t s) {
+                         const SItem* items, double* partial, cudaStream_t s) {
   k_gpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(psi, lam, P, items,
                                                                               partial);
   return cudaGetLastError();
 }
 
-cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const FItem* items,
-                         const DOp* gops, const Rot* coef, const RotT* rt, double* partial,
+cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const SItem* items,
+                         const DOp* gops, const double2* cs, const double* scale, double* partial,
                          cudaStream_t s) {
   k_bpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(
-      psi, lam, P, items, gops, coef, rt, partial);
+      psi, lam, P, items, gops, cs, scale, partial);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,202 @@
+// k_prep.cu -- what an evaluation of a planned circuit derives from its angles, in one launch.
+//
+// One block per fused pass or whole-state segment.  A pass's block turns each item into the
+// record the pass kernels stage (SItem), the product of the factors its RY and RX gates leave
+// out into the pass's scale, and the items' gradient factors; a segment's block writes the
+// segment's phase tables.  Done here once per evaluation instead of by every block of every
+// pass: each block's share was a chain of about 40 FP64 instructions by one warp (1.2 us at 64
+// clocks each), 10 to 20 % of a 17-qubit pass.
+#include "launch.h"
+#include "svqe_internal.cuh"
+
+namespace svqe {
+
+namespace {
+
+constexpr int kPT = 128;
+
+__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
+  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
+}
+
+__device__ __forceinline__ int fkind_of(int type) {
+  switch (type) {
+    case SV_GATE_H: return F_H;
+    case SV_GATE_RY: return F_RY;
+    case SV_GATE_RX: return F_RX;
+    case SV_GATE_SINGLE_EXC: case SV_GATE_DOUBLE_EXC: return F_EXC;
+    case SV_GATE_RZ: return F_ROTZ;
+    case SV_GATE_CZ: return F_NEG;
+    default: return F_SWAP;
+  }
+}
+
+// a * b for a value held as an unevaluated sum hi + lo (error about 2^-104).
+__device__ __forceinline__ void dd_mul(double& ah, double& al, double bh, double bl) {
+  const double p = ah * bh;
+  double e = fma(ah, bh, dneg(p));
+  e = fma(ah, bl, e);
+  e = fma(al, bh, e);
+  ah = p + e;
+  al = e - (ah - p);
+}
+
+__device__ __forceinline__ void angle_cs(const DOp* ops, int l, const double* theta, double& c,
+                                         double& s) {
+  const int param = ops[l].param;
+  sincos(0.5 * (param >= 0 ? theta[param] : ops[l].fixed), &s, &c);
+}
+
+// Items in chunks of 32, the last chunk first (the gradient factors are products over later
+// items), one lane each.
+__device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
+                          const double* theta, Rot* coefs, SItem* sitems, double* scales,
+                          double2* cs) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp > 0) {
+    // the other warps: (cos, sin) of the RZ gates of diagonal items
+    for (int i = u.first; i < u.first + u.count; ++i) {
+      if (items[i].kind != 1) continue;
+      for (int g = (warp - 1) * 32 + lane; g < items[i].count; g += kPT - 32) {
+        double c, s;
+        angle_cs(ops, items[i].op + g, theta, c, s);
+        cs[items[i].op + g] = make_double2(c, s);
+      }
+    }
+    return;
+  }
+  double sh = 1.0, sl = 0.0, fac = 1.0;
+  for (int base = (u.count - 1) / 32 * 32; base >= 0; base -= 32) {
+    const int i = base + lane;
+    const bool on = i < u.count;
+    SItem o;
+    o.p = o.q = 0.0;
+    o.mode = 0;
+    double f = 1.0, flo = 0.0;
+    if (on) {
+      const FItem it = items[u.first + i];
+      o.lo = (uint32_t)it.local.lo_or;
+      o.fl = (uint32_t)it.local.flip;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) o.sb[b] = it.local.sb[b];
+      o.k = (int16_t)it.local.k;
+      o.slot = (int16_t)it.slot;
+      o.op = it.op;
+      o.count = it.count;
+      o.kind = (int16_t)(it.kind == 1 ? F_DIAG : fkind_of(it.local.type));
+      if (o.kind == F_RY || o.kind == F_RX || o.kind == F_EXC || o.kind == F_ROTZ) {
+        double c, s;
+        angle_cs(ops, it.op, theta, c, s);
+        const Rot r = make_rot_cs(c, s);
+        coefs[it.op] = r;
+        if (o.kind == F_RY || o.kind == F_RX) {
+          const RotT t = make_rott(c, s);
+          o.p = t.t;
+          o.mode = (int16_t)t.mode;
+          f = t.f;
+          flo = t.flo;
+        } else {
+          o.p = r.a;
+          o.q = r.b;
+          o.mode = (int16_t)r.k;
+        }
+      }
+    }
+    // product of f^2 over the lanes above, times the later chunks'
+    double w = f * f;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const double v = __shfl_down_sync(0xffffffffu, w, d);
+      if (lane + d < 32) w *= v;
+    }
+    const double nx = __shfl_down_sync(0xffffffffu, w, 1);
+    o.f = fac * (lane == 31 ? 1.0 : nx);
+    fac *= __shfl_sync(0xffffffffu, w, 0);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const double h = __shfl_xor_sync(0xffffffffu, f, d);
+      const double l = __shfl_xor_sync(0xffffffffu, flo, d);
+      dd_mul(f, flo, h, l);
+    }
+    dd_mul(sh, sl, __shfl_sync(0xffffffffu, f, 0), __shfl_sync(0xffffffffu, flo, 0));
+    if (on) sitems[u.first + i] = o;
+  }
+  if (lane == 0) scales[u.idx] = sh;
+}
+
+__device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, int n, int bl,
+                        double2* tab) {
+  // (cos, sin) of the angle sum of each index bit's RZ gates
+  __shared__ double2 cs[32];
+  __shared__ double2 op_cs[64];
+  __shared__ int op_bit[64];
+  __shared__ unsigned has;
+  if (threadIdx.x == 0) has = 0u;
+  for (int g = threadIdx.x; g < u.count; g += kPT) {
+    int bit = -1;
+    if (ops[u.first + g].type == SV_GATE_RZ) {
+      double c, s;
+      angle_cs(ops, u.first + g, theta, c, s);
+      op_cs[g] = make_double2(c, s);
+      bit = ops[u.first + g].bit0;
+    }
+    op_bit[g] = bit;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < n) {
+    double2 p = make_double2(1.0, 0.0);
+    bool any = false;
+    for (int g = 0; g < u.count; ++g) {
+      if (op_bit[g] != (int)threadIdx.x) continue;
+      p = any ? cmul(p, op_cs[g]) : op_cs[g];
+      any = true;
+    }
+    cs[threadIdx.x] = p;
+    if (any) atomicOr(&has, 1u << threadIdx.x);
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < kDpTab; j += kPT) {
+    int b0, b1;
+    uint32_t v;
+    if (j < 128) {
+      b0 = 0; b1 = kDpThreadLog; v = j;
+    } else if (j < 136) {
+      b0 = kDpThreadLog; b1 = bl; v = j - 128;
+    } else {
+      const int t = (j - 136) >> 7;
+      b0 = bl + 7 * t; b1 = min(b0 + 7, n); v = (j - 136) & 127;
+    }
+    double2 p = make_double2(1.0, 0.0);
+    for (int b = b0; b < b1; ++b, v >>= 1)
+      if ((has >> b) & 1u) p = cmul(p, make_double2(cs[b].x, v & 1u ? cs[b].y : dneg(cs[b].y)));
+    tab[(size_t)u.idx * kDpTab + j] = p;
+  }
+}
+
+__global__ void __launch_bounds__(kPT) k_prep(const PrepUnit* __restrict__ units,
+                                              const DOp* __restrict__ ops,
+                                              const FItem* __restrict__ items,
+                                              const double* __restrict__ theta, int n, int bl,
+                                              Rot* __restrict__ coefs, SItem* __restrict__ sitems,
+                                              double* __restrict__ scales,
+                                              double2* __restrict__ cs,
+                                              double2* __restrict__ dptab) {
+  const PrepUnit u = units[blockIdx.x];
+  if (u.dp) prep_dp(u, ops, theta, n, bl, dptab);
+  else prep_pass(u, ops, items, theta, coefs, sitems, scales, cs);
+}
+
+}  // namespace
+
+static_assert(kDpMaxRz + kDpMaxCz <= 64, "a segment's diagonal ops fit prep_dp's arrays");
+
+cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,
+                        const double* theta, int n, Rot* coefs, SItem* sitems, double* scales,
+                        double2* cs, double2* dptab, cudaStream_t s) {
+  if (n_units <= 0) return cudaSuccess;
+  k_prep<<<n_units, kPT, 0, s>>>(units, ops, items, theta, n, n >= kDpMinQubits ? dp_block_log(n) : n,
+                                 coefs, sitems, scales, cs, dptab);
+  return cudaGetLastError();
+}
+
+}  // namespace svqe

@@ -63,26 +63,9 @@ __global__ void k_init_basis(double2* __restrict__ psi, uint64_t N, uint64_t b) 
 }
 
 __global__ void k_prep_coefs(const DOp* __restrict__ ops, int n_ops,
-                             const double* __restrict__ theta, Rot* __restrict__ coefs,
-                             RotT* __restrict__ rt) {
+                             const double* __restrict__ theta, Rot* __restrict__ coefs) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_ops) return;
-  const int type = ops[g].type, param = ops[g].param;
-  Rot r{0.0, 0.0, 0, 0};
-  RotT u{0.0, 1.0, 0.0, 0, 0};
-  if (is_param_type(type)) {
-    double s, c;
-    sincos(0.5 * (param >= 0 ? theta[param] : ops[g].fixed), &s, &c);
-    r = make_rot_cs(c, s);
-    if (type == SV_GATE_RZ) {
-      u.t = c;
-      u.c = s;
-    } else if (type == SV_GATE_RY || type == SV_GATE_RX) {
-      u = make_rott(c, s);
-    }
-  }
-  coefs[g] = r;
-  if (rt) rt[g] = u;
+  if (g < n_ops) coefs[g] = make_coef(ops[g], theta).r;
 }
 
 template <int KIND>
@@ -416,9 +399,9 @@ cudaError_t launch_init_basis(double2* psi, int n, uint64_t b, cudaStream_t s) {
 }
 
 cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Rot* coefs,
-                              RotT* rt, cudaStream_t s) {
+                              cudaStream_t s) {
   if (n_ops <= 0) return cudaSuccess;
-  k_prep_coefs<<<(n_ops + 31) / 32, 32, 0, s>>>(ops, n_ops, theta, coefs, rt);
+  k_prep_coefs<<<(n_ops + 31) / 32, 32, 0, s>>>(ops, n_ops, theta, coefs);
   return cudaGetLastError();
 }
 

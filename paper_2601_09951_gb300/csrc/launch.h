@@ -13,10 +13,14 @@ constexpr int kRedBlocks = 1216;  // 152 SMs x 8
 constexpr int kThreads = 256;
 
 cudaError_t launch_init_basis(double2* psi, int n, uint64_t b, cudaStream_t s);
-// Coefficients of every op at theta: the lifting form, and (rt != nullptr) the unnormalised form
-// that the fused passes use.
 cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Rot* coefs,
-                              RotT* rt, cudaStream_t s);
+                              cudaStream_t s);
+// Everything of a planned circuit that depends on theta, one block per unit (k_prep.cu): the
+// ops' lifting coefficients, the passes' items and scales, (cos, sin) of the RZ gates and the
+// phase tables (kDpTab entries each) of the whole-state segments on n qubits.
+cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,
+                        const double* theta, int n, Rot* coefs, SItem* sitems, double* scales,
+                        double2* cs, double2* dptab, cudaStream_t s);
 // Apply (inv = false) or un-apply one op on psi; coef points at the op's Rot.
 cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef, bool inv,
                             cudaStream_t s);
@@ -44,73 +48,59 @@ namespace svqe {
 
 // Fused passes of the single-state path (k_fused.cu).  Tiles of fused_tile_bits() bits (all
 // of the state when it is smaller); used for registers of at least kFusedMinQubits qubits.
-// Whole-state diagonal + permutation segments (k_dp.cu, blocks of 2048 amplitudes) need at
-// least kDpMinQubits.
+// Whole-state diagonal + permutation segments (k_dp.cu) are used from kDpMinQubits: below,
+// a layer's RZ and CNOT gates fit one fused pass or two.
 constexpr int kFusedMinQubits = 1;
-constexpr int kDpMinQubits = 14;
+constexpr int kDpMinQubits = 12;
 int fused_tile_bits();
 cudaError_t fused_prepare();
-cudaError_t launch_fpass(double2* psi, const FPass& P, const FItem* items, const DOp* gops,
-                         const Rot* coef, const RotT* rt, cudaStream_t s);
+// items, scale (the pass's place) and cs as launch_prep wrote them.
+cudaError_t launch_fpass(double2* psi, const FPass& P, const SItem* items, const DOp* gops,
+                         const double2* cs, const double* scale, cudaStream_t s);
 // The pass's items inverted and in reverse order, on v (un-applying the pass).
-cudaError_t launch_fpass_inv(double2* v, const FPass& P, const FItem* items, const DOp* gops,
-                             const Rot* coef, const RotT* rt, cudaStream_t s);
+cudaError_t launch_fpass_inv(double2* v, const FPass& P, const SItem* items, const DOp* gops,
+                             const double2* cs, const double* scale, cudaStream_t s);
 // Blocks a pass launches: one per tile, at most kRedBlocks.
 int pass_blocks(const FPass& P);
 // Whole-state diagonal + permutation segment of the single-state path (k_dp.cu): a run of
 // RZ/CZ gates followed by a run of CNOT/X gates, applied in one out-of-place streaming pass
-// for n >= 14.  perm: the permutation P of the CNOT/X run (gates in order) as three
-// 2048-entry tables over index bits [0, 11), [11, 22), [22, 31) (the first including P(0));
-// phase tables (written by launch_dp_setup from theta): e^{-i sum phi s(k)} of
-// the RZ gates over the 11 low bits, and over block-index bits [0, 10) and [10, 20).
+// for n >= kDpMinQubits.  The permutation P of the CNOT/X run (gates in order) is
+// P(k) = c0 ^ the XOR of col[b] over the set bits b of k.
 constexpr int kDpMaxRz = 32;
 constexpr int kDpMaxCz = 16;
 struct DpArgs {
-  uint64_t N;
   int n;
-  const uint32_t* perm;
-  const double2* phase_lo;
-  const double2* phase_b1;
-  const double2* phase_b2;
-  double2* phase_lo_w;
-  double2* phase_b1_w;
-  double2* phase_b2_w;
+  uint32_t c0;
+  uint32_t col[31];
+  uint32_t delta;            // M^-1 e_0, M the linear part of P
   int n_cz;
   uint32_t cz_mask[kDpMaxCz];
   int n_rz;                  // parameterised RZ ops: gradient targets
   int rz_op[kDpMaxRz];
   int rz_bit[kDpMaxRz];
-  int n_rz_all;              // every RZ op of the diagonal part: phase factors
-  int rz_all[kDpMaxRz];
-  // Block pairing of the gather/scatter.  The amplitude P(k) ^ 1, which shares P(k)'s 32-byte
-  // sector, is P(k ^ delta) with delta = M^-1 e_0 (M the linear part of P); pair is the block
-  // part delta >> 11 and pair_hi its highest set bit.  With pair > 1 the kernels visit block
-  // B(t) for t = 0, 1, ..., where B(t) and B(t ^ 1) differ by pair, so adjacent CTAs read (or
-  // write) the two halves of the same sectors in the same round.
-  uint32_t pair;
-  int pair_hi;
+  const double2* tab;        // the segment's phase tables
 };
-constexpr size_t kDpTableWords = 3 * 2048;     // uint32 per permutation
-constexpr size_t kDpPhaseEntries = 2048 + 2048;  // double2 per segment (low + two block tables)
-cudaError_t dp_prepare();
-cudaError_t launch_dp_setup(const DpArgs& a, const DOp* ops, const double* theta, cudaStream_t s);
+// CTAs of a segment's kernels on n qubits (a power of two).
+int dp_blocks(int n);
+// log2 of the amplitudes per block of a segment's kernels on n qubits
+int dp_block_log(int n);
 // out[P(k)] = phase(k) in[k]
 cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s);
 // out[k] = conj(phase(k)) in[P(k)]
 cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s);
 // out[k] = conj(phase(k)) lam[P(k)]; RZ gradient shares from w_k = Im(conj(out[k]) psi_b[k])
-// into partial[op * kRedBlocks + block]
+// into partial[op * kRedBlocks + block], block < dp_blocks(n)
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
                               const DpArgs& a, double* partial, cudaStream_t s);
 
 // Gradient shares only (psi and lambda unchanged) of a pass whose items are single ops:
 // partial[op * kRedBlocks + b] as for launch_bpass.
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const FItem* items, double* partial, cudaStream_t s);
+                         const SItem* items, double* partial, cudaStream_t s);
 // Backward pass: partial[op * kRedBlocks + b] receives block b's gradient share of every
 // parameterised op of the pass, for the pass_blocks(P) blocks launched.
-cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const FItem* items,
-                         const DOp* gops, const Rot* coef, const RotT* rt, double* partial,
+cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const SItem* items,
+                         const DOp* gops, const double2* cs, const double* scale, double* partial,
                          cudaStream_t s);
 
 // One instance of a compiled batch (device record).  steps, lr and etraj_off are used when

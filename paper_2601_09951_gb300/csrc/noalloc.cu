@@ -236,7 +236,7 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
                                        flag);
   NA_CUDA(cudaGetLastError());
   NA_CUDA(launch_init_basis(psi, n, ref, s));
-  NA_CUDA(launch_prep_coefs(ops, n_ops, theta_dev, coef, nullptr, s));
+  NA_CUDA(launch_prep_coefs(ops, n_ops, theta_dev, coef, s));
   for (int l = 0; l < n_ops; ++l) NA_CUDA(launch_apply_op(psi, n, hc.ops[l], coef + l, false, s));
   NA_CUDA(launch_hpsi(psi, lam, n, groups, n_groups, (const double2*)tables_dev, epart, s));
   for (int l = n_ops - 1; l >= 0; --l) {

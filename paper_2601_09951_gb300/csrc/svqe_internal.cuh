@@ -70,9 +70,14 @@ __device__ __forceinline__ Rot make_rot(double phi) {
   return make_rot_cs(c, s);
 }
 
-// The unnormalised form (see RotT) from c = cos phi, s = sin phi.  The factor is that of the
-// rounded t: r = 1 / sqrt(1 + t^2) with 1 + t^2 held in two doubles, and one Newton step for
-// the low part.
+// R(phi) without its normalisation (see SItem) from c = cos phi, s = sin phi.  The factor
+// f + flo is that of the rounded t, +-1 / sqrt(1 + t^2) to about 2^-100 (1 + t^2 held in two
+// doubles, and one Newton step for the low part), so that a pass's product of factors keeps the
+// norm of its amplitudes to one rounding.
+struct RotT {
+  double t, f, flo;
+  int mode;
+};
 __device__ __forceinline__ RotT make_rott(double c, double s) {
   RotT o;
   o.mode = fabs(s) > fabs(c) ? 1 : 0;
@@ -86,15 +91,13 @@ __device__ __forceinline__ RotT make_rott(double c, double s) {
   res = fma(dneg(r2e), a, res);
   res = fma(dneg(r2), al, res);
   const double lo = 0.5 * r * res;
-  double h = r + lo, l = lo - (h - r);
+  o.f = r + lo;
+  o.flo = lo - (o.f - r);
   if (den < 0.0) {
-    h = dneg(h);
-    l = dneg(l);
+    o.f = dneg(o.f);
+    o.flo = dneg(o.flo);
   }
   o.t = t;
-  o.c = h;
-  o.clo = l;
-  o.pad = 0;
   return o;
 }
 

@@ -41,19 +41,6 @@ struct Rot {
 };
 static_assert(sizeof(Rot) == 24, "Rot layout");
 
-// The same rotation without its normalisation, for the fused passes of the single-state path:
-// with mode 0 (|cos| >= |sin|) t = tan phi and R(phi) = c [[1, -t], [t, 1]], c = cos phi; with
-// mode 1 t = cot phi and R(phi) = c [[t, -1], [1, t]], c = sin phi.  c + clo is the factor of
-// the rounded t to about 2^-100, +-1 / sqrt(1 + t^2), so that a pass which multiplies its
-// amplitudes by the product of its factors keeps their norm to one rounding.  For an RZ gate
-// t = cos phi and c = sin phi.
-struct RotT {
-  double t, c, clo;
-  int32_t mode;
-  int32_t pad;
-};
-static_assert(sizeof(RotT) == 32, "RotT layout");
-
 // An X-mask group of Pauli terms, (H psi)[k] += f(k) psi[k ^ x]:
 //   cls 0/1/2: f(k) = table[toff + pext(k, zu)], a real / imaginary / complex table over the
 //              kz bits of the union zu of the group's z masks;
@@ -139,6 +126,37 @@ struct FItem {
   DOp local;
 };
 static_assert(sizeof(FItem) == 64, "FItem layout");
+
+// An item as the pass kernels read it (written by the preparation kernel from its FItem and the
+// angles, forward orientation).  RY and RX gates are stored without their normalisation: with
+// mode 0 (|cos phi| >= |sin phi|) p = tan phi and R(phi) = c [[1, -p], [p, 1]], c = cos phi;
+// with mode 1 p = cot phi and R(phi) = c [[p, -1], [1, p]], c = sin phi.  The pass multiplies its
+// amplitudes once by the product of its factors c.  Excitations and single RZ gates: p, q and
+// mode are Rot's a, b and k.
+enum ItemKind { F_SWAP = 0, F_H = 1, F_EXC = 2, F_ROTZ = 3, F_NEG = 4, F_RY = 5, F_RX = 6,
+                F_DIAG = 7 };
+struct SItem {
+  double p, q;
+  double f;  // factor of the item's gradient sum: the product of c^2 over the items after it
+  uint32_t lo, fl;
+  uint8_t sb[4];
+  int16_t kind, k;
+  int16_t mode, slot;
+  int32_t op, count;
+};
+static_assert(sizeof(SItem) == 56, "SItem layout");
+
+// What the preparation kernel does for one fused pass (items [first, first + count) to the
+// same SItem places, its scale to place idx) or one whole-state segment (RZ/CZ ops [first,
+// first + count), its phase tables to place idx).
+struct PrepUnit {
+  int32_t dp;
+  int32_t first, count, idx;
+};
+// Phase tables of a whole-state segment: the thread's 128 phases, the 8 of a thread's slots, and
+// three tables of 128 over block-index bits.
+constexpr int kDpThreadLog = 7;
+constexpr int kDpTab = 128 + 8 + 3 * 128;
 
 __host__ __device__ __forceinline__ bool is_param_type(int t) {
   return t == SV_GATE_RX || t == SV_GATE_RY || t == SV_GATE_RZ || t == SV_GATE_SINGLE_EXC ||
