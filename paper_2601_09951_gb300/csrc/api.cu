@@ -220,7 +220,7 @@ sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
     return SV_ENOMEM;
   }
   c->ref = 0;
-  if (fused_prepare() != cudaSuccess ||
+  if (fused_prepare() != cudaSuccess || dp_prepare() != cudaSuccess ||
       launch_init_basis(c->psi, n, 0, c->stream) != cudaSuccess) {
     set_error("init kernel launch failed");
     sv_destroy(c);
@@ -690,10 +690,12 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
                       c->scales, c->cs, c->dptab, c->stream), c);
   if (!c->chunks.empty()) {
     double2* psi = c->psi;
+    bool ov = false;  // the first kernel after the preparation waits for it
     for (const sv_ctx::Chunk& ch : c->chunks) {
       if (ch.kind == sv_ctx::CH_DP) {
         double2* dst = free_buffer(c, psi, nullptr);
-        SV_CUDA(launch_dp_fwd(psi, dst, ch.dp, c->stream), c);
+        SV_CUDA(launch_dp_fwd(psi, dst, ch.dp, c->stream, ov), c);
+        ov = true;
         psi = dst;
         continue;
       }
@@ -703,10 +705,12 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
       for (int p = ch.p0; p < ch.p1; ++p) {
         const int op = single_op(c, p);
         if (op >= 0)
-          SV_CUDA(launch_apply_op(psi, c->n, hc.ops[op], c->coef + op, false, c->stream), c);
+          SV_CUDA(launch_apply_op(psi, c->n, hc.ops[op], c->coef + op, false, c->stream,
+                                  ov), c);
         else
           SV_CUDA(launch_fpass(psi, c->plan.passes[p], c->sitems, c->ops, c->cs, c->scales + p,
-                               c->stream), c);
+                               c->stream, ov), c);
+        ov = true;
       }
     }
     *psi_out = psi;
@@ -832,9 +836,9 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
   sv_status st = forward(c, hc, theta_dev, true, &psi);
   if (st != SV_OK) return st;
   double2* lam = psi == c->lam ? c->psi : c->lam;
-  SV_CUDA(launch_hpsi(psi, lam, c->n, H->groups, H->n_groups, H->tables, c->epart,
-                      c->stream), c);
   const int n_ops = (int)hc.ops.size();
+  SV_CUDA(launch_hpsi(psi, lam, c->n, H->groups, H->n_groups, H->tables, c->epart,
+                      c->stream, n_ops > 0), c);
   if (!c->chunks.empty()) {
     for (int ci = (int)c->chunks.size() - 1; ci >= 0; --ci) {
       const sv_ctx::Chunk& ch = c->chunks[ci];
@@ -844,10 +848,10 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
           if (op >= 0) {
             double* part = hc.ops[op].param >= 0 ? c->gpart + (size_t)op * kRedBlocks : nullptr;
             SV_CUDA(launch_adjoint_op(psi, lam, c->n, hc.ops[op], c->coef + op, part,
-                                      c->stream), c);
+                                      c->stream, true), c);
           } else {
             SV_CUDA(launch_bpass(psi, lam, c->plan.passes[p], c->sitems, c->ops, c->cs,
-                                 c->scales + p, c->gpart, c->stream), c);
+                                 c->scales + p, c->gpart, c->stream, true), c);
           }
         }
       } else if (ch.kind == sv_ctx::CH_LAYER) {
@@ -855,18 +859,19 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
         // end, then the layer un-applied to lambda alone; psi before the layer is the
         // checkpoint itself (the buffer is not needed again in this sweep)
         for (int p = ch.p0; p < ch.p1; ++p)
-          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->sitems, c->gpart, c->stream), c);
+          SV_CUDA(launch_gpass(psi, lam, c->plan.passes[p], c->sitems, c->gpart, c->stream,
+                               true), c);
         for (int p = ch.p1 - 1; p >= ch.p0; --p)
           SV_CUDA(launch_fpass_inv(lam, c->plan.passes[p], c->sitems, c->ops, c->cs,
-                                   c->scales + p, c->stream), c);
+                                   c->scales + p, c->stream, true), c);
         psi = c->ck[ch.ck];
       } else {
         // diagonal + permutation: psi gathered and un-phased into a free buffer, then lambda
         // likewise with the RZ gradients from the two un-phased states
         double2* psi_b = free_buffer(c, psi, lam);
-        SV_CUDA(launch_dp_bwd_psi(psi, psi_b, ch.dp, c->stream), c);
+        SV_CUDA(launch_dp_bwd_psi(psi, psi_b, ch.dp, c->stream, true), c);
         double2* lam_b = free_buffer(c, psi_b, lam);
-        SV_CUDA(launch_dp_bwd_lam(lam, psi_b, lam_b, ch.dp, c->gpart, c->stream), c);
+        SV_CUDA(launch_dp_bwd_lam(lam, psi_b, lam_b, ch.dp, c->gpart, c->stream, true), c);
         psi = psi_b;
         lam = lam_b;
       }
@@ -883,7 +888,7 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
     }
   }
   SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, energy_dev,
-                        theta_upd, lr, traj, c->stream), c);
+                        theta_upd, lr, traj, c->stream, true), c);
   return SV_OK;
 }
 

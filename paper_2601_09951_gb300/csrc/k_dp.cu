@@ -124,9 +124,11 @@ __global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
   __shared__ DpShared<NA> S;
   constexpr int BL = kDTLog + (NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0);
   const DpThread T = dp_start(a);
+  dp_rounds(S, a, 0, 1u << (a.n - BL));
+  pdl_begin();
   const uint32_t nblk = 1u << (a.n - BL);
   for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
-    dp_rounds(S, a, r0, nblk);
+    if (r0) dp_rounds(S, a, r0, nblk);
     for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
       const uint32_t base = (S.blk[r] << BL) | threadIdx.x, pc = S.pc[r] ^ T.pt;
       double2 v[NA];
@@ -188,6 +190,8 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
   constexpr int NL = NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0;
   constexpr int BL = kDTLog + NL;
   const DpThread T = dp_start(a);
+  dp_rounds(S, a, 0, 1u << (a.n - BL));
+  pdl_begin();
   const uint32_t nblk = 1u << (a.n - BL);
   const int lg = 31 - __clz((int)gridDim.x);
   const int nrb = a.n - BL - lg;  // round bits
@@ -195,7 +199,7 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
 #pragma unroll
   for (int b = 0; b < kMaxRound; ++b) hr[b] = 0.0;
   for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
-    dp_rounds(S, a, r0, nblk);
+    if (r0) dp_rounds(S, a, r0, nblk);
     for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
       const uint32_t base = (S.blk[r] << BL) | threadIdx.x, pc = S.pc[r] ^ T.pt;
       double wb = 0.0;
@@ -315,30 +319,46 @@ int dp_na(int n) { return n >= 17 ? 8 : n == 16 ? 4 : n == 15 ? 2 : 1; }
 int dp_block_log(int n) { return kDTLog + (n >= 17 ? 3 : n == 16 ? 2 : n == 15 ? 1 : 0); }
 int dp_blocks(int n) { return (int)std::min<uint64_t>(1ull << (n - dp_block_log(n)), 1024); }
 
-#define DP_LAUNCH(K, ...)                                          \
-  switch (dp_na(a.n)) {                                            \
-    case 8: K(8)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
-    case 4: K(4)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
-    case 2: K(2)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;            \
-    default: K(1)<<<g, kDT, 0, s>>>(__VA_ARGS__); break;           \
-  }                                                                \
-  return cudaGetLastError();
+cudaError_t dp_prepare() {
+  const void* ks[] = {(const void*)k_dp<1, false>, (const void*)k_dp<2, false>,
+                      (const void*)k_dp<4, false>, (const void*)k_dp<8, false>,
+                      (const void*)k_dp<1, true>,  (const void*)k_dp<2, true>,
+                      (const void*)k_dp<4, true>,  (const void*)k_dp<8, true>,
+                      (const void*)k_dp_lam<1>,    (const void*)k_dp_lam<2>,
+                      (const void*)k_dp_lam<4>,    (const void*)k_dp_lam<8>};
+  for (const void* k : ks) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnePerSm);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+#define DP_LAUNCH(K, ...)                                                                     \
+  switch (dp_na(a.n)) {                                                                       \
+    case 8: return launch_overlapped(K(8), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);               \
+    case 4: return launch_overlapped(K(4), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);               \
+    case 2: return launch_overlapped(K(2), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);               \
+    default: return launch_overlapped(K(1), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);              \
+  }
 #define DP_FWD(NA) k_dp<NA, false>
 #define DP_BWD(NA) k_dp<NA, true>
 #define DP_LAM(NA) k_dp_lam<NA>
 
-cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s) {
+cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
+                          bool overlap) {
   const int g = dp_blocks(a.n);
   DP_LAUNCH(DP_FWD, in, out, a)
 }
 
-cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s) {
+cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
+                              bool overlap) {
   const int g = dp_blocks(a.n);
   DP_LAUNCH(DP_BWD, in, out, a)
 }
 
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
-                              const DpArgs& a, double* partial, cudaStream_t s) {
+                              const DpArgs& a, double* partial, cudaStream_t s, bool overlap) {
   const int g = dp_blocks(a.n);
   DP_LAUNCH(DP_LAM, lam, psi_b, out, a, partial)
 }

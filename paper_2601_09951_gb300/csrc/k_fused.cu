@@ -409,22 +409,19 @@ __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPa
   const TileMap T = tile_map(P);
   const double f = *scale;
   items += P.first_item;
-  bool staged = false;
+  if (nch == 1 && threadIdx.x < 32) stage_items(its, items, P.n_items, INV);
+  if (P.diag >= 0) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
+  pdl_begin();
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
       if (i < T.cnt) cp_async16(&tile[threadIdx.x + i * nt], &psi[outer | tile_idx(T, i)]);
-    if (P.diag >= 0) {
-      if (!staged) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
-      diag_tile(D, P, outer);
-    }
+    if (P.diag >= 0) diag_tile(D, P, outer);
     for (int ch = 0; ch < nch; ++ch) {
       const int base = (INV ? nch - 1 - ch : ch) * kChunk;
       const int cnt = min(kChunk, P.n_items - base);
-      if (!staged || nch > 1) {
-        if (threadIdx.x < 32) stage_items(its, items + base, cnt, INV);
-      }
+      if (nch > 1 && threadIdx.x < 32) stage_items(its, items + base, cnt, INV);
       if (ch == 0) cp_async_wait_all();
       __syncthreads();
       for (int ii = 0; ii < cnt;) {
@@ -451,7 +448,6 @@ __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPa
         __syncthreads();
       }
     }
-    staged = true;
     // (two loops: a select would issue the multiplications of an unscaled pass too)
     if (f == 1.0) {
 #pragma unroll
@@ -492,7 +488,27 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
   const double f = *scale;
   items += P.first_item;
   for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
-  bool staged = false;
+  if (nch == 1 && tid < 32) stage_items(its, items, P.n_items, true);
+  // op and gradient factor of each slot
+  for (int i = tid; i < P.n_items; i += nt) {
+    const int slot = items[i].slot;
+    if (slot >= 0 && items[i].kind != F_DIAG) {
+      s_op[slot] = items[i].op;
+      s_fac[slot] = items[i].f;
+    }
+  }
+  if (P.diag >= 0) {
+    diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
+    if (tid == 0) {
+      int sl = items[P.diag].slot;
+      for (int g = 0; g < D.m_rz; ++g) {
+        if (!D.par[g]) continue;
+        s_op[sl] = items[P.diag].op + g;
+        s_fac[sl++] = items[P.diag].f;
+      }
+    }
+  }
+  pdl_begin();
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
@@ -502,22 +518,11 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
         cp_async16(&tp[tid + i * nt], &psi[k]);
         cp_async16(&tlam[tid + i * nt], &lam[k]);
       }
-    if (P.diag >= 0) {
-      if (!staged) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
-      diag_tile(D, P, outer);
-    }
+    if (P.diag >= 0) diag_tile(D, P, outer);
     for (int ch = nch - 1; ch >= 0; --ch) {
       const int base = ch * kChunk;
       const int cnt = min(kChunk, P.n_items - base);
-      if (!staged || nch > 1) {
-        if (tid < 32) {
-          stage_items(its, items + base, cnt, true);
-          if (!staged && tid < cnt && its[tid].slot >= 0 && its[tid].kind != F_DIAG) {
-            s_op[its[tid].slot] = its[tid].op;
-            s_fac[its[tid].slot] = its[tid].f;
-          }
-        }
-      }
+      if (nch > 1 && tid < 32) stage_items(its, items + base, cnt, true);
       if (ch == nch - 1) cp_async_wait_all();
       __syncthreads();
       for (int i = cnt - 1; i >= 0;) {
@@ -549,10 +554,6 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
               v = lb == lt ? hi[0] : lb == lt + 1 ? hi[1] : hi[2];
             }
             accp[sl * nt + tid] += v;
-            if (!staged && tid == 0) {
-              s_op[sl] = s.op + g;
-              s_fac[sl] = s.f;
-            }
             ++sl;
           }
           --i;
@@ -581,7 +582,6 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
         __syncthreads();
       }
     }
-    staged = true;
     if (f == 1.0) {
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -630,6 +630,7 @@ __global__ void __launch_bounds__(kFT) k_gpass(const double2* __restrict__ psi,
   const TileMap T = tile_map(P);
   items += P.first_item;
   for (int s = 0; s < P.n_slots; ++s) accp[s * nt + tid] = 0.0;
+  pdl_begin();
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
@@ -692,46 +693,49 @@ int pass_blocks(const FPass& P) {
 }
 
 cudaError_t fused_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(k_fpass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)fpass_smem(11));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_fpass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)fpass_smem(11));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_gpass, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bpass_smem(11, kMaxSlotsDev));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_bpass, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)bpass_smem(11, kMaxSlotsDev));
+  const int most = (int)std::max(kOnePerSm, bpass_smem(11, kMaxSlotsDev));
+  const void* ks[] = {(const void*)k_fpass<false>, (const void*)k_fpass<true>,
+                      (const void*)k_gpass, (const void*)k_bpass};
+  for (const void* k : ks) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
+namespace {
+template <class... P, class... A>
+cudaError_t launch_pass(void (*k)(P...), const FPass& F, size_t smem, cudaStream_t s, bool overlap,
+                        A... args) {
+  const int g = pass_blocks(F);
+  return launch_overlapped(k, g, pass_threads(F.m), spread_smem(smem, g), s, overlap, args...);
+}
+}  // namespace
+
 cudaError_t launch_fpass(double2* psi, const FPass& P, const SItem* items, const DOp* gops,
-                         const double2* cs, const double* scale, cudaStream_t s) {
-  k_fpass<false><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(psi, P, items, gops,
-                                                                           cs, scale);
-  return cudaGetLastError();
+                         const double2* cs, const double* scale, cudaStream_t s, bool overlap) {
+  return launch_pass(k_fpass<false>, P, fpass_smem(P.m), s, overlap, psi, P, items, gops, cs,
+                     scale);
 }
 
 cudaError_t launch_fpass_inv(double2* v, const FPass& P, const SItem* items, const DOp* gops,
-                             const double2* cs, const double* scale, cudaStream_t s) {
-  k_fpass<true><<<pass_blocks(P), pass_threads(P.m), fpass_smem(P.m), s>>>(v, P, items, gops,
-                                                                          cs, scale);
-  return cudaGetLastError();
+                             const double2* cs, const double* scale, cudaStream_t s,
+                             bool overlap) {
+  return launch_pass(k_fpass<true>, P, fpass_smem(P.m), s, overlap, v, P, items, gops, cs, scale);
 }
 
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const SItem* items, double* partial, cudaStream_t s) {
-  k_gpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(psi, lam, P, items,
-                                                                              partial);
-  return cudaGetLastError();
+                         const SItem* items, double* partial, cudaStream_t s, bool overlap) {
+  return launch_pass(k_gpass, P, bpass_smem(P.m, P.n_slots), s, overlap, psi, lam, P, items,
+                     partial);
 }
 
 cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const SItem* items,
                          const DOp* gops, const double2* cs, const double* scale, double* partial,
-                         cudaStream_t s) {
-  k_bpass<<<pass_blocks(P), pass_threads(P.m), bpass_smem(P.m, P.n_slots), s>>>(
-      psi, lam, P, items, gops, cs, scale, partial);
-  return cudaGetLastError();
+                         cudaStream_t s, bool overlap) {
+  return launch_pass(k_bpass, P, bpass_smem(P.m, P.n_slots), s, overlap, psi, lam, P, items, gops,
+                     cs, scale, partial);
 }
 
 }  // namespace svqe

@@ -72,6 +72,7 @@ template <int KIND>
 __global__ void __launch_bounds__(kThreads, 4) k_apply(double2* __restrict__ psi, uint64_t npairs,
                                                     DOp op, const Rot* __restrict__ coef,
                                                     int inv) {
+  pdl_begin();
   Rot r = *coef;
   if (inv) r = rot_inverse(r);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(double2* __restrict__ psi,
                                                       DOp op, const Rot* __restrict__ coef,
                                                       double* __restrict__ partial) {
   __shared__ double red[kThreads / 32];
+  pdl_begin();
   const Rot r = rot_inverse(*coef);
   const bool want = partial != nullptr;
   double acc = 0.0;
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(kThreads) k_hpsi(const double2* __restrict__ p
                                                    double* __restrict__ partial) {
   __shared__ DGroup sg[128];
   __shared__ double red[kThreads / 32];
+  pdl_begin();
   double e = 0.0;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t tile = kUnroll * stride;
@@ -245,6 +248,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_expval(const double2* __restric
                                                         const double2* __restrict__ tables,
                                                         double* __restrict__ partial) {
   __shared__ double red[kThreads / 32];
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int h_log = n - 1;  // N/2 pairs per group
   const int c_log = min(h_log, 5 + kEULog);
@@ -351,6 +355,7 @@ __global__ void k_finish(const DOp* __restrict__ ops, int n_ops,
                          double* __restrict__ energy, double* __restrict__ theta_upd, double lr,
                          double* __restrict__ traj) {
   __shared__ double red[32];
+  pdl_begin();
   if (blockIdx.x == gridDim.x - 1) {
     if (!epart) return;
     double v = 0.0;
@@ -406,16 +411,16 @@ cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Ro
 }
 
 cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef, bool inv,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool overlap) {
   const uint64_t npairs = 1ull << (n - op.k);
   const int g = grid_for(npairs);
   switch (kind_of(op.type)) {
-    case K_SWAP: k_apply<K_SWAP><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
-    case K_H: k_apply<K_H><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
-    case K_ROTY: k_apply<K_ROTY><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
-    case K_ROTX: k_apply<K_ROTX><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
-    case K_ROTZ: k_apply<K_ROTZ><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
-    case K_NEG: k_apply<K_NEG><<<g, kThreads, 0, s>>>(psi, npairs, op, coef, inv); break;
+    case K_SWAP: return launch_overlapped(k_apply<K_SWAP>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
+    case K_H: return launch_overlapped(k_apply<K_H>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
+    case K_ROTY: return launch_overlapped(k_apply<K_ROTY>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
+    case K_ROTX: return launch_overlapped(k_apply<K_ROTX>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
+    case K_ROTZ: return launch_overlapped(k_apply<K_ROTZ>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
+    case K_NEG: return launch_overlapped(k_apply<K_NEG>, g, kThreads, 0, s, overlap, psi, npairs, op, coef, inv);
   }
   return cudaGetLastError();
 }
@@ -423,28 +428,29 @@ cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef,
 int adjoint_blocks(int n, const DOp& op) { return grid_for(1ull << (n - op.k)); }
 
 cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, const Rot* coef,
-                              double* partial, cudaStream_t s) {
+                              double* partial, cudaStream_t s, bool overlap) {
   const uint64_t npairs = 1ull << (n - op.k);
   const int g = grid_for(npairs);
   switch (kind_of(op.type)) {
-    case K_SWAP: k_adjoint<K_SWAP><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, nullptr); break;
-    case K_H: k_adjoint<K_H><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, nullptr); break;
-    case K_ROTY: k_adjoint<K_ROTY><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, partial); break;
-    case K_ROTX: k_adjoint<K_ROTX><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, partial); break;
-    case K_ROTZ: k_adjoint<K_ROTZ><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, partial); break;
-    case K_NEG: k_adjoint<K_NEG><<<g, kThreads, 0, s>>>(psi, lam, npairs, op, coef, nullptr); break;
+    case K_SWAP: return launch_overlapped(k_adjoint<K_SWAP>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, (double*)nullptr);
+    case K_H: return launch_overlapped(k_adjoint<K_H>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, (double*)nullptr);
+    case K_ROTY: return launch_overlapped(k_adjoint<K_ROTY>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, partial);
+    case K_ROTX: return launch_overlapped(k_adjoint<K_ROTX>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, partial);
+    case K_ROTZ: return launch_overlapped(k_adjoint<K_ROTZ>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, partial);
+    case K_NEG: return launch_overlapped(k_adjoint<K_NEG>, g, kThreads, 0, s, overlap, psi, lam, npairs, op, coef, (double*)nullptr);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_hpsi(const double2* psi, double2* lam, int n, const DGroup* groups,
-                        int n_groups, const double2* tables, double* partial, cudaStream_t s) {
+                        int n_groups, const double2* tables, double* partial, cudaStream_t s,
+                        bool overlap) {
   const uint64_t N = 1ull << n;
   if (!lam && partial)
-    k_expval<<<kRedBlocks, kThreads, 0, s>>>(psi, n, groups, n_groups, tables, partial);
-  else
-    k_hpsi<<<kRedBlocks, kThreads, 0, s>>>(psi, lam, N, groups, n_groups, tables, partial);
-  return cudaGetLastError();
+    return launch_overlapped(k_expval, kRedBlocks, kThreads, 0, s, overlap, psi, n, groups, n_groups,
+                             tables, partial);
+  return launch_overlapped(k_hpsi, kRedBlocks, kThreads, 0, s, overlap, psi, lam, N, groups, n_groups,
+                           tables, partial);
 }
 
 cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream_t s) {
@@ -454,11 +460,10 @@ cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream
 
 cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
                           double* grad, const double* epart, double* energy, double* theta_upd,
-                          double lr, double* traj, cudaStream_t s) {
+                          double lr, double* traj, cudaStream_t s, bool overlap) {
   const int per = kThreads / 32;
-  k_finish<<<(n_params + per - 1) / per + 1, kThreads, 0, s>>>(
-      ops, n_ops, partial, n_params, grad, epart, energy, theta_upd, lr, traj);
-  return cudaGetLastError();
+  return launch_overlapped(k_finish, (n_params + per - 1) / per + 1, kThreads, 0, s, overlap, ops,
+                           n_ops, partial, n_params, grad, epart, energy, theta_upd, lr, traj);
 }
 
 }  // namespace svqe

@@ -12,9 +12,41 @@ namespace svqe {
 constexpr int kRedBlocks = 1216;  // 152 SMs x 8
 constexpr int kThreads = 256;
 
+// Launch a kernel that calls pdl_begin so that its blocks start, and run up to pdl_begin, while
+// the preceding kernel of the stream drains (programmatic dependent launch).  The gap between
+// two dependent kernels and the successor's set-up (staged items, index maps) are 4 to 6 us of
+// every pass over a state that sits in L2.
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t s,
+                              bool overlap, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
+// Shared memory that keeps a kernel to one block per SM.  An overlapped kernel's blocks are placed
+// while its predecessor's still run, so a grid of at most one block per SM would double up on the
+// SMs that free first and leave others idle: at 17 qubits (128 blocks, FP64-bound) that cost
+// 15 % of an evaluation.
+constexpr int kSms = 152;
+constexpr size_t kOnePerSm = 116 * 1024;
+inline size_t spread_smem(size_t smem, int grid) {
+  return grid <= kSms && smem < kOnePerSm ? kOnePerSm : smem;
+}
+
 cudaError_t launch_init_basis(double2* psi, int n, uint64_t b, cudaStream_t s);
 cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Rot* coefs,
                               cudaStream_t s);
+// Launchers below that take `overlap` must not be given it for the first kernel that reads what
+// launch_prep wrote.
 // Everything of a planned circuit that depends on theta, one block per unit (k_prep.cu): the
 // ops' lifting coefficients, the passes' items and scales, (cos, sin) of the RZ gates and the
 // phase tables (kDpTab entries each) of the whole-state segments on n qubits.
@@ -23,15 +55,16 @@ cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, cons
                         double2* cs, double2* dptab, cudaStream_t s);
 // Apply (inv = false) or un-apply one op on psi; coef points at the op's Rot.
 cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef, bool inv,
-                            cudaStream_t s);
+                            cudaStream_t s, bool overlap = false);
 // Adjoint step for one op: if the op is parameterised, partial[b] (b < adjoint_blocks(n, op))
 // receives block b's share of 2 Im<lambda|G|psi>; then psi and lambda are un-applied.
 int adjoint_blocks(int n, const DOp& op);
 cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, const Rot* coef,
-                              double* partial, cudaStream_t s);
+                              double* partial, cudaStream_t s, bool overlap = false);
 // lambda = H psi (if lam != nullptr) and partial[b] = block b's share of Re<psi|H psi>.
 cudaError_t launch_hpsi(const double2* psi, double2* lam, int n, const DGroup* groups,
-                        int n_groups, const double2* tables, double* partial, cudaStream_t s);
+                        int n_groups, const double2* tables, double* partial, cudaStream_t s,
+                        bool overlap = false);
 // out[0] = sum of partial[0..count) in a fixed order.
 cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream_t s);
 // The end of an evaluation, in one launch: grad[p] = sum over ops l with param p (in op order)
@@ -40,7 +73,7 @@ cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream
 // theta_upd[p] -= lr * grad[p] and (traj != nullptr) traj[0] = the energy.
 cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
                           double* grad, const double* epart, double* energy, double* theta_upd,
-                          double lr, double* traj, cudaStream_t s);
+                          double lr, double* traj, cudaStream_t s, bool overlap = false);
 
 }  // namespace svqe
 
@@ -56,10 +89,11 @@ int fused_tile_bits();
 cudaError_t fused_prepare();
 // items, scale (the pass's place) and cs as launch_prep wrote them.
 cudaError_t launch_fpass(double2* psi, const FPass& P, const SItem* items, const DOp* gops,
-                         const double2* cs, const double* scale, cudaStream_t s);
+                         const double2* cs, const double* scale, cudaStream_t s, bool overlap);
 // The pass's items inverted and in reverse order, on v (un-applying the pass).
 cudaError_t launch_fpass_inv(double2* v, const FPass& P, const SItem* items, const DOp* gops,
-                             const double2* cs, const double* scale, cudaStream_t s);
+                             const double2* cs, const double* scale, cudaStream_t s,
+                             bool overlap);
 // Blocks a pass launches: one per tile, at most kRedBlocks.
 int pass_blocks(const FPass& P);
 // Whole-state diagonal + permutation segment of the single-state path (k_dp.cu): a run of
@@ -82,26 +116,29 @@ struct DpArgs {
 };
 // CTAs of a segment's kernels on n qubits (a power of two).
 int dp_blocks(int n);
+cudaError_t dp_prepare();
 // log2 of the amplitudes per block of a segment's kernels on n qubits
 int dp_block_log(int n);
 // out[P(k)] = phase(k) in[k]
-cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s);
+cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
+                          bool overlap);
 // out[k] = conj(phase(k)) in[P(k)]
-cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s);
+cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
+                              bool overlap);
 // out[k] = conj(phase(k)) lam[P(k)]; RZ gradient shares from w_k = Im(conj(out[k]) psi_b[k])
 // into partial[op * kRedBlocks + block], block < dp_blocks(n)
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
-                              const DpArgs& a, double* partial, cudaStream_t s);
+                              const DpArgs& a, double* partial, cudaStream_t s, bool overlap);
 
 // Gradient shares only (psi and lambda unchanged) of a pass whose items are single ops:
 // partial[op * kRedBlocks + b] as for launch_bpass.
 cudaError_t launch_gpass(const double2* psi, const double2* lam, const FPass& P,
-                         const SItem* items, double* partial, cudaStream_t s);
+                         const SItem* items, double* partial, cudaStream_t s, bool overlap);
 // Backward pass: partial[op * kRedBlocks + b] receives block b's gradient share of every
 // parameterised op of the pass, for the pass_blocks(P) blocks launched.
 cudaError_t launch_bpass(double2* psi, double2* lam, const FPass& P, const SItem* items,
                          const DOp* gops, const double2* cs, const double* scale, double* partial,
-                         cudaStream_t s);
+                         cudaStream_t s, bool overlap);
 
 // One instance of a compiled batch (device record).  steps, lr and etraj_off are used when
 // BatchArgs::n_steps < 0 (per-instance step counts, as the serving loop runs them).

@@ -251,6 +251,16 @@ __device__ __forceinline__ int group_value(const DGroup& G, uint64_t k, const do
   return G.cls;
 }
 
+// ------------------------------------------------------------------------------ launch overlap
+// A kernel launched with launch_overlapped starts while its predecessor on the stream runs.
+// Before pdl_begin it may read only what kernels before that predecessor wrote (a kernel lets
+// its successor start after its own pdl_begin, so everything older is complete by then) and may
+// write no global memory.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ------------------------------------------------------------------------------ reductions
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
