@@ -74,6 +74,11 @@ struct sv_ctx {
     DpArgs dp;         // CH_DP
   };
   std::vector<Chunk> chunks;
+  // small registers (k_small): checkpoints, and pinned host memory the kernel writes results to
+  double2* ckpt = nullptr;
+  size_t ckpt_cap = 0;
+  double* pin = nullptr;
+  size_t pin_cap = 0;
   int tune = 0;         // sv_set_autotune
   int tile_bits = 11;   // tile size of the staged circuit's fused passes
 };
@@ -84,6 +89,7 @@ struct sv_ham {
   int n_groups = 0;
   DGroup* groups = nullptr;
   double2* tables = nullptr;
+  int n_table = 0;  // table entries
   size_t groups_cap = 0, tables_cap = 0;  // allocated records / table entries
   uint64_t bytes = 0;
   double l1 = 0.0;
@@ -221,6 +227,7 @@ sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
   }
   c->ref = 0;
   if (fused_prepare() != cudaSuccess || dp_prepare() != cudaSuccess ||
+      small_prepare() != cudaSuccess ||
       launch_init_basis(c->psi, n, 0, c->stream) != cudaSuccess) {
     set_error("init kernel launch failed");
     sv_destroy(c);
@@ -250,6 +257,8 @@ sv_status sv_destroy(sv_ctx* c) {
   cudaFree(c->etraj);
   for (double2* p : c->ck) cudaFree(p);
   cudaFree(c->scratch);
+  cudaFree(c->ckpt);
+  if (c->pin) cudaFreeHost(c->pin);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   cudaGetLastError();
   delete c;
@@ -277,6 +286,7 @@ static sv_status ham_fill(sv_ctx* c, sv_ham* H, const sv_paulisum* h) {
   H->n = c->n;
   H->device = c->device;
   H->n_groups = (int)hh.groups.size();
+  H->n_table = (int)hh.tables.size();
   H->l1 = hh.l1;
   H->bytes = H->groups_cap * sizeof(DGroup) + H->tables_cap * sizeof(double2);
   if (!hh.groups.empty())
@@ -458,14 +468,15 @@ static int single_op(const sv_ctx* c, int p);
 // fewer contiguous low bits (the state sits in L2, where a 16- or 32-byte access costs no burst)
 // leave its other bits for gate wires: two passes still cover every qubit of a layer.  Runs of
 // gates on many wires (excitations) that the smaller tile would cut into over half as many
-// passes again keep the larger one, a pass costing a few microseconds whatever its tiles.
+// passes again (and more than one) keep the larger one, a pass costing a few microseconds
+// whatever its tiles.
 static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan& plan) {
   plan_passes(ops, n, tile_bits, plan);
   const int m = std::max({n - 7, (n + 1) / 2, 4 + kMinLowBitsL2});  // (a gate has up to 4 wires)
   if (n > 17 || m >= tile_bits) return;
   HostPlan small;
   plan_passes(ops, n, m, small, std::max(0, std::min(kMinLowBitsL2, 2 * m - n)));
-  if (2 * small.passes.size() <= 3 * plan.passes.size()) std::swap(plan, small);
+  if (2 * small.passes.size() <= 3 * plan.passes.size() + 2) std::swap(plan, small);
 }
 
 // Fused-pass plan of a staged circuit with tiles of tile_bits bits (see stage_circuit), and its
@@ -826,6 +837,119 @@ sv_status sv_tile_bits(const sv_ctx* c, int32_t* tile_bits) {
   return SV_OK;
 }
 
+// ------------------------------------------------------------------------------ small registers
+// Small registers are evaluated by one block in one launch (k_small, the batched kernel's
+// routine) instead of some twenty launches; descent steps loop inside it.  A context does so up
+// to kSmallQubits: one block's time doubles with each qubit and the passes' does not (four
+// hardware-efficient layers, one block against passes: 113 and 188 us at 8 qubits, 187 and 303
+// at 10, 313 and 292 at 11, 573 and 244 at 12).  The call without device allocation, which has
+// no passes and launches every gate, does up to the 12 qubits the routine holds.
+static constexpr int kSmallQubits = 10;
+static constexpr int64_t kSmallCkptAmps = 1 << 19;  // 8 MiB of checkpoint scratch at most
+
+bool svqe::pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
+                      const double* theta, SmallPack& out) {
+  if (hc.n > SV_BATCH_MAX_QUBITS) return false;
+  std::vector<DOp> ops(hc.ops);
+  std::vector<Seg> segs;
+  const int n_ckpt = segment_ops(ops, 2, 3, segs);
+  out.ckpt_amps = team_ckpt_amps(n_ckpt, hc.n);
+  const int P = hc.n_params, G = (int)ops.size();
+  auto align = [](size_t v) { return (v + 15) / 16 * 16; };
+  const size_t o_ops = sizeof(BInst);
+  const size_t o_segs = align(o_ops + G * sizeof(DOp));
+  const size_t o_pptr = align(o_segs + segs.size() * sizeof(Seg));
+  const size_t o_pops = align(o_pptr + ((size_t)P + 1) * sizeof(int32_t));
+  const size_t o_theta = align(o_pops + (size_t)G * sizeof(int32_t));
+  const size_t bytes = align(o_theta + (theta ? (size_t)P * sizeof(double) : 0));
+  if (out.ckpt_amps > kSmallCkptAmps || bytes > (100u << 10) ||
+      small_smem(hc.n, G, P, (int)bytes) > (200u << 10))
+    return false;
+  SmallArgs& A = out.args;
+  std::memset(&A, 0, offsetof(SmallArgs, blob));
+  unsigned char* b = A.blob;
+  if (bytes > kSmallBlob) {
+    out.blob.resize(bytes);
+    b = out.blob.data();
+  }
+  BInst I{};
+  I.n = hc.n;
+  I.n_ops = G;
+  I.n_params = P;
+  I.n_segs = (int)segs.size();
+  I.n_ckpt = n_ckpt;
+  I.ref = ref;
+  I.n_groups = n_groups;
+  I.tab_n = n_table;
+  std::memcpy(b, &I, sizeof I);
+  if (G) std::memcpy(b + o_ops, ops.data(), G * sizeof(DOp));
+  if (!segs.empty()) std::memcpy(b + o_segs, segs.data(), segs.size() * sizeof(Seg));
+  // parameter -> ops using it, in op order (CSR)
+  int32_t* pptr = reinterpret_cast<int32_t*>(b + o_pptr);
+  int32_t* pops = reinterpret_cast<int32_t*>(b + o_pops);
+  std::fill(pptr, pptr + P + 1, 0);
+  for (const DOp& op : ops)
+    if (op.param >= 0) ++pptr[op.param + 1];
+  for (int p = 0; p < P; ++p) pptr[p + 1] += pptr[p];
+  std::vector<int32_t> at(pptr, pptr + P);
+  for (int l = 0; l < G; ++l)
+    if (ops[l].param >= 0) pops[at[ops[l].param]++] = l;
+  if (theta && P) std::memcpy(b + o_theta, theta, (size_t)P * sizeof(double));
+  A.nw = small_warps(hc.n);
+  A.n = hc.n;
+  A.n_ops = G;
+  A.n_params = P;
+  A.blob_bytes = (int)bytes;
+  A.o_ops = (int)o_ops;
+  A.o_segs = (int)o_segs;
+  A.o_pptr = (int)o_pptr;
+  A.o_pops = (int)o_pops;
+  A.o_theta = theta ? (int)o_theta : -1;
+  A.a.n_inst = 1;
+  return true;
+}
+
+static sv_status grow_pinned(sv_ctx* c, size_t need) {
+  if (need <= c->pin_cap) return SV_OK;
+  if (c->pin) cudaFreeHost(c->pin);
+  c->pin = nullptr;
+  c->pin_cap = 0;
+  const size_t cap = std::max<size_t>(need, 512);
+  if (cudaHostAlloc((void**)&c->pin, cap * sizeof(double), cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    c->pin = nullptr;
+    set_error("pinned allocation of %llu bytes failed", (unsigned long long)(cap * sizeof(double)));
+    return SV_ENOMEM;
+  }
+  c->pin_cap = cap;
+  return SV_OK;
+}
+
+// Launch a packed circuit on the context (see pack_small): energy and gradient (nullptr: not
+// wanted) of one evaluation, or n_steps > 0 descent steps with their energies in etraj.
+static sv_status run_small(sv_ctx* c, SmallPack& S, const sv_ham* H, double* energy, double* grad,
+                           int n_steps, double lr, double* etraj) {
+  SmallArgs& A = S.args;
+  SV_CUDA(grow(c->ckpt, c->ckpt_cap, (size_t)S.ckpt_amps), c);
+  if (!S.blob.empty()) {
+    SV_CUDA(grow(c->blob, c->blob_cap, S.blob.size()), c);
+    SV_CUDA(cudaMemcpyAsync(c->blob, S.blob.data(), S.blob.size(), cudaMemcpyHostToDevice,
+                            c->stream), c);
+    A.blob_dev = c->blob;
+  }
+  A.a.groups = H->groups;
+  A.a.tables = H->tables;
+  A.a.ckpt = c->ckpt;
+  A.a.energy = energy;
+  A.a.grad = grad;
+  A.a.n_steps = n_steps;
+  A.a.lr = lr;
+  A.a.etraj = etraj;
+  A.ref_out = c->psi;
+  SV_CUDA(launch_small(A, c->stream), c);
+  return SV_OK;
+}
+
 // psi = |ref>, forward, lambda = H psi, adjoint sweep; energy -> energy_dev[0], gradient ->
 // grad_dev; with theta_upd set also the descent step (see launch_finish).  Everything stream-ordered on c->stream.
 sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
@@ -952,6 +1076,11 @@ sv_status sv_adjoint_grad_dev(sv_ctx* c, const sv_circuit* circ, const double* t
   sv_status st = lower_circuit(circ, c->n, hc);
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && (!theta_dev || !grad_dev)) { set_error("theta/grad is NULL"); return SV_EINVAL; }
+  SmallPack sp;
+  if (c->n <= kSmallQubits && pack_small(hc, c->ref, H->n_groups, H->n_table, nullptr, sp)) {
+    sp.args.a.theta = const_cast<double*>(theta_dev);
+    return run_small(c, sp, H, energy_dev, grad_dev, 0, 0.0, nullptr);
+  }
   if ((st = stage_circuit(c, hc, true)) != SV_OK) return st;
   return adjoint_core(c, hc, H, theta_dev, energy_dev, grad_dev);
 }
@@ -966,6 +1095,16 @@ sv_status sv_adjoint_grad(sv_ctx* c, const sv_circuit* circ, const double* theta
   sv_status st = lower_circuit(circ, c->n, hc);
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && (!theta || !grad_out)) { set_error("theta/grad is NULL"); return SV_EINVAL; }
+  SmallPack sp;
+  if (c->n <= kSmallQubits &&
+      pack_small(hc, c->ref, H->n_groups, H->n_table, hc.n_params ? theta : nullptr, sp)) {
+    if ((st = grow_pinned(c, (size_t)hc.n_params + 1)) != SV_OK) return st;
+    if ((st = run_small(c, sp, H, c->pin, c->pin + 1, 0, 0.0, nullptr)) != SV_OK) return st;
+    SV_CUDA(cudaStreamSynchronize(c->stream), c);
+    *energy_out = c->pin[0];
+    if (hc.n_params) std::memcpy(grad_out, c->pin + 1, hc.n_params * sizeof(double));
+    return SV_OK;
+  }
   if ((st = stage_circuit(c, hc, true)) != SV_OK) return st;
   if (hc.n_params)
     SV_CUDA(cudaMemcpyAsync(c->theta, theta, hc.n_params * sizeof(double),
@@ -1015,6 +1154,20 @@ sv_status vqe_step(sv_ctx* c, const sv_circuit* circ, const sv_ham* H, double* t
   sv_status st = lower_circuit(circ, c->n, hc);
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && !theta_inout) { set_error("theta is NULL"); return SV_EINVAL; }
+  SmallPack sp;
+  if (n_steps > 0 && c->n <= kSmallQubits &&
+      pack_small(hc, c->ref, H->n_groups, H->n_table, hc.n_params ? theta_inout : nullptr, sp)) {
+    // theta moves in shared memory from step to step; it and the energies come back pinned
+    const size_t P = (size_t)hc.n_params;
+    if ((st = grow_pinned(c, P + n_steps + 1)) != SV_OK) return st;
+    sp.args.theta_out = P ? c->pin : nullptr;
+    if ((st = run_small(c, sp, H, c->pin + P, nullptr, n_steps, lr, c->pin + P + 1)) != SV_OK)
+      return st;
+    SV_CUDA(cudaStreamSynchronize(c->stream), c);
+    if (P) std::memcpy(theta_inout, c->pin, P * sizeof(double));
+    if (energy_out) std::memcpy(energy_out, c->pin + P + 1, n_steps * sizeof(double));
+    return SV_OK;
+  }
   if ((st = vqe_enqueue(c, hc, H, theta_inout, lr, n_steps, theta_inout, energy_out)) != SV_OK)
     return st;
   SV_CUDA(cudaStreamSynchronize(c->stream), c);

@@ -26,6 +26,17 @@ sv_status adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
 // are written when the stream reaches them (pinned host memory for real asynchrony).
 sv_status vqe_enqueue(sv_ctx* c, const HostCircuit& hc, const sv_ham* H, const double* theta_in,
                       double lr, int32_t n_steps, double* theta_out, double* energy_out);
+// A circuit packed for launch_small: the argument block (a.ckpt, a.theta, results and the
+// Hamiltonian's arrays are the caller's to set), the blob when it exceeds kSmallBlob, and the
+// amplitudes of checkpoint scratch it needs.  theta (host, or nullptr) goes into the blob.
+// Returns false for a register or circuit that k_small does not take.
+struct SmallPack {
+  SmallArgs args;
+  std::vector<unsigned char> blob;
+  int64_t ckpt_amps;
+};
+bool pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
+                const double* theta, SmallPack& out);
 cudaStream_t ctx_stream(sv_ctx* c);
 // Replace the Pauli sum held by H (lowered for c's register), reusing H's device buffers when
 // they are large enough, so that a pooled context takes a new request without allocating.

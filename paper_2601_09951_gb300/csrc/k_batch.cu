@@ -1092,7 +1092,63 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch(BatchArgs a) {
   }
 }
 
+// One instance, one team, one block (see SmallArgs).
+__global__ void __launch_bounds__(kBatchThreads, 1) k_small(const __grid_constant__ SmallArgs p) {
+  extern __shared__ double2 sm[];
+  __shared__ TeamS S;
+  const uint32_t N = 1u << p.n;
+  // psi, lambda, the blob, coefficients, per-op gradients, gradient
+  unsigned char* blob = reinterpret_cast<unsigned char*>(sm + 2 * N);
+  const int bw = (p.blob_bytes + 15) >> 4;
+  const uint4* src = reinterpret_cast<const uint4*>(p.blob_dev ? p.blob_dev : p.blob);
+  for (int i = threadIdx.x; i < bw; i += blockDim.x) reinterpret_cast<uint4*>(blob)[i] = src[i];
+  BatchArgs a = p.a;
+  a.inst = reinterpret_cast<const BInst*>(blob);
+  a.ops = reinterpret_cast<const DOp*>(blob + p.o_ops);
+  a.segs = reinterpret_cast<const Seg*>(blob + p.o_segs);
+  a.pptr = reinterpret_cast<const int32_t*>(blob + p.o_pptr);
+  a.pops = reinterpret_cast<const int32_t*>(blob + p.o_pops);
+  if (p.o_theta >= 0) a.theta = reinterpret_cast<double*>(blob + p.o_theta);
+  a.coef = reinterpret_cast<Rot*>(blob + 16 * (size_t)bw);
+  a.contrib = reinterpret_cast<double*>(a.coef + p.n_ops);
+  if (!a.grad) a.grad = a.contrib + p.n_ops;
+  Team T;
+  T.nw = p.nw;
+  T.size = p.nw * 32;
+  T.log_size = 31 - __clz(T.size);
+  T.rank = threadIdx.x;
+  T.w = threadIdx.x >> 5;
+  T.bar = 1;
+  __syncthreads();
+  run_instance(a, 0, T, S, sm, a.ckpt);
+  if (p.theta_out)
+    for (int i = threadIdx.x; i < p.n_params; i += blockDim.x) p.theta_out[i] = a.theta[i];
+  if (p.ref_out) {
+    const uint32_t ref = (uint32_t)a.inst->ref;
+    for (uint32_t k = threadIdx.x; k < N; k += blockDim.x)
+      p.ref_out[k] = make_double2(k == ref ? 1.0 : 0.0, 0.0);
+  }
+}
+
 }  // namespace
+
+// A warp per 32 to 64 amplitudes: below, lanes idle while every FP64 instruction still takes a
+// warp's issue slots; above, one SMSP's pipe does what four could.
+int small_warps(int n) { return n <= 5 ? 1 : n <= 7 ? 2 : n == 8 ? 4 : 8; }
+
+size_t small_smem(int n, int n_ops, int n_params, int blob_bytes) {
+  return ((size_t)2 << n) * sizeof(double2) + (size_t)((blob_bytes + 15) / 16) * 16 +
+         (size_t)n_ops * (sizeof(Rot) + sizeof(double)) + (size_t)n_params * sizeof(double) + 16;
+}
+
+cudaError_t small_prepare() {
+  return cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+}
+
+cudaError_t launch_small(const SmallArgs& a, cudaStream_t s) {
+  k_small<<<1, 32 * a.nw, small_smem(a.n, a.n_ops, a.n_params, a.blob_bytes), s>>>(a);
+  return cudaGetLastError();
+}
 
 size_t batch_smem_bytes(int nmax) {
   (void)nmax;

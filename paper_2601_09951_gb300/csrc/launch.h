@@ -84,7 +84,7 @@ namespace svqe {
 // Whole-state diagonal + permutation segments (k_dp.cu) are used from kDpMinQubits: below,
 // a layer's RZ and CNOT gates fit one fused pass or two.
 constexpr int kFusedMinQubits = 1;
-constexpr int kDpMinQubits = 12;
+constexpr int kDpMinQubits = 11;
 int fused_tile_bits();
 cudaError_t fused_prepare();
 // items, scale (the pass's place) and cs as launch_prep wrote them.
@@ -212,6 +212,30 @@ constexpr int kDpAuxAmps = 176;
 inline int64_t team_ckpt_amps(int n_ckpt, int n) {
   return (int64_t)n_ckpt * ((int64_t(1) << n) + kDpAuxAmps);
 }
+
+// One instance alone, in one launch of one team (k_small): the single-state path of small
+// registers.  Its records (BInst, ops, segments, parameter uses and, for host callers, theta)
+// travel as a launch argument when they fit kSmallBlob bytes, else from blob_dev, and live in
+// shared memory with the coefficients, so a step reads nothing from global memory but the
+// Hamiltonian and its checkpoints.  Byte offsets into the blob; o_theta < 0: a.theta is used.
+constexpr int kSmallBlob = 3584;
+struct SmallArgs {
+  BatchArgs a;  // inst, ops, segs, pptr, pops, coef and contrib are set by the kernel
+  int nw;       // warps
+  int n, n_ops, blob_bytes;
+  int o_ops, o_segs, o_pptr, o_pops, o_theta;
+  int n_params;
+  const unsigned char* blob_dev;
+  double* theta_out;  // final theta, or nullptr
+  double2* ref_out;   // 2^n amplitudes that receive the reference state, or nullptr
+  alignas(16) unsigned char blob[kSmallBlob];
+};
+static_assert(sizeof(SmallArgs) <= 4096, "the argument block stays within 4 KB");
+// Warps of an n-qubit instance run alone, and the shared memory of such a launch.
+int small_warps(int n);
+size_t small_smem(int n, int n_ops, int n_params, int blob_bytes);
+cudaError_t small_prepare();
+cudaError_t launch_small(const SmallArgs& a, cudaStream_t s);
 
 // Threads per CTA of the batched kernel and its dynamic shared memory for nmax qubits.
 constexpr int kBatchThreads = 256;

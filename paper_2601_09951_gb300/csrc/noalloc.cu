@@ -23,9 +23,12 @@
 // psi, lambda or the caller's table.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cstring>
 #include <mutex>
 
 #include "../../include/svqe.h"
+#include "api_internal.h"
 #include "host_compile.h"
 #include "launch.h"
 #include "svqe_types.h"
@@ -96,16 +99,28 @@ sv_status scratch_address(unsigned char** out) {
     }                                                                                    \
   } while (0)
 
-// Op records travel to the device as kernel parameters (by value, copied at launch), so the
+// Records travel to the device as kernel parameters (by value, copied at launch), so the
 // upload reads no host memory after the call returns.
-constexpr int kOpChunk = 64;
-struct OpChunk {
-  DOp op[kOpChunk];
+constexpr int kPutWords = 250;  // 16-byte words
+struct PutChunk {
+  uint4 w[kPutWords];
 };
-static_assert(sizeof(OpChunk) <= 4096, "op chunk must stay a small kernel parameter");
+static_assert(sizeof(PutChunk) <= 4064, "a chunk must stay a small kernel parameter");
 
-__global__ void k_na_put_ops(OpChunk c, DOp* __restrict__ dst, int count) {
-  for (int i = threadIdx.x; i < count; i += blockDim.x) dst[i] = c.op[i];
+__global__ void k_na_put(const __grid_constant__ PutChunk c, uint4* __restrict__ dst, int count) {
+  for (int i = threadIdx.x; i < count; i += blockDim.x) dst[i] = c.w[i];
+}
+
+cudaError_t put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  for (size_t o = 0; o < bytes; o += sizeof(PutChunk)) {
+    PutChunk c;
+    const size_t cnt = std::min(sizeof(PutChunk), bytes - o);
+    std::memcpy(&c, (const unsigned char*)src + o, cnt);
+    k_na_put<<<1, 256, 0, s>>>(c, (uint4*)((unsigned char*)dst + o), (int)((cnt + 15) / 16));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Checks every caller record (x_mask and z_union inside the n-qubit register, a known class,
@@ -224,17 +239,34 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
   unsigned* flag = (unsigned*)(base + kOffFlag);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n_ops = (int)hc.ops.size();
-  for (DOp& op : hc.ops) op.flags = adjoint_blocks(n, op);
-  for (int i0 = 0; i0 < n_ops; i0 += kOpChunk) {
-    OpChunk c;
-    const int cnt = n_ops - i0 < kOpChunk ? n_ops - i0 : kOpChunk;
-    for (int i = 0; i < cnt; ++i) c.op[i] = hc.ops[i0 + i];
-    k_na_put_ops<<<1, kOpChunk, 0, s>>>(c, ops + i0, cnt);
-    NA_CUDA(cudaGetLastError());
-  }
   k_na_check_groups<<<1, 1024, 0, s>>>(groups_dev, n_groups, n, (long long)n_table, groups,
                                        flag);
   NA_CUDA(cudaGetLastError());
+  // Small registers run in one launch (k_small), its checkpoints and records in the part of the
+  // array that holds states and partials otherwise.
+  SmallPack sp;
+  const int n_pref = (int)std::min<int64_t>(n_table, 1 << 20);
+  if (pack_small(hc, ref, n_groups, n_pref, nullptr, sp) &&
+      align256(sp.blob.size()) + (size_t)sp.ckpt_amps * sizeof(double2) <= kOffGroups) {
+    SmallArgs& A = sp.args;
+    if (!sp.blob.empty()) {
+      NA_CUDA(put_bytes(base, sp.blob.data(), sp.blob.size(), s));
+      A.blob_dev = base;
+    }
+    A.a.groups = groups;
+    A.a.tables = (const double2*)tables_dev;
+    A.a.ckpt = (double2*)(base + align256(sp.blob.size()));
+    A.a.theta = const_cast<double*>(theta_dev);
+    A.a.energy = energy_dev;
+    A.a.grad = grad_dev;
+    NA_CUDA(small_prepare());
+    NA_CUDA(launch_small(A, s));
+    k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
+    NA_CUDA(cudaGetLastError());
+    return SV_OK;
+  }
+  for (DOp& op : hc.ops) op.flags = adjoint_blocks(n, op);
+  NA_CUDA(put_bytes(ops, hc.ops.data(), n_ops * sizeof(DOp), s));
   NA_CUDA(launch_init_basis(psi, n, ref, s));
   NA_CUDA(launch_prep_coefs(ops, n_ops, theta_dev, coef, s));
   for (int l = 0; l < n_ops; ++l) NA_CUDA(launch_apply_op(psi, n, hc.ops[l], coef + l, false, s));

@@ -1,4 +1,6 @@
-"""GPU parity of the fused passes at the edges of their rules: registers on both sides of the tile
+"""GPU parity of the single-state path at the edges of its rules: registers on both sides of the
+one-block limit (10 qubits; records that fit the launch's arguments and records that do not) and
+of the tile
 rule (tiles of n - 7 bits below 18 qubits), angles on both sides of the quarter turns where the
 unnormalised rotations change form, RY and RX gates that share a trip or repeat a qubit, and
 passes of more items than are staged at a time.  Tolerances as in tests/parity.py."""
@@ -45,7 +47,8 @@ def _circuit(n, rng, n_rot, n_swap):
 
 
 @pytest.mark.parametrize("n,n_rot,n_swap", [(1, 6, 3), (2, 9, 70), (5, 12, 33), (6, 20, 40),
-                                            (7, 20, 0), (12, 24, 35), (13, 24, 70), (14, 20, 3),
+                                            (7, 20, 0), (7, 150, 9), (8, 20, 3), (9, 60, 2),
+                                            (10, 12, 3), (10, 120, 70), (11, 30, 8), (12, 24, 35), (13, 24, 70), (14, 20, 3),
                                             (17, 10, 40), (18, 8, 0)])
 def test_pass_edges(n, n_rot, n_swap):
     rng = np.random.default_rng(900 + n)
@@ -73,3 +76,24 @@ def test_pass_edges(n, n_rot, n_swap):
     e0, g0 = oracle.energy_grad(inst)
     assert_energy(e, e0, inst["ham"], f"n={n}")
     assert_grad(g, g0, inst["ham"], f"n={n}")
+
+
+@pytest.mark.parametrize("n,layers", [(3, 1), (5, 30), (8, 2), (10, 3), (11, 2)])
+def test_descent_steps_match_single_evaluations(n, layers):
+    """vqe_step's trajectory (inside one launch up to 10 qubits) against adjoint_grad at each of
+    its own points, and the reference state left behind."""
+    inst = W.tfim_instance(n, layers)
+    ctx = svqe.Context(n)
+    ctx.init_reference(1)
+    H = svqe.Ham(ctx, inst["ham"])
+    lr = 0.3 / np.abs(inst["ham"]["coeff"]).sum()
+    theta, energies = ctx.vqe_step(inst["circuit"], H, inst["theta"], lr, 6)
+    ref = np.zeros(1 << n, np.complex128)
+    ref[1] = 1.0
+    assert np.max(np.abs(ctx.get_state() - ref)) <= PSI_TOL
+    th = np.array(inst["theta"])
+    for e_step in energies:
+        e, g = ctx.adjoint_grad(inst["circuit"], th, H)
+        assert_energy(e_step, e, inst["ham"])
+        th = th - lr * g
+    np.testing.assert_allclose(theta, th, rtol=0, atol=1e-11)
