@@ -205,12 +205,14 @@ int segment_ops(std::vector<DOp>& ops, int min_layer, int min_diag_rz,
   for (Seg& s : merged)
     s.ckpt = (s.kind == SEG_GATES || (s.kind == SEG_RLAYER && s.split == 1)) ? -1 : ckpt++;
   segs.swap(merged);
-  for (DOp& op : ops) op.flags &= ~kOpCS;
+  for (DOp& op : ops) op.flags &= ~(kOpCS | kOpT);
   for (const Seg& s : segs) {
     if (s.kind == SEG_RLAYER && s.split == 1) {
       for (int l = s.first; l < s.first + s.count; ++l) ops[l].flags |= kOpCS;
       continue;
     }
+    if (s.kind == SEG_RLAYER)
+      for (int l = s.first; l < s.first + s.count; ++l) ops[l].flags |= kOpT;
     if (s.kind != SEG_DIAG && s.kind != SEG_DIAGPERM) continue;
     const int nd = s.kind == SEG_DIAG ? s.count : s.split;
     for (int l = s.first; l < s.first + nd; ++l)

@@ -31,11 +31,12 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kM = 16;  // values reduced at once (kMaxLayer)
 constexpr int kWarps = kBatchThreads / 32;
 
-// A single-qubit gate of a commuting layer: its coefficients, type and qubit bit.
+// A single-qubit gate of a commuting layer: its unnormalised rotation (see RotT), type and
+// qubit bit.
 struct LOp {
-  Rot r;
-  int type;
-  int bit;
+  double t;
+  int mode, type, bit;
+  int pad;
 };
 
 // Per-team scratch in static shared memory.  Its first kDpBlockAmps x 16 bytes (tl .. n_rz)
@@ -311,8 +312,10 @@ __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;"
 __device__ __forceinline__ void layer_setup(const Team& T, TeamS& S, const DOp* ops,
                                             const Rot* coef, const Seg& sg) {
   if (T.rank < sg.count) {
+    const Rot r = coef[sg.first + T.rank];
     LOp o;
-    o.r = coef[sg.first + T.rank];
+    o.t = r.a;
+    o.mode = r.k;
     o.type = ops[sg.first + T.rank].type;
     o.bit = ops[sg.first + T.rank].bit0;
     S.lop[T.rank] = o;
@@ -320,38 +323,54 @@ __device__ __forceinline__ void layer_setup(const Team& T, TeamS& S, const DOp* 
   T.sync();
 }
 
+// The product of the factors a commuting layer's gates leave out, by one warp (at most 16
+// gates), the same value in every lane.
+__device__ __forceinline__ double layer_scale(const Rot* coef, const Seg& sg) {
+  const int lane = threadIdx.x & 31;
+  double h = 1.0, l = 0.0;
+  if (lane < sg.count) {
+    const Rot r = coef[sg.first + lane];
+    h = r.b;
+    l = (double)__int_as_float(r.pad);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const double bh = __shfl_xor_sync(kFull, h, o), bl = __shfl_xor_sync(kFull, l, o);
+    dd_mul(h, l, bh, bl);
+  }
+  return __shfl_sync(kFull, h + l, 0);
+}
+
 // One staged layer gate on v (inv: its inverse).
 __device__ __forceinline__ void lop_pass(const Team& T, double2* v, uint32_t N, const LOp& o,
                                          bool inv) {
   const uint32_t fl = 1u << o.bit, low = fl - 1u;
+  const bool rx = o.type == SV_GATE_RX;
+  const int mode = inv && o.mode ? 2 : o.mode;
+  const double t = inv && !o.mode ? dneg(o.t) : o.t;
+  const RotY r = make_roty(o.t, o.mode, fl, inv);
   for (uint32_t p = T.rank; p < (N >> 1); p += T.size) {
     const uint32_t i = ((p & ~low) << 1) | (p & low);
-    double2 x = v[i], y = v[i | fl];
-    pair_apply(o.type, o.r, inv, x, y);
+    const uint32_t j = rx ? i : i ^ r.swap;
+    double2 x = v[j], y = v[j ^ fl];
+    if (rx) {
+      pair_t<true>(mode, t, x, y);
+    } else {
+      rot_y(r.t, x, y);
+      x = flip_sign(x, r.neg0);
+      y = flip_sign(y, r.neg1);
+    }
     v[i] = x;
     v[i | fl] = y;
   }
 }
 
-// One layer gate on a pair, with the rotation (and its inverse, for RX) prepared: RY rotates
-// (re x, re y) and (im x, im y) by R(phi); RX rotates (re x, im y) by R(-phi) and (im x, re y)
-// by R(phi).
-template <bool ROTX>
-__device__ __forceinline__ void layer_pair(const Rot& r, const Rot& m, double2& x, double2& y) {
-  if (ROTX) {
-    rot_apply(m, x.x, y.y);
-    rot_apply(r, x.y, y.x);
-  } else {
-    rot_apply(r, x.x, y.x);
-    rot_apply(r, x.y, y.y);
-  }
-}
-
 // Two staged layer gates on distinct bits in one pass: each thread takes the four amplitudes of
 // a block (both bits 0, either, both 1), rotates them for the first gate, then for the second,
-// in registers (inverse: inverted, in reverse order).  A layer is all RY or all RX.  If ckout
-// is set, the amplitudes are also stored there unchanged first: the pass doubles as the
-// checkpoint copy.
+// in registers (inv: both inverted).  A layer is all RY or all RX.  If ckout is set, the
+// amplitudes are also stored there unchanged first: the pass doubles as the checkpoint copy.
+// With a branch on the rotations' form in the loop the passes, two FMAs per pair against three,
+// were slower than the shears; RY gates therefore take theirs through addresses and signs.
 template <bool ROTX>
 __device__ __forceinline__ void lop_pass2_k(const Team& T, double2* v, uint32_t N, const LOp& o1,
                                             const LOp& o2, bool inv, double2* ckout) {
@@ -359,27 +378,33 @@ __device__ __forceinline__ void lop_pass2_k(const Team& T, double2* v, uint32_t 
   uint8_t sb[2];
   sb[0] = (uint8_t)min(o1.bit, o2.bit);
   sb[1] = (uint8_t)max(o1.bit, o2.bit);
-  const Rot r1 = inv ? rot_inverse(o1.r) : o1.r, r2 = inv ? rot_inverse(o2.r) : o2.r;
-  const Rot m1 = rot_inverse(r1), m2 = rot_inverse(r2);
+  const int m1 = inv && o1.mode ? 2 : o1.mode, m2 = inv && o2.mode ? 2 : o2.mode;
+  const double t1 = inv && !o1.mode ? dneg(o1.t) : o1.t, t2 = inv && !o2.mode ? dneg(o2.t) : o2.t;
+  const RotY r1 = make_roty(o1.t, o1.mode, b1, inv), r2 = make_roty(o2.t, o2.mode, b2, inv);
+  const uint32_t sw = ROTX ? 0u : r1.swap ^ r2.swap;
   for (uint32_t p = T.rank; p < (N >> 2); p += T.size) {
-    const uint32_t i = insert_zeros32(p, sb, 2);
-    double2 a = v[i], b = v[i | b1], c = v[i | b2], d = v[i | b1 | b2];
+    const uint32_t i = insert_zeros32(p, sb, 2), j = i ^ sw;
+    double2 a = v[j], b = v[j ^ b1], c = v[j ^ b2], d = v[j ^ b1 ^ b2];
     if (ckout) {
-      ckout[i] = a;
-      ckout[i | b1] = b;
-      ckout[i | b2] = c;
-      ckout[i | b1 | b2] = d;
+      ckout[j] = a;
+      ckout[j ^ b1] = b;
+      ckout[j ^ b2] = c;
+      ckout[j ^ b1 ^ b2] = d;
     }
-    if (!inv) {
-      layer_pair<ROTX>(r1, m1, a, b);
-      layer_pair<ROTX>(r1, m1, c, d);
-      layer_pair<ROTX>(r2, m2, a, c);
-      layer_pair<ROTX>(r2, m2, b, d);
+    if (ROTX) {
+      pair_t<true>(m1, t1, a, b);
+      pair_t<true>(m1, t1, c, d);
+      pair_t<true>(m2, t2, a, c);
+      pair_t<true>(m2, t2, b, d);
     } else {
-      layer_pair<ROTX>(r2, m2, a, c);
-      layer_pair<ROTX>(r2, m2, b, d);
-      layer_pair<ROTX>(r1, m1, a, b);
-      layer_pair<ROTX>(r1, m1, c, d);
+      rot_y(r1.t, a, b);
+      rot_y(r1.t, c, d);
+      rot_y(r2.t, a, c);
+      rot_y(r2.t, b, d);
+      a = flip_sign(a, r1.neg0 ^ r2.neg0);
+      b = flip_sign(b, r1.neg1 ^ r2.neg0);
+      c = flip_sign(c, r1.neg0 ^ r2.neg1);
+      d = flip_sign(d, r1.neg1 ^ r2.neg1);
     }
     v[i] = a;
     v[i | b1] = b;
@@ -394,10 +419,35 @@ __device__ __forceinline__ void lop_pass2(const Team& T, double2* v, uint32_t N,
   else lop_pass2_k<false>(T, v, N, o1, o2, inv, ckout);
 }
 
+// A staged layer on v (inv: its inverse; the gates commute), the result multiplied by scale.
+// Ends with the team synchronised.
+__device__ __forceinline__ void layer_pass(const Team& T, TeamS& S, double2* v, uint32_t N,
+                                           int count, bool inv, double scale, double2* ckout) {
+  int g = 0;
+  for (; g + 1 < count; g += 2) {
+    lop_pass2(T, v, N, S.lop[g], S.lop[g + 1], inv, g == 0 ? ckout : nullptr);
+    T.sync();
+  }
+  if (g < count) {
+    lop_pass(T, v, N, S.lop[g], inv);
+    T.sync();
+  }
+  // (a loop of its own: inside the passes it becomes multiplications that always issue)
+  if (scale != 1.0) {
+    for (uint32_t k = T.rank; k < N; k += T.size) {
+      const double2 a = v[k];
+      v[k] = make_double2(scale * a.x, scale * a.y);
+    }
+    T.sync();
+  }
+}
+
 // Build the diagonal segment's half tables: th[hi] * tl[lo] = prod_RZ e^{-i phi s(k)}, and
 // the list of its CZ masks.
+// The high table is multiplied by scale, the factor that a commuting layer right before the
+// segment left out.
 __device__ __noinline__ int diag_setup(const Team& T, TeamS& S, const DOp* ops,
-                                          const Rot* coef, const Seg& sg, int n) {
+                                          const Rot* coef, const Seg& sg, int n, double scale) {
   // The segment's ops (at most kM RZ and kM CZ gates) are read in parallel by the lanes of the
   // team's first warp; a ballot gives each RZ (CZ) gate its slot in gate order.
   if (T.w == 0) {
@@ -432,7 +482,7 @@ __device__ __noinline__ int diag_setup(const Team& T, TeamS& S, const DOp* ops,
   for (int j = T.rank; j < nl + nh; j += T.size) {
     const bool hi = j >= nl;
     const int jj = hi ? j - nl : j;
-    double2 p = make_double2(1.0, 0.0);
+    double2 p = make_double2(hi ? scale : 1.0, 0.0);
     for (int g = 0; g < m; ++g) {
       const int b = S.rz_bit[g];
       if ((b >= hl) != hi) continue;
@@ -550,6 +600,11 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         r.k = 0;
         r.pad = 0;
         coef[g] = r;
+      } else if (op.flags & kOpT) {
+        double sn, cs;
+        sincos(0.5 * (op.param >= 0 ? theta[op.param] : op.fixed), &sn, &cs);
+        const RotT u = make_rott(cs, sn);
+        coef[g] = Rot{u.t, u.f, u.mode, __float_as_int((float)u.flo)};
       } else {
         coef[g] = make_coef(op, theta).r;
       }
@@ -562,6 +617,26 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
       team_prefetch_l2(T, a.tables + I.tab_off, (int64_t)I.tab_n * (int64_t)sizeof(double2));
     }
     T.sync();
+    // The factor of every layer whose gates run without it, kept in the gradient place of the
+    // layer's first op until the sweep takes the layer's gradients.
+    for (int s = T.w; s < I.n_segs; s += T.nw) {
+      const Seg sg = segs[s];
+      if (sg.kind != SEG_RLAYER || sg.split == 1) continue;
+      const double sc = layer_scale(coef, sg);
+      if ((threadIdx.x & 31) == 0) contrib[sg.first] = sc;
+    }
+    T.sync();
+    // what a diagonal segment's tables (prev: the segment before it) or a layer's last pass
+    // (next: the segment after it) multiply by
+    auto diag_scale = [&](int s) {
+      return s > 0 && segs[s - 1].kind == SEG_RLAYER && segs[s - 1].split != 1
+                 ? contrib[segs[s - 1].first] : 1.0;
+    };
+    auto own_scale = [&](int s) {
+      return s + 1 < I.n_segs &&
+                     (segs[s + 1].kind == SEG_DIAG || segs[s + 1].kind == SEG_DIAGPERM)
+                 ? 1.0 : contrib[segs[s].first];
+    };
 
     // ---------------------------------------------------------------- forward
     for (int s = 0; s < I.n_segs; ++s) {
@@ -573,7 +648,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
       if (sg.kind == SEG_DIAGPERM) {
         // one pass: checkpoint psi[k], apply the phase, scatter to P k (the gates' conditional
         // flips in order)
-        diag_setup(T, S, ops, coef, diag_part(sg), n);
+        diag_setup(T, S, ops, coef, diag_part(sg), n, diag_scale(s));
         perm_setup(T, S, ops, perm_part(sg), false, N);
         dp_save(T, S, aux + (size_t)sg.ckpt * kDpAuxAmps);
         const int ncz = S.n_cz;
@@ -599,7 +674,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         psi = lam;
         lam = t;
       } else if (sg.kind == SEG_DIAG) {
-        diag_setup(T, S, ops, coef, sg, n);
+        diag_setup(T, S, ops, coef, sg, n, diag_scale(s));
         const int ncz = S.n_cz;
         for (uint32_t k = tid; k < N; k += TS) {
           const double2 ph = cmul(S.th[k >> hl], S.tl[k & lmask]);
@@ -616,16 +691,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
       } else if (sg.kind == SEG_RLAYER) {
         // the layer's first pass also writes the checkpoint (a layer has at least two gates)
         layer_setup(T, S, ops, coef, sg);
-        int g = 0;
-        for (; g + 1 < sg.count; g += 2) {
-          lop_pass2(T, psi, N, S.lop[g], S.lop[g + 1], false,
-                    g == 0 ? ck + (size_t)sg.ckpt * N : nullptr);
-          T.sync();
-        }
-        if (g < sg.count) {
-          lop_pass(T, psi, N, S.lop[g], false);
-          T.sync();
-        }
+        layer_pass(T, S, psi, N, sg.count, false, own_scale(s), ck + (size_t)sg.ckpt * N);
       } else {
         for (int l = sg.first; l < sg.first + sg.count; ++l) {
           op_pass(T, psi, N, ops[l], coef[l], false);
@@ -964,6 +1030,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
           for (int q = 0; q < kM; ++q)
             if (q == g) v[q] = acc;
         }
+        const double sc = sg.split == 1 ? 1.0 : own_scale(s);
         const double tot = team_sum16(T, S, v, sg.count);
         if (tid < sg.count) contrib[sg.first + tid] = tot;
         if (sg.split == 1) {  // a product layer: nothing before it needs psi or lambda
@@ -973,20 +1040,12 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         // psi before the layer: the checkpoint copy runs while the layer is un-applied to
         // lambda (its gates commute: pairs in forward order, inverted), which leaves psi alone
         async_copy(T, psi, ck + (size_t)sg.ckpt * N, N);
-        g = 0;
-        for (; g + 1 < sg.count; g += 2) {
-          lop_pass2(T, lam, N, S.lop[g], S.lop[g + 1], true, nullptr);
-          T.sync();
-        }
-        if (g < sg.count) {
-          lop_pass(T, lam, N, S.lop[g], true);
-          T.sync();
-        }
+        layer_pass(T, S, lam, N, sg.count, true, sc, nullptr);
         async_wait();
         T.sync();
         continue;
       } else {  // SEG_DIAG
-        const int m = diag_setup(T, S, ops, coef, sg, n);
+        const int m = diag_setup(T, S, ops, coef, sg, n, diag_scale(s));
         const int ncz = S.n_cz;
         // Signed sums per bit: the bits below log_size are fixed within a thread (one running
         // sum W suffices); at most kHB higher bits vary across the thread's amplitudes.

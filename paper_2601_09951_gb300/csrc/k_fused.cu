@@ -182,34 +182,6 @@ __device__ __forceinline__ void stage_items(SItem* S, const SItem* src, int cnt,
   S[lane] = o;
 }
 
-// (x, y) <- the rotation without its factor.
-__device__ __forceinline__ void rot_t(int mode, double t, double& x, double& y) {
-  const double u = x, v = y;
-  if (mode == 0) {
-    x = fma(dneg(t), v, u);
-    y = fma(t, u, v);
-  } else if (mode == 1) {
-    x = fma(t, u, dneg(v));
-    y = fma(t, v, u);
-  } else {
-    x = fma(t, u, v);
-    y = fma(t, v, dneg(u));
-  }
-}
-
-template <bool ROTX>
-__device__ __forceinline__ void pair_t(int mode, double t, double2& x, double2& y) {
-  if (ROTX) {
-    // x' = c x - i s y, y' = c y - i s x: R(phi) on (im x, re y), R(-phi) on (re x, im y), the
-    // latter as R(phi) on (im y, re x)
-    rot_t(mode, t, y.y, x.x);
-    rot_t(mode, t, x.y, y.x);
-  } else {
-    rot_t(mode, t, x.x, y.x);
-    rot_t(mode, t, x.y, y.y);
-  }
-}
-
 // One pair of one of the normalised kinds.
 template <int KIND>
 __device__ __forceinline__ void fapply(const SItem& s, double2& x, double2& y) {

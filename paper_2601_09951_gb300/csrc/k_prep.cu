@@ -31,16 +31,6 @@ __device__ __forceinline__ int fkind_of(int type) {
   }
 }
 
-// a * b for a value held as an unevaluated sum hi + lo (error about 2^-104).
-__device__ __forceinline__ void dd_mul(double& ah, double& al, double bh, double bl) {
-  const double p = ah * bh;
-  double e = fma(ah, bh, dneg(p));
-  e = fma(ah, bl, e);
-  e = fma(al, bh, e);
-  ah = p + e;
-  al = e - (ah - p);
-}
-
 __device__ __forceinline__ void angle_cs(const DOp* ops, int l, const double* theta, double& c,
                                          double& s) {
   const int param = ops[l].param;
@@ -121,7 +111,7 @@ __device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
     dd_mul(sh, sl, __shfl_sync(0xffffffffu, f, 0), __shfl_sync(0xffffffffu, flo, 0));
     if (on) sitems[u.first + i] = o;
   }
-  if (lane == 0) scales[u.idx] = sh;
+  if (lane == 0) scales[u.idx] = sh + sl;
 }
 
 __device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, int n, int bl,

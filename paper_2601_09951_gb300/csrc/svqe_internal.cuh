@@ -70,10 +70,11 @@ __device__ __forceinline__ Rot make_rot(double phi) {
   return make_rot_cs(c, s);
 }
 
-// R(phi) without its normalisation (see SItem) from c = cos phi, s = sin phi.  The factor
-// f + flo is that of the rounded t, +-1 / sqrt(1 + t^2) to about 2^-100 (1 + t^2 held in two
-// doubles, and one Newton step for the low part), so that a pass's product of factors keeps the
-// norm of its amplitudes to one rounding.
+// R(phi) without its normalisation from c = cos phi, s = sin phi: with mode 0 (|c| >= |s|)
+// t = tan phi and R(phi) = f [[1, -t], [t, 1]], with mode 1 t = cot phi and
+// R(phi) = f [[t, -1], [1, t]].  The factor f + flo is that of the rounded t,
+// +-1 / sqrt(1 + t^2) to about 2^-100 (one Newton step from the cosine, 1 + t^2 held in two
+// doubles), so that a product of factors keeps the norm of the amplitudes to one rounding.
 struct RotT {
   double t, f, flo;
   int mode;
@@ -81,24 +82,80 @@ struct RotT {
 __device__ __forceinline__ RotT make_rott(double c, double s) {
   RotT o;
   o.mode = fabs(s) > fabs(c) ? 1 : 0;
-  const double num = o.mode ? c : s, den = o.mode ? s : c;
-  const double t = num / den;
+  const double num = o.mode ? c : s, f = o.mode ? s : c;
+  const double t = num / f;
   const double p = t * t, e = fma(t, t, dneg(p));
   const double a = 1.0 + p, al = (p - (a - 1.0)) + e;
-  const double r = 1.0 / sqrt(a);
-  const double r2 = r * r, r2e = fma(r, r, dneg(r2));
+  const double r2 = f * f, r2e = fma(f, f, dneg(r2));
   double res = fma(dneg(r2), a, 1.0);
   res = fma(dneg(r2e), a, res);
   res = fma(dneg(r2), al, res);
-  const double lo = 0.5 * r * res;
-  o.f = r + lo;
-  o.flo = lo - (o.f - r);
-  if (den < 0.0) {
-    o.f = dneg(o.f);
-    o.flo = dneg(o.flo);
-  }
   o.t = t;
+  o.f = f;
+  o.flo = 0.5 * f * res;
   return o;
+}
+// (x, y) <- R(phi) (x, y) without the factor, or with mode 2 (from mode 1, t unchanged) or a
+// negated t (mode 0) its inverse without the same factor: 2 FMA per real pair.
+__device__ __forceinline__ void rot_t(int mode, double t, double& x, double& y) {
+  const double u = x, v = y;
+  if (mode == 0) {
+    x = fma(dneg(t), v, u);
+    y = fma(t, u, v);
+  } else if (mode == 1) {
+    x = fma(t, u, dneg(v));
+    y = fma(t, v, u);
+  } else {
+    x = fma(t, u, v);
+    y = fma(t, v, dneg(u));
+  }
+}
+// The rotation on a pair of complex amplitudes: RY, or (ROTX) RX.
+template <bool ROTX>
+__device__ __forceinline__ void pair_t(int mode, double t, double2& x, double2& y) {
+  if (ROTX) {
+    // x' = c x - i s y, y' = c y - i s x: R(phi) on (im x, re y) and on (im y, re x)
+    rot_t(mode, t, y.y, x.x);
+    rot_t(mode, t, x.y, y.x);
+  } else {
+    rot_t(mode, t, x.x, y.x);
+    rot_t(mode, t, x.y, y.y);
+  }
+}
+// The same for RY gates without a branch on the mode.  R(phi) of mode 1 is the mode-0 form with
+// its t on the swapped pair (y, x), the result for x (its inverse: for y, with -t) negated.  So
+// a kernel loads the pair from swapped addresses, applies rot_y, and flips the sign of the
+// amplitudes whose bit has the value `neg` when it stores them.
+struct RotY {
+  double t;
+  uint32_t swap, neg0, neg1;  // address mask of the swap; sign masks of bit values 0 and 1
+};
+__device__ __forceinline__ RotY make_roty(double t, int mode, uint32_t bit, bool inv) {
+  RotY r;
+  r.t = inv ? dneg(t) : t;
+  r.swap = mode ? bit : 0u;
+  r.neg0 = mode && !inv ? 0x80000000u : 0u;
+  r.neg1 = mode && inv ? 0x80000000u : 0u;
+  return r;
+}
+__device__ __forceinline__ void rot_y(double t, double2& x, double2& y) {
+  const double2 u = x, v = y;
+  x.x = fma(dneg(t), v.x, u.x);
+  x.y = fma(dneg(t), v.y, u.y);
+  y.x = fma(t, u.x, v.x);
+  y.y = fma(t, u.y, v.y);
+}
+__device__ __forceinline__ double2 flip_sign(const double2& v, uint32_t m) {
+  return make_double2(__hiloint2double(__double2hiint(v.x) ^ (int)m, __double2loint(v.x)),
+                      __hiloint2double(__double2hiint(v.y) ^ (int)m, __double2loint(v.y)));
+}
+// (ah + al) *= (bh + bl), both unevaluated sums, to about 2^-104.
+__device__ __forceinline__ void dd_mul(double& ah, double& al, double bh, double bl) {
+  const double p = ah * bh;
+  double e = fma(ah, bh, dneg(p));
+  e = fma(ah, bl, e);
+  al = fma(al, bh, e);
+  ah = p;
 }
 
 // Coefficients of R(-phi) from those of R(phi).

@@ -30,6 +30,9 @@ static_assert(sizeof(DOp) == 48, "DOp layout");
 // product-state layer: for an op with this flag its coefficient slot holds
 // Rot{a = cos phi, b = sin phi, k = 0}.
 constexpr int32_t kOpCS = 1;
+// The RY and RX gates of a (non-product) commuting layer run without their normalisation (RotT):
+// the coefficient slot holds Rot{a = t, b = f, k = mode, pad = flo as a float}.
+constexpr int32_t kOpT = 2;
 
 // Lifting form of the rotation R(phi) = [[c, -s], [s, c]] (phi = theta/2):
 // R(phi) = L(a) S(b) L(a) R(k pi/2), a = -tan(r/2), b = sin(r), r = phi - k pi/2 in
@@ -64,7 +67,10 @@ static_assert(sizeof(DGroup) == 32, "DGroup layout");
 //               on the forward pass.  With split = 1 (the first segment, RY gates only) the
 //               layer acts on the reference basis state, so its output is a product state,
 //               written directly from two half tables; the sweep takes its gradients and stops
-//               there (no un-apply, no checkpoint).
+//               there (no un-apply, no checkpoint).  The other layers' gates run without their
+//               normalisation (kOpT); the product of the factors goes into the phase tables of
+//               the diagonal segment that follows, or else multiplies the state after
+//               the layer.
 //   SEG_DIAG  : RZ and CZ gates (diagonal, mutually commuting), applied as one phase
 //               e^{-i sum_q phi_q s_q(k)} (+-1 for CZ) per amplitude from two half tables;
 //               gradients from w_k = Im(conj(lambda_k) psi_k); psi reloaded from a checkpoint.
