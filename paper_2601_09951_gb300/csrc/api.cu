@@ -1235,6 +1235,28 @@ std::vector<BItem> svqe::batch_items(const std::vector<BInst>& bi,
   std::vector<int> order(n);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return cost[a] > cost[c]; });
+  // Teams per item: as many as fit a CTA, or fewer (halved, the largest first) while the items
+  // then still fit one per SM: an SM's FP64 pipe is shared by the teams of an item, so a small
+  // batch's instances run faster apart (100 one-warp instances: 13 CTAs of eight or 100 of one).
+  int cnt[kNumClasses] = {0}, per[kNumClasses];
+  for (int i = 0; i < n; ++i) ++cnt[cls[i]];
+  for (int c = 0; c < kNumClasses; ++c) per[c] = 8 / kClassWarps[c];
+  auto n_items = [&]() {
+    int t = 0;
+    for (int c = 0; c < kNumClasses; ++c) t += (cnt[c] + per[c] - 1) / per[c];
+    return t;
+  };
+  for (;;) {
+    int big = -1;
+    for (int c = 0; c < kNumClasses; ++c)
+      if (cnt[c] > 1 && per[c] > 1 && (big < 0 || per[c] > per[big])) big = c;
+    if (big < 0) break;
+    per[big] /= 2;
+    if (n_items() > kSms) {
+      per[big] *= 2;
+      break;
+    }
+  }
   std::vector<BItem> items;
   std::vector<double> icost;
   BItem open[kNumClasses];
@@ -1243,7 +1265,7 @@ std::vector<BItem> svqe::batch_items(const std::vector<BInst>& bi,
     open[c].cls = c;
     for (int t = 0; t < 8; ++t) open[c].inst[t] = -1;
     fill[c] = 0;
-    cap[c] = 8 / kClassWarps[c];
+    cap[c] = per[c];
   }
   std::vector<double> first_cost(kNumClasses, 0.0);
   for (int i : order) {
@@ -1275,7 +1297,7 @@ std::vector<BItem> svqe::batch_items(const std::vector<BInst>& bi,
 // one 8 (and 2 per amplitude for the layer's factor when no diagonal segment takes it), gradient
 // 8 per pair, H gate 8 per pair; a diagonal segment (alone or fused with the permutation after it) 12 per
 // amplitude forward and 16 + (RZ gates on bits >= 8) backward; a product layer 1 per amplitude
-// forward and its gradients (8 per pair) backward; a commuting layer un-applies lambda only; groups 4 (real or imaginary table) or 8
+// forward and 6 backward (its gradients); a commuting layer un-applies lambda only; groups 4 (real or imaginary table) or 8
 // (complex) per amplitude plus 4 for the energy.
 double svqe::batch_instance_flops(const HostCircuit& hc, const HostHam& hh,
                             const std::vector<Seg>& segs) {
@@ -1290,13 +1312,13 @@ double svqe::batch_instance_flops(const HostCircuit& hc, const HostHam& hh,
         if (rot) f += pairs * (12 + 24 + (op.param >= 0 ? 8 : 0));
         else if (op.type == SV_GATE_H) f += pairs * (8 + 16);
       } else if (s.kind == SEG_RLAYER) {
-        f += pairs * (s.split == 1 ? 8 : 8 + 8 + 8);
+        f += s.split == 1 ? 0.0 : pairs * (8 + 8 + 8);
       }
     }
     if (s.kind == SEG_RLAYER && s.split != 1 &&
         !(&s != &segs.back() && ((&s)[1].kind == SEG_DIAG || (&s)[1].kind == SEG_DIAGPERM)))
       f += N * (2 + 2);
-    if (s.kind == SEG_RLAYER && s.split == 1) f += N;  // the product state, one DMUL/amp
+    if (s.kind == SEG_RLAYER && s.split == 1) f += N * (1 + 5);  // one DMUL forward, contractions
     if (s.kind == SEG_DIAG || s.kind == SEG_DIAGPERM) {
       int hi = 0;
       for (int l = s.first; l < s.first + s.count; ++l)

@@ -333,8 +333,7 @@ __device__ __forceinline__ double layer_scale(const Rot* coef, const Seg& sg) {
     h = r.b;
     l = (double)__int_as_float(r.pad);
   }
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) {
+  for (int o = sg.count > 8 ? 8 : sg.count > 4 ? 4 : sg.count > 2 ? 2 : 1; o > 0; o >>= 1) {
     const double bh = __shfl_xor_sync(kFull, h, o), bl = __shfl_xor_sync(kFull, l, o);
     dd_mul(h, l, bh, bl);
   }
@@ -516,8 +515,9 @@ __device__ __forceinline__ GRec grec(const DGroup& G) {
 // bit with r_b = 0, (-sin phi, cos phi) for r_b = 1, and [k_b == r_b] on a bit without a gate.
 // The factors of bits [0, hl) and [hl, n) are multiplied out into the half tables tl and th
 // (real parts), so psi[k] = tl[k & lmask] * th[k >> hl].
-__device__ __noinline__ void product_setup(const Team& T, TeamS& S, const DOp* ops,
-                                           const Rot* coef, const Seg& sg, uint64_t ref, int n) {
+__device__ __forceinline__ void product_factors(const Team& T, TeamS& S, const DOp* ops,
+                                                const Rot* coef, const Seg& sg, uint64_t ref,
+                                                int n) {
   if (T.rank < n) {
     const bool r1 = (ref >> T.rank) & 1ull;
     S.cs[T.rank] = r1 ? make_double2(0.0, 1.0) : make_double2(1.0, 0.0);
@@ -530,19 +530,79 @@ __device__ __noinline__ void product_setup(const Team& T, TeamS& S, const DOp* o
     S.cs[b] = r1 ? make_double2(dneg(r.b), r.a) : make_double2(r.a, r.b);
   }
   T.sync();
+}
+
+// The product of the factors of bits [b0, b1) at the bit values j.
+__device__ __forceinline__ double product_of(const TeamS& S, int b0, int b1, uint32_t j) {
+  double p = 1.0;
+  for (int b = b0; b < b1; ++b, j >>= 1) {
+    const double2 f = S.cs[b];
+    p *= (j & 1u) ? f.y : f.x;
+  }
+  return p;
+}
+
+__device__ __noinline__ void product_setup(const Team& T, TeamS& S, const DOp* ops,
+                                           const Rot* coef, const Seg& sg, uint64_t ref, int n) {
+  product_factors(T, S, ops, coef, sg, ref, n);
   const int hl = n < 6 ? n : 6;
   const int nl = 1 << hl, nh = 1 << (n - hl);
   for (int j = T.rank; j < nl + nh; j += T.size) {
     const bool hi = j >= nl;
-    const int jj = hi ? j - nl : j;
-    const int b0 = hi ? hl : 0, b1 = hi ? n : hl;
-    double p = 1.0;
-    for (int b = b0; b < b1; ++b) {
-      const double2 f = S.cs[b];
-      p *= ((jj >> (b - b0)) & 1) ? f.y : f.x;
-    }
-    if (hi) S.th[jj] = make_double2(p, 0.0); else S.tl[jj] = make_double2(p, 0.0);
+    const double p = hi ? product_of(S, hl, n, j - nl) : product_of(S, 0, hl, j);
+    if (hi) S.th[j - nl] = make_double2(p, 0.0); else S.tl[j] = make_double2(p, 0.0);
   }
+  T.sync();
+}
+
+// Gradients of a product layer, sum_k Re lambda[k ^ b] psi[k] signed by bit b of k, from lambda
+// alone: psi is real and psi[k] = lo[tid] hi[u] for k = tid + u TS, so lambda is contracted once
+// with hi over a thread's slots (B, one value per thread) and once with lo over the threads
+// (A, at most 16 values), and each gate's sum runs over B or A: 3 FP64 operations per amplitude
+// for the whole layer instead of 2 per gate.  bb: scratch of 2^n doubles.
+__device__ __noinline__ void product_grads(const Team& T, TeamS& S, const DOp* ops,
+                                           const Rot* coef, const Seg& sg, uint64_t ref, int n,
+                                           const double2* lam, double* bb, double* contrib) {
+  product_factors(T, S, ops, coef, sg, ref, n);
+  const int lb = n < T.log_size ? n : T.log_size, nhb = n - lb, nu = 1 << nhb;
+  const uint32_t tid = T.rank;
+  const bool on = tid < (1u << lb);
+  if ((int)tid < nu) S.tl[tid].x = product_of(S, lb, n, tid);
+  const double lo = on ? product_of(S, 0, lb, tid) : 0.0;
+  T.sync();
+  double B = 0.0, v[kM];
+#pragma unroll
+  for (int u = 0; u < kM; ++u) {
+    v[u] = 0.0;
+    if (u < nu && on) {
+      const double r = lam[tid + u * T.size].x;
+      B = fma(r, S.tl[u].x, B);
+      v[u] = r * lo;
+    }
+  }
+  const double A = team_sum16(T, S, v, nu);
+  if ((int)tid < nu) S.th[tid].x = A;
+  if (on) bb[tid] = B;
+  T.sync();
+#pragma unroll
+  for (int g = 0; g < kM; ++g) {
+    v[g] = 0.0;
+    if (g < sg.count) {
+      const int b = S.lop[g].bit;
+      double w = 0.0;
+      uint32_t bit = 0;
+      if (b < lb) {
+        w = on ? bb[tid ^ (1u << b)] * lo : 0.0;
+        bit = (tid >> b) & 1u;
+      } else if ((int)tid < nu) {
+        w = S.th[tid ^ (1u << (b - lb))].x * S.tl[tid].x;
+        bit = (tid >> (b - lb)) & 1u;
+      }
+      v[g] = bit ? dneg(w) : w;
+    }
+  }
+  const double tot = team_sum16(T, S, v, sg.count);
+  if ((int)tid < sg.count) contrib[sg.first + tid] = tot;
   T.sync();
 }
 
@@ -591,23 +651,25 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
   const double lr = per_inst ? I.lr : (a.lr_inst ? a.lr_inst[idx] : a.lr);
 
   for (int step = 0; step < steps; ++step) {
+    // one sincos per op whatever form it takes (lanes of one warp hold ops of every form, and
+    // each would run its own)
     for (int g = tid; g < I.n_ops; g += TS) {
       const DOp op = ops[g];
-      if (op.flags & kOpCS) {
-        const double t = op.param >= 0 ? theta[op.param] : op.fixed;
-        Rot r;
-        sincos(0.5 * t, &r.b, &r.a);
-        r.k = 0;
-        r.pad = 0;
-        coef[g] = r;
-      } else if (op.flags & kOpT) {
+      Rot r{0.0, 0.0, 0, 0};
+      if (is_param_type(op.type)) {
         double sn, cs;
         sincos(0.5 * (op.param >= 0 ? theta[op.param] : op.fixed), &sn, &cs);
-        const RotT u = make_rott(cs, sn);
-        coef[g] = Rot{u.t, u.f, u.mode, __float_as_int((float)u.flo)};
-      } else {
-        coef[g] = make_coef(op, theta).r;
+        if (op.flags & kOpCS) {
+          r.a = cs;
+          r.b = sn;
+        } else if (op.flags & kOpT) {
+          const RotT u = make_rott(cs, sn);
+          r = Rot{u.t, u.f, u.mode, __float_as_int((float)u.flo)};
+        } else {
+          r = make_rot_cs(cs, sn);
+        }
       }
+      coef[g] = r;
     }
     for (uint32_t k = tid; k < N; k += TS)
       psi[k] = make_double2(k == (uint32_t)I.ref ? 1.0 : 0.0, 0.0);
@@ -626,6 +688,14 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
       if ((threadIdx.x & 31) == 0) contrib[sg.first] = sc;
     }
     T.sync();
+    // A product layer's gradients are contracted from lambda when each thread holds at least
+    // eight amplitudes; with fewer the contraction's set-up and two reductions cost more than the
+    // pair terms (ten steps of an 8-qubit chain: 467 against 412 us).  A segment right after
+    // such a layer needs no checkpoint.
+    const bool contract = N >= 8u * (uint32_t)TS;
+    auto after_product = [&](int s) {
+      return contract && s == 1 && segs[0].kind == SEG_RLAYER && segs[0].split == 1;
+    };
     // what a diagonal segment's tables (prev: the segment before it) or a layer's last pass
     // (next: the segment after it) multiply by
     auto diag_scale = [&](int s) {
@@ -653,9 +723,10 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         dp_save(T, S, aux + (size_t)sg.ckpt * kDpAuxAmps);
         const int ncz = S.n_cz;
         double2* c = ck + (size_t)sg.ckpt * N;
+        const bool keep = !after_product(s);
         for (uint32_t k = tid; k < N; k += TS) {
           const double2 p0 = psi[k];
-          c[k] = p0;
+          if (keep) c[k] = p0;
           const double2 ph = cmul(S.th[k >> hl], S.tl[k & lmask]);
           double2 v = cmul(p0, ph);
           if (ncz && cz_sign(S, ncz, k)) v = make_double2(dneg(v.x), dneg(v.y));
@@ -953,7 +1024,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         }
         T.sync();
         // psi before the segment: the checkpoint copy overlaps the stores and the reduction
-        async_copy(T, psi, ck + (size_t)sg.ckpt * N, N);
+        if (!after_product(s)) async_copy(T, psi, ck + (size_t)sg.ckpt * N, N);
 #pragma unroll
         for (int u = 0; u < kHU; ++u) {
           if (u >= nu) break;
@@ -982,10 +1053,14 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
                      aux + (size_t)segs[s - 1].ckpt * kDpAuxAmps, kDpBlockAmps);
           pre_dp = s - 1;
         }
+        layer_setup(T, S, ops, coef, sg);
+        if (sg.split == 1 && contract) {  // nothing before it needs psi or lambda
+          product_grads(T, S, ops, coef, sg, I.ref, n, lam, reinterpret_cast<double*>(psi), contrib);
+          continue;
+        }
         // gradients of every gate from (psi, lambda) at the layer's end, two gates per pass:
         // each thread reads a block of four amplitudes of psi and lambda and accumulates both
         // gates' pair terms from it
-        layer_setup(T, S, ops, coef, sg);
         int g = 0;
         for (; g + 1 < sg.count; g += 2) {
           const LOp& o1 = S.lop[g];
@@ -1033,7 +1108,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         const double sc = sg.split == 1 ? 1.0 : own_scale(s);
         const double tot = team_sum16(T, S, v, sg.count);
         if (tid < sg.count) contrib[sg.first + tid] = tot;
-        if (sg.split == 1) {  // a product layer: nothing before it needs psi or lambda
+        if (sg.split == 1) {
           T.sync();
           continue;
         }
@@ -1084,6 +1159,13 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
     }
 
     // ---------------------------------------------------------------- gradients, update
+    // Adam's bias corrections, both powers at once: beta1's in even lanes, beta2's in odd ones
+    double c1 = 0.0, c2 = 0.0;
+    if (gd && a.opt == 1) {
+      const double pw = 1.0 - ipow((threadIdx.x & 1) ? a.beta2 : a.beta1, a.adam_t0 + step + 1);
+      c1 = __shfl_sync(kFull, pw, 0);
+      c2 = __shfl_sync(kFull, pw, 1);
+    }
     for (int p = tid; p < I.n_params; p += TS) {
       double g = 0.0;
       for (int j = a.pptr[I.pp_off + p]; j < a.pptr[I.pp_off + p + 1]; ++j)
@@ -1097,9 +1179,8 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
           const double v = fma(a.beta2, a.adam_v[q], (1.0 - a.beta2) * g * g);
           a.adam_m[q] = m;
           a.adam_v[q] = v;
-          const int t = a.adam_t0 + step + 1;
-          const double mh = m / (1.0 - ipow(a.beta1, t));
-          const double vh = v / (1.0 - ipow(a.beta2, t));
+          const double mh = m / c1;
+          const double vh = v / c2;
           theta[p] -= lr * mh / (sqrt(vh) + a.eps);
         } else {
           theta[p] = fma(-lr, g, theta[p]);
