@@ -50,6 +50,12 @@ struct sv_ctx {
   double* scales = nullptr;
   double2* dptab = nullptr;
   size_t coef_cap = 0, cs_cap = 0, sitems_cap = 0, scales_cap = 0, dptab_cap = 0;
+  double* prod = nullptr;     // contraction parts of the product prefix's gradients
+  size_t prod_cap = 0;
+  // psi holds exactly |ref>: set by sv_init_reference, cleared by everything that writes psi;
+  // never set again once the caller has psi's address
+  bool psi_is_ref = false;
+  bool psi_shared = false;
   double* gpart = nullptr;    // n_ops x kRedBlocks gradient partials
   size_t gpart_cap = 0;
   double* theta = nullptr;
@@ -65,13 +71,13 @@ struct sv_ctx {
   // whole-state diagonal + permutation segments (k_dp.cu) need a third state buffer
   double2* scratch = nullptr;
   bool scratch_failed = false;
-  enum { CH_PASSES = 0, CH_LAYER = 1, CH_DP = 2 };
+  enum { CH_PASSES = 0, CH_LAYER = 1, CH_DP = 2, CH_PROD = 3 };
   struct Chunk {
     int kind;
     int first, count;  // ops
-    int ck;            // CH_LAYER: its checkpoint buffer
+    int ck;            // CH_LAYER: its checkpoint buffer; CH_PROD: ops of the prefix
     int p0, p1;        // CH_PASSES / CH_LAYER: passes [p0, p1) of plan
-    DpArgs dp;         // CH_DP
+    DpArgs dp;         // CH_DP, CH_PROD
   };
   std::vector<Chunk> chunks;
   // small registers (k_small): checkpoints, and pinned host memory the kernel writes results to
@@ -251,6 +257,7 @@ sv_status sv_destroy(sv_ctx* c) {
   cudaFree(c->sitems);
   cudaFree(c->scales);
   cudaFree(c->dptab);
+  cudaFree(c->prod);
   cudaFree(c->gpart);
   cudaFree(c->theta);
   cudaFree(c->grad);
@@ -440,14 +447,15 @@ sv_status sv_init_reference(sv_ctx* c, uint64_t b) {
   if (b >= c->N) { set_error("basis index %llu >= 2^%d", (unsigned long long)b, c->n); return SV_EINVAL; }
   c->ref = b;
   SV_CUDA(launch_init_basis(c->psi, c->n, b, c->stream), c);
+  c->psi_is_ref = !c->psi_shared;
   return SV_OK;
 }
 
 // Upload a lowered circuit's ops and make sure every circuit-sized buffer fits.
-static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits);
+static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, bool from_ref);
 static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc);
 
-sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune) {
+sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune, bool from_ref) {
   const size_t n_ops = hc.ops.size();
   SV_CUDA(grow(c->coef, c->coef_cap, n_ops), c);
   SV_CUDA(grow(c->cs, c->cs_cap, n_ops), c);
@@ -457,7 +465,7 @@ sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune) {
   int m = fused_tile_bits();
   if (may_tune && c->tune && c->n >= kFusedMinQubits && n_ops > 0) m = tune_tile_bits(c, hc);
   if (m <= 0) return SV_ECUDA;
-  return plan_circuit(c, hc, m);
+  return plan_circuit(c, hc, m, from_ref);
 }
 
 static int single_op(const sv_ctx* c, int p);
@@ -479,9 +487,25 @@ static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan
   if (2 * small.passes.size() <= 3 * plan.passes.size() + 2) std::swap(plan, small);
 }
 
+// Length of the circuit's product prefix, its leading one-qubit gates, or 0: it is used from the
+// registers that have whole-state segments, when it saves at least a pass or so.
+static int product_prefix(const HostCircuit& hc) {
+  if (hc.n < kDpMinQubits) return 0;
+  std::vector<int> per(hc.n, 0);
+  int m = 0;
+  for (; m < (int)hc.ops.size(); ++m) {
+    const DOp& op = hc.ops[m];
+    if (op.type != SV_GATE_X && op.type != SV_GATE_H && op.type != SV_GATE_RX &&
+        op.type != SV_GATE_RY && op.type != SV_GATE_RZ)
+      break;
+    if (++per[op.bit0] > kMaxQubitGates) return 0;
+  }
+  return 2 * m >= hc.n ? m : 0;
+}
+
 // Fused-pass plan of a staged circuit with tiles of tile_bits bits (see stage_circuit), and its
 // upload.
-static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
+static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, bool from_ref) {
   const size_t n_ops = hc.ops.size();
   c->tile_bits = tile_bits;
   c->plan.passes.clear();
@@ -489,7 +513,11 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
   c->chunks.clear();
   if (c->n >= kFusedMinQubits && n_ops > 0) {
     // commuting layers that get a psi checkpoint: as many as the budget (and the device) allow
+    const int n_prod = from_ref ? product_prefix(hc) : 0;
     std::vector<std::pair<int, int>> layers = commuting_layers(hc.ops, 2);
+    layers.erase(std::remove_if(layers.begin(), layers.end(),
+                                [&](const std::pair<int, int>& l) { return l.first < n_prod; }),
+                 layers.end());
     const uint64_t sb = sv_state_bytes(c->n);
     size_t n_ck = std::min<size_t>(layers.size(), (size_t)(c->ck_budget / sb));
     while (c->ck.size() < n_ck) {
@@ -554,6 +582,26 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
       ch.p1 = (int)c->plan.passes.size();
       c->chunks.push_back(ch);
     };
+    // P of the CNOT/X run [l0, l1), the gates' conditional flips in order, affine over GF(2)
+    auto map_args = [&](DpArgs& d, int l0, int l1) {
+      d.n = c->n;
+      auto P = [&](uint32_t k) {
+        for (int l = l0; l < l1; ++l) {
+          const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
+          if ((k & lo) == lo) k ^= fl;
+        }
+        return k;
+      };
+      d.c0 = P(0);
+      for (int b = 0; b < c->n; ++b) d.col[b] = P(1u << b) ^ d.c0;
+      // delta = M^-1 e_0: the linear parts of the gates (a CNOT flips its target where its
+      // control is set; an X is a constant) applied to e_0 in reverse order
+      d.delta = 1u;
+      for (int l = l1 - 1; l >= l0; --l) {
+        const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
+        if (lo && (d.delta & lo) == lo) d.delta ^= fl;
+      }
+    };
     auto dp_chunk = [&](int first, int split, int len) {
       sv_ctx::Chunk ch{};
       ch.kind = sv_ctx::CH_DP;
@@ -574,29 +622,25 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
           d.cz_mask[d.n_cz++] = (uint32_t)op.lo_or;
         }
       }
-      // P(k): the CNOT/X gates' conditional flips in order, affine over GF(2)
-      auto P = [&](uint32_t k) {
-        for (int l = first + split; l < first + len; ++l) {
-          const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
-          if ((k & lo) == lo) k ^= fl;
-        }
-        return k;
-      };
-      d.c0 = P(0);
-      for (int b = 0; b < c->n; ++b) d.col[b] = P(1u << b) ^ d.c0;
-      // delta = M^-1 e_0: the linear parts of the gates (a CNOT flips its target where its
-      // control is set; an X is a constant) applied to e_0 in reverse order
-      d.delta = 1u;
-      for (int l = first + len - 1; l >= first + split; --l) {
-        const uint32_t lo = (uint32_t)hc.ops[l].lo_or, fl = (uint32_t)hc.ops[l].flip;
-        if (lo && (d.delta & lo) == lo) d.delta ^= fl;
-      }
+      map_args(d, first + split, first + len);
       c->chunks.push_back(ch);
     };
     int i = 0, pass_start = 0;
     auto flush = [&](int end) {
       if (end > pass_start) plan_chunk(sv_ctx::CH_PASSES, pass_start, end - pass_start, -1);
     };
+    if (n_prod > 0) {
+      // the prefix, and the CNOT/X run after it
+      int e = n_prod;
+      while (e < (int)n_ops && is_perm(hc.ops[e].type)) ++e;
+      sv_ctx::Chunk ch{};
+      ch.kind = sv_ctx::CH_PROD;
+      ch.count = e;
+      ch.ck = n_prod;
+      map_args(ch.dp, n_prod, e);
+      c->chunks.push_back(ch);
+      i = pass_start = e;
+    }
     while (i < (int)n_ops) {
       int split = 0, len = 0;
       if (layer_at[i] >= 0) {
@@ -621,8 +665,9 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
   std::vector<DOp> ops(hc.ops);
   for (size_t l = 0; l < n_ops; ++l) ops[l].flags = adjoint_blocks(c->n, ops[l]);
   for (const sv_ctx::Chunk& ch : c->chunks) {
-    if (ch.kind == sv_ctx::CH_DP) {
-      for (int l = ch.first; l < ch.first + ch.count; ++l) ops[l].flags = dp_blocks(c->n);
+    if (ch.kind == sv_ctx::CH_DP || ch.kind == sv_ctx::CH_PROD) {
+      for (int l = ch.first; l < ch.first + ch.count; ++l)
+        ops[l].flags = ch.kind == sv_ctx::CH_DP ? dp_blocks(c->n) : 1;
       continue;
     }
     for (int p = ch.p0; p < ch.p1; ++p) {
@@ -641,10 +686,13 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
       while (split < ch.count && (hc.ops[ch.first + split].type == SV_GATE_RZ ||
                                   hc.ops[ch.first + split].type == SV_GATE_CZ))
         ++split;
-      units.push_back(PrepUnit{1, ch.first, split, n_dp++});
+      units.push_back(PrepUnit{PREP_DP, ch.first, split, n_dp++});
+    } else if (ch.kind == sv_ctx::CH_PROD) {
+      units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++});
+      SV_CUDA(grow(c->prod, c->prod_cap, prod_scratch(c->n)), c);
     }
     for (int p = ch.p0; p < ch.p1; ++p)
-      units.push_back(PrepUnit{0, c->plan.passes[p].first_item, c->plan.passes[p].n_items, p});
+      units.push_back(PrepUnit{PREP_PASS, c->plan.passes[p].first_item, c->plan.passes[p].n_items, p});
   }
   auto align = [](size_t v) { return (v + 255) / 256 * 256; };
   const size_t o_items = align(n_ops * sizeof(DOp));
@@ -668,7 +716,8 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits) {
   c->n_units = (int)units.size();
   n_dp = 0;
   for (sv_ctx::Chunk& ch : c->chunks)
-    if (ch.kind == sv_ctx::CH_DP) ch.dp.tab = c->dptab + (size_t)kDpTab * n_dp++;
+    if (ch.kind == sv_ctx::CH_DP || ch.kind == sv_ctx::CH_PROD)
+      ch.dp.tab = c->dptab + (size_t)kDpTab * n_dp++;
   return SV_OK;
 }
 
@@ -697,8 +746,8 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
                          double2** psi_out) {
   const int n_ops = (int)hc.ops.size();
   *psi_out = c->psi;
-  SV_CUDA(launch_prep(c->units, c->n_units, c->ops, c->items, theta_dev, c->n, c->coef, c->sitems,
-                      c->scales, c->cs, c->dptab, c->stream), c);
+  SV_CUDA(launch_prep(c->units, c->n_units, c->ops, c->items, theta_dev, c->n, c->ref, c->coef,
+                      c->sitems, c->scales, c->cs, c->dptab, c->stream), c);
   if (!c->chunks.empty()) {
     double2* psi = c->psi;
     bool ov = false;  // the first kernel after the preparation waits for it
@@ -708,6 +757,11 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
         SV_CUDA(launch_dp_fwd(psi, dst, ch.dp, c->stream, ov), c);
         ov = true;
         psi = dst;
+        continue;
+      }
+      if (ch.kind == sv_ctx::CH_PROD) {  // (the first chunk) psi from the tables alone
+        SV_CUDA(launch_prod_fwd(psi, ch.dp, c->stream, ov), c);
+        ov = true;
         continue;
       }
       if (save && ch.kind == sv_ctx::CH_LAYER)
@@ -793,7 +847,7 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc) {
   float best_ms = 1e30f;
   bool ok = true;
   for (int m = 9; m <= 11 && ok; ++m) {
-    ok = plan_circuit(c, hc, m) == SV_OK;
+    ok = plan_circuit(c, hc, m, true) == SV_OK;
     float ms = 0.0f;
     for (int rep = 0; rep < 2 && ok; ++rep) {
       double2* out = nullptr;
@@ -955,7 +1009,9 @@ static sv_status run_small(sv_ctx* c, SmallPack& S, const sv_ham* H, double* ene
 sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
                        const double* theta_dev, double* energy_dev, double* grad_dev,
                        double* theta_upd, double lr, double* traj) {
-  SV_CUDA(launch_init_basis(c->psi, c->n, c->ref, c->stream), c);
+  const bool prod = !c->chunks.empty() && c->chunks[0].kind == sv_ctx::CH_PROD;
+  c->psi_is_ref = false;
+  if (!prod) SV_CUDA(launch_init_basis(c->psi, c->n, c->ref, c->stream), c);
   double2* psi = nullptr;
   sv_status st = forward(c, hc, theta_dev, true, &psi);
   if (st != SV_OK) return st;
@@ -978,6 +1034,9 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
                                  c->scales + p, c->gpart, c->stream, true), c);
           }
         }
+      } else if (ch.kind == sv_ctx::CH_PROD) {
+        SV_CUDA(launch_prod_grads(lam, ch.dp, c->ops, ch.ck, c->cs, c->ref, c->prod, c->gpart,
+                                  c->stream, true), c);
       } else if (ch.kind == sv_ctx::CH_LAYER) {
         // a checkpointed commuting layer: every gradient from (psi, lambda) at the layer's
         // end, then the layer un-applied to lambda alone; psi before the layer is the
@@ -1001,7 +1060,10 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
       }
     }
     // psi is back at the reference state; it lives in the context's psi buffer between calls
-    if (psi != c->psi)
+    // (a product prefix is not un-applied: the state is written)
+    if (prod)
+      SV_CUDA(launch_init_basis(c->psi, c->n, c->ref, c->stream), c);
+    else if (psi != c->psi)
       SV_CUDA(cudaMemcpyAsync(c->psi, psi, sv_state_bytes(c->n), cudaMemcpyDeviceToDevice,
                               c->stream), c);
   } else {
@@ -1012,7 +1074,7 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
     }
   }
   SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, energy_dev,
-                        theta_upd, lr, traj, c->stream, true), c);
+                        theta_upd, lr, traj, c->stream, !prod), c);
   return SV_OK;
 }
 
@@ -1024,7 +1086,8 @@ sv_status sv_apply_circuit(sv_ctx* c, const sv_circuit* circ, const double* thet
   sv_status st = lower_circuit(circ, c->n, hc);
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && !theta) { set_error("theta is NULL"); return SV_EINVAL; }
-  if ((st = stage_circuit(c, hc)) != SV_OK) return st;
+  if ((st = stage_circuit(c, hc, false, c->psi_is_ref)) != SV_OK) return st;
+  c->psi_is_ref = false;
   if (hc.n_params)
     SV_CUDA(cudaMemcpyAsync(c->theta, theta, hc.n_params * sizeof(double),
                             cudaMemcpyHostToDevice, c->stream), c);
@@ -1081,7 +1144,7 @@ sv_status sv_adjoint_grad_dev(sv_ctx* c, const sv_circuit* circ, const double* t
     sp.args.a.theta = const_cast<double*>(theta_dev);
     return run_small(c, sp, H, energy_dev, grad_dev, 0, 0.0, nullptr);
   }
-  if ((st = stage_circuit(c, hc, true)) != SV_OK) return st;
+  if ((st = stage_circuit(c, hc, true, true)) != SV_OK) return st;
   return adjoint_core(c, hc, H, theta_dev, energy_dev, grad_dev);
 }
 
@@ -1105,7 +1168,7 @@ sv_status sv_adjoint_grad(sv_ctx* c, const sv_circuit* circ, const double* theta
     if (hc.n_params) std::memcpy(grad_out, c->pin + 1, hc.n_params * sizeof(double));
     return SV_OK;
   }
-  if ((st = stage_circuit(c, hc, true)) != SV_OK) return st;
+  if ((st = stage_circuit(c, hc, true, true)) != SV_OK) return st;
   if (hc.n_params)
     SV_CUDA(cudaMemcpyAsync(c->theta, theta, hc.n_params * sizeof(double),
                             cudaMemcpyHostToDevice, c->stream), c);
@@ -1121,7 +1184,7 @@ sv_status sv_adjoint_grad(sv_ctx* c, const sv_circuit* circ, const double* theta
 
 sv_status svqe::vqe_enqueue(sv_ctx* c, const HostCircuit& hc, const sv_ham* H, const double* theta_in,
                       double lr, int32_t n_steps, double* theta_out, double* energy_out) {
-  sv_status st = stage_circuit(c, hc, true);
+  sv_status st = stage_circuit(c, hc, true, true);
   if (st != SV_OK) return st;
   SV_CUDA(grow(c->etraj, c->etraj_cap, (size_t)std::max(1, n_steps)), c);
   if (hc.n_params)
@@ -1188,6 +1251,7 @@ sv_status sv_set_state(sv_ctx* c, const void* host_in) {
   clear_error();
   if (!c || !host_in) { set_error("NULL argument"); return SV_EINVAL; }
   SV_CHECK_STICKY(c);
+  c->psi_is_ref = false;
   SV_CUDA(cudaMemcpyAsync(c->psi, host_in, sv_state_bytes(c->n), cudaMemcpyHostToDevice,
                           c->stream), c);
   SV_CUDA(cudaStreamSynchronize(c->stream), c);
@@ -1196,6 +1260,8 @@ sv_status sv_set_state(sv_ctx* c, const void* host_in) {
 
 sv_status sv_state_device_ptr(sv_ctx* c, void** psi_dev) {
   if (!c || !psi_dev) { set_error("NULL argument"); return SV_EINVAL; }
+  c->psi_shared = true;
+  c->psi_is_ref = false;
   *psi_dev = c->psi;
   return SV_OK;
 }

@@ -16,7 +16,9 @@ namespace svqe {
 // (sv_set_autotune), a circuit structure not seen before has its tile size measured first
 // (the forward pass is run on the context's psi, so only callers that re-initialise psi
 // afterwards pass true).
-sv_status stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune = false);
+// from_ref: psi is the reference state when the circuit runs, so that its leading one-qubit gates
+// may be written as a product state.
+sv_status stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune, bool from_ref);
 // psi = |ref>, forward, lambda = H psi, adjoint sweep; stream-ordered.
 sv_status adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
                        const double* theta_dev, double* energy_dev, double* grad_dev,

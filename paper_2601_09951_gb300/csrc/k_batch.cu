@@ -171,24 +171,6 @@ __device__ __forceinline__ double team_sum(const Team& T, TeamS& S, double v) {
   return t;
 }
 
-// Sum over the warp of 16 values per lane by recursive halving (16 DADD per lane instead of
-// 80); afterwards lanes 2j and 2j+1 hold the warp total of value j.
-__device__ __forceinline__ double warp_sum16(double (&v)[kM]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int o = 16 >> s, h = 8 >> s;
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const double send = up ? v[i] : v[i + h];
-      const double keep = up ? v[i + h] : v[i];
-      v[i] = keep + __shfl_xor_sync(kFull, send, o);
-    }
-  }
-  return v[0] + __shfl_xor_sync(kFull, v[0], 1);
-}
-
 // Team totals of v[0..m): team rank j < m returns the total of value j, others 0.  Ends with
 // the team synchronised.
 __device__ __forceinline__ double team_sum16(const Team& T, TeamS& S, double (&v)[kM], int m) {
@@ -227,13 +209,6 @@ __device__ __forceinline__ void pair_grad_acc(int type, const double2& lx, const
     acc = fma(dneg(lx.x), py.x, acc);
     acc = fma(dneg(lx.y), py.y, acc);
   }
-}
-
-__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ double2 cmul_conj(const double2& a, const double2& b) {  // a * conj(b)
-  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, dneg(a.x) * b.y));
 }
 
 // Apply one pair op to buffer v (forward or inverse), pairs strided over the team, two pairs

@@ -11,6 +11,8 @@
 //   * the RZ gradients 2 Im<lambda|Z_q/2|psi> = sum_k s_q(k) w_k, w_k = Im(conj(lambda_k)
 //     psi_k), are the same at either end of the diagonal part (the phase cancels in w_k), so
 //     they are taken from the un-phased lambda and psi.
+// A circuit's leading one-qubit gates make a product state, written and differentiated with the
+// same index split (k_dp<DP_MAKE>, k_prod_lam, k_prod_fin).
 // Blocks of 128 NA consecutive amplitudes are handled by 128 threads, NA (1 to 8) amplitudes
 // each (k = base + tid + 128 i), so P and the phase of an amplitude split into a part per
 // thread, one per i and one per block: a thread keeps its own part in registers, and the block
@@ -36,13 +38,6 @@ constexpr int kDT = 128;       // threads per CTA
 constexpr int kDTLog = kDpThreadLog;
 constexpr int kChunk = 32;     // rounds tabulated at a time
 constexpr int kMaxRound = 11;  // round bits (31 qubits: 2^21 blocks on 2^10 CTAs)
-
-__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ double2 cmul_conj(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, dneg(a.x) * b.y));
-}
 
 // The block of visit index t: bit 0 of t selects pair, bit pair_hi of t selects block bit 0,
 // every other bit of t is the same block bit.  A bijection on the block indices, because pair
@@ -117,8 +112,10 @@ __device__ __forceinline__ void dp_rounds(DpShared<NA>& S, const DpArgs& a, uint
   __syncthreads();
 }
 
-// Forward (BWD false): out[P(k)] = phase(k) in[k].  Backward: out[k] = conj(phase(k)) in[P(k)].
-template <int NA, bool BWD>
+// DP_FWD: out[P(k)] = phase(k) in[k].  DP_BWD: out[k] = conj(phase(k)) in[P(k)].  DP_MAKE:
+// out[P(k)] = phase(k), the tables holding the factors of a product state.
+enum { DP_FWD = 0, DP_BWD = 1, DP_MAKE = 2 };
+template <int NA, int MODE>
 __global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
                                                double2* __restrict__ out, DpArgs a) {
   __shared__ DpShared<NA> S;
@@ -132,13 +129,15 @@ __global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
     for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
       const uint32_t base = (S.blk[r] << BL) | threadIdx.x, pc = S.pc[r] ^ T.pt;
       double2 v[NA];
+      if (MODE != DP_MAKE) {
 #pragma unroll
-      for (int i = 0; i < NA; ++i) {
-        uint32_t p = pc;
+        for (int i = 0; i < NA; ++i) {
+          uint32_t p = pc;
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
-          if ((i >> b) & 1) p ^= a.col[kDTLog + b];
-        v[i] = in[BWD ? p : base | (i * kDT)];
+          for (int b = 0; b < 3; ++b)
+            if ((i >> b) & 1) p ^= a.col[kDTLog + b];
+          v[i] = in[MODE == DP_BWD ? p : base | (i * kDT)];
+        }
       }
 #pragma unroll
       for (int i = 0; i < NA; ++i) {
@@ -148,30 +147,14 @@ __global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
           if ((i >> b) & 1) p ^= a.col[kDTLog + b];
         const uint32_t k = base | (i * kDT);
         const double2 ph = cmul(T.ph, S.q[r * NA + i]);
-        double2 w = BWD ? cmul_conj(v[i], ph) : cmul(v[i], ph);
+        double2 w = ph;
+        if (MODE == DP_FWD) w = cmul(v[i], ph);
+        if (MODE == DP_BWD) w = cmul_conj(v[i], ph);
         if (a.n_cz && dp_cz(a, k)) w = make_double2(dneg(w.x), dneg(w.y));
-        out[BWD ? k : p] = w;
+        out[MODE == DP_BWD ? k : p] = w;
       }
     }
   }
-}
-
-// Sum over the warp of 16 values per lane by recursive halving (16 DADD per lane instead of
-// 80); afterwards lanes 2j and 2j+1 hold the warp total of value j.
-__device__ __forceinline__ double warp_sum16(double (&v)[16]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int o = 16 >> s, h = 8 >> s;
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const double send = up ? v[i] : v[i + h];
-      const double keep = up ? v[i + h] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Backward, lambda: out[k] = conj(phase(k)) lam[P(k)], and the RZ gradient shares from
@@ -310,6 +293,228 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
   }
 }
 
+// ------------------------------------------------------------------------------ product prefix
+// Gradients of one-qubit gates on a product state psi = prod_b f_b(k_b): with
+// Lambda_b[v] = sum over k with k_b = v of lambda[k] prod_{c != b} conj f_c(k_c), a gate of qubit
+// b that makes f_b's derivative g_b contributes 2 Re sum_v conj(Lambda_b[v]) g_b[v].  One pass over lambda
+// replaces the un-phasing and un-applying of two states: k_prod_lam contracts it with the factors
+// of all bits but the slots' (A), the threads' (B) or the blocks' (D), about 11 FP64 operations
+// per amplitude against 170 for a layer of 24 RY and 24 RZ gates; k_prod_fin finishes every
+// qubit from those.
+//   part: A[4 CTAs][16] (a warp's 8 slots), B[CTAs][128], D[blocks][4] (a block's 4 warps).
+template <int NA>
+__global__ void __launch_bounds__(kDT, 4) k_prod_lam(const double2* __restrict__ lam, DpArgs a,
+                                                     double* __restrict__ part) {
+  __shared__ double2 so[kChunk], spi[8];
+  __shared__ uint32_t sblk[kChunk], spc[kChunk];
+  constexpr int BL = kDTLog + (NA == 8 ? 3 : NA == 4 ? 2 : NA == 2 ? 1 : 0);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t nblk = 1u << (a.n - BL), pair = a.delta >> BL;
+  double* pA = part;
+  double2* pB = reinterpret_cast<double2*>(part + (size_t)gridDim.x * 64);
+  double2* pD = pB + (size_t)gridDim.x * kDT;
+  const DpThread T = dp_start(a);
+  if (tid < NA) spi[tid] = a.tab[128 + tid];
+  double2 A[NA], B = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int i = 0; i < NA; ++i) A[i] = make_double2(0.0, 0.0);
+  pdl_begin();
+  for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
+    __syncthreads();
+    const uint32_t t = blockIdx.x + (r0 + tid) * gridDim.x;
+    if (tid < kChunk && t < nblk) {
+      const uint32_t b = dp_block(pair, t);
+      uint32_t c = a.c0;
+      for (int i = BL; i < a.n; ++i)
+        if ((b >> (i - BL)) & 1u) c ^= a.col[i];
+      sblk[tid] = b;
+      spc[tid] = c;
+      double2 p = a.tab[136 + (b & 127u)];
+      if (a.n > BL + 7) p = cmul(p, a.tab[264 + ((b >> 7) & 127u)]);
+      if (a.n > BL + 14) p = cmul(p, a.tab[392 + (b >> 14)]);
+      so[tid] = p;
+    }
+    __syncthreads();
+    for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
+      const uint32_t pc = spc[r] ^ T.pt;
+      double2 v[NA];
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        uint32_t p = pc;
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if ((i >> b) & 1) p ^= a.col[kDTLog + b];
+        v[i] = lam[p];
+      }
+      const double2 o = so[r], tb = cmul(T.ph, o);
+      double2 d = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        cmac_conj(A[i], v[i], tb);
+        cmac_conj(d, v[i], spi[i]);
+      }
+      cmac_conj(B, d, o);
+      double2 e = cmul_conj(d, T.ph);
+      e.x = warp_sum(e.x);
+      e.y = warp_sum(e.y);
+      if (lane == 0) pD[(size_t)sblk[r] * 4 + warp] = e;
+    }
+  }
+  double v[16];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    v[2 * i] = i < NA ? A[i < NA ? i : 0].x : 0.0;
+    v[2 * i + 1] = i < NA ? A[i < NA ? i : 0].y : 0.0;
+  }
+  const double t = warp_sum16(v);
+  if ((lane & 1) == 0) pA[((size_t)blockIdx.x * 4 + warp) * 16 + (lane >> 1)] = t;
+  pB[(size_t)blockIdx.x * kDT + tid] = B;
+}
+
+constexpr int kFT = 256;
+
+// One CTA per qubit (index bit): Lambda_b from the parts, then the qubit's gates.
+__global__ void __launch_bounds__(kFT) k_prod_fin(const double* __restrict__ part, int n_cta,
+                                                  DpArgs a, int bl, const DOp* __restrict__ ops,
+                                                  int n_ops, const double2* __restrict__ cs,
+                                                  uint64_t ref, double* __restrict__ partial) {
+  __shared__ double2 sx[kFT], st[3][128];
+  __shared__ double red[kFT / 32][16];
+  __shared__ double2 s_lam[2], s_cs[kMaxQubitGates];
+  __shared__ int s_op[kMaxQubitGates], s_type[kMaxQubitGates], s_m;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int b = blockIdx.x, n = a.n;
+  const double* pA = part;
+  const double2* pB = reinterpret_cast<const double2*>(part + (size_t)n_cta * 64);
+  const double2* pD = pB + (size_t)n_cta * kDT;
+  const double2* f = a.tab + kDpStates;
+  // this qubit's gates, in order
+  if (warp == 0) {
+    int m = 0;
+    for (int g0 = 0; g0 < n_ops; g0 += 32) {
+      const bool hit = g0 + lane < n_ops && ops[g0 + lane].bit0 == b;
+      const unsigned bal = __ballot_sync(0xffffffffu, hit);
+      if (hit) {
+        const int j = m + __popc(bal & ((1u << lane) - 1u));
+        s_op[j] = g0 + lane;
+        s_type[j] = ops[g0 + lane].type;
+        s_cs[j] = is_param_type(ops[g0 + lane].type) ? cs[g0 + lane] : make_double2(1.0, 0.0);
+      }
+      m += __popc(bal);
+    }
+    if (lane == 0) s_m = m;
+  }
+  // products of the factors of bits [b0, b1) but b
+  auto others = [&](int b0, int b1, uint32_t v) {
+    double2 p = make_double2(1.0, 0.0);
+    for (int c = b0; c < b1; ++c, v >>= 1)
+      if (c != b) p = cmul(p, f[2 * c + (v & 1u)]);
+    return p;
+  };
+  if (b >= bl)
+    for (int j = tid; j < 384; j += kFT) {
+      const int b0 = bl + 7 * (j >> 7);
+      st[j >> 7][j & 127] = others(b0, min(b0 + 7, n), j & 127);
+    }
+  pdl_begin();
+  double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+  if (b < kDTLog) {
+    double2 x = make_double2(0.0, 0.0);
+    for (int c = tid >> kDTLog; c < n_cta; c += kFT / kDT) {
+      const double2 v = pB[(size_t)c * kDT + (tid & (kDT - 1))];
+      x.x += v.x;
+      x.y += v.y;
+    }
+    sx[tid] = x;
+    __syncthreads();
+    if (tid < kDT) {
+      x = make_double2(sx[tid].x + sx[tid + kDT].x, sx[tid].y + sx[tid + kDT].y);
+      const double2 y = cmul_conj(x, others(0, kDTLog, tid));
+      if ((tid >> b) & 1) acc[1] = y; else acc[0] = y;
+    }
+  } else if (b < bl) {
+    double v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = 0.0;
+    for (int e = tid; e < 4 * n_cta; e += kFT)
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] += pA[(size_t)e * 16 + j];
+    const double t = warp_sum16(v);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = t;
+    __syncthreads();
+    if (tid < 16) {
+      double u = 0.0;
+      for (int w = 0; w < kFT / 32; ++w) u += red[w][tid];
+      reinterpret_cast<double*>(sx)[tid] = u;
+    }
+    __syncthreads();
+    if (tid < (1 << (bl - kDTLog))) {
+      const double2 y = cmul_conj(sx[tid], others(kDTLog, bl, tid));
+      if ((tid >> (b - kDTLog)) & 1) acc[1] = y; else acc[0] = y;
+    }
+  } else {
+    __syncthreads();
+    const uint32_t nblk = 1u << (n - bl), bit = 1u << (b - bl);
+    for (uint32_t k = tid; k < nblk; k += kFT) {
+      double2 x = pD[(size_t)k * 4];
+#pragma unroll
+      for (int w = 1; w < 4; ++w) {
+        const double2 y = pD[(size_t)k * 4 + w];
+        x.x += y.x;
+        x.y += y.y;
+      }
+      double2 p = st[0][k & 127u];
+      if (n > bl + 7) p = cmul(p, st[1][(k >> 7) & 127u]);
+      if (n > bl + 14) p = cmul(p, st[2][k >> 14]);
+      if (k & bit) cmac_conj(acc[1], x, p);
+      else cmac_conj(acc[0], x, p);
+    }
+  }
+  __syncthreads();
+  double w[4] = {acc[0].x, acc[0].y, acc[1].x, acc[1].y};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    w[j] = warp_sum(w[j]);
+    if (lane == 0) red[warp][j] = w[j];
+  }
+  __syncthreads();
+  if (tid < 4) {
+    double u = 0.0;
+    for (int q = 0; q < kFT / 32; ++q) u += red[q][tid];
+    reinterpret_cast<double*>(s_lam)[tid] = u;
+  }
+  __syncthreads();
+  // gate j: 2 Re <Lambda, (the gates after it) (-i G_j) (the gates up to it) |ref>>
+  if (tid < s_m && ops[s_op[tid]].param >= 0) {
+    double2 x = make_double2(1.0, 0.0), y = make_double2(0.0, 0.0);
+    if ((ref >> b) & 1ull) {
+      x.x = 0.0;
+      y.x = 1.0;
+    }
+    for (int j = 0; j < s_m; ++j) {
+      qubit_apply(s_type[j], s_cs[j], x, y);
+      if (j != tid) continue;
+      // 2 (-i G): RY (-y, x), RX (-i y, -i x), RZ (-i x, i y)
+      const double2 u = x, v = y;
+      if (s_type[j] == SV_GATE_RY) {
+        x = make_double2(dneg(v.x), dneg(v.y));
+        y = u;
+      } else if (s_type[j] == SV_GATE_RX) {
+        x = make_double2(v.y, dneg(v.x));
+        y = make_double2(u.y, dneg(u.x));
+      } else {
+        x = make_double2(u.y, dneg(u.x));
+        y = make_double2(dneg(v.y), v.x);
+      }
+    }
+    double g = s_lam[0].x * x.x;
+    g = fma(s_lam[0].y, x.y, g);
+    g = fma(s_lam[1].x, y.x, g);
+    g = fma(s_lam[1].y, y.y, g);
+    partial[(size_t)s_op[tid] * kRedBlocks] = g;
+  }
+}
+
 // Amplitudes per thread: as many as leave 128 blocks, up to eight (a block's set-up costs what
 // four hundred amplitudes do; one amplitude per thread in 1024 blocks took 11 us at 17 qubits).
 int dp_na(int n) { return n >= 17 ? 8 : n == 16 ? 4 : n == 15 ? 2 : 1; }
@@ -320,12 +525,11 @@ int dp_block_log(int n) { return kDTLog + (n >= 17 ? 3 : n == 16 ? 2 : n == 15 ?
 int dp_blocks(int n) { return (int)std::min<uint64_t>(1ull << (n - dp_block_log(n)), 1024); }
 
 cudaError_t dp_prepare() {
-  const void* ks[] = {(const void*)k_dp<1, false>, (const void*)k_dp<2, false>,
-                      (const void*)k_dp<4, false>, (const void*)k_dp<8, false>,
-                      (const void*)k_dp<1, true>,  (const void*)k_dp<2, true>,
-                      (const void*)k_dp<4, true>,  (const void*)k_dp<8, true>,
-                      (const void*)k_dp_lam<1>,    (const void*)k_dp_lam<2>,
-                      (const void*)k_dp_lam<4>,    (const void*)k_dp_lam<8>};
+#define DP_ALL(NA)                                                                \
+  (const void*)k_dp<NA, DP_FWD>, (const void*)k_dp<NA, DP_BWD>,                  \
+      (const void*)k_dp<NA, DP_MAKE>, (const void*)k_dp_lam<NA>, (const void*)k_prod_lam<NA>
+  const void* ks[] = {DP_ALL(1), DP_ALL(2), DP_ALL(4), DP_ALL(8)};
+#undef DP_ALL
   for (const void* k : ks) {
     const cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnePerSm);
@@ -341,26 +545,53 @@ cudaError_t dp_prepare() {
     case 2: return launch_overlapped(K(2), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);               \
     default: return launch_overlapped(K(1), g, kDT, spread_smem(0, g), s, overlap, __VA_ARGS__);              \
   }
-#define DP_FWD(NA) k_dp<NA, false>
-#define DP_BWD(NA) k_dp<NA, true>
-#define DP_LAM(NA) k_dp_lam<NA>
+#define DP_K_FWD(NA) k_dp<NA, DP_FWD>
+#define DP_K_BWD(NA) k_dp<NA, DP_BWD>
+#define DP_K_MAKE(NA) k_dp<NA, DP_MAKE>
+#define DP_K_LAM(NA) k_dp_lam<NA>
+#define DP_K_PROD(NA) k_prod_lam<NA>
 
 cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
                           bool overlap) {
   const int g = dp_blocks(a.n);
-  DP_LAUNCH(DP_FWD, in, out, a)
+  DP_LAUNCH(DP_K_FWD, in, out, a)
 }
 
 cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
                               bool overlap) {
   const int g = dp_blocks(a.n);
-  DP_LAUNCH(DP_BWD, in, out, a)
+  DP_LAUNCH(DP_K_BWD, in, out, a)
 }
 
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
                               const DpArgs& a, double* partial, cudaStream_t s, bool overlap) {
   const int g = dp_blocks(a.n);
-  DP_LAUNCH(DP_LAM, lam, psi_b, out, a, partial)
+  DP_LAUNCH(DP_K_LAM, lam, psi_b, out, a, partial)
+}
+
+cudaError_t launch_prod_fwd(double2* out, const DpArgs& a, cudaStream_t s, bool overlap) {
+  const int g = dp_blocks(a.n);
+  DP_LAUNCH(DP_K_MAKE, (const double2*)nullptr, out, a)
+}
+
+size_t prod_scratch(int n) {
+  const size_t g = (size_t)dp_blocks(n), nblk = (size_t)1 << (n - dp_block_log(n));
+  return g * 64 + g * 2 * kDT + nblk * 8;
+}
+
+static cudaError_t prod_lam(const double2* lam, const DpArgs& a, double* part, cudaStream_t s,
+                            bool overlap) {
+  const int g = dp_blocks(a.n);
+  DP_LAUNCH(DP_K_PROD, lam, a, part)
+}
+
+cudaError_t launch_prod_grads(const double2* lam, const DpArgs& a, const DOp* ops, int n_ops,
+                              const double2* cs, uint64_t ref, double* part, double* partial,
+                              cudaStream_t s, bool overlap) {
+  const cudaError_t e = prod_lam(lam, a, part, s, overlap);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(k_prod_fin, a.n, kFT, 0, s, true, (const double*)part, dp_blocks(a.n), a,
+                           dp_block_log(a.n), ops, n_ops, cs, ref, partial);
 }
 
 }  // namespace svqe

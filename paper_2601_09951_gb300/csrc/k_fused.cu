@@ -44,12 +44,6 @@ struct DiagS {
   int hl;
 };
 
-__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ double2 cmul_conj(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, dneg(a.x) * b.y));
-}
 __device__ __forceinline__ double2 rz_factor(const double2& cs, int bit) {
   return make_double2(cs.x, bit ? cs.y : dneg(cs.y));  // e^{-i phi} on |0>, e^{+i phi} on |1>
 }

@@ -1,6 +1,6 @@
 // k_prep.cu -- what an evaluation of a planned circuit derives from its angles, in one launch.
 //
-// One block per fused pass or whole-state segment.  A pass's block turns each item into the
+// One block per fused pass, whole-state segment or product prefix.  A pass's block turns each item into the
 // record the pass kernels stage (SItem), the product of the factors its RY and RX gates leave
 // out into the pass's scale, and the items' gradient factors; a segment's block writes the
 // segment's phase tables.  Done here once per evaluation instead of by every block of every
@@ -14,10 +14,6 @@ namespace svqe {
 namespace {
 
 constexpr int kPT = 128;
-
-__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
-  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
-}
 
 __device__ __forceinline__ int fkind_of(int type) {
   switch (type) {
@@ -114,6 +110,18 @@ __device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
   if (lane == 0) scales[u.idx] = sh + sl;
 }
 
+// Index bits [b0, b1) and their values v of entry j of a segment's tables.
+__device__ __forceinline__ void tab_bits(int j, int bl, int n, int& b0, int& b1, uint32_t& v) {
+  if (j < 128) {
+    b0 = 0; b1 = kDpThreadLog; v = j;
+  } else if (j < 136) {
+    b0 = kDpThreadLog; b1 = bl; v = j - 128;
+  } else {
+    const int t = (j - 136) >> 7;
+    b0 = bl + 7 * t; b1 = min(b0 + 7, n); v = (j - 136) & 127;
+  }
+}
+
 __device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, int n, int bl,
                         double2* tab) {
   // (cos, sin) of the angle sum of each index bit's RZ gates
@@ -145,17 +153,10 @@ __device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, 
     if (any) atomicOr(&has, 1u << threadIdx.x);
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < kDpTab; j += kPT) {
+  for (int j = threadIdx.x; j < kDpStates; j += kPT) {
     int b0, b1;
     uint32_t v;
-    if (j < 128) {
-      b0 = 0; b1 = kDpThreadLog; v = j;
-    } else if (j < 136) {
-      b0 = kDpThreadLog; b1 = bl; v = j - 128;
-    } else {
-      const int t = (j - 136) >> 7;
-      b0 = bl + 7 * t; b1 = min(b0 + 7, n); v = (j - 136) & 127;
-    }
+    tab_bits(j, bl, n, b0, b1, v);
     double2 p = make_double2(1.0, 0.0);
     for (int b = b0; b < b1; ++b, v >>= 1)
       if ((has >> b) & 1u) p = cmul(p, make_double2(cs[b].x, v & 1u ? cs[b].y : dneg(cs[b].y)));
@@ -163,16 +164,65 @@ __device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, 
   }
 }
 
+// The product prefix: ops [0, count) act on single qubits of the reference state, so their
+// result is a product of qubit states; the tables hold products of its factors.
+__device__ void prep_prod(const PrepUnit& u, const DOp* ops, const double* theta, int n, int bl,
+                          uint64_t ref, double2* cs, double2* tab) {
+  __shared__ double2 s_cs[kPT];
+  __shared__ int s_type[kPT], s_bit[kPT];
+  __shared__ double2 s_f[32][2];
+  const int tid = threadIdx.x;
+  double2 x = make_double2(1.0, 0.0), y = make_double2(0.0, 0.0);
+  if ((ref >> (tid & 31)) & 1ull) {
+    x.x = 0.0;
+    y.x = 1.0;
+  }
+  for (int g0 = 0; g0 < u.count; g0 += kPT) {
+    const int g = g0 + tid;
+    __syncthreads();
+    if (g < u.count) {
+      double2 v = make_double2(1.0, 0.0);
+      if (is_param_type(ops[g].type)) {
+        angle_cs(ops, g, theta, v.x, v.y);
+        cs[g] = v;
+      }
+      s_cs[tid] = v;
+      s_type[tid] = ops[g].type;
+      s_bit[tid] = ops[g].bit0;
+    }
+    __syncthreads();
+    if (tid < n)
+      for (int j = 0; j < min(kPT, u.count - g0); ++j)
+        if (s_bit[j] == tid) qubit_apply(s_type[j], s_cs[j], x, y);
+  }
+  double2* t = tab + (size_t)u.idx * kDpTab;
+  if (tid < n) {
+    s_f[tid][0] = t[kDpStates + 2 * tid] = x;
+    s_f[tid][1] = t[kDpStates + 2 * tid + 1] = y;
+  }
+  __syncthreads();
+  for (int j = tid; j < kDpStates; j += kPT) {
+    int b0, b1;
+    uint32_t v;
+    tab_bits(j, bl, n, b0, b1, v);
+    double2 p = make_double2(1.0, 0.0);
+    for (int b = b0; b < b1; ++b, v >>= 1) p = cmul(p, s_f[b][v & 1u]);
+    t[j] = p;
+  }
+}
+
 __global__ void __launch_bounds__(kPT) k_prep(const PrepUnit* __restrict__ units,
                                               const DOp* __restrict__ ops,
                                               const FItem* __restrict__ items,
                                               const double* __restrict__ theta, int n, int bl,
+                                              uint64_t ref,
                                               Rot* __restrict__ coefs, SItem* __restrict__ sitems,
                                               double* __restrict__ scales,
                                               double2* __restrict__ cs,
                                               double2* __restrict__ dptab) {
   const PrepUnit u = units[blockIdx.x];
-  if (u.dp) prep_dp(u, ops, theta, n, bl, dptab);
+  if (u.kind == PREP_DP) prep_dp(u, ops, theta, n, bl, dptab);
+  else if (u.kind == PREP_PROD) prep_prod(u, ops, theta, n, bl, ref, cs, dptab);
   else prep_pass(u, ops, items, theta, coefs, sitems, scales, cs);
 }
 
@@ -181,11 +231,11 @@ __global__ void __launch_bounds__(kPT) k_prep(const PrepUnit* __restrict__ units
 static_assert(kDpMaxRz + kDpMaxCz <= 64, "a segment's diagonal ops fit prep_dp's arrays");
 
 cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,
-                        const double* theta, int n, Rot* coefs, SItem* sitems, double* scales,
-                        double2* cs, double2* dptab, cudaStream_t s) {
+                        const double* theta, int n, uint64_t ref, Rot* coefs, SItem* sitems,
+                        double* scales, double2* cs, double2* dptab, cudaStream_t s) {
   if (n_units <= 0) return cudaSuccess;
   k_prep<<<n_units, kPT, 0, s>>>(units, ops, items, theta, n, n >= kDpMinQubits ? dp_block_log(n) : n,
-                                 coefs, sitems, scales, cs, dptab);
+                                 ref, coefs, sitems, scales, cs, dptab);
   return cudaGetLastError();
 }
 

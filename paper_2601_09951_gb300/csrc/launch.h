@@ -51,8 +51,8 @@ cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Ro
 // ops' lifting coefficients, the passes' items and scales, (cos, sin) of the RZ gates and the
 // phase tables (kDpTab entries each) of the whole-state segments on n qubits.
 cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,
-                        const double* theta, int n, Rot* coefs, SItem* sitems, double* scales,
-                        double2* cs, double2* dptab, cudaStream_t s);
+                        const double* theta, int n, uint64_t ref, Rot* coefs, SItem* sitems,
+                        double* scales, double2* cs, double2* dptab, cudaStream_t s);
 // Apply (inv = false) or un-apply one op on psi; coef points at the op's Rot.
 cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef, bool inv,
                             cudaStream_t s, bool overlap = false);
@@ -129,6 +129,19 @@ cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, 
 // into partial[op * kRedBlocks + block], block < dp_blocks(n)
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
                               const DpArgs& a, double* partial, cudaStream_t s, bool overlap);
+
+// The product prefix (k_dp.cu): a circuit's leading one-qubit gates on the reference state make
+// a product state, and the CNOT/X run after them (if any) permutes it.  a: the run's map (the
+// identity without one) and the product's tables.
+// out[P(k)] = prod(k)
+cudaError_t launch_prod_fwd(double2* out, const DpArgs& a, cudaStream_t s, bool overlap);
+// Gradients of the prefix's parameterised ops [0, n_ops) from lambda after the run:
+// partial[op * kRedBlocks] = the whole of 2 Im<lambda|G|psi>.  part: prod_scratch(n) doubles.
+size_t prod_scratch(int n);
+cudaError_t launch_prod_grads(const double2* lam, const DpArgs& a, const DOp* ops, int n_ops,
+                              const double2* cs, uint64_t ref, double* part, double* partial,
+                              cudaStream_t s, bool overlap);
+constexpr int kMaxQubitGates = 64;  // gates of one qubit in a product prefix
 
 // Gradient shares only (psi and lambda unchanged) of a pass whose items are single ops:
 // partial[op * kRedBlocks + b] as for launch_bpass.

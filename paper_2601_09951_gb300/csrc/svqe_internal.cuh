@@ -308,6 +308,64 @@ __device__ __forceinline__ int group_value(const DGroup& G, uint64_t k, const do
   return G.cls;
 }
 
+__device__ __forceinline__ double2 cmul(const double2& a, const double2& b) {
+  return make_double2(fma(a.x, b.x, dneg(a.y) * b.y), fma(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ double2 cmul_conj(const double2& a, const double2& b) {  // a conj(b)
+  return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, dneg(a.x) * b.y));
+}
+// acc += a conj(b)
+__device__ __forceinline__ void cmac_conj(double2& acc, const double2& a, const double2& b) {
+  acc.x = fma(a.x, b.x, acc.x);
+  acc.x = fma(a.y, b.y, acc.x);
+  acc.y = fma(a.y, b.x, acc.y);
+  acc.y = fma(dneg(a.x), b.y, acc.y);
+}
+
+// Sum over the warp of 16 values per lane by recursive halving (16 DADD per lane instead of
+// 80); afterwards lanes 2j and 2j+1 hold the warp total of value j.
+__device__ __forceinline__ double warp_sum16(double (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int o = 16 >> s, h = 8 >> s;
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = up ? v[i] : v[i + h];
+      const double keep = up ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// One-qubit gate with (cos phi, sin phi) = cs on a single qubit's state (x, y).
+__device__ __forceinline__ void qubit_apply(int type, const double2& cs, double2& x, double2& y) {
+  const double2 a = x, b = y;
+  switch (type) {
+    case SV_GATE_X: x = b; y = a; break;
+    case SV_GATE_H: {
+      const double r = 0.70710678118654752440;
+      x = make_double2(r * (a.x + b.x), r * (a.y + b.y));
+      y = make_double2(r * (a.x - b.x), r * (a.y - b.y));
+    } break;
+    case SV_GATE_RY:
+      x = make_double2(fma(cs.x, a.x, dneg(cs.y) * b.x), fma(cs.x, a.y, dneg(cs.y) * b.y));
+      y = make_double2(fma(cs.y, a.x, cs.x * b.x), fma(cs.y, a.y, cs.x * b.y));
+      break;
+    case SV_GATE_RX:  // x' = c x - i s y, y' = c y - i s x
+      x = make_double2(fma(cs.x, a.x, cs.y * b.y), fma(cs.x, a.y, dneg(cs.y) * b.x));
+      y = make_double2(fma(cs.x, b.x, cs.y * a.y), fma(cs.x, b.y, dneg(cs.y) * a.x));
+      break;
+    case SV_GATE_RZ:
+      x = cmul_conj(a, cs);
+      y = cmul(b, cs);
+      break;
+    default: break;
+  }
+}
+
 // ------------------------------------------------------------------------------ launch overlap
 // A kernel launched with launch_overlapped starts while its predecessor on the stream runs.
 // Before pdl_begin it may read only what kernels before that predecessor wrote (a kernel lets

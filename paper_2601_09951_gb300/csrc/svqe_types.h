@@ -152,17 +152,20 @@ struct SItem {
 };
 static_assert(sizeof(SItem) == 56, "SItem layout");
 
-// What the preparation kernel does for one fused pass (items [first, first + count) to the
-// same SItem places, its scale to place idx) or one whole-state segment (RZ/CZ ops [first,
-// first + count), its phase tables to place idx).
+// What the preparation kernel does for one unit: a fused pass (items [first, first + count) to
+// the same SItem places, its scale to place idx), a whole-state segment (RZ/CZ ops [first, first
+// + count), its phase tables to table idx) or the product prefix (ops [0, count), its tables and
+// qubit states to table idx).
+enum { PREP_PASS = 0, PREP_DP = 1, PREP_PROD = 2 };
 struct PrepUnit {
-  int32_t dp;
+  int32_t kind;
   int32_t first, count, idx;
 };
-// Phase tables of a whole-state segment: the thread's 128 phases, the 8 of a thread's slots, and
-// three tables of 128 over block-index bits.
+// Tables of a whole-state segment over 128 thread indices, a thread's 8 slots and three times 7
+// block-index bits, then (product prefix) the states of up to 32 qubits.
 constexpr int kDpThreadLog = 7;
-constexpr int kDpTab = 128 + 8 + 3 * 128;
+constexpr int kDpStates = 128 + 8 + 3 * 128;
+constexpr int kDpTab = kDpStates + 64;
 
 __host__ __device__ __forceinline__ bool is_param_type(int t) {
   return t == SV_GATE_RX || t == SV_GATE_RY || t == SV_GATE_RZ || t == SV_GATE_SINGLE_EXC ||
