@@ -198,6 +198,15 @@ uint64_t sv_ctx_device_bytes(int32_t n) {
   return 2 * sv_state_bytes(n) + (uint64_t)(kRedBlocks + 8) * sizeof(double);
 }
 
+// ------------------------------------------------------------------------------ small registers
+// Small registers are evaluated by one block in one launch (k_small, the batched kernel's
+// routine) instead of some twenty launches; descent steps loop inside it.  A context does so up
+// to kSmallQubits: one block's time doubles with each qubit and the passes' does not (four
+// hardware-efficient layers, one block against passes: 113 and 188 us at 8 qubits, 187 and 303
+// at 10, 313 and 292 at 11, 573 and 244 at 12).  The call without device allocation, which has
+// no passes and launches every gate, does up to the 12 qubits the routine holds.
+static constexpr int kSmallQubits = 10;
+
 // ------------------------------------------------------------------------------ contexts
 sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
   clear_error();
@@ -232,8 +241,8 @@ sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
     return SV_ENOMEM;
   }
   c->ref = 0;
-  if (fused_prepare() != cudaSuccess || dp_prepare() != cudaSuccess ||
-      small_prepare() != cudaSuccess ||
+  if (fused_prepare() != cudaSuccess || dp_prepare(n) != cudaSuccess ||
+      (n <= kSmallQubits && small_prepare() != cudaSuccess) ||
       launch_init_basis(c->psi, n, 0, c->stream) != cudaSuccess) {
     set_error("init kernel launch failed");
     sv_destroy(c);
@@ -678,21 +687,47 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
           ops[c->plan.items[i].op + g].flags = pass_blocks(P);
     }
   }
+  // A chunk of passes right before a whole-state segment leaves its scale to the segment's phase
+  // tables, which saves 2 of a pass's 16 to 24 FP64 operations per amplitude and state (a pass of
+  // one gate runs that gate's own, normalised kernel: such a chunk keeps its scales).
+  auto folds = [&](size_t ci) {
+    if (ci + 1 >= c->chunks.size() || c->chunks[ci].kind != sv_ctx::CH_PASSES ||
+        c->chunks[ci + 1].kind != sv_ctx::CH_DP)
+      return false;
+    int items = 0;
+    for (int p = c->chunks[ci].p0; p < c->chunks[ci].p1; ++p) {
+      if (single_op(c, p) >= 0) return false;
+      items += c->plan.passes[p].n_items;
+    }
+    return items > 0 && items <= kMaxFoldItems;
+  };
   std::vector<PrepUnit> units;
   int n_dp = 0;
-  for (const sv_ctx::Chunk& ch : c->chunks) {
+  int cf = 0, cl = 0;  // items of the chunk whose scale the next segment takes
+  for (size_t ci = 0; ci < c->chunks.size(); ++ci) {
+    const sv_ctx::Chunk& ch = c->chunks[ci];
     if (ch.kind == sv_ctx::CH_DP) {
       int split = 0;
       while (split < ch.count && (hc.ops[ch.first + split].type == SV_GATE_RZ ||
                                   hc.ops[ch.first + split].type == SV_GATE_CZ))
         ++split;
-      units.push_back(PrepUnit{PREP_DP, ch.first, split, n_dp++});
-    } else if (ch.kind == sv_ctx::CH_PROD) {
-      units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++});
+      units.push_back(PrepUnit{PREP_DP, ch.first, split, n_dp++, cf, cl});
+      cf = cl = 0;
+      continue;
+    }
+    if (ch.kind == sv_ctx::CH_PROD) {
+      units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++, 0, 0});
       SV_CUDA(grow(c->prod, c->prod_cap, prod_scratch(c->n)), c);
+      continue;
+    }
+    cf = cl = 0;
+    if (folds(ci)) {
+      cf = c->plan.passes[ch.p0].first_item;
+      cl = c->plan.passes[ch.p1 - 1].first_item + c->plan.passes[ch.p1 - 1].n_items;
     }
     for (int p = ch.p0; p < ch.p1; ++p)
-      units.push_back(PrepUnit{PREP_PASS, c->plan.passes[p].first_item, c->plan.passes[p].n_items, p});
+      units.push_back(PrepUnit{PREP_PASS, c->plan.passes[p].first_item,
+                               c->plan.passes[p].n_items, p, cf, cl});
   }
   auto align = [](size_t v) { return (v + 255) / 256 * 256; };
   const size_t o_items = align(n_ops * sizeof(DOp));
@@ -891,14 +926,6 @@ sv_status sv_tile_bits(const sv_ctx* c, int32_t* tile_bits) {
   return SV_OK;
 }
 
-// ------------------------------------------------------------------------------ small registers
-// Small registers are evaluated by one block in one launch (k_small, the batched kernel's
-// routine) instead of some twenty launches; descent steps loop inside it.  A context does so up
-// to kSmallQubits: one block's time doubles with each qubit and the passes' does not (four
-// hardware-efficient layers, one block against passes: 113 and 188 us at 8 qubits, 187 and 303
-// at 10, 313 and 292 at 11, 573 and 244 at 12).  The call without device allocation, which has
-// no passes and launches every gate, does up to the 12 qubits the routine holds.
-static constexpr int kSmallQubits = 10;
 static constexpr int64_t kSmallCkptAmps = 1 << 19;  // 8 MiB of checkpoint scratch at most
 
 bool svqe::pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,

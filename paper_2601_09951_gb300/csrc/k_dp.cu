@@ -289,6 +289,8 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
     double v = 0.0;
 #pragma unroll
     for (int w = 0; w < kDT / 32; ++w) v += red[w][j];
+    // (psi and lambda carry the scale that the passes before the segment left out)
+    v *= a.tab[kDpStates].x;
     partial[(size_t)a.rz_op[tid] * kRedBlocks + blockIdx.x] = neg ? dneg(v) : v;
   }
 }
@@ -524,18 +526,27 @@ int dp_na(int n) { return n >= 17 ? 8 : n == 16 ? 4 : n == 15 ? 2 : 1; }
 int dp_block_log(int n) { return kDTLog + (n >= 17 ? 3 : n == 16 ? 2 : n == 15 ? 1 : 0); }
 int dp_blocks(int n) { return (int)std::min<uint64_t>(1ull << (n - dp_block_log(n)), 1024); }
 
-cudaError_t dp_prepare() {
-#define DP_ALL(NA)                                                                \
-  (const void*)k_dp<NA, DP_FWD>, (const void*)k_dp<NA, DP_BWD>,                  \
-      (const void*)k_dp<NA, DP_MAKE>, (const void*)k_dp_lam<NA>, (const void*)k_prod_lam<NA>
-  const void* ks[] = {DP_ALL(1), DP_ALL(2), DP_ALL(4), DP_ALL(8)};
-#undef DP_ALL
+template <int NA>
+static cudaError_t prepare_na() {
+  const void* ks[] = {(const void*)k_dp<NA, DP_FWD>, (const void*)k_dp<NA, DP_BWD>,
+                      (const void*)k_dp<NA, DP_MAKE>, (const void*)k_dp_lam<NA>,
+                      (const void*)k_prod_lam<NA>};
   for (const void* k : ks) {
     const cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnePerSm);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+cudaError_t dp_prepare(int n) {
+  if (n < kDpMinQubits || dp_blocks(n) > kSms) return cudaSuccess;
+  switch (dp_na(n)) {
+    case 8: return prepare_na<8>();
+    case 4: return prepare_na<4>();
+    case 2: return prepare_na<2>();
+    default: return prepare_na<1>();
+  }
 }
 
 #define DP_LAUNCH(K, ...)                                                                     \

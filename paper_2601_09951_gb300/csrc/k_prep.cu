@@ -33,12 +33,34 @@ __device__ __forceinline__ void angle_cs(const DOp* ops, int l, const double* th
   sincos(0.5 * (param >= 0 ? theta[param] : ops[l].fixed), &s, &c);
 }
 
+// The factor an item leaves out, as an unevaluated sum (1 for items that leave none).
+__device__ __forceinline__ void item_factor(const FItem& it, const DOp* ops, const double* theta,
+                                            double& f, double& flo) {
+  f = 1.0;
+  flo = 0.0;
+  if (it.kind == 0 && (it.local.type == SV_GATE_RY || it.local.type == SV_GATE_RX)) {
+    double c, s;
+    angle_cs(ops, it.op, theta, c, s);
+    const RotT t = make_rott(c, s);
+    f = t.f;
+    flo = t.flo;
+  }
+}
+
 // Items in chunks of 32, the last chunk first (the gradient factors are products over later
 // items), one lane each.
 __device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
                           const double* theta, Rot* coefs, SItem* sitems, double* scales,
                           double2* cs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool folded = u.cl > u.cf;
+  __shared__ double s_f2[kPT];  // folded: f^2 of the chunk's items (at most kPT)
+  if (folded) {
+    double f = 1.0, flo;
+    if (u.cf + (int)threadIdx.x < u.cl) item_factor(items[u.cf + threadIdx.x], ops, theta, f, flo);
+    s_f2[threadIdx.x] = f * f;
+    __syncthreads();
+  }
   if (warp > 0) {
     // the other warps: (cos, sin) of the RZ gates of diagonal items
     for (int i = u.first; i < u.first + u.count; ++i) {
@@ -98,6 +120,11 @@ __device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
     const double nx = __shfl_down_sync(0xffffffffu, w, 1);
     o.f = fac * (lane == 31 ? 1.0 : nx);
     fac *= __shfl_sync(0xffffffffu, w, 0);
+    if (folded && on) {
+      double g = 1.0;
+      for (int j = 0; j <= u.first + i - u.cf; ++j) g *= s_f2[j];
+      o.f = 1.0 / g;
+    }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
       const double h = __shfl_xor_sync(0xffffffffu, f, d);
@@ -107,7 +134,7 @@ __device__ void prep_pass(const PrepUnit& u, const DOp* ops, const FItem* items,
     dd_mul(sh, sl, __shfl_sync(0xffffffffu, f, 0), __shfl_sync(0xffffffffu, flo, 0));
     if (on) sitems[u.first + i] = o;
   }
-  if (lane == 0) scales[u.idx] = sh + sl;
+  if (lane == 0) scales[u.idx] = folded ? 1.0 : sh + sl;
 }
 
 // Index bits [b0, b1) and their values v of entry j of a segment's tables.
@@ -122,8 +149,30 @@ __device__ __forceinline__ void tab_bits(int j, int bl, int n, int& b0, int& b1,
   }
 }
 
-__device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, int n, int bl,
-                        double2* tab) {
+__device__ void prep_dp(const PrepUnit& u, const DOp* ops, const FItem* items,
+                        const double* theta, int n, int bl, double2* tab) {
+  // the product of the factors the chunk of passes before it left out
+  double scale = 1.0;
+  if (u.cl > u.cf) {
+    __shared__ double s_h[kPT / 32], s_l[kPT / 32];
+    double f = 1.0, flo = 0.0;
+    if (u.cf + (int)threadIdx.x < u.cl) item_factor(items[u.cf + threadIdx.x], ops, theta, f, flo);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const double h = __shfl_xor_sync(0xffffffffu, f, d);
+      const double l = __shfl_xor_sync(0xffffffffu, flo, d);
+      dd_mul(f, flo, h, l);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      s_h[threadIdx.x >> 5] = f;
+      s_l[threadIdx.x >> 5] = flo;
+    }
+    __syncthreads();
+    double h = s_h[0], l = s_l[0];
+#pragma unroll
+    for (int w = 1; w < kPT / 32; ++w) dd_mul(h, l, s_h[w], s_l[w]);
+    scale = h + l;
+  }
   // (cos, sin) of the angle sum of each index bit's RZ gates
   __shared__ double2 cs[32];
   __shared__ double2 op_cs[64];
@@ -157,11 +206,13 @@ __device__ void prep_dp(const PrepUnit& u, const DOp* ops, const double* theta, 
     int b0, b1;
     uint32_t v;
     tab_bits(j, bl, n, b0, b1, v);
-    double2 p = make_double2(1.0, 0.0);
+    double2 p = make_double2(j < 128 ? scale : 1.0, 0.0);
     for (int b = b0; b < b1; ++b, v >>= 1)
       if ((has >> b) & 1u) p = cmul(p, make_double2(cs[b].x, v & 1u ? cs[b].y : dneg(cs[b].y)));
     tab[(size_t)u.idx * kDpTab + j] = p;
   }
+  if (threadIdx.x == 0)
+    tab[(size_t)u.idx * kDpTab + kDpStates] = make_double2(1.0 / (scale * scale), 0.0);
 }
 
 // The product prefix: ops [0, count) act on single qubits of the reference state, so their
@@ -221,13 +272,14 @@ __global__ void __launch_bounds__(kPT) k_prep(const PrepUnit* __restrict__ units
                                               double2* __restrict__ cs,
                                               double2* __restrict__ dptab) {
   const PrepUnit u = units[blockIdx.x];
-  if (u.kind == PREP_DP) prep_dp(u, ops, theta, n, bl, dptab);
+  if (u.kind == PREP_DP) prep_dp(u, ops, items, theta, n, bl, dptab);
   else if (u.kind == PREP_PROD) prep_prod(u, ops, theta, n, bl, ref, cs, dptab);
   else prep_pass(u, ops, items, theta, coefs, sitems, scales, cs);
 }
 
 }  // namespace
 
+static_assert(kMaxFoldItems <= kPT, "one thread per item of a folded chunk");
 static_assert(kDpMaxRz + kDpMaxCz <= 64, "a segment's diagonal ops fit prep_dp's arrays");
 
 cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,

@@ -50,6 +50,7 @@ cudaError_t launch_prep_coefs(const DOp* ops, int n_ops, const double* theta, Ro
 // Everything of a planned circuit that depends on theta, one block per unit (k_prep.cu): the
 // ops' lifting coefficients, the passes' items and scales, (cos, sin) of the RZ gates and the
 // phase tables (kDpTab entries each) of the whole-state segments on n qubits.
+constexpr int kMaxFoldItems = 128;
 cudaError_t launch_prep(const PrepUnit* units, int n_units, const DOp* ops, const FItem* items,
                         const double* theta, int n, uint64_t ref, Rot* coefs, SItem* sitems,
                         double* scales, double2* cs, double2* dptab, cudaStream_t s);
@@ -116,7 +117,7 @@ struct DpArgs {
 };
 // CTAs of a segment's kernels on n qubits (a power of two).
 int dp_blocks(int n);
-cudaError_t dp_prepare();
+cudaError_t dp_prepare(int n);  // (attributes of the kernels an n-qubit state uses)
 // log2 of the amplitudes per block of a segment's kernels on n qubits
 int dp_block_log(int n);
 // out[P(k)] = phase(k) in[k]

@@ -137,13 +137,15 @@ static_assert(sizeof(FItem) == 64, "FItem layout");
 // angles, forward orientation).  RY and RX gates are stored without their normalisation: with
 // mode 0 (|cos phi| >= |sin phi|) p = tan phi and R(phi) = c [[1, -p], [p, 1]], c = cos phi;
 // with mode 1 p = cot phi and R(phi) = c [[p, -1], [1, p]], c = sin phi.  The pass multiplies its
-// amplitudes once by the product of its factors c.  Excitations and single RZ gates: p, q and
+// amplitudes once by the product of its factors c, or (folded) leaves that to the whole-state
+// segment after its chunk of passes.  Excitations and single RZ gates: p, q and
 // mode are Rot's a, b and k.
 enum ItemKind { F_SWAP = 0, F_H = 1, F_EXC = 2, F_ROTZ = 3, F_NEG = 4, F_RY = 5, F_RX = 6,
                 F_DIAG = 7 };
 struct SItem {
   double p, q;
-  double f;  // factor of the item's gradient sum: the product of c^2 over the items after it
+  double f;  // factor of the item's gradient sum: the product of c^2 over the pass's items after
+             // it; in a folded chunk 1 / that over the chunk's items up to and with it
   uint32_t lo, fl;
   uint8_t sb[4];
   int16_t kind, k;
@@ -155,14 +157,17 @@ static_assert(sizeof(SItem) == 56, "SItem layout");
 // What the preparation kernel does for one unit: a fused pass (items [first, first + count) to
 // the same SItem places, its scale to place idx), a whole-state segment (RZ/CZ ops [first, first
 // + count), its phase tables to table idx) or the product prefix (ops [0, count), its tables and
-// qubit states to table idx).
+// qubit states to table idx).  A pass and the segment that takes its chunk's scale (folded) have
+// the chunk's items as [cf, cl); otherwise cf = cl.
 enum { PREP_PASS = 0, PREP_DP = 1, PREP_PROD = 2 };
 struct PrepUnit {
   int32_t kind;
   int32_t first, count, idx;
+  int32_t cf, cl;
 };
 // Tables of a whole-state segment over 128 thread indices, a thread's 8 slots and three times 7
-// block-index bits, then (product prefix) the states of up to 32 qubits.
+// block-index bits, then the states of up to 32 qubits (product prefix) or, in the first entry, the
+// factor of the segment's gradients (folded scale).
 constexpr int kDpThreadLog = 7;
 constexpr int kDpStates = 128 + 8 + 3 * 128;
 constexpr int kDpTab = kDpStates + 64;
