@@ -1100,8 +1100,8 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
       SV_CUDA(launch_adjoint_op(c->psi, c->lam, c->n, op, c->coef + l, part, c->stream), c);
     }
   }
-  SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, energy_dev,
-                        theta_upd, lr, traj, c->stream, !prod), c);
+  SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, hpsi_blocks(c->n),
+                        energy_dev, theta_upd, lr, traj, c->stream, !prod), c);
   return SV_OK;
 }
 
@@ -1147,8 +1147,7 @@ sv_status sv_expval_paulisum(sv_ctx* c, const sv_ham* H, double* energy_out) {
   if (!c || !H || !energy_out) { set_error("NULL argument"); return SV_EINVAL; }
   SV_CHECK_STICKY(c);
   if (H->n != c->n) { set_error("Hamiltonian has %d qubits, context %d", H->n, c->n); return SV_EINVAL; }
-  SV_CUDA(launch_hpsi(c->psi, nullptr, c->n, H->groups, H->n_groups, H->tables, c->epart,
-                      c->stream), c);
+  SV_CUDA(launch_expval(c->psi, c->n, H->groups, H->n_groups, H->tables, c->epart, c->stream), c);
   SV_CUDA(launch_sum(c->epart, kRedBlocks, c->scal, c->stream), c);
   SV_CUDA(cudaMemcpyAsync(energy_out, c->scal, sizeof(double), cudaMemcpyDeviceToHost,
                           c->stream), c);

@@ -415,8 +415,8 @@ __global__ void __launch_bounds__(kFT) k_prod_fin(const double* __restrict__ par
   };
   if (b >= bl)
     for (int j = tid; j < 384; j += kFT) {
-      const int b0 = bl + 7 * (j >> 7);
-      st[j >> 7][j & 127] = others(b0, min(b0 + 7, n), j & 127);
+      const int b0 = bl + 7 * (j >> 7), b1 = min(b0 + 7, n);
+      if (b0 < b1 && (j & 127) < (1 << (b1 - b0))) st[j >> 7][j & 127] = others(b0, b1, j & 127);
     }
   pdl_begin();
   double2 acc[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};

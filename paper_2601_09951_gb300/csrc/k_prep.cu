@@ -222,6 +222,7 @@ __device__ void prep_prod(const PrepUnit& u, const DOp* ops, const double* theta
   __shared__ double2 s_cs[kPT];
   __shared__ int s_type[kPT], s_bit[kPT];
   __shared__ double2 s_f[32][2];
+  __shared__ uint8_t s_list[32][kMaxQubitGates];
   const int tid = threadIdx.x;
   double2 x = make_double2(1.0, 0.0), y = make_double2(0.0, 0.0);
   if ((ref >> (tid & 31)) & 1ull) {
@@ -242,9 +243,13 @@ __device__ void prep_prod(const PrepUnit& u, const DOp* ops, const double* theta
       s_bit[tid] = ops[g].bit0;
     }
     __syncthreads();
+    // each qubit's gates are listed first and then applied by all qubits at once: applied as they
+    // are met, every gate would be a step of its own for the whole warp
+    int m = 0;
     if (tid < n)
       for (int j = 0; j < min(kPT, u.count - g0); ++j)
-        if (s_bit[j] == tid) qubit_apply(s_type[j], s_cs[j], x, y);
+        if (s_bit[j] == tid) s_list[tid][m++] = (uint8_t)j;
+    for (int j = 0; j < m; ++j) qubit_apply(s_type[s_list[tid][j]], s_cs[s_list[tid][j]], x, y);
   }
   double2* t = tab + (size_t)u.idx * kDpTab;
   if (tid < n) {

@@ -4,6 +4,8 @@
 // thread, 64-bit indices.  Gate arithmetic follows svqe_internal.cuh (lifting rotations,
 // integer sign flips).  Reductions use a fixed grid of kRedBlocks blocks and fixed-order
 // sums, so results do not depend on scheduling.
+#include <algorithm>
+
 #include "launch.h"
 #include "svqe_internal.cuh"
 
@@ -171,56 +173,184 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(double2* __restrict__ psi,
   }
 }
 
+// A group as the threads of one tile read it: masks over the tile's bits, and the part of the
+// table offset (or of the sign) that the tile's index decides.
+struct HRec {
+  uint32_t x;     // (all bits)
+  uint32_t zlow;  // z mask over the tile's bits
+  int32_t cls;
+  int32_t pad;
+  int64_t toff;   // tables: offset of the entry at tile-bit index 0
+  double c;       // one term: its coefficient, the tile's sign applied
+};
+
+// acc += f v of a one-term group: the sign (-1)^popc(zu & k) as the thread's part and a mask per
+// bit of u; IMAG: (i f) v = (-f v.y, f v.x).
+template <int U, int UB, bool IMAG>
+__device__ __forceinline__ void hpsi_term(const HRec& G, uint32_t t, uint32_t zu,
+                                          const double2 (&v)[U], double2 (&acc)[U]) {
+  const uint32_t s0 = (uint32_t)(__popc(t & G.zlow) & 1) << 31;
+  const int chi = __double2hiint(G.c), clo = __double2loint(G.c);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    uint32_t s = s0;
+#pragma unroll
+    for (int b = 0; b < UB; ++b)
+      if ((u >> b) & 1) s ^= (zu << (31 - b)) & 0x80000000u;
+    const double f = __hiloint2double(chi ^ (int)s, clo);
+    if constexpr (IMAG) {
+      acc[u].x = fma(dneg(f), v[u].y, acc[u].x);
+      acc[u].y = fma(f, v[u].x, acc[u].y);
+    } else {
+      acc[u].x = fma(f, v[u].x, acc[u].x);
+      acc[u].y = fma(f, v[u].y, acc[u].y);
+    }
+  }
+}
+
+// acc += f v of a tabulated group: the table index as the thread's part and an offset per bit
+// of u.
+template <int U, int TB, int UB, int CLS>
+__device__ __forceinline__ void hpsi_table(const HRec& G, uint32_t t,
+                                           const double2* __restrict__ tables,
+                                           const double2 (&v)[U], double2 (&acc)[U]) {
+  const uint32_t tl = G.zlow & ((1u << TB) - 1u), zu = G.zlow >> TB;
+  const uint32_t ti0 = pext64(t, tl);
+  const int sh = __popc(tl);
+  uint32_t d[3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b) d[b] = ((zu >> b) & 1u) << (sh + __popc(zu & ((1u << b) - 1u)));
+  const double* tab = reinterpret_cast<const double*>(tables + G.toff);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    uint32_t ti = ti0;
+#pragma unroll
+    for (int b = 0; b < UB; ++b)
+      if ((u >> b) & 1) ti += d[b];
+    if constexpr (CLS == 0) {
+      const double f = tab[2 * ti];
+      acc[u].x = fma(f, v[u].x, acc[u].x);
+      acc[u].y = fma(f, v[u].y, acc[u].y);
+    } else if constexpr (CLS == 1) {
+      const double f = tab[2 * ti + 1];
+      acc[u].x = fma(dneg(f), v[u].y, acc[u].x);
+      acc[u].y = fma(f, v[u].x, acc[u].y);
+    } else {
+      group_madd(2, make_double2(tab[2 * ti], tab[2 * ti + 1]), v[u], acc[u]);
+    }
+  }
+}
+
 // lambda[k] = sum_g f_g(k) psi[k ^ x_g];  partial[b] = block share of Re<psi|lambda>.
-__global__ void __launch_bounds__(kThreads) k_hpsi(const double2* __restrict__ psi,
-                                                   double2* __restrict__ lam, uint64_t N,
-                                                   const DGroup* __restrict__ groups,
-                                                   int n_groups,
-                                                   const double2* __restrict__ tables,
-                                                   double* __restrict__ partial) {
-  __shared__ DGroup sg[128];
+//
+// A block takes tiles of 256 U / S amplitudes: its threads are S slices of the group list times
+// 256 / S amplitudes, U amplitudes each (k = tile base + t + u 256 / S), and the slices' sums are
+// added in slice order.  S splits the groups when the state has too few amplitudes for the chip:
+// at 13 qubits 32 blocks walked 100 groups one by one, 34 us.  Records are staged per tile with
+// everything that only the tile's index decides, so an amplitude costs one load of psi, an
+// integer op or two and two FMAs per group.  On a large state FP64 binds (2 FMA per amplitude
+// and group); a software pext per amplitude and a branch on the class inside the amplitude loop
+// had kept that pipe at 75 %.
+template <int U, int S>
+__global__ void __launch_bounds__(kThreads, U == 8 ? 2 : U == 4 ? 3 : 4) k_hpsi(
+    const double2* __restrict__ psi, double2* __restrict__ lam, int n,
+    const DGroup* __restrict__ groups, int n_groups, const double2* __restrict__ tables,
+    double* __restrict__ partial) {
+  constexpr int T = kThreads / S;
+  constexpr int TB = T == 256 ? 8 : T == 128 ? 7 : T == 64 ? 6 : 5;
+  constexpr int UB = U == 8 ? 3 : U == 4 ? 2 : U == 2 ? 1 : 0;
+  constexpr int kStage = 128;
+  __shared__ HRec sg[kStage];
+  __shared__ double2 sacc[S > 1 ? kThreads * U : 1];
   __shared__ double red[kThreads / 32];
   pdl_begin();
+  const int tid = threadIdx.x, slice = tid >> TB;
+  const uint32_t t = tid & (T - 1);
+  const uint32_t ntiles = n > TB + UB ? 1u << (n - TB - UB) : 1u;
+  const uint32_t N = n >= 32 ? 0xffffffffu : 1u << n;
   double e = 0.0;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t tile = kUnroll * stride;
-  for (uint64_t base = blockIdx.x * (uint64_t)blockDim.x; base < N; base += tile) {
-    const uint64_t k0 = base + threadIdx.x;
-    double2 acc[kUnroll];
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const uint32_t base = tile << (TB + UB);
+    double2 acc[U];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) acc[u] = make_double2(0.0, 0.0);
-    for (int g0 = 0; g0 < n_groups; g0 += 128) {
-      const int cnt = min(128, n_groups - g0);
+    for (int u = 0; u < U; ++u) acc[u] = make_double2(0.0, 0.0);
+    for (int g0 = 0; g0 < n_groups; g0 += kStage) {
+      const int cnt = min(kStage, n_groups - g0);
       __syncthreads();
-      for (int t = threadIdx.x; t < cnt; t += blockDim.x) sg[t] = groups[g0 + t];
+      if (tid < cnt) {
+        const DGroup G = groups[g0 + tid];
+        HRec h;
+        h.x = (uint32_t)G.x;
+        h.zlow = (uint32_t)G.zu & ((1u << (TB + UB)) - 1u);
+        h.cls = G.cls;
+        h.pad = 0;
+        h.toff = G.toff;
+        h.c = 0.0;
+        const uint32_t zhi = (uint32_t)G.zu >> (TB + UB);
+        if (G.cls >= 4) {
+          const double2 f = tables[G.toff];
+          h.c = G.cls == 4 ? f.x : f.y;
+          if (__popc(tile & zhi) & 1) h.c = dneg(h.c);
+        } else {
+          h.toff += (int64_t)pext64(tile, zhi) << __popc(h.zlow);
+        }
+        sg[tid] = h;
+      }
       __syncthreads();
-      for (int g = 0; g < cnt; ++g) {
-        const DGroup G = sg[g];
+      for (int g = slice; g < cnt; g += S) {
+        const HRec& G = sg[g];
+        const uint32_t kx = (base | t) ^ G.x, zu = G.zlow >> TB;
+        double2 v[U];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const uint64_t k = k0 + u * stride;
-          if (k < N) {
-            const double2 v = psi[k ^ G.x];
-            double2 f;
-            const int cls = group_value(G, k, tables, f);
-            group_madd(cls, f, v, acc[u]);
-          }
+        for (int u = 0; u < U; ++u) {
+          const uint32_t k = kx ^ (uint32_t)(u << TB);
+          v[u] = k < N ? psi[k] : make_double2(0.0, 0.0);
+        }
+        // (one loop per class: with the class tested inside the loop the FMAs of every class issue)
+        switch (G.cls) {
+          case 0: hpsi_table<U, TB, UB, 0>(G, t, tables, v, acc); break;
+          case 1: hpsi_table<U, TB, UB, 1>(G, t, tables, v, acc); break;
+          case 2: hpsi_table<U, TB, UB, 2>(G, t, tables, v, acc); break;
+          case 4: hpsi_term<U, UB, false>(G, t, zu, v, acc); break;
+          default: hpsi_term<U, UB, true>(G, t, zu, v, acc); break;
         }
       }
     }
+    if (S > 1) {
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const uint64_t k = k0 + u * stride;
-      if (k < N) {
-        const double2 p = psi[k];
-        e = fma(p.x, acc[u].x, e);
-        e = fma(p.y, acc[u].y, e);
-        if (lam) lam[k] = acc[u];
+      for (int u = 0; u < U; ++u) sacc[(slice * U + u) * T + t] = acc[u];
+      __syncthreads();
+      for (int i = tid; i < T * U; i += kThreads) {
+        double2 a = sacc[i];
+#pragma unroll
+        for (int s = 1; s < S; ++s) {
+          const double2 b = sacc[s * U * T + i];
+          a.x += b.x;
+          a.y += b.y;
+        }
+        const uint32_t k = base + i;  // i = u T + t
+        if (k < N) {
+          const double2 p = psi[k];
+          e = fma(p.x, a.x, e);
+          e = fma(p.y, a.y, e);
+          lam[k] = a;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t k = (base | t) + (uint32_t)(u << TB);
+        if (k < N) {
+          const double2 p = psi[k];
+          e = fma(p.x, acc[u].x, e);
+          e = fma(p.y, acc[u].y, e);
+          lam[k] = acc[u];
+        }
       }
     }
   }
-  const double t = block_sum(e, red);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
+  const double s = block_sum(e, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
 // Energy only: E = <psi|H|psi> (Eq. 2), H the Pauli sum of Eq. 3 grouped by X mask:
@@ -248,7 +378,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_expval(const double2* __restric
                                                         const double2* __restrict__ tables,
                                                         double* __restrict__ partial) {
   __shared__ double red[kThreads / 32];
-  pdl_begin();
   const int lane = threadIdx.x & 31;
   const int h_log = n - 1;  // N/2 pairs per group
   const int c_log = min(h_log, 5 + kEULog);
@@ -352,14 +481,14 @@ __global__ void k_sum(const double* __restrict__ partial, int count, double* __r
 __global__ void k_finish(const DOp* __restrict__ ops, int n_ops,
                          const double* __restrict__ partial, int n_params,
                          double* __restrict__ grad, const double* __restrict__ epart,
-                         double* __restrict__ energy, double* __restrict__ theta_upd, double lr,
+                         int n_epart, double* __restrict__ energy, double* __restrict__ theta_upd, double lr,
                          double* __restrict__ traj) {
   __shared__ double red[32];
   pdl_begin();
   if (blockIdx.x == gridDim.x - 1) {
     if (!epart) return;
     double v = 0.0;
-    for (int i = threadIdx.x; i < kRedBlocks; i += blockDim.x) v += epart[i];
+    for (int i = threadIdx.x; i < n_epart; i += blockDim.x) v += epart[i];
     const double t = block_sum(v, red);
     if (threadIdx.x == 0) {
       energy[0] = t;
@@ -442,15 +571,40 @@ cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, 
   return cudaGetLastError();
 }
 
+namespace {
+// log2 of the tile of k_hpsi on n qubits: 1024 tiles or more from 15 qubits, so that the last
+// round of the SMs is short.
+int hpsi_tile_log(int n) { return n >= 22 ? 11 : n >= 20 ? 10 : n >= 15 ? n - 10 : 5; }
+}  // namespace
+
+int hpsi_blocks(int n) {
+  const int l = hpsi_tile_log(n);
+  return n <= l ? 1 : (int)std::min<uint64_t>(1ull << (n - l), kRedBlocks);
+}
+
 cudaError_t launch_hpsi(const double2* psi, double2* lam, int n, const DGroup* groups,
                         int n_groups, const double2* tables, double* partial, cudaStream_t s,
                         bool overlap) {
-  const uint64_t N = 1ull << n;
-  if (!lam && partial)
-    return launch_overlapped(k_expval, kRedBlocks, kThreads, 0, s, overlap, psi, n, groups, n_groups,
-                             tables, partial);
-  return launch_overlapped(k_hpsi, kRedBlocks, kThreads, 0, s, overlap, psi, lam, N, groups, n_groups,
-                           tables, partial);
+  const int g = hpsi_blocks(n);
+#define HPSI(U, S)                                                                              \
+  return launch_overlapped(k_hpsi<U, S>, g, kThreads, 0, s, overlap, psi, lam, n, groups, n_groups, \
+                           tables, partial)
+  switch (hpsi_tile_log(n)) {
+    case 11: HPSI(8, 1);
+    case 10: HPSI(4, 1);
+    case 9: HPSI(2, 1);
+    case 8: HPSI(2, 2);
+    case 7: HPSI(2, 4);
+    case 6: HPSI(2, 8);
+    default: HPSI(1, 8);
+  }
+#undef HPSI
+}
+
+cudaError_t launch_expval(const double2* psi, int n, const DGroup* groups, int n_groups,
+                          const double2* tables, double* partial, cudaStream_t s) {
+  k_expval<<<kRedBlocks, kThreads, 0, s>>>(psi, n, groups, n_groups, tables, partial);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream_t s) {
@@ -459,11 +613,11 @@ cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream
 }
 
 cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
-                          double* grad, const double* epart, double* energy, double* theta_upd,
-                          double lr, double* traj, cudaStream_t s, bool overlap) {
+                          double* grad, const double* epart, int n_epart, double* energy,
+                          double* theta_upd, double lr, double* traj, cudaStream_t s, bool overlap) {
   const int per = kThreads / 32;
   return launch_overlapped(k_finish, (n_params + per - 1) / per + 1, kThreads, 0, s, overlap, ops,
-                           n_ops, partial, n_params, grad, epart, energy, theta_upd, lr, traj);
+                           n_ops, partial, n_params, grad, epart, n_epart, energy, theta_upd, lr, traj);
 }
 
 }  // namespace svqe

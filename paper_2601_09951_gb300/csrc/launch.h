@@ -62,19 +62,23 @@ cudaError_t launch_apply_op(double2* psi, int n, const DOp& op, const Rot* coef,
 int adjoint_blocks(int n, const DOp& op);
 cudaError_t launch_adjoint_op(double2* psi, double2* lam, int n, const DOp& op, const Rot* coef,
                               double* partial, cudaStream_t s, bool overlap = false);
-// lambda = H psi (if lam != nullptr) and partial[b] = block b's share of Re<psi|H psi>.
+// lambda = H psi, and partial[b] = block b's share of Re<psi|H psi>, b < hpsi_blocks(n).
+int hpsi_blocks(int n);
 cudaError_t launch_hpsi(const double2* psi, double2* lam, int n, const DGroup* groups,
                         int n_groups, const double2* tables, double* partial, cudaStream_t s,
                         bool overlap = false);
+// The energy alone: partial[b] = block b's share, b < kRedBlocks.
+cudaError_t launch_expval(const double2* psi, int n, const DGroup* groups, int n_groups,
+                          const double2* tables, double* partial, cudaStream_t s);
 // out[0] = sum of partial[0..count) in a fixed order.
 cudaError_t launch_sum(const double* partial, int count, double* out, cudaStream_t s);
 // The end of an evaluation, in one launch: grad[p] = sum over ops l with param p (in op order)
 // of sum_b partial[l * kRedBlocks + b] over the op's ops[l].flags blocks, and (epart != nullptr)
-// energy[0] = the sum of epart[0..kRedBlocks).  With theta_upd set also the descent step
+// energy[0] = the sum of epart[0..n_epart).  With theta_upd set also the descent step
 // theta_upd[p] -= lr * grad[p] and (traj != nullptr) traj[0] = the energy.
 cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int n_params,
-                          double* grad, const double* epart, double* energy, double* theta_upd,
-                          double lr, double* traj, cudaStream_t s, bool overlap = false);
+                          double* grad, const double* epart, int n_epart, double* energy,
+                          double* theta_upd, double lr, double* traj, cudaStream_t s, bool overlap = false);
 
 }  // namespace svqe
 

@@ -275,7 +275,8 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
     double* part = hc.ops[l].param >= 0 ? gpart + (size_t)l * kRedBlocks : nullptr;
     NA_CUDA(launch_adjoint_op(psi, lam, n, hc.ops[l], coef + l, part, s));
   }
-  NA_CUDA(launch_finish(ops, n_ops, gpart, hc.n_params, grad_dev, epart, energy_dev, nullptr, 0.0,
+  NA_CUDA(launch_finish(ops, n_ops, gpart, hc.n_params, grad_dev, epart, hpsi_blocks(n), energy_dev,
+                        nullptr, 0.0,
                         nullptr, s));
   k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
   NA_CUDA(cudaGetLastError());
