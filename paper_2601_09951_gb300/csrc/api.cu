@@ -944,7 +944,7 @@ bool svqe::pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_t
   const size_t o_theta = align(o_pops + (size_t)G * sizeof(int32_t));
   const size_t bytes = align(o_theta + (theta ? (size_t)P * sizeof(double) : 0));
   if (out.ckpt_amps > kSmallCkptAmps || bytes > (100u << 10) ||
-      small_smem(hc.n, G, P, (int)bytes) > (200u << 10))
+      small_smem(hc.n, G, P, (int)bytes) > kSmallSmem)
     return false;
   SmallArgs& A = out.args;
   std::memset(&A, 0, offsetof(SmallArgs, blob));
@@ -986,6 +986,8 @@ bool svqe::pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_t
   A.o_pptr = (int)o_pptr;
   A.o_pops = (int)o_pops;
   A.o_theta = theta ? (int)o_theta : -1;
+  const size_t ham = (size_t)n_groups * sizeof(DGroup) + (size_t)n_table * sizeof(double2);
+  A.ham_bytes = small_smem(hc.n, G, P, (int)bytes) + ham <= kSmallSmem ? (int)ham : 0;
   A.a.n_inst = 1;
   return true;
 }

@@ -315,9 +315,9 @@ __device__ __forceinline__ double layer_scale(const Rot* coef, const Seg& sg) {
   return __shfl_sync(kFull, h + l, 0);
 }
 
-// One staged layer gate on v (inv: its inverse).
+// One staged layer gate on v (inv: its inverse); ckout as for lop_pass2_k.
 __device__ __forceinline__ void lop_pass(const Team& T, double2* v, uint32_t N, const LOp& o,
-                                         bool inv) {
+                                         bool inv, double2* ckout) {
   const uint32_t fl = 1u << o.bit, low = fl - 1u;
   const bool rx = o.type == SV_GATE_RX;
   const int mode = inv && o.mode ? 2 : o.mode;
@@ -327,6 +327,10 @@ __device__ __forceinline__ void lop_pass(const Team& T, double2* v, uint32_t N, 
     const uint32_t i = ((p & ~low) << 1) | (p & low);
     const uint32_t j = rx ? i : i ^ r.swap;
     double2 x = v[j], y = v[j ^ fl];
+    if (ckout) {
+      ckout[j] = x;
+      ckout[j ^ fl] = y;
+    }
     if (rx) {
       pair_t<true>(mode, t, x, y);
     } else {
@@ -398,12 +402,16 @@ __device__ __forceinline__ void lop_pass2(const Team& T, double2* v, uint32_t N,
 __device__ __forceinline__ void layer_pass(const Team& T, TeamS& S, double2* v, uint32_t N,
                                            int count, bool inv, double scale, double2* ckout) {
   int g = 0;
-  for (; g + 1 < count; g += 2) {
-    lop_pass2(T, v, N, S.lop[g], S.lop[g + 1], inv, g == 0 ? ckout : nullptr);
-    T.sync();
-  }
-  if (g < count) {
-    lop_pass(T, v, N, S.lop[g], inv);
+  if (T.size <= (int)(N >> 2))
+    for (; g + 1 < count; g += 2) {
+      lop_pass2(T, v, N, S.lop[g], S.lop[g + 1], inv, g == 0 ? ckout : nullptr);
+      T.sync();
+    }
+  // the last gate of an odd layer; or every gate when the team has a thread per pair (a warp's
+  // FP64 instruction takes 64 clocks however many lanes take part, and pairs fill twice as many
+  // as blocks of four)
+  for (; g < count; ++g) {
+    lop_pass(T, v, N, S.lop[g], inv, g == 0 ? ckout : nullptr);
     T.sync();
   }
   // (a loop of its own: inside the passes it becomes multiplications that always issue)
@@ -600,8 +608,9 @@ __device__ __forceinline__ bool cz_sign(const TeamS& S, int ncz, uint32_t k) {
   return par & 1u;
 }
 
+// room: bytes of the team's shared memory at sm, psi and lambda (first) included.
 __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& S, double2* sm,
-                             double2* ck) {
+                             size_t room, double2* ck) {
   const BInst I = a.inst[idx];
   const int n = I.n;
   const uint32_t N = 1u << n;
@@ -609,6 +618,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
   double2* lam = sm + N;
   const DOp* ops = a.ops + I.op_off;
   const DGroup* groups = a.groups + I.grp_off;
+  const double2* tables = a.tables;
   const Seg* segs = a.segs + I.seg_off;
   Rot* coef = a.coef + I.coef_off;
   double* contrib = a.contrib + I.contrib_off;
@@ -624,6 +634,27 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
   const int steps = per_inst ? I.steps : (a.n_steps > 0 ? a.n_steps : 1);
   const bool gd = a.n_steps != 0;
   const double lr = per_inst ? I.lr : (a.lr_inst ? a.lr_inst[idx] : a.lr);
+
+  // The Hamiltonian in the rest of the team's shared memory when it fits, once for all steps:
+  // with few amplitudes per thread a group is over before its table entry arrives from L2 (100
+  // terms on 8 qubits: 870 clocks per group, of which 256 are arithmetic).
+  const size_t head = (size_t)2 * N * sizeof(double2);
+  const size_t gbytes = (size_t)I.n_groups * sizeof(DGroup);
+  const bool staged =
+      N <= 4u * (uint32_t)TS && head + gbytes + (size_t)I.tab_n * sizeof(double2) <= room;
+  if (staged) {
+    DGroup* sgr = reinterpret_cast<DGroup*>(sm + 2 * N);
+    double2* stab = reinterpret_cast<double2*>(sgr + I.n_groups);
+    const double2* t0 = a.tables + I.tab_off;
+    for (int g = tid; g < I.n_groups; g += TS) {
+      DGroup G = groups[g];
+      G.toff -= I.tab_off;
+      sgr[g] = G;
+    }
+    for (int j = tid; j < I.tab_n; j += TS) stab[j] = t0[j];
+    groups = sgr;
+    tables = stab;
+  }
 
   for (int step = 0; step < steps; ++step) {
     // one sincos per op whatever form it takes (lanes of one warp hold ops of every form, and
@@ -649,7 +680,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
     for (uint32_t k = tid; k < N; k += TS)
       psi[k] = make_double2(k == (uint32_t)I.ref ? 1.0 : 0.0, 0.0);
     // the group records and tables are first read by lambda = H psi, after the forward pass
-    if (step == 0) {
+    if (step == 0 && !staged) {
       team_prefetch_l2(T, groups, (int64_t)I.n_groups * (int64_t)sizeof(DGroup));
       team_prefetch_l2(T, a.tables + I.tab_off, (int64_t)I.tab_n * (int64_t)sizeof(double2));
     }
@@ -771,13 +802,13 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         if (ng > 0) {
           Gn = grec(groups[0]);
           Gnn = grec(groups[ng > 1 ? 1 : 0]);
-          cn = a.tables[Gn.toff];
+          cn = tables[Gn.toff];
         }
         for (int g = 0; g < ng; ++g) {
           const GRec G = Gn;
           const double2 c = cn;
           Gn = Gnn;
-          cn = a.tables[Gn.toff];
+          cn = tables[Gn.toff];
           Gnn = grec(groups[g + 2 < ng ? g + 2 : ng - 1]);
           const uint32_t x = G.x, zu = G.zu;
           if (G.cls == 4) {
@@ -818,7 +849,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
             for (int b = 0; b < 4; ++b)
               d[b] = ((zh >> b) & 1u) << (sh + __popc(zh & ((1u << b) - 1u)));
             // a real or imaginary table is read one component at a time (8 bytes per entry)
-            const double* tab = reinterpret_cast<const double*>(a.tables + G.toff);
+            const double* tab = reinterpret_cast<const double*>(tables + G.toff);
             if (G.cls == 0) {
   #pragma unroll
               for (int u = 0; u < kHU; ++u) {
@@ -861,7 +892,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
   #pragma unroll
                   for (int b = 0; b < 4; ++b)
                     if ((u >> b) & 1) ti += d[b];
-                  group_madd(2, a.tables[G.toff + ti], psi[k ^ x], acc[u]);
+                  group_madd(2, tables[G.toff + ti], psi[k ^ x], acc[u]);
                 }
               }
             }
@@ -1037,7 +1068,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         // each thread reads a block of four amplitudes of psi and lambda and accumulates both
         // gates' pair terms from it
         int g = 0;
-        for (; g + 1 < sg.count; g += 2) {
+        for (; TS <= (int)(N >> 2) && g + 1 < sg.count; g += 2) {
           const LOp& o1 = S.lop[g];
           const LOp& o2 = S.lop[g + 1];
           const uint32_t b1 = 1u << o1.bit, b2 = 1u << o2.bit;
@@ -1068,7 +1099,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
             if (q == g + 1) v[q] = a2;
           }
         }
-        if (g < sg.count) {
+        for (; g < sg.count; ++g) {
           const LOp& o = S.lop[g];
           const uint32_t fl = 1u << o.bit, low = fl - 1u;
           double acc = 0.0;
@@ -1201,7 +1232,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch(BatchArgs a) {
       double2* region = sm + (size_t)team * (a.smem_amps / nteams);
       double2* ck = a.ckpt + (size_t)blockIdx.x * a.ckpt_slot +
                     (size_t)team * (a.ckpt_slot / nteams);
-      run_instance(a, inst, T, S[team], region, ck);
+      run_instance(a, inst, T, S[team], region, (a.smem_amps / nteams) * sizeof(double2), ck);
     }
     __syncthreads();
   }
@@ -1212,8 +1243,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_small(const __grid_constan
   extern __shared__ double2 sm[];
   __shared__ TeamS S;
   const uint32_t N = 1u << p.n;
-  // psi, lambda, the blob, coefficients, per-op gradients, gradient
-  unsigned char* blob = reinterpret_cast<unsigned char*>(sm + 2 * N);
+  // psi, lambda, the Hamiltonian (p.ham_bytes, if it fits), the blob, coefficients, per-op
+  // gradients, gradient
+  unsigned char* blob = reinterpret_cast<unsigned char*>(sm + 2 * N) + p.ham_bytes;
   const int bw = (p.blob_bytes + 15) >> 4;
   const uint4* src = reinterpret_cast<const uint4*>(p.blob_dev ? p.blob_dev : p.blob);
   for (int i = threadIdx.x; i < bw; i += blockDim.x) reinterpret_cast<uint4*>(blob)[i] = src[i];
@@ -1235,7 +1267,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_small(const __grid_constan
   T.w = threadIdx.x >> 5;
   T.bar = 1;
   __syncthreads();
-  run_instance(a, 0, T, S, sm, a.ckpt);
+  run_instance(a, 0, T, S, sm, 2 * N * sizeof(double2) + p.ham_bytes, a.ckpt);
   if (p.theta_out)
     for (int i = threadIdx.x; i < p.n_params; i += blockDim.x) p.theta_out[i] = a.theta[i];
   if (p.ref_out) {
@@ -1257,11 +1289,13 @@ size_t small_smem(int n, int n_ops, int n_params, int blob_bytes) {
 }
 
 cudaError_t small_prepare() {
-  return cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  return cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kSmallSmem);
 }
 
 cudaError_t launch_small(const SmallArgs& a, cudaStream_t s) {
-  k_small<<<1, 32 * a.nw, small_smem(a.n, a.n_ops, a.n_params, a.blob_bytes), s>>>(a);
+  k_small<<<1, 32 * a.nw, small_smem(a.n, a.n_ops, a.n_params, a.blob_bytes) + a.ham_bytes, s>>>(
+      a);
   return cudaGetLastError();
 }
 

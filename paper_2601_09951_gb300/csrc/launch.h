@@ -241,6 +241,7 @@ struct SmallArgs {
   BatchArgs a;  // inst, ops, segs, pptr, pops, coef and contrib are set by the kernel
   int nw;       // warps
   int n, n_ops, blob_bytes;
+  int ham_bytes;  // shared memory for the Hamiltonian (a multiple of 16), or 0: read from L2
   int o_ops, o_segs, o_pptr, o_pops, o_theta;
   int n_params;
   const unsigned char* blob_dev;
@@ -252,6 +253,7 @@ static_assert(sizeof(SmallArgs) <= 4096, "the argument block stays within 4 KB")
 // Warps of an n-qubit instance run alone, and the shared memory of such a launch.
 int small_warps(int n);
 size_t small_smem(int n, int n_ops, int n_params, int blob_bytes);
+constexpr size_t kSmallSmem = 200 * 1024;
 cudaError_t small_prepare();
 cudaError_t launch_small(const SmallArgs& a, cudaStream_t s);
 
