@@ -11,6 +11,7 @@
 #include <mutex>
 #include <new>
 #include <numeric>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -85,6 +86,7 @@ struct sv_ctx {
   size_t ckpt_cap = 0;
   double* pin = nullptr;
   size_t pin_cap = 0;
+  bool fixed = false;   // every buffer is the caller's (adjoint_fixed): nothing may grow
   int tune = 0;         // sv_set_autotune
   int tile_bits = 11;   // tile size of the staged circuit's fused passes
 };
@@ -172,6 +174,23 @@ static cudaError_t grow(T*& p, size_t& cap, size_t need) {
   return e;
 }
 
+// Room for `need` entries in a context's buffer: grown, or (fixed) SV_ENOMEM.
+template <class T>
+static sv_status room(sv_ctx* c, T*& p, size_t& cap, size_t need) {
+  if (c->fixed) {
+    if (need <= cap) return SV_OK;
+    set_error("the working memory is too small for this circuit");
+    return SV_ENOMEM;
+  }
+  SV_CUDA(grow(p, cap, need), c);
+  return SV_OK;
+}
+#define SV_ROOM(p, cap, need)                                 \
+  do {                                                        \
+    const sv_status r_ = room(c, c->p, c->cap, need);         \
+    if (r_ != SV_OK) return r_;                               \
+  } while (0)
+
 const char* sv_status_str(sv_status s) {
   switch (s) {
     case SV_OK: return "SV_OK";
@@ -203,9 +222,7 @@ uint64_t sv_ctx_device_bytes(int32_t n) {
 // routine) instead of some twenty launches; descent steps loop inside it.  A context does so up
 // to kSmallQubits: one block's time doubles with each qubit and the passes' does not (four
 // hardware-efficient layers, one block against passes: 113 and 188 us at 8 qubits, 187 and 303
-// at 10, 313 and 292 at 11, 573 and 244 at 12).  The call without device allocation, which has
-// no passes and launches every gate, does up to the 12 qubits the routine holds.
-static constexpr int kSmallQubits = 10;
+// at 10, 313 and 292 at 11, 573 and 244 at 12).
 
 // ------------------------------------------------------------------------------ contexts
 sv_status sv_create(sv_ctx** out, int32_t n, void* stream) {
@@ -466,11 +483,13 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc);
 
 sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune, bool from_ref) {
   const size_t n_ops = hc.ops.size();
-  SV_CUDA(grow(c->coef, c->coef_cap, n_ops), c);
-  SV_CUDA(grow(c->cs, c->cs_cap, n_ops), c);
-  SV_CUDA(grow(c->gpart, c->gpart_cap, std::max<size_t>(1, n_ops) * kRedBlocks), c);
-  SV_CUDA(grow(c->theta, c->theta_cap, (size_t)hc.n_params), c);
-  SV_CUDA(grow(c->grad, c->grad_cap, (size_t)hc.n_params), c);
+  SV_ROOM(coef, coef_cap, n_ops);
+  SV_ROOM(cs, cs_cap, n_ops);
+  SV_ROOM(gpart, gpart_cap, std::max<size_t>(1, n_ops) * kRedBlocks);
+  if (!c->fixed) {
+    SV_CUDA(grow(c->theta, c->theta_cap, (size_t)hc.n_params), c);
+    SV_CUDA(grow(c->grad, c->grad_cap, (size_t)hc.n_params), c);
+  }
   int m = fused_tile_bits();
   if (may_tune && c->tune && c->n >= kFusedMinQubits && n_ops > 0) m = tune_tile_bits(c, hc);
   if (m <= 0) return SV_ECUDA;
@@ -717,7 +736,7 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
     }
     if (ch.kind == sv_ctx::CH_PROD) {
       units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++, 0, 0});
-      SV_CUDA(grow(c->prod, c->prod_cap, prod_scratch(c->n)), c);
+      SV_ROOM(prod, prod_cap, prod_scratch(c->n));
       continue;
     }
     cf = cl = 0;
@@ -738,11 +757,13 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
     std::memcpy(blob.data() + o_items, c->plan.items.data(), c->plan.items.size() * sizeof(FItem));
   if (!units.empty())
     std::memcpy(blob.data() + o_units, units.data(), units.size() * sizeof(PrepUnit));
-  SV_CUDA(grow(c->blob, c->blob_cap, blob.size()), c);
-  SV_CUDA(grow(c->sitems, c->sitems_cap, c->plan.items.size()), c);
-  SV_CUDA(grow(c->scales, c->scales_cap, c->plan.passes.size()), c);
-  if (n_dp) SV_CUDA(grow(c->dptab, c->dptab_cap, (size_t)n_dp * kDpTab), c);
-  if (!blob.empty())
+  SV_ROOM(blob, blob_cap, blob.size());
+  SV_ROOM(sitems, sitems_cap, c->plan.items.size());
+  SV_ROOM(scales, scales_cap, c->plan.passes.size());
+  if (n_dp) SV_ROOM(dptab, dptab_cap, (size_t)n_dp * kDpTab);
+  if (c->fixed)  // (no copy from pageable memory on a caller's stream)
+    SV_CUDA(put_bytes(c->blob, blob.data(), blob.size(), c->stream), c);
+  else if (!blob.empty())
     SV_CUDA(cudaMemcpyAsync(c->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice,
                             c->stream), c);
   c->ops = (DOp*)c->blob;
@@ -1090,7 +1111,10 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
     }
     // psi is back at the reference state; it lives in the context's psi buffer between calls
     // (a product prefix is not un-applied: the state is written)
-    if (prod)
+    // (nobody sees the psi of a fixed context)
+    if (c->fixed)
+      (void)psi;
+    else if (prod)
       SV_CUDA(launch_init_basis(c->psi, c->n, c->ref, c->stream), c);
     else if (psi != c->psi)
       SV_CUDA(cudaMemcpyAsync(c->psi, psi, sv_state_bytes(c->n), cudaMemcpyDeviceToDevice,
@@ -1103,7 +1127,7 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
     }
   }
   SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, hpsi_blocks(c->n),
-                        energy_dev, theta_upd, lr, traj, c->stream, !prod), c);
+                        energy_dev, theta_upd, lr, traj, c->stream, c->fixed || !prod), c);
   return SV_OK;
 }
 
@@ -1230,6 +1254,55 @@ sv_status svqe::vqe_enqueue(sv_ctx* c, const HostCircuit& hc, const sv_ham* H, c
     SV_CUDA(cudaMemcpyAsync(energy_out, c->etraj, n_steps * sizeof(double),
                             cudaMemcpyDeviceToHost, c->stream), c);
   return SV_OK;
+}
+
+sv_status svqe::adjoint_fixed(const HostCircuit& hc, uint64_t ref, const DGroup* groups,
+                              int n_groups, const double2* tables, const double* theta_dev,
+                              double* energy_dev, double* grad_dev, unsigned char* mem,
+                              size_t bytes, cudaStream_t s) {
+  const size_t G = std::max<size_t>(1, hc.ops.size());
+  sv_ctx c;
+  c.fixed = true;
+  c.n = hc.n;
+  c.N = 1ull << hc.n;
+  c.ref = ref;
+  c.stream = s;
+  size_t at = 0;
+  auto take = [&](auto*& p, size_t& cap, size_t count) {
+    using T = std::remove_reference_t<decltype(*p)>;
+    p = reinterpret_cast<T*>(mem + at);
+    cap = count;
+    at += (count * sizeof(T) + 255) / 256 * 256;
+  };
+  size_t none = 0;
+  take(c.psi, none, c.N);
+  take(c.lam, none, c.N);
+  if (hc.n >= kDpMinQubits) take(c.scratch, none, c.N);
+  take(c.epart, none, kRedBlocks);
+  take(c.gpart, c.gpart_cap, G * kRedBlocks);
+  take(c.coef, c.coef_cap, G);
+  take(c.cs, c.cs_cap, G);
+  take(c.sitems, c.sitems_cap, G);
+  take(c.scales, c.scales_cap, G);
+  take(c.blob, c.blob_cap, G * (sizeof(DOp) + sizeof(FItem) + sizeof(PrepUnit)) + 1024);
+  if (hc.n >= kDpMinQubits) take(c.prod, c.prod_cap, prod_scratch(hc.n));
+  if (at >= bytes) {
+    set_error("the working memory is too small for this circuit");
+    return SV_ENOMEM;
+  }
+  take(c.dptab, c.dptab_cap, (bytes - at) / sizeof(double2));
+  sv_ham H;
+  H.n = hc.n;
+  H.n_groups = n_groups;
+  H.groups = const_cast<DGroup*>(groups);
+  H.tables = const_cast<double2*>(tables);
+  if (fused_prepare() != cudaSuccess || dp_prepare(hc.n) != cudaSuccess) {
+    set_error("kernel attributes could not be set");
+    return SV_ECUDA;
+  }
+  const sv_status st = stage_circuit(&c, hc, false, true);
+  if (st != SV_OK) return st;
+  return adjoint_core(&c, hc, &H, theta_dev, energy_dev, grad_dev);
 }
 
 cudaStream_t svqe::ctx_stream(sv_ctx* c) { return c->stream; }

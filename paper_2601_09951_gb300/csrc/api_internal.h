@@ -28,6 +28,8 @@ sv_status adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
 // are written when the stream reaches them (pinned host memory for real asynchrony).
 sv_status vqe_enqueue(sv_ctx* c, const HostCircuit& hc, const sv_ham* H, const double* theta_in,
                       double lr, int32_t n_steps, double* theta_out, double* energy_out);
+// Registers up to this size run in one launch of one block (see api.cu).
+constexpr int kSmallQubits = 10;
 // A circuit packed for launch_small: the argument block (a.ckpt, a.theta, results and the
 // Hamiltonian's arrays are the caller's to set), the blob when it exceeds kSmallBlob, and the
 // amplitudes of checkpoint scratch it needs.  theta (host, or nullptr) goes into the blob.
@@ -40,6 +42,15 @@ struct SmallPack {
 bool pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
                 const double* theta, SmallPack& out);
 cudaStream_t ctx_stream(sv_ctx* c);
+// sv_adjoint_grad_dev's evaluation with every buffer in the caller's `bytes` of device memory at
+// mem (256-byte aligned), nothing allocated and nothing copied from pageable host memory.
+// SV_ENOMEM, with nothing enqueued, when the circuit needs more.
+sv_status adjoint_fixed(const HostCircuit& hc, uint64_t ref, const DGroup* groups, int n_groups,
+                        const double2* tables, const double* theta_dev, double* energy_dev,
+                        double* grad_dev, unsigned char* mem, size_t bytes, cudaStream_t s);
+// Copy host bytes to the device as kernel arguments (dst 16-byte aligned, its length rounded up
+// to 16 bytes): stream-ordered, and src is not read after the call.
+cudaError_t put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s);
 // Replace the Pauli sum held by H (lowered for c's register), reusing H's device buffers when
 // they are large enough, so that a pooled context takes a new request without allocating.
 sv_status ham_reload(sv_ctx* c, sv_ham* H, const sv_paulisum* h);

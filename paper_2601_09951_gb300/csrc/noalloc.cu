@@ -52,9 +52,9 @@ constexpr size_t kOffEpart =
 // A register of n qubits has at most 2^n distinct X masks, hence at most 2^n groups.
 constexpr int kMaxGroups = 1 << SV_NOALLOC_MAX_QUBITS;
 constexpr size_t kOffGroups = kOffEpart + align256(sizeof(double) * kRedBlocks);
-constexpr size_t kOffFlag = kOffGroups + align256(sizeof(DGroup) * (size_t)kMaxGroups);
-constexpr size_t kScratchBytes = kOffFlag + 256;
-static_assert(kScratchBytes <= SV_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds its stated size");
+constexpr size_t kOffFlag = SV_NOALLOC_SCRATCH_BYTES - 256;
+static_assert(kOffGroups + align256(sizeof(DGroup) * (size_t)kMaxGroups) <= kOffFlag,
+              "scratch layout exceeds its stated size");
 
 // The scratch itself.  In host code this name is only a host-side stand-in: its device address
 // comes from cudaGetSymbolAddress (see scratch_address).
@@ -101,26 +101,14 @@ sv_status scratch_address(unsigned char** out) {
 
 // Records travel to the device as kernel parameters (by value, copied at launch), so the
 // upload reads no host memory after the call returns.
-constexpr int kPutWords = 250;  // 16-byte words
+constexpr int kPutWords = 1000;  // 16-byte words
 struct PutChunk {
   uint4 w[kPutWords];
 };
-static_assert(sizeof(PutChunk) <= 4064, "a chunk must stay a small kernel parameter");
+static_assert(sizeof(PutChunk) <= 32000, "a chunk must fit the kernel parameters");
 
 __global__ void k_na_put(const __grid_constant__ PutChunk c, uint4* __restrict__ dst, int count) {
   for (int i = threadIdx.x; i < count; i += blockDim.x) dst[i] = c.w[i];
-}
-
-cudaError_t put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s) {
-  for (size_t o = 0; o < bytes; o += sizeof(PutChunk)) {
-    PutChunk c;
-    const size_t cnt = std::min(sizeof(PutChunk), bytes - o);
-    std::memcpy(&c, (const unsigned char*)src + o, cnt);
-    k_na_put<<<1, 256, 0, s>>>(c, (uint4*)((unsigned char*)dst + o), (int)((cnt + 15) / 16));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
 }
 
 // Checks every caller record (x_mask and z_union inside the n-qubit register, a known class,
@@ -175,6 +163,19 @@ __global__ void k_na_poison(const unsigned* __restrict__ flag, double* __restric
 }
 
 }  // namespace
+
+cudaError_t put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  for (size_t o = 0; o < bytes; o += sizeof(PutChunk)) {
+    PutChunk c;
+    const size_t cnt = std::min(sizeof(PutChunk), bytes - o);
+    std::memcpy(&c, (const unsigned char*)src + o, cnt);
+    k_na_put<<<1, 256, 0, s>>>(c, (uint4*)((unsigned char*)dst + o), (int)((cnt + 15) / 16));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 }  // namespace svqe
 
 using namespace svqe;
@@ -235,19 +236,35 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
   Rot* coef = (Rot*)(base + kOffCoef);
   double* gpart = (double*)(base + kOffGpart);
   double* epart = (double*)(base + kOffEpart);
-  DGroup* groups = (DGroup*)(base + kOffGroups);
+  // the call's groups lie at the array's end, so that the rest is one piece
+  const size_t off_groups = kOffFlag - align256(sizeof(DGroup) * (size_t)n_groups);
+  DGroup* groups = (DGroup*)(base + off_groups);
   unsigned* flag = (unsigned*)(base + kOffFlag);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int n_ops = (int)hc.ops.size();
   k_na_check_groups<<<1, 1024, 0, s>>>(groups_dev, n_groups, n, (long long)n_table, groups,
                                        flag);
   NA_CUDA(cudaGetLastError());
-  // Small registers run in one launch (k_small), its checkpoints and records in the part of the
-  // array that holds states and partials otherwise.
+  auto poison = [&]() -> sv_status {
+    k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
+    NA_CUDA(cudaGetLastError());
+    return SV_OK;
+  };
+  // From kSmallQubits + 1 qubits: the passes of the ordinary path, in the array.  A circuit whose
+  // tables do not fit it goes on below.
+  if (n > kSmallQubits) {
+    st = adjoint_fixed(hc, ref, groups, n_groups, (const double2*)tables_dev, theta_dev, energy_dev,
+                       grad_dev, base, off_groups, s);
+    if (st == SV_OK) return poison();
+    if (st != SV_ENOMEM) return st;
+    clear_error();
+  }
+  // Small registers (and, failing the above, up to 12 qubits) run in one launch (k_small), its
+  // checkpoints and records in the array.
   SmallPack sp;
   const int n_pref = (int)std::min<int64_t>(n_table, 1 << 20);
   if (pack_small(hc, ref, n_groups, n_pref, nullptr, sp) &&
-      align256(sp.blob.size()) + (size_t)sp.ckpt_amps * sizeof(double2) <= kOffGroups) {
+      align256(sp.blob.size()) + (size_t)sp.ckpt_amps * sizeof(double2) <= off_groups) {
     SmallArgs& A = sp.args;
     if (!sp.blob.empty()) {
       NA_CUDA(put_bytes(base, sp.blob.data(), sp.blob.size(), s));
@@ -261,10 +278,9 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
     A.a.grad = grad_dev;
     NA_CUDA(small_prepare());
     NA_CUDA(launch_small(A, s));
-    k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
-    NA_CUDA(cudaGetLastError());
-    return SV_OK;
+    return poison();
   }
+  // What is left launches every gate.
   for (DOp& op : hc.ops) op.flags = adjoint_blocks(n, op);
   NA_CUDA(put_bytes(ops, hc.ops.data(), n_ops * sizeof(DOp), s));
   NA_CUDA(launch_init_basis(psi, n, ref, s));
@@ -276,9 +292,6 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
     NA_CUDA(launch_adjoint_op(psi, lam, n, hc.ops[l], coef + l, part, s));
   }
   NA_CUDA(launch_finish(ops, n_ops, gpart, hc.n_params, grad_dev, epart, hpsi_blocks(n), energy_dev,
-                        nullptr, 0.0,
-                        nullptr, s));
-  k_na_poison<<<1, 256, 0, s>>>(flag, energy_dev, grad_dev, hc.n_params);
-  NA_CUDA(cudaGetLastError());
-  return SV_OK;
+                        nullptr, 0.0, nullptr, s));
+  return poison();
 }

@@ -97,3 +97,46 @@ def test_descent_steps_match_single_evaluations(n, layers):
         assert_energy(e_step, e, inst["ham"])
         th = th - lr * g
     np.testing.assert_allclose(theta, th, rtol=0, atol=1e-11)
+
+
+def _bad_records_give_nan(torch, svqe_call, rec):
+    wide = rec.copy()
+    wide["x_mask"][0] |= np.uint64(1) << np.uint64(40)
+    e, g = svqe_call(wide)
+    assert np.isnan(e) and np.all(np.isnan(g))
+
+
+@pytest.mark.parametrize("make", [
+    lambda: W.hea_instance(10, 4, 80, 51), lambda: W.hea_instance(11, 5, 80, 52),
+    lambda: W.hea_instance(12, 5, 80, 53, ring=True), lambda: W.hea_instance(13, 4, 60, 54),
+    lambda: W.hea_instance(14, 4, 60, 55, ring=True),
+    lambda: W.uccsd_instance(n=13, n_elec=6, n_singles=20, n_doubles=80, n_terms=200, seed=56),
+    lambda: W.uccsd_instance(n=14, n_elec=7, n_singles=56, n_doubles=200, n_terms=100, seed=57)])
+def test_without_device_allocation_every_route(make):
+    """The call without device allocation on both sides of the one-block limit, at its qubit and
+    gate limits, against adjoint_grad; a bad record still gives NaN, and the next call is right."""
+    torch = pytest.importorskip("torch")
+    inst = make()
+    n, theta = inst["circuit"]["n"], np.asarray(inst["theta"])
+    rec, table = svqe.group_records(inst["ham"], n)
+    t_d = torch.as_tensor(table.view(np.float64)).cuda()
+    th_d = torch.as_tensor(theta).cuda()
+
+    def call(records):
+        g_d = torch.as_tensor(records.view(np.uint8).reshape(-1)).cuda()
+        e_d = torch.zeros(1, dtype=torch.float64, device="cuda")
+        gr_d = torch.zeros(len(theta), dtype=torch.float64, device="cuda")
+        svqe.adjoint_grad_noalloc(inst["circuit"], inst["ref"], n, g_d.data_ptr(), len(records),
+                                  t_d.data_ptr(), len(table), th_d.data_ptr(), e_d.data_ptr(),
+                                  gr_d.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        return float(e_d.item()), gr_d.cpu().numpy()
+
+    ctx = svqe.Context(n)
+    ctx.init_reference(inst["ref"])
+    e0, g0 = ctx.adjoint_grad(inst["circuit"], theta, svqe.Ham(ctx, inst["ham"]))
+    for _ in range(2):
+        _bad_records_give_nan(torch, call, rec)
+        e, g = call(rec)
+        assert_energy(e, e0, inst["ham"])
+        assert_grad(g, g0, inst["ham"])
