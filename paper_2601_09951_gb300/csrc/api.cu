@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -498,21 +499,55 @@ sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune, b
 
 static int single_op(const sv_ctx* c, int p);
 
-// Tile size and lowest contiguous bits of the fused passes of a run of ops.  Tiles of tile_bits
-// bits leave a small state in fewer tiles than the 152 SMs, one block each (17 qubits: 64 tiles
-// of 2^11, 24 us per 9-gate pass).  Below 18 qubits a tile of n - 7 bits gives 128 blocks, and
-// fewer contiguous low bits (the state sits in L2, where a 16- or 32-byte access costs no burst)
-// leave its other bits for gate wires: two passes still cover every qubit of a layer.  Runs of
-// gates on many wires (excitations) that the smaller tile would cut into over half as many
-// passes again (and more than one) keep the larger one, a pass costing a few microseconds
-// whatever its tiles.
+// Estimated time (us) of a plan's passes, forward and backward, on an n-qubit state: two launches
+// with their round trips to L2 (85 passes of a 14-qubit excitation circuit take 13 us each), a
+// barrier or two per item, and the FP64 work of the SM with most tiles
+// (2 operations per clock; 8 per amplitude of an RY gate in both directions, excitations by the
+// amplitudes they touch).
+static double plan_cost(const HostPlan& plan, double* fp64_us) {
+  double us = 0.0, fp64 = 0.0;
+  for (const FPass& P : plan.passes) {
+    double flops = 0.0;
+    for (int i = P.first_item; i < P.first_item + P.n_items; ++i) {
+      const FItem& it = plan.items[i];
+      if (it.kind == 1) flops += 20.0;
+      else if (it.local.type == SV_GATE_RY || it.local.type == SV_GATE_RX) flops += 8.0;
+      else if (it.local.type == SV_GATE_RZ) flops += 11.0;
+      else if (is_param_type(it.local.type)) flops += 11.0 / (1 << (it.local.k - 1));
+      else flops += 1.0;
+    }
+    const double tiles = (double)(1ull << __builtin_popcountll(P.outer_mask));
+    us += 11.0 + 0.4 * P.n_items;
+    fp64 += std::ceil(tiles / kSms) * (double)(1u << P.m) * flops / (2.0 * 2070.0);
+  }
+  if (fp64_us) *fp64_us = fp64;
+  return us + fp64;
+}
+
+// Fused passes of a run of ops.  Tiles of tile_bits bits leave a small state in fewer tiles than
+// the 152 SMs, one block each (17 qubits: 64 tiles of 2^11, 24 us per 9-gate pass).  Below 18
+// qubits a tile of n - 7 bits gives 128 blocks, and fewer contiguous low bits (the state sits in
+// L2, where a 16- or 32-byte access costs no burst) leave its other bits for gate wires: two
+// passes still cover every qubit of a layer.  Gates on many wires (excitations) need more of the
+// smaller passes, so the sizes are compared by plan_cost.
 static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan& plan) {
   plan_passes(ops, n, tile_bits, plan);
   const int m = std::max({n - 7, (n + 1) / 2, 4 + kMinLowBitsL2});  // (a gate has up to 4 wires)
   if (n > 17 || m >= tile_bits) return;
-  HostPlan small;
-  plan_passes(ops, n, m, small, std::max(0, std::min(kMinLowBitsL2, 2 * m - n)));
-  if (2 * small.passes.size() <= 3 * plan.passes.size() + 2) std::swap(plan, small);
+  // (planning 300 gates again takes 30 us: not when too little of the time could be saved)
+  double fp64 = 0.0;
+  double best = plan_cost(plan, &fp64);
+  if (fp64 < 0.4 * best) return;
+  for (const int t : {m, (m + tile_bits) / 2}) {
+    HostPlan p;
+    plan_passes(ops, n, t, p, std::max(0, std::min(kMinLowBitsL2, 2 * t - n)));
+    const double c = plan_cost(p, nullptr);
+    if (c < best) {
+      std::swap(plan, p);
+      if (c < 0.8 * best) break;  // (clearly: planning again costs microseconds too)
+      best = c;
+    }
+  }
 }
 
 // Length of the circuit's product prefix, its leading one-qubit gates, or 0: it is used from the
