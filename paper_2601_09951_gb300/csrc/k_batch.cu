@@ -62,6 +62,7 @@ struct TeamS {
   uint32_t pm_lo[kMaxPerm];  // condition and flip masks of a permutation segment's gates
   uint32_t pm_fl[kMaxPerm];
   LOp lop[kM];               // the gates of a commuting layer, staged once per segment
+  int gop[kM];               // ops whose gradients wait to be reduced (plain gates)
 };
 constexpr int kDpBlockAmps = 173;
 static_assert(offsetof(TeamS, pad) + sizeof(int) * 2 == kDpBlockAmps * sizeof(double2),
@@ -211,38 +212,147 @@ __device__ __forceinline__ void pair_grad_acc(int type, const double2& lx, const
   }
 }
 
-// Apply one pair op to buffer v (forward or inverse), pairs strided over the team, two pairs
-// per iteration (both loaded before either is stored, so their chains overlap).
-__device__ __forceinline__ void op_pass(const Team& T, double2* v, uint32_t N, const DOp& op,
-                                        const Rot& r, bool inv) {
-  const uint32_t np = N >> op.k;
-  const uint32_t lo = (uint32_t)op.lo_or;
-  if (op.type == SV_GATE_CZ) {
-    for (uint32_t p = T.rank; p < np; p += T.size) {
-      const uint32_t i = insert_zeros32(p, op.sb, op.k) | lo;
-      v[i] = make_double2(dneg(v[i].x), dneg(v[i].y));
-    }
-    return;
+// The arithmetic of a plain gate, chosen once per gate.
+enum GKind { G_SWAP, G_H, G_ROT, G_ROTX, G_ROTZ, G_NEG };
+__device__ __forceinline__ int gkind(int type) {
+  switch (type) {
+    case SV_GATE_H: return G_H;
+    case SV_GATE_RY: case SV_GATE_SINGLE_EXC: case SV_GATE_DOUBLE_EXC: return G_ROT;
+    case SV_GATE_RX: return G_ROTX;
+    case SV_GATE_RZ: return G_ROTZ;
+    case SV_GATE_CZ: return G_NEG;
+    default: return G_SWAP;
   }
-  const uint32_t fl = (uint32_t)op.flip;
-  for (uint32_t p = T.rank; p < np; p += 2 * T.size) {
-    const uint32_t p2 = p + T.size;
+}
+template <int KIND>
+__device__ __forceinline__ void gate_pair(const Rot& r, double2& x, double2& y) {
+  constexpr int type = KIND == G_H ? SV_GATE_H : KIND == G_ROT ? SV_GATE_RY : KIND == G_ROTX
+                       ? SV_GATE_RX : KIND == G_ROTZ ? SV_GATE_RZ : SV_GATE_X;
+  pair_apply(type, r, false, x, y);
+}
+
+// One plain gate on v, pairs strided over the team.
+template <int KIND>
+__device__ __forceinline__ void gate_fwd(const Team& T, double2* v, uint32_t N, const DOp& op,
+                                         const Rot& r) {
+  const uint32_t np = N >> op.k, lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
+  for (uint32_t p = T.rank; p < np; p += T.size) {
     const uint32_t i = insert_zeros32(p, op.sb, op.k) | lo;
-    const uint32_t i2 = insert_zeros32(p2, op.sb, op.k) | lo;
-    double2 x = v[i], y = v[i ^ fl];
-    double2 x2, y2;
-    const bool two = p2 < np;
-    if (two) {
-      x2 = v[i2];
-      y2 = v[i2 ^ fl];
+    if (KIND == G_NEG) {
+      v[i] = make_double2(dneg(v[i].x), dneg(v[i].y));
+    } else {
+      double2 x = v[i], y = v[i ^ fl];
+      gate_pair<KIND>(r, x, y);
+      v[i] = x;
+      v[i ^ fl] = y;
     }
-    pair_apply(op.type, r, inv, x, y);
-    if (two) pair_apply(op.type, r, inv, x2, y2);
-    v[i] = x;
-    v[i ^ fl] = y;
-    if (two) {
-      v[i2] = x2;
-      v[i2 ^ fl] = y2;
+  }
+}
+
+// Its step of the sweep on psi and lambda, r inverted: returns the thread's share of
+// 2 Im<lambda|G|psi> (if pg).
+template <int KIND>
+__device__ __forceinline__ double gate_bwd(const Team& T, double2* psi, double2* lam, uint32_t N,
+                                           const DOp& op, const Rot& r, bool pg) {
+  const uint32_t np = N >> op.k, lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
+  double acc = 0.0;
+  for (uint32_t p = T.rank; p < np; p += T.size) {
+    const uint32_t i = insert_zeros32(p, op.sb, op.k) | lo, j = i ^ fl;
+    if (KIND == G_NEG) {
+      psi[i] = make_double2(dneg(psi[i].x), dneg(psi[i].y));
+      lam[i] = make_double2(dneg(lam[i].x), dneg(lam[i].y));
+      continue;
+    }
+    double2 px = psi[i], py = psi[j], lx = lam[i], ly = lam[j];
+    if (KIND == G_ROT && pg) pair_grad_acc(SV_GATE_RY, lx, ly, px, py, acc);
+    if (KIND == G_ROTX && pg) pair_grad_acc(SV_GATE_RX, lx, ly, px, py, acc);
+    if (KIND == G_ROTZ && pg) pair_grad_acc(SV_GATE_RZ, lx, ly, px, py, acc);
+    gate_pair<KIND>(r, px, py);
+    gate_pair<KIND>(r, lx, ly);
+    psi[i] = px;
+    psi[j] = py;
+    lam[i] = lx;
+    lam[j] = ly;
+  }
+  return acc;
+}
+
+// A SEG_GATES segment forward: the next gate's record and coefficients are read while the
+// current one is applied.
+__device__ __noinline__ void gates_fwd(const Team& T, double2* psi, uint32_t N, const DOp* ops,
+                                       const Rot* coef, int first, int count) {
+  DOp nop = ops[first];
+  Rot nr = coef[first];
+  for (int l = first; l < first + count; ++l) {
+    const DOp op = nop;
+    const Rot r = nr;
+    if (l + 1 < first + count) {
+      nop = ops[l + 1];
+      nr = coef[l + 1];
+    }
+    switch (gkind(op.type)) {
+      case G_SWAP: gate_fwd<G_SWAP>(T, psi, N, op, r); break;
+      case G_H: gate_fwd<G_H>(T, psi, N, op, r); break;
+      case G_ROT: gate_fwd<G_ROT>(T, psi, N, op, r); break;
+      case G_ROTX: gate_fwd<G_ROTX>(T, psi, N, op, r); break;
+      case G_ROTZ: gate_fwd<G_ROTZ>(T, psi, N, op, r); break;
+      default: gate_fwd<G_NEG>(T, psi, N, op, r); break;
+    }
+    T.sync();
+  }
+}
+
+// The same in the sweep.  Gradients are reduced sixteen gates at a time: one by one, each cost
+// ten dependent FP64 adds of 64 clocks and two barriers.
+__device__ __noinline__ void gates_bwd(const Team& T, TeamS& S, double2* psi, double2* lam,
+                                       uint32_t N, const DOp* ops, const Rot* coef, int first,
+                                       int count, double* contrib) {
+  double v[kM];
+#pragma unroll
+  for (int q = 0; q < kM; ++q) v[q] = 0.0;
+  int nq = 0;
+  DOp nop = ops[first + count - 1];
+  Rot nr = coef[first + count - 1];
+  for (int l = first + count - 1; l >= first; --l) {
+    const DOp op = nop;
+    const Rot r = rot_inverse(nr);
+    if (l > first) {
+      nop = ops[l - 1];
+      nr = coef[l - 1];
+    }
+    const bool pg = op.param >= 0;
+    double acc = 0.0;
+    switch (gkind(op.type)) {
+      case G_SWAP: gate_bwd<G_SWAP>(T, psi, lam, N, op, r, false); break;
+      case G_H: gate_bwd<G_H>(T, psi, lam, N, op, r, false); break;
+      case G_ROT: acc = gate_bwd<G_ROT>(T, psi, lam, N, op, r, pg); break;
+      case G_ROTX: acc = gate_bwd<G_ROTX>(T, psi, lam, N, op, r, pg); break;
+      case G_ROTZ: acc = gate_bwd<G_ROTZ>(T, psi, lam, N, op, r, pg); break;
+      default: gate_bwd<G_NEG>(T, psi, lam, N, op, r, false); break;
+    }
+    if (count == 1) {  // (alone: five adds instead of sixteen)
+      if (pg) {
+        const double tot = team_sum(T, S, acc);
+        if (T.rank == 0) contrib[l] = tot;
+      }
+      T.sync();
+      return;
+    }
+    if (pg) {
+#pragma unroll
+      for (int q = 0; q < kM; ++q)
+        if (q == nq) v[q] = acc;
+      if (T.rank == 0) S.gop[nq] = l;
+      ++nq;
+    }
+    T.sync();
+    if (nq == kM || (l == first && nq > 0)) {
+      const double tot = team_sum16(T, S, v, nq);
+      if (T.rank < nq) contrib[S.gop[T.rank]] = tot;
+      T.sync();
+#pragma unroll
+      for (int q = 0; q < kM; ++q) v[q] = 0.0;
+      nq = 0;
     }
   }
 }
@@ -770,10 +880,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
         layer_setup(T, S, ops, coef, sg);
         layer_pass(T, S, psi, N, sg.count, false, own_scale(s), ck + (size_t)sg.ckpt * N);
       } else {
-        for (int l = sg.first; l < sg.first + sg.count; ++l) {
-          op_pass(T, psi, N, ops[l], coef[l], false);
-          T.sync();
-        }
+        gates_fwd(T, psi, N, ops, coef, sg.first, sg.count);
       }
     }
 
@@ -921,36 +1028,7 @@ __device__ void run_instance(const BatchArgs& a, int idx, const Team& T, TeamS& 
     for (int s = I.n_segs - 1; s >= 0; --s) {
       const Seg sg = segs[s];
       if (sg.kind == SEG_GATES) {
-        for (int l = sg.first + sg.count - 1; l >= sg.first; --l) {
-          const DOp op = ops[l];
-          const Rot r = coef[l];
-          const uint32_t np = N >> op.k;
-          const bool pg = op.param >= 0;
-          const uint32_t lo = (uint32_t)op.lo_or, fl = (uint32_t)op.flip;
-          double acc = 0.0;
-          for (uint32_t p = tid; p < np; p += TS) {
-            const uint32_t i = insert_zeros32(p, op.sb, op.k) | lo;
-            if (op.type == SV_GATE_CZ) {
-              psi[i] = make_double2(dneg(psi[i].x), dneg(psi[i].y));
-              lam[i] = make_double2(dneg(lam[i].x), dneg(lam[i].y));
-            } else {
-              const uint32_t j = i ^ fl;
-              double2 px = psi[i], py = psi[j], lx = lam[i], ly = lam[j];
-              if (pg) pair_grad_acc(op.type, lx, ly, px, py, acc);
-              pair_apply(op.type, r, true, px, py);
-              pair_apply(op.type, r, true, lx, ly);
-              psi[i] = px;
-              psi[j] = py;
-              lam[i] = lx;
-              lam[j] = ly;
-            }
-          }
-          if (pg) {
-            const double t = team_sum(T, S, acc);
-            if (tid == 0) contrib[l] = t;
-          }
-          T.sync();
-        }
+        gates_bwd(T, S, psi, lam, N, ops, coef, sg.first, sg.count, contrib);
         continue;
       }
       if (sg.kind == SEG_PERM) {
