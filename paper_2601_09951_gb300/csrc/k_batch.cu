@@ -62,6 +62,10 @@ struct TeamS {
   uint32_t pm_lo[kMaxPerm];  // condition and flip masks of a permutation segment's gates
   uint32_t pm_fl[kMaxPerm];
   LOp lop[kM];               // the gates of a commuting layer, staged once per segment
+  double2 bcs[12];           // (cos, sin) of the one RZ gate on each index bit, or (1, 0)
+  double2 sub[32];           // phases over three bits each
+  int dup;                   // some bit has several RZ gates
+  int pad2[3];
   int gop[kM];               // ops whose gradients wait to be reduced (plain gates)
 };
 constexpr int kDpBlockAmps = 173;
@@ -546,12 +550,16 @@ __device__ __noinline__ int diag_setup(const Team& T, TeamS& S, const DOp* ops,
     const int lane = threadIdx.x & 31;
     int type = -1;
     DOp op;
+    if (lane < 12) S.bcs[lane] = make_double2(1.0, 0.0);
+    __syncwarp();
     if (lane < sg.count) {
       op = ops[sg.first + lane];
       type = op.type;
     }
     const unsigned brz = __ballot_sync(kFull, type == SV_GATE_RZ);
     const unsigned bcz = __ballot_sync(kFull, type == SV_GATE_CZ);
+    const unsigned same = __match_any_sync(kFull, type == SV_GATE_RZ ? op.bit0 : -1 - lane);
+    const unsigned dup = __ballot_sync(kFull, type == SV_GATE_RZ && (same & (same - 1u)) != 0u);
     const unsigned below = (1u << lane) - 1u;
     if (type == SV_GATE_RZ) {
       const int i = __popc(brz & below);
@@ -559,29 +567,54 @@ __device__ __noinline__ int diag_setup(const Team& T, TeamS& S, const DOp* ops,
       S.rz_bit[i] = op.bit0;
       const Rot r = coef[sg.first + lane];  // (cos phi, sin phi), set up with the step's coefficients
       S.cs[i] = make_double2(r.a, r.b);
+      S.bcs[op.bit0] = make_double2(r.a, r.b);
     } else if (type == SV_GATE_CZ) {
       S.cz_mask[__popc(bcz & below)] = (uint32_t)op.lo_or;
     }
     if (lane == 0) {
       S.n_rz = __popc(brz);
       S.n_cz = __popc(bcz);
+      S.dup = dup != 0u;
     }
   }
   T.sync();
   const int m = S.n_rz;
   const int hl = n < 6 ? n : 6;
   const int nl = 1 << hl, nh = 1 << (n - hl);
+  if (S.dup) {
+    for (int j = T.rank; j < nl + nh; j += T.size) {
+      const bool hi = j >= nl;
+      const int jj = hi ? j - nl : j;
+      double2 p = make_double2(hi ? scale : 1.0, 0.0);
+      for (int g = 0; g < m; ++g) {
+        const int b = S.rz_bit[g];
+        if ((b >= hl) != hi) continue;
+        const int bit = (jj >> (hi ? b - hl : b)) & 1;
+        const double2 f = make_double2(S.cs[g].x, bit ? S.cs[g].y : dneg(S.cs[g].y));
+        p = cmul(p, f);
+      }
+      if (hi) S.th[jj] = p; else S.tl[jj] = p;
+    }
+    T.sync();
+    return m;
+  }
+  // one gate per bit at most: phases over bits [0, 3), [3, 6), [6, 9) and [9, 12) (eight each),
+  // then their products (3 complex multiplications in a row instead of 6)
+  for (int j = T.rank; j < 32; j += T.size) {
+    const int b0 = 3 * (j >> 3);
+    auto f = [&](int i) {
+      const double2 c = S.bcs[b0 + i];
+      return make_double2(c.x, (j >> i) & 1 ? c.y : dneg(c.y));
+    };
+    double2 p = cmul(cmul(f(0), f(1)), f(2));
+    if (b0 == 6) p = make_double2(scale * p.x, scale * p.y);
+    S.sub[j] = p;
+  }
+  T.sync();
   for (int j = T.rank; j < nl + nh; j += T.size) {
     const bool hi = j >= nl;
-    const int jj = hi ? j - nl : j;
-    double2 p = make_double2(hi ? scale : 1.0, 0.0);
-    for (int g = 0; g < m; ++g) {
-      const int b = S.rz_bit[g];
-      if ((b >= hl) != hi) continue;
-      const int bit = (jj >> (hi ? b - hl : b)) & 1;
-      const double2 f = make_double2(S.cs[g].x, bit ? S.cs[g].y : dneg(S.cs[g].y));
-      p = cmul(p, f);
-    }
+    const int jj = hi ? j - nl : j, o = hi ? 16 : 0;
+    const double2 p = cmul(S.sub[o + (jj & 7)], S.sub[o + 8 + (jj >> 3)]);
     if (hi) S.th[jj] = p; else S.tl[jj] = p;
   }
   T.sync();
