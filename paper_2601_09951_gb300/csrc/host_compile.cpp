@@ -350,6 +350,13 @@ void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan, int 
       --left;
     }
     P.n_slots = slot;
+    // A pass of gates on two or more wires reads and writes only what they touch (a
+    // DoubleExcitation an eighth of the tile, four of them 40 %) when the state makes more tiles
+    // than the chip runs at once: its time is then the L2's.  With fewer, finding what is touched
+    // costs more than the copies (18 qubits, 128 tiles: 1.25 ms for 300 excitations against 1.42).
+    P.sparse = __builtin_popcountll(P.outer_mask) >= kSparseTilesLog && P.diag < 0;
+    for (int i = P.first_item; i < P.first_item + P.n_items; ++i)
+      P.sparse = P.sparse && plan.items[i].local.k >= 2;
     plan.passes.push_back(P);
   }
 }

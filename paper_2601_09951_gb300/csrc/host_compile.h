@@ -58,6 +58,7 @@ std::vector<std::pair<int, int>> commuting_layers(const std::vector<DOp>& ops, i
 // Every tile includes the min_low lowest bits; min_low < 0 selects kMinLowBits (kMinLowBitsL2
 // for n <= kL2Qubits).
 constexpr int kMaxSlots = kMaxSlotsDev;
+constexpr int kSparseTilesLog = 8;
 struct HostPlan {
   std::vector<FPass> passes;
   std::vector<FItem> items;

@@ -176,6 +176,25 @@ __device__ __forceinline__ void stage_items(SItem* S, const SItem* src, int cnt,
   S[lane] = o;
 }
 
+// Which of the thread's amplitudes (bit i: j = tid + i nt) some item of a sparse pass touches: the
+// others are neither read nor written (see FPass::sparse).
+__device__ __forceinline__ uint32_t touched(const SItem* its, int n_items, const TileMap& T) {
+  uint32_t need = 0;
+  for (int q = 0; q < n_items; ++q) {
+    const SItem& s = its[q];
+    uint32_t wires = 0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (t < s.k) wires |= 1u << s.sb[t];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t w = (threadIdx.x + i * blockDim.x) & wires;
+      if (i < T.cnt && (w == s.lo || w == (s.lo ^ s.fl))) need |= 1u << i;
+    }
+  }
+  return need;
+}
+
 // One pair of one of the normalised kinds.
 template <int KIND>
 __device__ __forceinline__ void fapply(const SItem& s, double2& x, double2& y) {
@@ -361,7 +380,7 @@ __device__ __forceinline__ bool can_pair(const SItem& a, const SItem& b) {
 
 // INV: apply the pass's items inverted, in reverse order (un-applying the pass).
 template <bool INV>
-__global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPass P,
+__global__ void __launch_bounds__(kFT, 4) k_fpass(double2* __restrict__ psi, FPass P,
                                                const SItem* __restrict__ items,
                                                const DOp* __restrict__ gops,
                                                const double2* __restrict__ cs,
@@ -377,12 +396,18 @@ __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPa
   items += P.first_item;
   if (nch == 1 && threadIdx.x < 32) stage_items(its, items, P.n_items, INV);
   if (P.diag >= 0) diag_setup(D, P, items[P.diag].op, items[P.diag].count, gops, cs);
+  uint32_t need = (1u << T.cnt) - 1u;
+  if (P.sparse && nch == 1) {
+    __syncthreads();
+    need = touched(its, P.n_items, T);
+  }
   pdl_begin();
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (i < T.cnt) cp_async16(&tile[threadIdx.x + i * nt], &psi[outer | tile_idx(T, i)]);
+      if ((need >> i) & 1u)
+        cp_async16(&tile[threadIdx.x + i * nt], &psi[outer | tile_idx(T, i)]);
     if (P.diag >= 0) diag_tile(D, P, outer);
     for (int ch = 0; ch < nch; ++ch) {
       const int base = (INV ? nch - 1 - ch : ch) * kChunk;
@@ -418,7 +443,7 @@ __global__ void __launch_bounds__(kFT, 5) k_fpass(double2* __restrict__ psi, FPa
     if (f == 1.0) {
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        if (i < T.cnt) psi[outer | tile_idx(T, i)] = tile[threadIdx.x + i * nt];
+        if ((need >> i) & 1u) psi[outer | tile_idx(T, i)] = tile[threadIdx.x + i * nt];
     } else {
 #pragma unroll
       for (int i = 0; i < 8; ++i)
@@ -474,12 +499,17 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
       }
     }
   }
+  uint32_t need = (1u << T.cnt) - 1u;
+  if (P.sparse && nch == 1) {
+    __syncthreads();
+    need = touched(its, P.n_items, T);
+  }
   pdl_begin();
   for (uint64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const uint32_t outer = pdep32((uint32_t)t, (uint32_t)P.outer_mask);
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (i < T.cnt) {
+      if ((need >> i) & 1u) {
         const uint32_t k = outer | tile_idx(T, i);
         cp_async16(&tp[tid + i * nt], &psi[k]);
         cp_async16(&tlam[tid + i * nt], &lam[k]);
@@ -551,7 +581,7 @@ __global__ void __launch_bounds__(kFT, 2) k_bpass(double2* __restrict__ psi,
     if (f == 1.0) {
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        if (i < T.cnt) {
+        if ((need >> i) & 1u) {
           const uint32_t k = outer | tile_idx(T, i);
           psi[k] = tp[tid + i * nt];
           lam[k] = tlam[tid + i * nt];

@@ -117,7 +117,8 @@ struct FPass {
   int32_t first_item, n_items;
   int32_t n_slots;  // gradient slots used by the pass's parameterised items
   int32_t diag;     // index of the pass's diagonal item (kind 1), or -1
-  int32_t pad[2];
+  int32_t sparse;   // no item touches all of a tile, and skipping the rest pays (see plan_passes)
+  int32_t pad;
 };
 static_assert(sizeof(FPass) == 48, "FPass layout");
 
