@@ -162,8 +162,9 @@ __global__ void __launch_bounds__(kDT, 7) k_dp(const double2* __restrict__ in,
 // partial[op * kRedBlocks + block] for every parameterised RZ op of the segment.  The number of
 // CTAs is a power of two, G: CTA c takes visit indices t = c, c + G, c + 2G, ..., so the bits of
 // t below log2 G are fixed per CTA (their signs apply to the CTA's total) and the bits above
-// are bits of the round r (one sum each, at most kMaxRound).
-template <int NA>
+// are bits of the round r (one sum each, at most MR: 5 up to 25 qubits, which saves twelve
+// registers and the spills).
+template <int NA, int MR>
 __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ lam,
                                                    const double2* __restrict__ psi_b,
                                                    double2* __restrict__ out, DpArgs a,
@@ -178,9 +179,9 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
   const uint32_t nblk = 1u << (a.n - BL);
   const int lg = 31 - __clz((int)gridDim.x);
   const int nrb = a.n - BL - lg;  // round bits
-  double W = 0.0, mid[3] = {0.0, 0.0, 0.0}, hr[kMaxRound];
+  double W = 0.0, mid[3] = {0.0, 0.0, 0.0}, hr[MR];
 #pragma unroll
-  for (int b = 0; b < kMaxRound; ++b) hr[b] = 0.0;
+  for (int b = 0; b < MR; ++b) hr[b] = 0.0;
   for (uint32_t r0 = 0; blockIdx.x + r0 * gridDim.x < nblk; r0 += kChunk) {
     if (r0) dp_rounds(S, a, r0, nblk);
     for (int r = 0; r < kChunk && blockIdx.x + (r0 + r) * gridDim.x < nblk; ++r) {
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
       }
       W += wb;
 #pragma unroll
-      for (int b = 0; b < kMaxRound; ++b)
+      for (int b = 0; b < MR; ++b)
         if (b < nrb) hr[b] += (((r0 + r) >> b) & 1u) ? dneg(wb) : wb;
     }
   }
@@ -250,10 +251,10 @@ __global__ void __launch_bounds__(kDT, 7) k_dp_lam(const double2* __restrict__ l
     const double t = warp_sum16(v);
     if ((lane & 1) == 0) red[warp][lane >> 1] = t;
   }
-  if (nrb > 5) {
+  if constexpr (MR > 5) {
     double v[16];
 #pragma unroll
-    for (int b = 0; b < 16; ++b) v[b] = b + 5 < kMaxRound ? hr[b + 5 < kMaxRound ? b + 5 : 0] : 0.0;
+    for (int b = 0; b < 16; ++b) v[b] = b + 5 < MR ? hr[b + 5 < MR ? b + 5 : 0] : 0.0;
     const double t = warp_sum16(v);
     if ((lane & 1) == 0) red[warp][16 + (lane >> 1)] = t;
   }
@@ -529,7 +530,7 @@ int dp_blocks(int n) { return (int)std::min<uint64_t>(1ull << (n - dp_block_log(
 template <int NA>
 static cudaError_t prepare_na() {
   const void* ks[] = {(const void*)k_dp<NA, DP_FWD>, (const void*)k_dp<NA, DP_BWD>,
-                      (const void*)k_dp<NA, DP_MAKE>, (const void*)k_dp_lam<NA>,
+                      (const void*)k_dp<NA, DP_MAKE>, (const void*)k_dp_lam<NA, 5>,
                       (const void*)k_prod_lam<NA>};
   for (const void* k : ks) {
     const cudaError_t e =
@@ -559,7 +560,7 @@ cudaError_t dp_prepare(int n) {
 #define DP_K_FWD(NA) k_dp<NA, DP_FWD>
 #define DP_K_BWD(NA) k_dp<NA, DP_BWD>
 #define DP_K_MAKE(NA) k_dp<NA, DP_MAKE>
-#define DP_K_LAM(NA) k_dp_lam<NA>
+#define DP_K_LAM(NA) k_dp_lam<NA, 5>
 #define DP_K_PROD(NA) k_prod_lam<NA>
 
 cudaError_t launch_dp_fwd(const double2* in, double2* out, const DpArgs& a, cudaStream_t s,
@@ -577,6 +578,9 @@ cudaError_t launch_dp_bwd_psi(const double2* in, double2* out, const DpArgs& a, 
 cudaError_t launch_dp_bwd_lam(const double2* lam, const double2* psi_b, double2* out,
                               const DpArgs& a, double* partial, cudaStream_t s, bool overlap) {
   const int g = dp_blocks(a.n);
+  if (a.n - dp_block_log(a.n) - 10 > 5)  // round bits: 1024 CTAs
+    return launch_overlapped(k_dp_lam<8, kMaxRound>, g, kDT, 0, s, overlap, lam, psi_b, out, a,
+                             partial);
   DP_LAUNCH(DP_K_LAM, lam, psi_b, out, a, partial)
 }
 
