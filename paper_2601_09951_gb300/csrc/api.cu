@@ -550,6 +550,9 @@ static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan
   }
 }
 
+// Whether the parts of the product prefix's gradients fit a state buffer (from 15 qubits).
+static bool prod_in_psi(int n) { return prod_scratch(n) * sizeof(double) <= sv_state_bytes(n); }
+
 // Length of the circuit's product prefix, its leading one-qubit gates, or 0: it is used from the
 // registers that have whole-state segments, when it saves at least a pass or so.
 static int product_prefix(const HostCircuit& hc) {
@@ -771,7 +774,7 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
     }
     if (ch.kind == sv_ctx::CH_PROD) {
       units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++, 0, 0});
-      SV_ROOM(prod, prod_cap, prod_scratch(c->n));
+      if (!prod_in_psi(c->n)) SV_ROOM(prod, prod_cap, prod_scratch(c->n));
       continue;
     }
     cf = cl = 0;
@@ -1120,7 +1123,9 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
           }
         }
       } else if (ch.kind == sv_ctx::CH_PROD) {
-        SV_CUDA(launch_prod_grads(lam, ch.dp, c->ops, ch.ck, c->cs, c->ref, c->prod, c->gpart,
+        // (nothing reads psi any more: it takes the contraction's parts where they fit)
+        double* part = prod_in_psi(c->n) ? reinterpret_cast<double*>(psi) : c->prod;
+        SV_CUDA(launch_prod_grads(lam, ch.dp, c->ops, ch.ck, c->cs, c->ref, part, c->gpart,
                                   c->stream, true), c);
       } else if (ch.kind == sv_ctx::CH_LAYER) {
         // a checkpointed commuting layer: every gradient from (psi, lambda) at the layer's
@@ -1320,7 +1325,7 @@ sv_status svqe::adjoint_fixed(const HostCircuit& hc, uint64_t ref, const DGroup*
   take(c.sitems, c.sitems_cap, G);
   take(c.scales, c.scales_cap, G);
   take(c.blob, c.blob_cap, G * (sizeof(DOp) + sizeof(FItem) + sizeof(PrepUnit)) + 1024);
-  if (hc.n >= kDpMinQubits) take(c.prod, c.prod_cap, prod_scratch(hc.n));
+  if (hc.n >= kDpMinQubits && !prod_in_psi(hc.n)) take(c.prod, c.prod_cap, prod_scratch(hc.n));
   if (at >= bytes) {
     set_error("the working memory is too small for this circuit");
     return SV_ENOMEM;

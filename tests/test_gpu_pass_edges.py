@@ -140,3 +140,48 @@ def test_without_device_allocation_every_route(make):
         e, g = call(rec)
         assert_energy(e, e0, inst["ham"])
         assert_grad(g, g0, inst["ham"])
+
+
+def test_states_the_caller_can_reach_are_not_taken_for_the_reference():
+    """A circuit applied right after sv_init_reference may start from a product state; one applied
+    to a state set by the caller, to an earlier circuit's result, or to a state whose address the
+    caller holds (and here overwrites) may not."""
+    torch = pytest.importorskip("torch")
+    n = 12
+    rng = np.random.default_rng(77)
+    inst = W.hea_instance(n, 2, 10, 78)
+    circ, theta = inst["circuit"], inst["theta"]
+    ctx = svqe.Context(n)
+    ctx.init_reference(5)
+    ctx.apply_circuit(circ, theta)
+    once = oracle.state(circ, theta, 5)
+    assert np.max(np.abs(ctx.get_state() - once)) <= PSI_TOL
+    ctx.apply_circuit(circ, theta)  # on its own result
+
+    def apply(psi):
+        for t, w, p, f in zip(circ["types"], circ["wires"], circ["params"], circ["fixed"]):
+            wires = [int(q) for q in w[:W.N_WIRES[int(t)]]]
+            psi = oracle.apply_gate(psi, n, int(t), wires, float(theta[p]) if p >= 0 else f)
+        return psi
+
+    assert np.max(np.abs(ctx.get_state() - apply(once))) <= PSI_TOL
+    psi = rng.normal(size=1 << n) + 1j * rng.normal(size=1 << n)
+    psi /= np.linalg.norm(psi)
+    want = apply(psi)
+    ctx.init_reference(5)
+    ctx.set_state(psi)
+    ctx.apply_circuit(circ, theta)
+    assert np.max(np.abs(ctx.get_state() - want)) <= PSI_TOL
+    stream = torch.cuda.current_stream().cuda_stream
+    own = svqe.Context(n, stream=stream)
+    ptr = own.state_ptr()
+    own.init_reference(5)
+
+    class Psi:  # the context's buffer as a torch tensor
+        __cuda_array_interface__ = {"shape": (1 << n,), "typestr": "<c16", "data": (ptr, False),
+                                    "version": 2}
+
+    torch.as_tensor(Psi(), device="cuda").copy_(torch.as_tensor(psi).cuda())
+    torch.cuda.synchronize()
+    own.apply_circuit(circ, theta)
+    assert np.max(np.abs(own.get_state() - want)) <= PSI_TOL
