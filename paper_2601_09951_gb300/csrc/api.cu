@@ -530,8 +530,28 @@ static double plan_cost(const HostPlan& plan, double* fp64_us) {
 // L2, where a 16- or 32-byte access costs no burst) leave its other bits for gate wires: two
 // passes still cover every qubit of a layer.  Gates on many wires (excitations) need more of the
 // smaller passes, so the sizes are compared by plan_cost.
+//
+// Above, one low bit fewer (128-byte runs of an HBM-resident state, 32-byte ones in L2) where that
+// saves a run of one-qubit gates a pass: a layer on 26 or 27 qubits (11 + 8 + 8 gates instead of
+// 11 + 7 + 7 + the rest) and on 21 (11 + 10).  Ten layers, an evaluation: 296 -> 272 ms at 26
+// qubits (whose pass of one gate also kept the layer's scale out of the segment), 570 -> 561 at
+// 27, 8.59 -> 7.97 at 21.
 static void plan_run(const std::vector<DOp>& ops, int n, int tile_bits, HostPlan& plan) {
   plan_passes(ops, n, tile_bits, plan);
+  if (n > 17 && plan.passes.size() > 1) {
+    uint64_t bits = 0;
+    for (const DOp& op : ops) {
+      if (op.k != 1) return;
+      bits |= 1ull << op.bit0;
+    }
+    const int low = (n <= kL2Qubits ? kMinLowBitsL2 : kMinLowBits) - 1;
+    const int rest = __builtin_popcountll(bits) - tile_bits, per = tile_bits - low;
+    if ((int)plan.passes.size() <= 1 + (std::max(0, rest) + per - 1) / per) return;
+    HostPlan p;
+    plan_passes(ops, n, tile_bits, p, low);
+    if (p.passes.size() < plan.passes.size()) std::swap(plan, p);
+    return;
+  }
   const int m = std::max({n - 7, (n + 1) / 2, 4 + kMinLowBitsL2});  // (a gate has up to 4 wires)
   if (n > 17 || m >= tile_bits) return;
   // (planning 300 gates again takes 30 us: not when too little of the time could be saved)

@@ -97,10 +97,11 @@ static_assert(sizeof(Seg) == 16, "Seg layout");
 constexpr int kMaxPerm = 32;
 // Gradient slots per fused pass (and RZ gates per diagonal item).
 constexpr int kMaxSlotsDev = 16;
-// Lowest contiguous bits every fused tile includes (runs of 2^kMinLowBits amplitudes, 256 B),
+// Lowest contiguous bits a fused tile includes (runs of 2^kMinLowBits amplitudes, 256 B),
 // so that tiles of an HBM-resident state move in long DRAM bursts.  A state small enough for
 // psi and lambda to stay in L2 (n <= kL2Qubits) needs only 32-byte sectors: its tiles include
 // kMinLowBitsL2 low bits, which leaves more of the tile's bits for gate wires (fewer passes).
+// plan_run (api.cu) goes one lower where that saves a pass, and below 18 qubits.
 constexpr int kMinLowBits = 4;
 constexpr int kMinLowBitsL2 = 2;
 constexpr int kL2Qubits = 21;

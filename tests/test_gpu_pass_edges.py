@@ -185,3 +185,34 @@ def test_states_the_caller_can_reach_are_not_taken_for_the_reference():
     torch.cuda.synchronize()
     own.apply_circuit(circ, theta)
     assert np.max(np.abs(own.get_state() - want)) <= PSI_TOL
+
+
+@pytest.mark.parametrize("n,odd", [(21, 0), (21, 1), (19, 0)])
+def test_layers_of_an_odd_number_of_tile_bits(n, odd):
+    """RY and RX layers planned with one low bit fewer (21 qubits: two passes instead of three;
+    with one gate left out and at 19 qubits the ordinary plan).  The state against the oracle,
+    three gradient entries against its parameter shift."""
+    rng = np.random.default_rng(2100 + n + odd)
+    cb = W.CircuitBuilder(n)
+    for layer, gate in enumerate((W.RX, W.RY, W.RX)):
+        for q in range(n - (odd if layer else 0)):
+            cb.add(gate, (q,), param="new")
+        for q in range(n):
+            cb.add(W.RZ, (q,), angle=float(rng.uniform(-3, 3)))
+        for q in range(n - 1):
+            cb.add(W.CNOT, (q, q + 1))
+    circ = cb.build()
+    theta = rng.uniform(-7, 7, circ["n_params"])
+    ham = W.tfim_instance(n)["ham"]
+    ctx = svqe.Context(n)
+    ctx.init_reference(3)
+    ctx.apply_circuit(circ, theta)
+    psi = oracle.state(circ, theta, 3)
+    assert np.max(np.abs(ctx.get_state() - psi)) <= PSI_TOL
+    H = svqe.Ham(ctx, ham)
+    e, g = ctx.adjoint_grad(circ, theta, H)
+    assert_energy(e, oracle.expval(psi, n, ham)[0], ham)
+    which = [0, n + n // 2, circ["n_params"] - 1]
+    inst = {"circuit": circ, "ham": ham, "ref": 3, "theta": theta}
+    want = oracle.energy_grad_subset(inst, which)[1]
+    assert_grad(g[which], [want[p] for p in which], ham)
