@@ -304,8 +304,9 @@ HBM_PEAK_GBS = 6678.2  # measured copy bandwidth (read + write) of a GB300
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_batch launch of the default workload,
 # from one ncu capture of that launch, keyed by a hash of the kernel's sources: once the
 # kernel changes the key no longer matches and traffic is null.
-KBATCH_TRAFFIC = {"fa0046678f00f781": 373.54e6 + 519.86e6,
-                  "69036a9ca5c72f5d": 373.48e6 + 519.67e6}
+# (The second key differs from the first by a comment in svqe_types.h.)
+KBATCH_TRAFFIC = {"ea31bb0808c4b826": 338.64e6 + 470.35e6,
+                  "4c6a29bd7dbf863d": 338.64e6 + 470.35e6}
 KBATCH_SOURCES = ("k_batch.cu", "svqe_internal.cuh", "svqe_types.h", "launch.h")
 
 
@@ -401,10 +402,10 @@ def kernel_table(svqe, W, torch, n, subset=None):
     layer = W.hea_circuit(n, 1, ring=True)
     lc = svqe.Circuit(layer)
     lth = np.random.default_rng(0).uniform(-3, 3, layer["n_params"])
-    # one HEA layer, fused passes: FP64 per amplitude = 6 per RY + 12 for the RZ run
+    # one HEA layer, fused passes: FP64 per amplitude = 4 per RY (unnormalised) + 12 for the RZ run
     n_pass, _ = svqe.circuit_plan(lc)
     timed(f"fused HEA layer, {n_pass} passes (a6, forward)",
-          lambda: ctx.apply_circuit(lc, lth), 32 * n_pass, 6 * n + 12)
+          lambda: ctx.apply_circuit(lc, lth), 32 * n_pass, 4 * n + 12)
     inst = W.hea_single(n, layers=1, n_terms=100)
     H = svqe.Ham(ctx, inst["ham"])
     G = H.info()[0]
@@ -553,9 +554,9 @@ def run_single(args):
 
 def per_circuit(insts, sample):
     """The plain one-circuit-per-launch path on the same instances: each instance's energy and
-    adjoint gradient through a single-state context (sv_adjoint_grad_dev: fused passes),
-    one after another on one stream, for the first `sample` instances.  evals/s from CUDA
-    events; launches per evaluation counted from the op lists."""
+    adjoint gradient through a single-state context (sv_adjoint_grad_dev: one launch up to 10
+    qubits, fused passes above), one after another on one stream, for the first `sample`
+    instances.  evals/s from CUDA events; launches per evaluation estimated from the op lists."""
     import torch
     from paper_2601_09951_gb300 import svqe
     stream = torch.cuda.Stream()
@@ -570,9 +571,9 @@ def per_circuit(insts, sample):
         th = torch.tensor(np.asarray(inst["theta"], dtype=np.float64), device="cuda")
         g = torch.zeros(max(C.n_params, 1), dtype=torch.float64, device="cuda")
         prepared.append((ctxs[n], C, th, H, g))
-        # init, coefficients, one forward and one backward kernel per fused pass, H psi + sum,
-        # the partials' reset, per-op contributions + per-parameter sums
-        launches += 2 * svqe.circuit_plan(inst["circuit"])[0] + 7
+        # one launch up to 10 qubits; above about one forward and one backward kernel per fused
+        # pass of the plain plan, the preparation, H psi, the final sums and psi's reset
+        launches += 1 if n <= 10 else 2 * svqe.circuit_plan(inst["circuit"])[0] + 4
     e = torch.zeros(1, dtype=torch.float64, device="cuda")
     for ctx, C, th, H, g in prepared:
         ctx.adjoint_grad_dev(C, th.data_ptr(), H, e.data_ptr(), g.data_ptr())

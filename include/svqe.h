@@ -111,9 +111,12 @@ const char* sv_last_error(void);
 int32_t sv_abi_version(void);
 /* Bytes of one n-qubit complex128 state, 2^n * 16 (Table 3); 0 if n is outside [0, 62]. */
 uint64_t sv_state_bytes(int32_t n_qubits);
-/* Device bytes a context of n qubits allocates: two state buffers (psi, lambda) plus
- * reduction scratch.  Unless checkpoints are enabled (sv_set_checkpoint_bytes), at most three
- * state-sized buffers are ever used (31 qubits fit). */
+/* Device bytes a context of n qubits allocates when it is created: two state buffers (psi,
+ * lambda) plus reduction scratch.  Circuits with whole-state segments or a product prefix (from
+ * 11 qubits, see sv_adjoint_grad) add a third state-sized buffer when first staged, and every
+ * circuit its own records and partial sums (about 10 KB per gate).  Unless checkpoints are
+ * enabled (sv_set_checkpoint_bytes), at most three state-sized buffers are ever used (31 qubits
+ * fit). */
 uint64_t sv_ctx_device_bytes(int32_t n_qubits);
 
 /* ---------------------------------------------------------------- contexts */
@@ -131,13 +134,13 @@ sv_status sv_destroy(sv_ctx* ctx);
  * bytes / (2^n * 16) such layers, the forward pass copies psi before the layer into its own
  * buffer.  The adjoint sweep then takes all of the layer's gradients at its end (the
  * layer's gates commute).  It un-applies the layer to lambda only and copies psi back:
- * 5 instead of 8 FP64 operations per amplitude per gate.  The paper's gradient (Algorithm 1)
- * is unchanged up to rounding.  Buffers are allocated when a circuit is staged, as far as
+ * 6 instead of 8 FP64 operations per amplitude per gate, both directions together.  The paper's
+ * gradient (Algorithm 1) is unchanged up to rounding.  Buffers are allocated when a circuit is staged, as far as
  * the device allows.  A smaller budget frees the buffers beyond it; SV_EINVAL for a NULL
  * handle. */
 sv_status sv_set_checkpoint_bytes(sv_ctx* ctx, uint64_t bytes);
 /* Autotuning of the fused-pass tile size; off by default
- * (tiles of 2^11 amplitudes).  When on, the first sv_adjoint_grad* / vqe_step call with a
+ * (tiles of 2^11 amplitudes; below 18 qubits smaller ones where they are estimated faster).  When on, the first sv_adjoint_grad* / vqe_step call with a
  * circuit structure not seen before in the process does the following.  Gate types and wires
  * count as structure; angles do not.  It times the forward pass with tiles of 2^9, 2^10 and
  * 2^11 amplitudes and keeps the fastest.  That call therefore runs three extra forward passes
@@ -145,7 +148,8 @@ sv_status sv_set_checkpoint_bytes(sv_ctx* ctx, uint64_t bytes);
  * process.  If the environment variable SVQE_TUNE_CACHE names a file, results are read from
  * and appended to it as "n key bits" lines.  SV_EINVAL for a NULL handle. */
 sv_status sv_set_autotune(sv_ctx* ctx, int32_t enable);
-/* Tile size (bits) of the fused passes of the last circuit staged on the context. */
+/* Tile size (bits) of the fused passes of the last circuit staged on the context: the largest
+ * it was planned with (passes of a register below 18 qubits may use smaller tiles). */
 sv_status sv_tile_bits(const sv_ctx* ctx, int32_t* tile_bits);
 
 /* ---------------------------------------------------------------- Hamiltonians */
@@ -214,8 +218,12 @@ sv_status sv_expval_paulisum(sv_ctx* ctx, const sv_ham* h, double* energy_out);
  * last sv_init_reference (|0> if none).  The paper differentiates by parameter shift; this
  * call reaches the same gradient by the adjoint method.  Forward pass, lambda = H psi, then the adjoint sweep
  * over gates in reverse: g_p += 2 Im<lambda|G_l|psi> for each gate l with parameter p, then
- * psi <- U_l^dag psi and lambda <- U_l^dag lambda.  Uses psi and lambda only, unless
- * checkpoints are enabled (sv_set_checkpoint_bytes).  energy_out:
+ * psi <- U_l^dag psi and lambda <- U_l^dag lambda.  Up to 10 qubits one launch evaluates the
+ * whole circuit in shared memory (with at most 8 MiB of checkpoints).  From 11 qubits, runs of
+ * RZ/CZ followed by CNOT/X gates are whole-state segments, and the circuit's leading one-qubit
+ * gates on |ref> a product state; both use a third state buffer beside psi and lambda, and the
+ * call falls back to two where it cannot be had.  Layer checkpoints: sv_set_checkpoint_bytes.
+ * psi holds |ref> again afterwards.  energy_out:
  * host double; grad_out: host array of n_params (gates sharing a parameter are summed). */
 sv_status sv_adjoint_grad(sv_ctx* ctx, const sv_circuit* circuit, const double* theta,
                           const sv_ham* h, double* energy_out, double* grad_out);
