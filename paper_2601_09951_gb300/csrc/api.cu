@@ -1,5 +1,6 @@
 // api.cu -- the C ABI of libsvqe.so (include/svqe.h): contexts, Hamiltonians, the single-state
-// path and batches.  Host code only; kernels live in k_state.cu and k_batch.cu.
+// path and batches.  Host code only; kernels live in k_prep.cu, k_state.cu, k_fused.cu, k_dp.cu
+// and k_batch.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -19,7 +19,7 @@
 // and i parts of 32 rounds are tabulated together.  The phases come from tables of 128 entries over
 // seven bits each (k_prep.cu).  Tables of 2048 entries staged per block (80 KB read through
 // 56 KB of shared memory) cost small states ten times their work and held large ones to four
-// blocks per SM: the lambda sweep took 94 us at 17 qubits and 610 us at 24, now 20 and 470.
+// blocks per SM: the lambda sweep took 94 us at 17 qubits and 610 us at 24, now 20 and 437.
 // Out of place: the gather/scatter needs a second buffer.
 //
 // Bound by the FP64 pipe on an HBM-resident state (8 operations per amplitude forward, 12.75 in
