@@ -28,6 +28,6 @@ def assert_grad(got, want, ham, what=""):
     want = np.asarray(want)
     assert got.shape == want.shape, (got.shape, want.shape)
     bound = G_TOL * np.maximum(np.abs(want), max(l1(ham), 1e-300))
-    bad = np.abs(got - want) > bound
+    bad = ~(np.abs(got - want) <= bound)  # (a NaN is a mismatch)
     assert not bad.any(), (f"{what} gradient mismatch at {np.flatnonzero(bad)[:8]}: "
                            f"{got[bad][:4]} vs {want[bad][:4]}")
