@@ -250,6 +250,7 @@ struct Unit {      // a schedulable unit: one op, or a run of RZ ops (diagonal i
   uint64_t pair;   // bits that must lie inside the tile
   uint64_t touch;  // bits the unit acts on
   int slots;       // gradient slots it needs
+  int rot;         // 1 for an RY or RX gate
 };
 }  // namespace
 
@@ -264,7 +265,7 @@ void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan, int 
       int e = l;
       while (e < n_ops && ops[e].type == SV_GATE_RZ && e - l < kMaxSlots) ++e;
       if (e - l >= 3) {
-        Unit u{1, l, e - l, 0, 0, 0};
+        Unit u{1, l, e - l, 0, 0, 0, 0};
         for (int q = l; q < e; ++q) {
           u.touch |= 1ull << ops[q].bit0;
           u.slots += ops[q].param >= 0;
@@ -277,30 +278,36 @@ void plan_passes(const std::vector<DOp>& ops, int n, int m, HostPlan& plan, int 
     const DOp& op = ops[l];
     uint64_t bits = 0;
     for (int a = 0; a < op.k; ++a) bits |= 1ull << op.sb[a];
-    units.push_back(Unit{0, l, 1, bits, bits, op.param >= 0 ? 1 : 0});
+    units.push_back(Unit{0, l, 1, bits, bits, op.param >= 0 ? 1 : 0,
+                         op.type == SV_GATE_RY || op.type == SV_GATE_RX});
     ++l;
   }
   m = std::min(m, n);
   const uint64_t low = (1ull << std::min(min_low, n)) - 1ull;
+  const uint64_t full = n >= 64 ? ~0ull : (1ull << n) - 1ull;
   std::vector<char> done(units.size(), 0);
-  size_t left = units.size();
+  size_t left = units.size(), next = 0;  // next: the first unit not taken yet
   while (left > 0) {
+    while (done[next]) ++next;
     uint64_t pair = 0, blocked = 0;
-    int slots = 0;
+    int slots = 0, rot = 0;
     bool have_diag = false;
     std::vector<int> take;
-    for (size_t u = 0; u < units.size(); ++u) {
+    for (size_t u = next; u < units.size(); ++u) {
       if (done[u]) continue;
       const Unit& U = units[u];
       bool ok = !(U.touch & blocked) && __builtin_popcountll(pair | U.pair | low) <= m &&
-                slots + U.slots <= kMaxSlots && !(U.kind == 1 && have_diag);
+                slots + U.slots <= kMaxSlots && rot + U.rot <= kMaxPassRot &&
+                !(U.kind == 1 && have_diag);
       if (!ok) {
         blocked |= U.touch;
+        if (blocked == full) break;  // (nothing later can be taken)
         continue;
       }
       take.push_back((int)u);
       pair |= U.pair;
       slots += U.slots;
+      rot += U.rot;
       have_diag |= U.kind == 1;
     }
     // Tile bits: the pass's pair bits plus the lowest free bits up to m (contiguous runs).

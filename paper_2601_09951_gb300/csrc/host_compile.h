@@ -54,10 +54,15 @@ std::vector<std::pair<int, int>> commuting_layers(const std::vector<DOp>& ops, i
 // greedily in order into the current pass while the pass's pair bits fit the tile; an op may
 // move ahead of ops skipped for this pass only if it shares no qubit with them (so it
 // commutes with them).  Runs of >= 3 consecutive RZ gates become one diagonal item (at most
-// one per pass, at most kMaxSlots RZ gates).  A pass holds at most kMaxSlots gradient slots.
+// one per pass, at most kMaxSlots RZ gates).  A pass holds at most kMaxSlots gradient slots and
+// kMaxPassRot RY/RX gates: those run without their normalisation, each growing the tile by up to
+// sqrt 2 until the pass stores it, and fixed-angle ones need no slot.  128 bound the growth of psi
+// and lambda by 2^64 each and keep the gradient factors (SItem::f) above 2^-128; without a bound
+// the amplitudes of 2048 gates, and the gradients of 1024, overflowed.
 // Every tile includes the min_low lowest bits; min_low < 0 selects kMinLowBits (kMinLowBitsL2
 // for n <= kL2Qubits).
 constexpr int kMaxSlots = kMaxSlotsDev;
+constexpr int kMaxPassRot = 128;
 constexpr int kSparseTilesLog = 8;
 struct HostPlan {
   std::vector<FPass> passes;

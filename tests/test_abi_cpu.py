@@ -207,6 +207,27 @@ def test_fused_plan_keeps_dependencies_and_fits_tiles(make):
     assert n_pass * 3 <= G
 
 
+@pytest.mark.parametrize("n", [6, 12, 24])
+def test_fused_plan_bounds_the_rotations_of_a_pass(n):
+    """RY and RX gates run unnormalised until their pass ends, so a pass holds at most 128 of
+    them, also of fixed-angle ones, which take no gradient slot; other gates may still join."""
+    rng = np.random.default_rng(n)
+    cb = W.CircuitBuilder(n)
+    cb.add(W.CNOT, (0, 1))
+    cb.add(W.RY, (2,), param="new")
+    for i in range(2200):
+        q = int(rng.integers(6))
+        cb.add(*((W.H, (q,)) if i % 5 == 4 else ((W.RY, W.RX)[i % 2], (q,))))
+    circ = cb.build()
+    n_pass, pog = svqe.circuit_plan(circ)
+    rot = np.isin(np.asarray(circ["types"]), (W.RY, W.RX))
+    per = np.bincount(pog[rot], minlength=n_pass)
+    assert per.max() <= 128 and n_pass == -(-int(rot.sum()) // 128)
+    for a in range(6):  # the gates of a qubit keep their order
+        mine = pog[[a in [int(q) for q in w if q >= 0] for w in circ["wires"]]]
+        assert np.all(np.diff(mine) >= 0)
+
+
 def test_layout_and_probe_calls_validate_their_arguments():
     """Host-side argument checks of the layout tuner's calls and the FP64 probe (no device
     work: every call below is rejected before a launch)."""

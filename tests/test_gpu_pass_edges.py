@@ -216,3 +216,32 @@ def test_layers_of_an_odd_number_of_tile_bits(n, odd):
     inst = {"circuit": circ, "ham": ham, "ref": 3, "theta": theta}
     want = oracle.energy_grad_subset(inst, which)[1]
     assert_grad(g[which], [want[p] for p in which], ham)
+
+
+@pytest.mark.parametrize("n,n_rot", [(6, 2200), (12, 1200), (12, 2200)])
+def test_long_runs_of_fixed_rotations(n, n_rot):
+    """Fixed-angle rotations take no gradient slot, and at odd multiples of a quarter turn each
+    leaves out a factor of 1 / sqrt 2: all in one pass, 1024 of them would overflow the gradient
+    of the free gate before them and 2048 the amplitudes.  (At 6 qubits the records of 2200 gates
+    exceed the one-launch path; the CNOT first keeps the product prefix out.)  n_rot roundings of
+    the angles and of the amplitudes stay below 2200 * 2^-52 = 5e-13."""
+    rng = np.random.default_rng(n_rot + n)
+    cb = W.CircuitBuilder(n)
+    cb.add(W.CNOT, (0, 1))
+    cb.add(W.RY, (2,), param="new")
+    for _ in range(n_rot):
+        cb.add((W.RY, W.RX)[int(rng.integers(2))], (int(rng.integers(6)),),
+               angle=float((2 * rng.integers(-3, 3) + 1) * np.pi / 2))
+    cb.add(W.RX, (3,), param="new")
+    circ = cb.build()
+    theta = rng.uniform(-3, 3, 2)
+    ctx = svqe.Context(n)
+    ctx.init_reference(5)
+    ctx.apply_circuit(circ, theta)
+    assert np.max(np.abs(ctx.get_state() - oracle.state(circ, theta, 5))) <= PSI_TOL
+    inst = {"circuit": circ, "ham": W.random_pauli_sum(rng, n, 12, 0.5, 4, 1.0), "ref": 5,
+            "theta": theta}
+    e, g = ctx.adjoint_grad(circ, theta, svqe.Ham(ctx, inst["ham"]))
+    e0, g0 = oracle.energy_grad(inst)
+    assert_energy(e, e0, inst["ham"])
+    assert_grad(g, g0, inst["ham"])
