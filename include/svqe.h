@@ -143,8 +143,8 @@ sv_status sv_set_checkpoint_bytes(sv_ctx* ctx, uint64_t bytes);
  * (tiles of 2^11 amplitudes; below 18 qubits smaller ones where they are estimated faster).  When on, the first sv_adjoint_grad* / vqe_step call with a
  * circuit structure not seen before in the process does the following.  Gate types and wires
  * count as structure; angles do not.  It times the forward pass with tiles of 2^9, 2^10 and
- * 2^11 amplitudes and keeps the fastest.  That call therefore runs three extra forward passes
- * on psi, which the evaluation re-initialises.  Results are shared by every context of the
+ * 2^11 amplitudes and keeps the fastest.  That call therefore runs three candidates' forward
+ * passes on psi (twice each), which holds |ref> again afterwards.  Results are shared by every context of the
  * process.  If the environment variable SVQE_TUNE_CACHE names a file, results are read from
  * and appended to it as "n key bits" lines.  SV_EINVAL for a NULL handle. */
 sv_status sv_set_autotune(sv_ctx* ctx, int32_t enable);

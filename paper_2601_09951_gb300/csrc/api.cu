@@ -961,6 +961,7 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc) {
   int best = fused_tile_bits();
   float best_ms = 1e30f;
   bool ok = true;
+  c->psi_is_ref = false;
   for (int m = 9; m <= 11 && ok; ++m) {
     ok = plan_circuit(c, hc, m, true) == SV_OK;
     float ms = 0.0f;
@@ -980,7 +981,10 @@ static int tune_tile_bits(sv_ctx* c, const HostCircuit& hc) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  // (a call without an evaluation, vqe_step of no steps, leaves psi as the tuner does)
+  ok = ok && launch_init_basis(c->psi, c->n, c->ref, c->stream) == cudaSuccess;
   if (!ok) return -1;
+  c->psi_is_ref = !c->psi_shared;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune[key] = best;
   if (path) {

@@ -245,3 +245,30 @@ def test_long_runs_of_fixed_rotations(n, n_rot):
     e0, g0 = oracle.energy_grad(inst)
     assert_energy(e, e0, inst["ham"])
     assert_grad(g, g0, inst["ham"])
+
+
+@pytest.mark.parametrize("first", [W.RY, W.CNOT])
+def test_tuner_leaves_the_reference_state(first):
+    """The tile tuner runs its candidates on psi; a call that tunes without evaluating (no descent
+    steps) leaves |ref>, from which a circuit with a product prefix (RY first) and one without
+    (CNOT first) both start."""
+    n = 12
+    cb = W.CircuitBuilder(n)
+    if first == W.CNOT:
+        cb.add(W.CNOT, (0, 1))
+    for q in range(n):
+        cb.add(W.RY, (q,), param="new")
+    for q in range(n - 1):
+        cb.add(W.CZ, (q, q + 1))
+        cb.add(W.RX, (q,), angle=0.3 + 0.01 * first + q)
+    circ = cb.build()
+    theta = np.random.default_rng(41).uniform(-3, 3, circ["n_params"])
+    ctx = svqe.Context(n)
+    ctx.set_autotune(True)
+    ctx.init_reference(5)
+    ctx.vqe_step(circ, svqe.Ham(ctx, W.tfim_instance(n)["ham"]), theta, 0.1, 0)
+    ref = np.zeros(1 << n, np.complex128)
+    ref[5] = 1.0
+    assert np.max(np.abs(ctx.get_state() - ref)) <= PSI_TOL
+    ctx.apply_circuit(circ, theta)
+    assert np.max(np.abs(ctx.get_state() - oracle.state(circ, theta, 5))) <= PSI_TOL
