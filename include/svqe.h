@@ -341,7 +341,9 @@ sv_status sv_batch_adam_dev(sv_batch* b, double* theta_dev, double lr, int32_t n
  * qubit count (at most max_active_large idle sets), so that steady-state admission and
  * completion allocate and free nothing on the device.  The admitted requests' footprints and
  * the idle buffers together never exceed the budget; idle buffers are freed when an admission
- * needs their room. */
+ * needs their room.  A large request's footprint is what its context allocates, the third state
+ * buffer included (see sv_adjoint_grad); a request whose footprint only fits the whole budget
+ * without that buffer runs without it, slower and equal up to rounding. */
 typedef struct {
   uint64_t hbm_budget_bytes;
   int32_t max_active_small;

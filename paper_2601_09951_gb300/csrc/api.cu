@@ -74,6 +74,7 @@ struct sv_ctx {
   // whole-state diagonal + permutation segments (k_dp.cu) need a third state buffer
   double2* scratch = nullptr;
   bool scratch_failed = false;
+  bool two_states = false;    // (ctx_two_states) use psi and lambda only
   enum { CH_PASSES = 0, CH_LAYER = 1, CH_DP = 2, CH_PROD = 3 };
   struct Chunk {
     int kind;
@@ -600,7 +601,8 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
   c->chunks.clear();
   if (c->n >= kFusedMinQubits && n_ops > 0) {
     // commuting layers that get a psi checkpoint: as many as the budget (and the device) allow
-    const int n_prod = from_ref ? product_prefix(hc) : 0;
+    const int n_prod =
+        from_ref && (!c->two_states || prod_in_psi(c->n)) ? product_prefix(hc) : 0;
     std::vector<std::pair<int, int>> layers = commuting_layers(hc.ops, 2);
     layers.erase(std::remove_if(layers.begin(), layers.end(),
                                 [&](const std::pair<int, int>& l) { return l.first < n_prod; }),
@@ -620,14 +622,14 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
     std::vector<int> layer_at(n_ops, -1);
     for (size_t j = 0; j < layers.size(); ++j) layer_at[layers[j].first] = (int)j;
     // diagonal + permutation runs need the third buffer
-    if (c->n >= kDpMinQubits && !c->scratch && !c->scratch_failed) {
+    if (c->n >= kDpMinQubits && !c->two_states && !c->scratch && !c->scratch_failed) {
       if (cudaMalloc((void**)&c->scratch, sb) != cudaSuccess) {
         cudaGetLastError();
         c->scratch = nullptr;
         c->scratch_failed = true;
       }
     }
-    const bool use_dp = c->scratch != nullptr && c->n >= kDpMinQubits;
+    const bool use_dp = c->scratch != nullptr && !c->two_states && c->n >= kDpMinQubits;
     auto is_diag = [&](int t) { return t == SV_GATE_RZ || t == SV_GATE_CZ; };
     auto is_perm = [&](int t) { return t == SV_GATE_CNOT || t == SV_GATE_X; };
     // a run of RZ/CZ (at most kDpMaxRz / kDpMaxCz) then at least two CNOT/X gates, from l
@@ -1371,6 +1373,32 @@ sv_status svqe::adjoint_fixed(const HostCircuit& hc, uint64_t ref, const DGroup*
 }
 
 cudaStream_t svqe::ctx_stream(sv_ctx* c) { return c->stream; }
+void svqe::ctx_two_states(sv_ctx* c, bool on) { c->two_states = on; }
+
+uint64_t svqe::ctx_request_bytes(const HostCircuit& hc, int32_t n_steps, bool two_states) {
+  const uint64_t G = hc.ops.size();
+  // (as grow does; a circuit of G ops has at most G items, passes and preparation units)
+  auto room = [](uint64_t count, uint64_t size) { return std::max<uint64_t>(count, 64) * size; };
+  uint64_t b = sv_ctx_device_bytes(hc.n);
+  b += room(G, sizeof(Rot)) + room(G, sizeof(double2)) + room(G, sizeof(SItem)) +
+       room(G, sizeof(double)) + room(G * (sizeof(DOp) + sizeof(FItem) + sizeof(PrepUnit)) + 512, 1) +
+       std::max<uint64_t>(1, G) * kRedBlocks * sizeof(double) +
+       2 * room((uint64_t)hc.n_params, sizeof(double)) +
+       room((uint64_t)std::max(1, n_steps), sizeof(double));
+  const bool prod = product_prefix(hc) > 0;
+  uint64_t tabs = prod && (!two_states || prod_in_psi(hc.n));
+  if (!two_states && hc.n >= kDpMinQubits) {
+    b += sv_state_bytes(hc.n);
+    if (prod && !prod_in_psi(hc.n)) b += room(prod_scratch(hc.n), sizeof(double));
+    // a segment ends with a run of two or more CNOT/X gates, and takes all of it
+    int run = 0;
+    for (const DOp& op : hc.ops) {
+      run = op.type == SV_GATE_CNOT || op.type == SV_GATE_X ? run + 1 : 0;
+      tabs += run == 2;
+    }
+  }
+  return b + (tabs ? room(tabs * kDpTab, sizeof(double2)) : 0);
+}
 
 sv_status vqe_step(sv_ctx* c, const sv_circuit* circ, const sv_ham* H, double* theta_inout,
                    double lr, int32_t n_steps, double* energy_out) {

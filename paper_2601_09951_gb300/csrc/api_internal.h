@@ -42,6 +42,12 @@ struct SmallPack {
 bool pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
                 const double* theta, SmallPack& out);
 cudaStream_t ctx_stream(sv_ctx* c);
+// Keep what is staged next to psi and lambda: no third state buffer, so no whole-state segments,
+// and the product prefix only where its scratch lies in psi.
+void ctx_two_states(sv_ctx* c, bool on);
+// Device bytes a context of hc.n > kSmallQubits qubits without checkpoints holds after a
+// vqe_enqueue of hc, at most.
+uint64_t ctx_request_bytes(const HostCircuit& hc, int32_t n_steps, bool two_states);
 // sv_adjoint_grad_dev's evaluation with every buffer in the caller's `bytes` of device memory at
 // mem (256-byte aligned), nothing allocated and nothing copied from pageable host memory.
 // SV_ENOMEM, with nothing enqueued, when the circuit needs more.

@@ -137,6 +137,7 @@ struct Req {
   size_t pin_cap = 0;
   cudaStream_t stream = nullptr;  // the context's stream (the server creates and destroys it)
   bool heavy = false;             // n >= heavy_qubits
+  bool two_states = false;        // the budget has no room for a third state buffer
 };
 
 // The device resources of a finished large request, kept for the next request of width n.
@@ -295,11 +296,9 @@ uint64_t small_footprint(const Req& r) {
 }
 
 uint64_t large_footprint(const Req& r) {
-  const uint64_t n_ops = r.hc.ops.size();
-  return sv_ctx_device_bytes(r.n) + (uint64_t)r.hh.groups.size() * sizeof(DGroup) +
-         (uint64_t)r.hh.tables.size() * sizeof(double2) +
-         n_ops * (sizeof(DOp) + sizeof(Rot) + 8 + (uint64_t)kRedBlocks * 8 + 2 * sizeof(FItem)) +
-         (uint64_t)r.hc.n_params * 16 + (uint64_t)r.steps * 8 + 4096;
+  return ctx_request_bytes(r.hc, r.steps, r.two_states) +
+         std::max<uint64_t>(r.hh.groups.size(), 64) * sizeof(DGroup) +
+         std::max<uint64_t>(r.hh.tables.size(), 64) * sizeof(double2);
 }
 
 void finish(sv_server* s, Req& r, int state, sv_status st, const char* msg) {
@@ -399,6 +398,7 @@ sv_status start_large(sv_server* s, Req& r) {
       return fail_cuda("request stream", e);
     if ((st = sv_create(&r.ctx, r.n, r.stream)) != SV_OK) return st;
   }
+  ctx_two_states(r.ctx, r.two_states);
   if ((st = sv_init_reference(r.ctx, r.ref)) != SV_OK) return st;
   sv_paulisum ps{r.n, (int32_t)r.hcoef.size(), r.hx.data(), r.hz.data(), r.hcoef.data()};
   if ((st = r.ham ? ham_reload(r.ctx, r.ham, &ps) : sv_ham_upload(r.ctx, &ps, &r.ham)) != SV_OK)
@@ -723,6 +723,10 @@ sv_status sv_server_submit(sv_server* s, const sv_instance* inst, const double* 
     r.hz.assign(inst->ham.z_mask, inst->ham.z_mask + inst->ham.n_terms);
     r.hcoef.assign(inst->ham.coeff, inst->ham.coeff + inst->ham.n_terms);
     r.footprint = large_footprint(r);
+    if (r.footprint > s->cfg.hbm_budget_bytes) {
+      r.two_states = true;
+      r.footprint = large_footprint(r);
+    }
   }
   if (r.footprint > s->cfg.hbm_budget_bytes) {
     set_error("request needs %llu device bytes, the server's budget is %llu",

@@ -184,3 +184,59 @@ def test_bench_stream_sampled_against_the_oracle():
     one.close()
     assert np.array_equal(out[big][0], th0) and np.array_equal(out[big][1], es0)
     assert_energy(out[big][1][0], oracle.energy(reqs[big]), reqs[big]["ham"], reqs[big]["name"])
+
+
+@pytest.mark.parametrize("n", [13, 14, 24])
+def test_footprint_covers_what_a_large_request_allocates(n):
+    """The footprint of a large request counts all three states, the records and partial sums of
+    every gate and, at 13 and 14 qubits, the scratch of the product prefix; at 24 qubits it is also
+    compared with the device memory that goes (the context stays, idle, when the request is
+    done).  48 MiB: a dozen allocations rounded up to 2 MiB, and the stream's own."""
+    torch = pytest.importorskip("torch")
+    req = W.hea_instance(n, 2, 40, 61)
+    srv = svqe.Server(hbm_budget_bytes=2 << 30)
+    # (a request of the batched path first: the libraries load their kernels on first use)
+    small = W.hea_instance(5, 1, 10, 62)
+    srv.wait(srv.submit(small, 1, 0.1), 60000)
+    svqe.Context(n).apply_circuit(req["circuit"], req["theta"])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    _, _, info = srv.wait(srv.submit(req, 1, 0.01), 60000)
+    taken = before - torch.cuda.mem_get_info()[0]
+    srv.close()
+    gates = len(req["circuit"]["types"])
+    counted = 3 * (16 << n) + gates * 1216 * 8 + {13: 167936, 14: 335872}.get(n, 0)
+    counted += 16 * len(svqe.group_records(req["ham"], n)[1])
+    assert counted <= info.footprint_bytes <= counted + gates * 512 + (100 << 10)
+    if n == 24:
+        assert taken <= info.footprint_bytes + (48 << 20)
+
+
+@pytest.mark.parametrize("n", [13, 16])
+def test_a_budget_without_room_for_a_third_state(n):
+    """A request that fits the budget with two states only runs with two: same results up to
+    rounding, alone and on a context that an earlier request left idle; without room for two it is
+    refused."""
+    req = W.hea_instance(n, 2, 40, 63)
+    out = []
+    srv = svqe.Server(serial=True)
+    th, es, info = srv.wait(srv.submit(req, 3, 0.02), 60000)
+    srv.close()
+    budget = int(info.footprint_bytes) - 1
+    srv = svqe.Server(serial=True, hbm_budget_bytes=budget)
+    for _ in range(2):
+        th2, es2, info2 = srv.wait(srv.submit(req, 3, 0.02), 60000)
+        assert info2.status == 0 and info2.footprint_bytes <= info.footprint_bytes - (16 << n)
+        out.append((th2, es2))
+        for a, b in zip(es2, es):
+            assert_energy(a, b, req["ham"])
+        assert_grad((np.asarray(req["theta"]) - th2) / 0.02, (np.asarray(req["theta"]) - th) / 0.02,
+                    req["ham"])
+    assert srv.stats().peak_bytes_in_use <= budget
+    srv.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    srv = svqe.Server(serial=True, hbm_budget_bytes=2 * (16 << n))
+    with pytest.raises(svqe.SvError) as e:
+        srv.submit(req, 3, 0.02)
+    assert e.value.status == svqe.SV_ENOMEM
+    srv.close()
