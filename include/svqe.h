@@ -140,16 +140,19 @@ sv_status sv_destroy(sv_ctx* ctx);
  * handle. */
 sv_status sv_set_checkpoint_bytes(sv_ctx* ctx, uint64_t bytes);
 /* Autotuning of the fused-pass tile size; off by default
- * (tiles of 2^11 amplitudes; below 18 qubits smaller ones where they are estimated faster).  When on, the first sv_adjoint_grad* / vqe_step call with a
- * circuit structure not seen before in the process does the following.  Gate types and wires
- * count as structure; angles do not.  It times the forward pass with tiles of 2^9, 2^10 and
+ * (tiles of 2^11 amplitudes; below 18 qubits smaller ones where they are estimated faster, also
+ * instead of the tuned size).  When on, the first sv_adjoint_grad* / vqe_step call with a
+ * circuit structure not seen before in the process does the following, unless it runs in one
+ * launch (up to 10 qubits, see sv_adjoint_grad): there are no passes to tune then.  Gate types
+ * and wires count as structure; angles do not.  It times the forward pass with tiles of 2^9, 2^10 and
  * 2^11 amplitudes and keeps the fastest.  That call therefore runs three candidates' forward
  * passes on psi (twice each), which holds |ref> again afterwards.  Results are shared by every context of the
  * process.  If the environment variable SVQE_TUNE_CACHE names a file, results are read from
  * and appended to it as "n key bits" lines.  SV_EINVAL for a NULL handle. */
 sv_status sv_set_autotune(sv_ctx* ctx, int32_t enable);
 /* Tile size (bits) of the fused passes of the last circuit staged on the context: the largest
- * it was planned with (passes of a register below 18 qubits may use smaller tiles). */
+ * it was planned with (passes of a register below 18 qubits may use smaller tiles); 11 after a
+ * call that ran in one launch. */
 sv_status sv_tile_bits(const sv_ctx* ctx, int32_t* tile_bits);
 
 /* ---------------------------------------------------------------- Hamiltonians */

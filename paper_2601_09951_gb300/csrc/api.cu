@@ -1099,6 +1099,7 @@ static sv_status grow_pinned(sv_ctx* c, size_t need) {
 static sv_status run_small(sv_ctx* c, SmallPack& S, const sv_ham* H, double* energy, double* grad,
                            int n_steps, double lr, double* etraj) {
   SmallArgs& A = S.args;
+  c->tile_bits = fused_tile_bits();  // (no passes: not those of an earlier circuit)
   SV_CUDA(grow(c->ckpt, c->ckpt_cap, (size_t)S.ckpt_amps), c);
   if (!S.blob.empty()) {
     SV_CUDA(grow(c->blob, c->blob_cap, S.blob.size()), c);

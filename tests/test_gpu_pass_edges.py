@@ -4,6 +4,10 @@ of the tile
 rule (tiles of n - 7 bits below 18 qubits), angles on both sides of the quarter turns where the
 unnormalised rotations change form, RY and RX gates that share a trip or repeat a qubit, and
 passes of more items than are staged at a time.  Tolerances as in tests/parity.py."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -272,3 +276,44 @@ def test_tuner_leaves_the_reference_state(first):
     assert np.max(np.abs(ctx.get_state() - ref)) <= PSI_TOL
     ctx.apply_circuit(circ, theta)
     assert np.max(np.abs(ctx.get_state() - oracle.state(circ, theta, 5))) <= PSI_TOL
+
+
+def test_tile_bits_after_a_call_in_one_launch(tmp_path):
+    """Up to 10 qubits a circuit whose records fit one launch has no passes: the tuner does not run
+    for it, and its tile size reads 11, not that of the last circuit that had passes (here one of
+    2200 gates, for which the tuner's cache file names tiles of 2^9)."""
+    code = """
+import sys
+import numpy as np
+from paper_2601_09951_gb300 import svqe, workloads as W
+n = 8
+big = W.CircuitBuilder(n)
+for i in range(2200):
+    big.add(W.RY, (i % n,), angle=0.1 * i)
+small = W.tfim_instance(n, 1)
+ctx = svqe.Context(n)
+ctx.set_autotune(True)
+H = svqe.Ham(ctx, small["ham"])
+out = []
+for circ, theta in ((big.build(), np.zeros(0)), (small["circuit"], small["theta"])):
+    ctx.adjoint_grad(circ, theta, H)
+    out.append(ctx.tile_bits())
+    ctx.vqe_step(circ, H, theta, 0.1, 2)
+    out.append(ctx.tile_bits())
+print("bits", *out)
+"""
+    cache = tmp_path / "tune.txt"
+    env = dict(os.environ, SVQE_TUNE_CACHE=str(cache))
+
+    def bits():
+        run = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True,
+                             timeout=300, cwd=os.path.dirname(os.path.dirname(__file__)))
+        assert run.returncode == 0, run.stderr
+        return [int(b) for b in run.stdout.split("bits")[1].split()]
+
+    first = bits()
+    assert first[0] == first[1] and first[2:] == [11, 11]
+    lines = cache.read_text().split()
+    assert len(lines) == 3 and lines[0] == "8"  # one structure tuned: the large circuit's
+    cache.write_text(f"8 {lines[1]} 9\n")
+    assert bits() == [9, 9, 11, 11]
