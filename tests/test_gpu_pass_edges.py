@@ -1,9 +1,10 @@
 """GPU parity of the single-state path at the edges of its rules: registers on both sides of the
 one-block limit (10 qubits; records that fit the launch's arguments and records that do not) and
-of the tile
-rule (tiles of n - 7 bits below 18 qubits), angles on both sides of the quarter turns where the
-unnormalised rotations change form, RY and RX gates that share a trip or repeat a qubit, and
-passes of more items than are staged at a time.  Tolerances as in tests/parity.py."""
+of the tile rule (tiles of n - 7 bits below 18 qubits), angles on both sides of the quarter turns
+where the unnormalised rotations change form, RY and RX gates that share a trip or repeat a qubit,
+forward passes of more items than are staged at a time, runs of more rotations than a pass takes,
+and the tile tuner's effect on psi and on the reported tile size.  (Backward passes of many items:
+test_gpu_pass_limits.py.)  Tolerances as in tests/parity.py."""
 import os
 import subprocess
 import sys
