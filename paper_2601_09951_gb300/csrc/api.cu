@@ -66,7 +66,7 @@ struct sv_ctx {
   size_t theta_cap = 0, grad_cap = 0;
   double* etraj = nullptr;
   size_t etraj_cap = 0;
-  HostPlan plan;              // fused passes of the staged circuit (empty: per-op kernels)
+  HostPlan plan;              // fused passes of the staged circuit
   // psi checkpoints of commuting layers (sv_set_checkpoint_bytes): the staged circuit's fused
   // passes are planned in chunks, each either a checkpointed layer or a run of other ops
   uint64_t ck_budget = 0;
@@ -494,7 +494,7 @@ sv_status svqe::stage_circuit(sv_ctx* c, const HostCircuit& hc, bool may_tune, b
     SV_CUDA(grow(c->grad, c->grad_cap, (size_t)hc.n_params), c);
   }
   int m = fused_tile_bits();
-  if (may_tune && c->tune && c->n >= kFusedMinQubits && n_ops > 0) m = tune_tile_bits(c, hc);
+  if (may_tune && c->tune && n_ops > 0) m = tune_tile_bits(c, hc);
   if (m <= 0) return SV_ECUDA;
   return plan_circuit(c, hc, m, from_ref);
 }
@@ -599,7 +599,7 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
   c->plan.passes.clear();
   c->plan.items.clear();
   c->chunks.clear();
-  if (c->n >= kFusedMinQubits && n_ops > 0) {
+  if (n_ops > 0) {
     // commuting layers that get a psi checkpoint: as many as the budget (and the device) allow
     const int n_prod =
         from_ref && (!c->two_states || prod_in_psi(c->n)) ? product_prefix(hc) : 0;
@@ -861,7 +861,6 @@ static double2* free_buffer(sv_ctx* c, const double2* a, const double2* b) {
 // into the checkpoint of every checkpointed layer before the layer runs.
 static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_dev, bool save,
                          double2** psi_out) {
-  const int n_ops = (int)hc.ops.size();
   *psi_out = c->psi;
   SV_CUDA(launch_prep(c->units, c->n_units, c->ops, c->items, theta_dev, c->n, c->ref, c->coef,
                       c->sitems, c->scales, c->cs, c->dptab, c->stream), c);
@@ -898,8 +897,6 @@ static sv_status forward(sv_ctx* c, const HostCircuit& hc, const double* theta_d
     *psi_out = psi;
     return SV_OK;
   }
-  for (int l = 0; l < n_ops; ++l)
-    SV_CUDA(launch_apply_op(c->psi, c->n, hc.ops[l], c->coef + l, false, c->stream), c);
   return SV_OK;
 }
 
@@ -1187,12 +1184,6 @@ sv_status svqe::adjoint_core(sv_ctx* c, const HostCircuit& hc, const sv_ham* H,
     else if (psi != c->psi)
       SV_CUDA(cudaMemcpyAsync(c->psi, psi, sv_state_bytes(c->n), cudaMemcpyDeviceToDevice,
                               c->stream), c);
-  } else {
-    for (int l = n_ops - 1; l >= 0; --l) {
-      const DOp& op = hc.ops[l];
-      double* part = op.param >= 0 ? c->gpart + (size_t)l * kRedBlocks : nullptr;
-      SV_CUDA(launch_adjoint_op(c->psi, c->lam, c->n, op, c->coef + l, part, c->stream), c);
-    }
   }
   SV_CUDA(launch_finish(c->ops, n_ops, c->gpart, hc.n_params, grad_dev, c->epart, hpsi_blocks(c->n),
                         energy_dev, theta_upd, lr, traj, c->stream, c->fixed || !prod), c);
@@ -1483,9 +1474,7 @@ static double thread_time(const BInst& B, int cls) {
   return per_thread * (6.0 * B.n_ops + 2.0 * B.n_groups + 8.0) + 150.0 * B.n_ops;
 }
 
-std::vector<BItem> svqe::batch_items(const std::vector<BInst>& bi,
-                                     const std::vector<double>& cost_in, const int* cls_of_n) {
-  (void)cost_in;
+std::vector<BItem> svqe::batch_items(const std::vector<BInst>& bi, const int* cls_of_n) {
   const int n = (int)bi.size();
   std::vector<int> cls(n);
   std::vector<double> cost(n);
@@ -1639,7 +1628,6 @@ static sv_status batch_build(const sv_instance* inst, int32_t n, void* stream,
   std::vector<double2> tables;
   std::vector<Seg> segs;
   std::vector<int32_t> pptr, pops;
-  std::vector<double> cost(n);
   double flops = 0.0, bytes = 0.0;
   int nmax = 1;
   int64_t theta_off = 0, ckpt_slot = 1;
@@ -1707,7 +1695,6 @@ static sv_status batch_build(const sv_instance* inst, int32_t n, void* stream,
     tables.insert(tables.end(), hh.tables.begin(), hh.tables.end());
     ops.insert(ops.end(), hc.ops.begin(), hc.ops.end());
     nmax = std::max(nmax, hc.n);
-    cost[i] = inst_flops + 64.0 * B.n_ops + 1.0;  // per-op latency matters for tiny states
   }
   sv_batch* b = new (std::nothrow) sv_batch();
   if (!b) { set_error("host allocation failed"); return SV_ENOMEM; }
@@ -1725,7 +1712,7 @@ static sv_status batch_build(const sv_instance* inst, int32_t n, void* stream,
     if (e != cudaSuccess) { set_error("cudaStreamCreate: %s", cudaGetErrorString(e)); delete b; return SV_ECUDA; }
     b->own_stream = true;
   }
-  const std::vector<BItem> items = batch_items(bi, cost, cls_of_n);
+  const std::vector<BItem> items = batch_items(bi, cls_of_n);
   b->n_items = (int)items.size();
   for (int q = 0; q <= SV_BATCH_MAX_QUBITS; ++q) b->lay[q] = BLayout{-1, 0, 0};
   for (int i = 0; i < n; ++i) b->lay[bi[i].n] = lay[bi[i].n];

@@ -77,12 +77,11 @@ struct BLayout {
 BLayout default_layout(int n);
 
 // Batched-kernel helpers: team class of an n-qubit instance under the fixed rule, teams per CTA
-// of that class, work items from per-instance costs (cls_of_n: team class per qubit count, or
+// of that class, work items, costliest first (cls_of_n: team class per qubit count, or
 // nullptr for the fixed rule), and the FP64 flop count of one instance.
 int batch_class(int n);
 int class_teams(int n);
-std::vector<BItem> batch_items(const std::vector<BInst>& bi, const std::vector<double>& cost,
-                               const int* cls_of_n = nullptr);
+std::vector<BItem> batch_items(const std::vector<BInst>& bi, const int* cls_of_n = nullptr);
 double batch_instance_flops(const HostCircuit& hc, const HostHam& hh,
                             const std::vector<Seg>& segs);
 

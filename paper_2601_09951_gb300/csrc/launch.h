@@ -85,10 +85,9 @@ cudaError_t launch_finish(const DOp* ops, int n_ops, const double* partial, int 
 namespace svqe {
 
 // Fused passes of the single-state path (k_fused.cu).  Tiles of fused_tile_bits() bits (all
-// of the state when it is smaller); used for registers of at least kFusedMinQubits qubits.
+// of the state when it is smaller).
 // Whole-state diagonal + permutation segments (k_dp.cu) are used from kDpMinQubits: below,
 // a layer's RZ and CNOT gates fit one fused pass or two.
-constexpr int kFusedMinQubits = 1;
 constexpr int kDpMinQubits = 11;
 int fused_tile_bits();
 cudaError_t fused_prepare();

@@ -117,7 +117,6 @@ struct Req {
   std::vector<double> hcoef;
   std::vector<Seg> segs;
   int n_ckpt = 0;
-  double cost = 0.0;
   std::vector<double> theta, etraj;
   uint64_t footprint = 0;
   int state = Q_QUEUED;
@@ -554,7 +553,6 @@ void worker_loop(sv_server* s) {
       }
       if (!tick_reqs.empty()) {
         std::vector<BInst> bi;
-        std::vector<double> cost;
         for (auto& rp : tick_reqs) {
           Req& r = *rp;
           const int k = std::min(s->cfg.steps_per_tick, r.steps - r.done_steps);
@@ -563,9 +561,8 @@ void worker_loop(sv_server* s) {
           B.steps = k;
           B.etraj_off = r.etraj_elem + r.done_steps;
           bi.push_back(B);
-          cost.push_back(r.cost * k);
         }
-        const std::vector<BItem> items = batch_items(bi, cost);
+        const std::vector<BItem> items = batch_items(bi);
         std::memcpy(s->h_inst, bi.data(), bi.size() * sizeof(BInst));
         std::memcpy(s->h_items, items.data(), items.size() * sizeof(BItem));
         BatchArgs a{};
@@ -716,7 +713,6 @@ sv_status sv_server_submit(sv_server* s, const sv_instance* inst, const double* 
                 "scratch holds", r.n_ckpt, r.n);
       return SV_EINVAL;
     }
-    r.cost = batch_instance_flops(r.hc, r.hh, r.segs) + 64.0 * r.hc.ops.size() + 1.0;
     r.footprint = small_footprint(r);
   } else {
     r.hx.assign(inst->ham.x_mask, inst->ham.x_mask + inst->ham.n_terms);
