@@ -304,9 +304,7 @@ HBM_PEAK_GBS = 6678.2  # measured copy bandwidth (read + write) of a GB300
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_batch launch of the default workload,
 # from one ncu capture of that launch, keyed by a hash of the kernel's sources: once the
 # kernel changes the key no longer matches and traffic is null.
-# (The second key differs from the first by a comment in svqe_types.h.)
-KBATCH_TRAFFIC = {"ea31bb0808c4b826": 338.64e6 + 470.35e6,
-                  "4c6a29bd7dbf863d": 338.64e6 + 470.35e6}
+KBATCH_TRAFFIC = {"722a89cb4a4cedd7": 339.67e6 + 470.91e6}
 KBATCH_SOURCES = ("k_batch.cu", "svqe_internal.cuh", "svqe_types.h", "launch.h")
 
 

@@ -112,9 +112,10 @@ int32_t sv_abi_version(void);
 /* Bytes of one n-qubit complex128 state, 2^n * 16 (Table 3); 0 if n is outside [0, 62]. */
 uint64_t sv_state_bytes(int32_t n_qubits);
 /* Device bytes a context of n qubits allocates when it is created: two state buffers (psi,
- * lambda) plus reduction scratch.  Circuits with whole-state segments or a product prefix (from
- * 11 qubits, see sv_adjoint_grad) add a third state-sized buffer when first staged, and every
- * circuit its own records and partial sums (about 10 KB per gate).  Unless checkpoints are
+ * lambda) plus reduction scratch.  From 11 qubits the first circuit staged adds a third
+ * state-sized buffer for whole-state segments (see sv_adjoint_grad; below 15 qubits a product
+ * prefix adds up to 328 KiB of its own), and every circuit its records and partial sums (about
+ * 10 KB per gate).  Unless checkpoints are
  * enabled (sv_set_checkpoint_bytes), at most three state-sized buffers are ever used (31 qubits
  * fit). */
 uint64_t sv_ctx_device_bytes(int32_t n_qubits);
@@ -222,10 +223,10 @@ sv_status sv_expval_paulisum(sv_ctx* ctx, const sv_ham* h, double* energy_out);
  * call reaches the same gradient by the adjoint method.  Forward pass, lambda = H psi, then the adjoint sweep
  * over gates in reverse: g_p += 2 Im<lambda|G_l|psi> for each gate l with parameter p, then
  * psi <- U_l^dag psi and lambda <- U_l^dag lambda.  Up to 10 qubits one launch evaluates the
- * whole circuit in shared memory (with at most 8 MiB of checkpoints).  From 11 qubits, runs of
- * RZ/CZ followed by CNOT/X gates are whole-state segments, and the circuit's leading one-qubit
- * gates on |ref> a product state; both use a third state buffer beside psi and lambda, and the
- * call falls back to two where it cannot be had.  Layer checkpoints: sv_set_checkpoint_bytes.
+ * whole circuit in shared memory (with at most 8 MiB of checkpoints).  From 11 qubits, the
+ * circuit's leading one-qubit gates on |ref> are a product state, and runs of RZ/CZ followed by
+ * CNOT/X gates whole-state segments; segments need a third state buffer beside psi and lambda,
+ * and where it cannot be had their gates run in passes on the two.  Layer checkpoints: sv_set_checkpoint_bytes.
  * psi holds |ref> again afterwards.  energy_out:
  * host double; grad_out: host array of n_params (gates sharing a parameter are summed). */
 sv_status sv_adjoint_grad(sv_ctx* ctx, const sv_circuit* circuit, const double* theta,

@@ -1,12 +1,14 @@
 // svqe_internal.cuh -- types and device arithmetic shared by the CUDA translation units.
 //
-// Design rule for GB300: FP64 issue rate is ~2 DFMA/clk/SM (measured 598 G DFMA/s on the
+// Design rule for GB300: FP64 issue rate is 2 DFMA/clk/SM (measured 628 G DFMA/s on the
 // whole chip) against ~64 integer and ~110 FP32 lane-ops/clk/SM.  Every kernel here is
 // therefore written to minimise FP64 instructions per amplitude:
 //   * sign flips and multiplications by +-1, +-i are integer bit operations or swaps;
-//   * a real 2x2 rotation is applied as three shears ("lifting", x += a*y; y += b*x;
-//     x += a*y), 3 DFMA per real pair instead of 2 DMUL + 2 DFMA, after reducing the angle
-//     to [-pi/4, pi/4] with an exact quarter-turn (a swap and sign flips);
+//   * the RY and RX gates of fused passes and commuting layers run without their normalisation
+//     (RotT, 2 DFMA per real pair), the product of the factors left out applied once;
+//   * any other real 2x2 rotation (a gate on its own, excitations) is three shears ("lifting",
+//     Rot: x += a*y; y += b*x; x += a*y), 3 DFMA per real pair instead of 2 DMUL + 2 DFMA, after
+//     reducing the angle to [-pi/4, pi/4] with an exact quarter-turn (a swap and sign flips);
 //   * Pauli groups are applied through tabulated f_g(i), one complex or real multiply-add
 //     per amplitude per group whatever the number of terms in the group.
 #pragma once
