@@ -223,7 +223,8 @@ sv_status sv_expval_paulisum(sv_ctx* ctx, const sv_ham* h, double* energy_out);
  * call reaches the same gradient by the adjoint method.  Forward pass, lambda = H psi, then the adjoint sweep
  * over gates in reverse: g_p += 2 Im<lambda|G_l|psi> for each gate l with parameter p, then
  * psi <- U_l^dag psi and lambda <- U_l^dag lambda.  Up to 10 qubits one launch evaluates the
- * whole circuit in shared memory (with at most 8 MiB of checkpoints).  From 11 qubits, the
+ * whole circuit in shared memory (with at most 8 MiB of checkpoints), unless the Hamiltonian has
+ * so many groups that one SM takes longer for them than the passes do.  From 11 qubits, the
  * circuit's leading one-qubit gates on |ref> are a product state, and runs of RZ/CZ followed by
  * CNOT/X gates whole-state segments; segments need a third state buffer beside psi and lambda,
  * and where it cannot be had their gates run in passes on the two.  Layer checkpoints: sv_set_checkpoint_bytes.

@@ -100,7 +100,8 @@ struct sv_ham {
   int n_groups = 0;
   DGroup* groups = nullptr;
   double2* tables = nullptr;
-  int n_table = 0;  // table entries
+  int n_table = 0;    // table entries
+  int n_complex = 0;  // groups with a complex table
   size_t groups_cap = 0, tables_cap = 0;  // allocated records / table entries
   uint64_t bytes = 0;
   double l1 = 0.0;
@@ -323,6 +324,8 @@ static sv_status ham_fill(sv_ctx* c, sv_ham* H, const sv_paulisum* h) {
   H->device = c->device;
   H->n_groups = (int)hh.groups.size();
   H->n_table = (int)hh.tables.size();
+  H->n_complex = 0;
+  for (const DGroup& g : hh.groups) H->n_complex += g.cls == 2;
   H->l1 = hh.l1;
   H->bytes = H->groups_cap * sizeof(DGroup) + H->tables_cap * sizeof(double2);
   if (!hh.groups.empty())
@@ -1011,6 +1014,21 @@ sv_status sv_tile_bits(const sv_ctx* c, int32_t* tile_bits) {
 
 static constexpr int64_t kSmallCkptAmps = 1 << 19;  // 8 MiB of checkpoint scratch at most
 
+// One block forms lambda = H psi with one SM's FP64 pipe and one group after another: (N + 200)
+// clocks for a group with a real or imaginary factor, 3.6 N or at least 2,300 for a complex table;
+// k_hpsi splits the amplitudes and the groups over 32 SMs and takes 100 to 200 clocks a group.
+// What one launch saves over the passes is 35 us and 0.6 us per gate (8 to 10 qubits, layers and
+// excitations of 20 to 170 gates).  Either side at 10 qubits and two layers, one block against
+// passes: 122 groups 167 and 167 us, 216 (28 complex) 235 and 168, 1023 complex 1947 and 258; at 9
+// qubits 192 (38 complex) 153 and 158, 512 complex 709 and 196; at 8, 88 (17 complex) 100 and 135,
+// 256 complex 340 and 153.
+bool svqe::small_pays(const HostCircuit& hc, int n_groups, int n_complex) {
+  if (hc.n > kSmallQubits) return false;
+  const double N = (double)(1 << hc.n);
+  const double ham_us = (n_groups * (N + 100.0) + n_complex * (1.6 * N + 900.0)) / 2070.0;
+  return ham_us <= 35.0 + 0.6 * (double)hc.ops.size();
+}
+
 bool svqe::pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
                       const double* theta, SmallPack& out) {
   if (hc.n > SV_BATCH_MAX_QUBITS) return false;
@@ -1251,7 +1269,8 @@ sv_status sv_adjoint_grad_dev(sv_ctx* c, const sv_circuit* circ, const double* t
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && (!theta_dev || !grad_dev)) { set_error("theta/grad is NULL"); return SV_EINVAL; }
   SmallPack sp;
-  if (c->n <= kSmallQubits && pack_small(hc, c->ref, H->n_groups, H->n_table, nullptr, sp)) {
+  if (small_pays(hc, H->n_groups, H->n_complex) &&
+      pack_small(hc, c->ref, H->n_groups, H->n_table, nullptr, sp)) {
     sp.args.a.theta = const_cast<double*>(theta_dev);
     return run_small(c, sp, H, energy_dev, grad_dev, 0, 0.0, nullptr);
   }
@@ -1270,7 +1289,7 @@ sv_status sv_adjoint_grad(sv_ctx* c, const sv_circuit* circ, const double* theta
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && (!theta || !grad_out)) { set_error("theta/grad is NULL"); return SV_EINVAL; }
   SmallPack sp;
-  if (c->n <= kSmallQubits &&
+  if (small_pays(hc, H->n_groups, H->n_complex) &&
       pack_small(hc, c->ref, H->n_groups, H->n_table, hc.n_params ? theta : nullptr, sp)) {
     if ((st = grow_pinned(c, (size_t)hc.n_params + 1)) != SV_OK) return st;
     if ((st = run_small(c, sp, H, c->pin, c->pin + 1, 0, 0.0, nullptr)) != SV_OK) return st;
@@ -1404,7 +1423,7 @@ sv_status vqe_step(sv_ctx* c, const sv_circuit* circ, const sv_ham* H, double* t
   if (st != SV_OK) return st;
   if (hc.n_params > 0 && !theta_inout) { set_error("theta is NULL"); return SV_EINVAL; }
   SmallPack sp;
-  if (n_steps > 0 && c->n <= kSmallQubits &&
+  if (n_steps > 0 && small_pays(hc, H->n_groups, H->n_complex) &&
       pack_small(hc, c->ref, H->n_groups, H->n_table, hc.n_params ? theta_inout : nullptr, sp)) {
     // theta moves in shared memory from step to step; it and the energies come back pinned
     const size_t P = (size_t)hc.n_params;

@@ -41,6 +41,9 @@ struct SmallPack {
 };
 bool pack_small(const HostCircuit& hc, uint64_t ref, int n_groups, int n_table,
                 const double* theta, SmallPack& out);
+// Whether one block is the faster way for this circuit and a Hamiltonian of n_groups X masks, of
+// which n_complex have complex tables: up to kSmallQubits qubits and not too many groups.
+bool small_pays(const HostCircuit& hc, int n_groups, int n_complex);
 cudaStream_t ctx_stream(sv_ctx* c);
 // Keep what is staged next to psi and lambda: no third state buffer, so no whole-state segments,
 // and the product prefix only where its scratch lies in psi.

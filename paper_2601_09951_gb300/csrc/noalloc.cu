@@ -250,16 +250,17 @@ extern "C" sv_status sv_adjoint_grad_noalloc(const sv_circuit* circuit, uint64_t
     NA_CUDA(cudaGetLastError());
     return SV_OK;
   };
-  // From kSmallQubits + 1 qubits: the passes of the ordinary path, in the array.  A circuit whose
-  // tables do not fit it goes on below.
-  if (n > kSmallQubits) {
+  // Where one block does not pay: the passes of the ordinary path, in the array.  A circuit whose
+  // tables do not fit it goes on below.  (The groups' classes are on the device: none is counted as
+  // complex, so that a little fewer calls leave the one block than in sv_adjoint_grad.)
+  if (!small_pays(hc, n_groups, 0)) {
     st = adjoint_fixed(hc, ref, groups, n_groups, (const double2*)tables_dev, theta_dev, energy_dev,
                        grad_dev, base, off_groups, s);
     if (st == SV_OK) return poison();
     if (st != SV_ENOMEM) return st;
     clear_error();
   }
-  // Small registers (and, failing the above, up to 12 qubits) run in one launch (k_small), its
+  // Small registers (and, failing the above, up to 12 qubits) in one launch (k_small), its
   // checkpoints and records in the array.
   SmallPack sp;
   const int n_pref = (int)std::min<int64_t>(n_table, 1 << 20);

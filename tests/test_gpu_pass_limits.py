@@ -152,3 +152,39 @@ def test_contexts_on_streams_of_their_own():
             e, g = oracle.energy_grad_subset(inst, [0, 1])
             assert_energy(out[0, 0], e, inst["ham"])
             assert_grad(out[0, 1:3], [g[0], g[1]], inst["ham"])
+
+
+@pytest.mark.parametrize("n,terms,p_zonly", [(6, 3000, 0.2), (7, 700, 0.0), (8, 300, 0.3),
+                                             (9, 260, 0.2), (9, 2000, 0.0), (10, 60, 0.5),
+                                             (10, 300, 0.5), (10, 3000, 0.0)])
+@pytest.mark.parametrize("layers", [1, 4])
+def test_hamiltonians_on_both_sides_of_the_one_block_limit(n, terms, p_zonly, layers):
+    """Up to 10 qubits a circuit runs in one block unless the Hamiltonian's groups take one SM
+    longer than the passes' launches: energy, gradient, a descent step and the call without device
+    allocation on either side, against the oracle and one another."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n * terms + layers)
+    inst = W.hea_instance(n, layers, 4, 80 + n)
+    circ, theta = inst["circuit"], np.asarray(inst["theta"])
+    ham = W.random_pauli_sum(rng, n, terms, p_zonly, n, 1.0)
+    ctx = svqe.Context(n)
+    ctx.init_reference(inst["ref"])
+    H = svqe.Ham(ctx, ham)
+    e, g = ctx.adjoint_grad(circ, theta, H)
+    which = [0, len(theta) // 2, len(theta) - 1]
+    e0, part = oracle.energy_grad_subset(dict(inst, ham=ham), which)
+    assert_energy(e, e0, ham)
+    assert_grad(g[which], [part[p] for p in which], ham)
+    th, es = ctx.vqe_step(circ, H, theta, 0.01, 2)
+    assert_energy(es[0], e, ham)
+    assert_energy(es[1], ctx.adjoint_grad(circ, theta - 0.01 * g, H)[0], ham)
+    rec, table = svqe.group_records(ham, n)
+    bufs = [torch.as_tensor(a).cuda() for a in (rec.view(np.uint8).reshape(-1),
+                                                table.view(np.float64), theta)]
+    out = torch.zeros(len(theta) + 1, dtype=torch.float64, device="cuda")
+    svqe.adjoint_grad_noalloc(circ, inst["ref"], n, bufs[0].data_ptr(), len(rec),
+                              bufs[1].data_ptr(), len(table), bufs[2].data_ptr(), out.data_ptr(),
+                              out[1:].data_ptr(), torch.cuda.current_stream().cuda_stream)
+    out = out.cpu().numpy()
+    assert_energy(out[0], e, ham)
+    assert_grad(out[1:], g, ham)
