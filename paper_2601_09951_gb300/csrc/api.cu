@@ -794,12 +794,12 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
       while (split < ch.count && (hc.ops[ch.first + split].type == SV_GATE_RZ ||
                                   hc.ops[ch.first + split].type == SV_GATE_CZ))
         ++split;
-      units.push_back(PrepUnit{PREP_DP, ch.first, split, n_dp++, cf, cl});
+      units.push_back(PrepUnit{PREP_DP, ch.first, split, n_dp++, cf, cl, -1});
       cf = cl = 0;
       continue;
     }
     if (ch.kind == sv_ctx::CH_PROD) {
-      units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++, 0, 0});
+      units.push_back(PrepUnit{PREP_PROD, 0, ch.ck, n_dp++, 0, 0, -1});
       if (!prod_in_psi(c->n)) SV_ROOM(prod, prod_cap, prod_scratch(c->n));
       continue;
     }
@@ -808,9 +808,12 @@ static sv_status plan_circuit(sv_ctx* c, const HostCircuit& hc, int tile_bits, b
       cf = c->plan.passes[ch.p0].first_item;
       cl = c->plan.passes[ch.p1 - 1].first_item + c->plan.passes[ch.p1 - 1].n_items;
     }
-    for (int p = ch.p0; p < ch.p1; ++p)
-      units.push_back(PrepUnit{PREP_PASS, c->plan.passes[p].first_item,
-                               c->plan.passes[p].n_items, p, cf, cl});
+    for (int p = ch.p0; p < ch.p1; ++p) {
+      const int op = ch.kind == sv_ctx::CH_PASSES ? single_op(c, p) : -1;
+      const FPass& P = c->plan.passes[p];
+      units.push_back(op >= 0 ? PrepUnit{PREP_COEF, op, 1, p, 0, 0, -1}
+                              : PrepUnit{PREP_PASS, P.first_item, P.n_items, p, cf, cl, P.diag});
+    }
   }
   auto align = [](size_t v) { return (v + 255) / 256 * 256; };
   const size_t o_items = align(n_ops * sizeof(DOp));

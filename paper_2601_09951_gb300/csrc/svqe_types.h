@@ -160,12 +160,14 @@ static_assert(sizeof(SItem) == 56, "SItem layout");
 // the same SItem places, its scale to place idx), a whole-state segment (RZ/CZ ops [first, first
 // + count), its phase tables to table idx) or the product prefix (ops [0, count), its tables and
 // qubit states to table idx).  A pass and the segment that takes its chunk's scale (folded) have
-// the chunk's items as [cf, cl); otherwise cf = cl.
-enum { PREP_PASS = 0, PREP_DP = 1, PREP_PROD = 2 };
+// the chunk's items as [cf, cl); otherwise cf = cl.  A pass that runs as its one gate's own kernel
+// needs that op's (first) lifting coefficients only.  diag: the pass's diagonal item, or -1.
+enum { PREP_PASS = 0, PREP_DP = 1, PREP_PROD = 2, PREP_COEF = 3 };
 struct PrepUnit {
   int32_t kind;
   int32_t first, count, idx;
   int32_t cf, cl;
+  int32_t diag;
 };
 // Tables of a whole-state segment over 128 thread indices, a thread's 8 slots and three times 7
 // block-index bits, then the states of up to 32 qubits (product prefix) or, in the first entry, the

@@ -188,3 +188,33 @@ def test_hamiltonians_on_both_sides_of_the_one_block_limit(n, terms, p_zonly, la
     out = out.cpu().numpy()
     assert_energy(out[0], e, ham)
     assert_grad(out[1:], g, ham)
+
+
+def test_checkpointed_layer_with_a_pass_of_one_gate():
+    """A layer of ten gates above the two low bits that every tile holds: passes of nine gates and
+    of one, which runs as the gate's own kernel forward and as a pass in the sweep."""
+    n = 19
+    rng = np.random.default_rng(19)
+    cb = W.CircuitBuilder(n)
+    cb.add(W.CNOT, (0, n - 1))
+    for gate in (W.RY, W.RX):
+        for q in range(10):
+            cb.add(gate, (q,), param="new")
+        cb.add(W.CZ, (0, 5))
+    circ = cb.build()
+    n_pass, pog = svqe.circuit_plan({**circ, "types": circ["types"][1:11],
+                                     "wires": circ["wires"][1:11], "params": circ["params"][1:11],
+                                     "fixed": circ["fixed"][1:11]})
+    assert sorted(np.bincount(pog)) == [1, 9]
+    theta = rng.uniform(-7, 7, circ["n_params"])
+    ham = W.tfim_instance(n)["ham"]
+    inst = {"circuit": circ, "ham": ham, "ref": 77, "theta": theta}
+    which = [0, 8, 9, 10, 19]
+    e0, part = oracle.energy_grad_subset(inst, which)
+    for budget in (0, 2 * (16 << n)):
+        ctx = svqe.Context(n)
+        ctx.set_checkpoint_bytes(budget)
+        ctx.init_reference(77)
+        e, g = ctx.adjoint_grad(circ, theta, svqe.Ham(ctx, ham))
+        assert_energy(e, e0, ham)
+        assert_grad(g[which], [part[p] for p in which], ham)
