@@ -89,6 +89,7 @@ namespace svqe {
 // Whole-state diagonal + permutation segments (k_dp.cu) are used from kDpMinQubits: below,
 // a layer's RZ and CNOT gates fit one fused pass or two.
 constexpr int kDpMinQubits = 11;
+constexpr int kDpSmallQubits = 14, kDpMinGates = 8;  // (see plan_circuit)
 int fused_tile_bits();
 cudaError_t fused_prepare();
 // items, scale (the pass's place) and cs as launch_prep wrote them.

@@ -218,3 +218,31 @@ def test_checkpointed_layer_with_a_pass_of_one_gate():
         e, g = ctx.adjoint_grad(circ, theta, svqe.Ham(ctx, ham))
         assert_energy(e, e0, ham)
         assert_grad(g[which], [part[p] for p in which], ham)
+
+
+@pytest.mark.parametrize("n", [11, 13, 14])
+@pytest.mark.parametrize("n_diag,n_perm", [(0, 2), (5, 2), (6, 2), (0, 7), (0, 8), (6, 1)])
+def test_segments_of_the_fewest_gates(n, n_diag, n_perm):
+    """RZ/CZ and CNOT/X runs on both sides of the least gates a whole-state segment takes, between
+    layers that end up in passes."""
+    rng = np.random.default_rng(n + 10 * n_diag + n_perm)
+    cb = W.CircuitBuilder(n)
+    cb.add(W.CNOT, (0, 1))
+    for layer in range(3):
+        for q in range(0, n, 2):
+            cb.add((W.RY, W.RX)[layer % 2], (q,), param="new")
+        for j in range(n_diag):
+            if j % 3 == 2:
+                cb.add(W.CZ, (j, (j + 3) % n))
+            else:
+                cb.add(W.RZ, (j,), param="new")
+        for j in range(n_perm):
+            if j % 4 == 3:
+                cb.add(W.X, (j,))
+            else:
+                cb.add(W.CNOT, (j, (j + 1 + layer) % n))
+    cb.add(W.H, (3,))
+    circ = cb.build()
+    theta = rng.uniform(-7, 7, circ["n_params"])
+    which = [int(p) for p in rng.choice(len(theta), 6, replace=False)]
+    _check(circ, theta, W.random_pauli_sum(rng, n, 12, 0.5, 4, 1.0), 3, which)
