@@ -226,8 +226,9 @@ sv_status sv_expval_paulisum(sv_ctx* ctx, const sv_ham* h, double* energy_out);
  * whole circuit in shared memory (with at most 8 MiB of checkpoints), unless the Hamiltonian has
  * so many groups that one SM takes longer for them than the passes do.  From 11 qubits, the
  * circuit's leading one-qubit gates on |ref> are a product state, and runs of RZ/CZ followed by
- * CNOT/X gates (below 14 qubits of eight gates or more) whole-state segments; segments need a third state buffer beside psi and lambda,
- * and where it cannot be had their gates run in passes on the two.  Layer checkpoints: sv_set_checkpoint_bytes.
+ * CNOT/X gates (below 14 qubits of eight gates or more) whole-state segments; segments need a
+ * third state buffer beside psi and lambda, and where it cannot be had their gates run in passes
+ * on the two.  Layer checkpoints: sv_set_checkpoint_bytes.
  * psi holds |ref> again afterwards.  energy_out:
  * host double; grad_out: host array of n_params (gates sharing a parameter are summed). */
 sv_status sv_adjoint_grad(sv_ctx* ctx, const sv_circuit* circuit, const double* theta,
